@@ -17,7 +17,9 @@
 //
 // Split-K: a phase's (tile, k-chunk) units are cut into equal contiguous ranges over its
 // CTAs; each CTA stores its fp32 partial tile with plain stores and the consuming phase
-// sums a tile's partials in CTA order (deterministic, no atomics).
+// sums a tile's partials in CTA order (deterministic, no atomics).  The gate / up projection is
+// column-owned instead: each CTA takes 16-feature units with the whole K and applies the SwiGLU
+// in its epilogue (no partials, no finalisation phase).
 //
 // Warp roles (352 threads, 11 warps):
 //   warp 0   W producer: bulk copies of pre-swizzled weight tiles and KV blocks
@@ -37,8 +39,8 @@
 //           than these products); the last split of a row to finish merges the splits
 //   3 O     att W_o^T -> partials           (a subset of the CTAs)
 //   4 FIN_O x += sum; x_g = x * g_mlp (bf16 hi/lo, blocked); per-row sum of squares
-//   5 GU    x_g W_gu^T -> partials          (gate / up interleaved in 64-row blocks)
-//   6 FIN_GU h = silu(r g) * (r u), r = 1/rms(x)  (bf16 hi/lo, blocked)
+//   6 GU    h = silu(r g) * (r u), g | u = x_g W_gu^T, r = 1/rms(x)  (bf16 hi/lo, blocked): gate
+//           and up rows alternate in blocks of 8, a CTA holds whole features (counter 5 is unused)
 //   7 DOWN  h W_down^T -> partials
 //   8 FIN_D x += sum; x_g = x * g_next; sum of squares
 // then lm_head over whole 256-token tiles fused with the Gumbel-max sampler: per (row, tile,
@@ -46,8 +48,8 @@
 //
 // Layouts (all chosen so that bulk copies land MMA operands in shared memory in the
 // 128-byte-swizzled K-major form the tensor core reads):
-//   weights       tiles of 256 rows (the last may have 128): [N/256][K/64][rows][64],
-//                 16-byte granule j of row r at granule j ^ (r % 8)
+//   weights       chunk-major [K/64][N][64], 16-byte granule j of row r at granule j ^ (r % 8):
+//                 any 8-aligned run of rows of a chunk is one contiguous copy
 //   activations   [K/64][2 rows16][64] bf16, 8-row groups alternating hi / lo parts, same swizzle
 //   KV cache      per (layer, slot, kv head, 128-position block): K as [d/64][128 pos][64 d]
 //                 and V transposed as [pos/64][128 d][64 pos], fp16, head dim padded to 128
@@ -71,8 +73,7 @@ constexpr int kMegaMaxSplits = 96;    // splits per row a merge handles (context
 constexpr int kPhasesPerLayer = 9;
 constexpr int kMaxCtaBlocks = 256;    // attention KV block ids a CTA keeps in shared memory
 // phases of a layer (counter index 1 + 9 l + phase)
-enum : int { kPhQKV = 0, kPhFinQ = 1, kPhAtt = 2, kPhO = 3, kPhFinO = 4, kPhGU = 5, kPhFinGU = 6, kPhDown = 7,
-             kPhFinD = 8 };
+enum : int { kPhQKV = 0, kPhFinQ = 1, kPhAtt = 2, kPhO = 3, kPhFinO = 4, kPhGU = 6, kPhDown = 7, kPhFinD = 8 };
 __device__ constexpr int kGemmPhases[4] = {kPhQKV, kPhO, kPhGU, kPhDown};
 constexpr int kSmallPhaseUnits = 2;   // QKV / O: units per participating CTA
 constexpr int kCntStride = 16;        // phase counters 128 bytes apart (one L2 line each)
@@ -158,7 +159,7 @@ struct MegaSmem {
     uint32_t tmem_base;
     int abort;
     int last_flag;
-    int rows, rows16, nx, nx_lg, n_items, att_span;  // nx = 2^nx_lg X stages
+    int rows, rows16, nx, nx_lg, xgroup, n_items, att_span;  // nx = 2^nx_lg X stages of xgroup chunks
     float rstd[128];
     // KV block ids: of this CTA's attention blocks (unit i's block j at ablk[aoff[i] + j]), and
     // of each row's current position (ablk_ok = 0: too many to hold, looked up in the table)
@@ -196,11 +197,8 @@ __host__ __device__ __forceinline__ int kv_v_off(int pp, int d) {
     const int c = pp & 63;
     return 32768 + (pp >> 6) * 16384 + d * 128 + ((((c >> 3) ^ (d & 7)) << 4) | ((c & 7) << 1));
 }
-// Byte offset of the (tile t, k-chunk kc) block of a blocked weight matrix [N][K].
-__host__ __device__ __forceinline__ int64_t wblk_off(int N, int K, int t, int kc) {
-    const int rows = (N - t * kTileN) < kTileN ? (N - t * kTileN) : kTileN;
-    return (int64_t)t * kTileN * K * 2 + (int64_t)kc * rows * 128;
-}
+// Byte offset of features col0.. (a multiple of 8) of k-chunk kc of a blocked weight matrix [N][K].
+__device__ __forceinline__ int64_t wblk_off(int N, int col0, int kc) { return ((int64_t)kc * N + col0) * 128; }
 
 // ------------------------------------------------------------------------------ waits
 // Bounded mbarrier wait that also gives up (returning false) once the CTA is aborting.
@@ -218,6 +216,12 @@ __device__ __forceinline__ bool mwait(uint64_t *bar, uint32_t parity, int *err, 
             }
         }
     }
+}
+
+// The same for a converged warp: one answer for all of its lanes.
+__device__ __forceinline__ bool mwait_warp(uint64_t *bar, uint32_t parity, int *err, volatile int *abort, uint64_t limit) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mwait(bar, parity, err, abort, limit));
 }
 
 // Spin until a phase counter reaches `target` (acquire loads);
@@ -244,6 +248,14 @@ __device__ __forceinline__ bool spin_counter(const unsigned long long *cnt, unsi
     }
 }
 
+// The same for a converged warp: one lane polls.
+__device__ __forceinline__ bool spin_counter_warp(const unsigned long long *cnt, unsigned long long target, int *err,
+                                                  volatile int *abort, uint64_t limit) {
+    bool r = false;
+    if (elect_one()) r = spin_counter(cnt, target, err, abort, limit);
+    return __any_sync(0xffffffffu, r);
+}
+
 // Counter value a wait on phase counter idx needs: every CTA of this launch arrived (the
 // test hook makes one counter's target unreachable, so its waits run into the time limit).
 __device__ __forceinline__ unsigned long long phase_target(const MegaParams &p, const MegaSmem &S, int idx) {
@@ -251,17 +263,27 @@ __device__ __forceinline__ unsigned long long phase_target(const MegaParams &p, 
 }
 
 // ------------------------------------------------------------------------------ phases
+// A GEMM phase: N output features, K inputs; unit widths below.  Two ways to split the work:
+//   K-split (own = false): (256-feature tile, 64-column chunk) units in equal contiguous ranges
+//     over the CTAs; each CTA stores its fp32 partial tiles and a finalisation phase sums them.
+//   column-owned (own = true): 16-feature units in equal contiguous ranges, each with the whole
+//     K, so that the CTA's epilogue applies the nonlinearity itself and no partials and no
+//     finalisation phase are needed.  More activation traffic (every CTA reads the whole
+//     operand) and fewer weight rows per MMA, but one phase barrier and one L2 round trip less.
 struct GemmPh {
     const uint8_t *w;
     int N, K, kch, T, Gp;
     const uint8_t *x;  // pair-blocked operand
     bool whole;  // whole tiles per CTA (lm_head: the argmax of a tile is finished in one CTA)
+    bool own;    // column-owned
 };
+constexpr int kOwnCols = 16;  // features per unit of a column-owned phase
 
 // GEMM phase k (kPhQKV, kPhO, kPhGU, kPhDown) of layer l; l == layers: lm_head.
 __device__ __forceinline__ GemmPh gemm_phase(const MegaParams &p, int l, int k) {
     GemmPh g;
     g.whole = false;
+    g.own = false;
     g.Gp = gridDim.x;
     if (l == p.layers) {
         g.w = p.w_lm; g.N = p.V; g.K = p.d; g.x = p.xg; g.whole = true;
@@ -270,37 +292,71 @@ __device__ __forceinline__ GemmPh gemm_phase(const MegaParams &p, int l, int k) 
     } else if (k == kPhO) {
         g.w = p.w_o + l * p.ls_o; g.N = p.d; g.K = p.H * p.hd; g.x = p.att; g.Gp = p.gp_o;
     } else if (k == kPhGU) {
-        g.w = p.w_gu + l * p.ls_gu; g.N = 2 * p.F; g.K = p.d; g.x = p.xg;
+        g.w = p.w_gu + l * p.ls_gu; g.N = 2 * p.F; g.K = p.d; g.x = p.xg; g.own = true;
     } else {
         g.w = p.w_down + l * p.ls_down; g.N = p.d; g.K = p.F; g.x = p.hm;
     }
     g.kch = g.K / 64;
-    g.T = (g.N + kTileN - 1) / kTileN;
+    g.T = g.own ? g.N / kOwnCols : (g.N + kTileN - 1) / kTileN;
     // at most one CTA per unit (tile for lm_head), so every participating CTA holds a
     // non-empty range and the CTAs between a tile's first and last owner all contributed
-    g.Gp = min(g.Gp, g.whole ? g.T : g.T * g.kch);
+    g.Gp = min(g.Gp, g.whole || g.own ? g.T : g.T * g.kch);
     return g;
 }
-__device__ __forceinline__ int tile_rows(const GemmPh &g, int t) { return min(kTileN, g.N - kTileN * t); }
 
-// This CTA's (tile, k-chunk) units: an equal contiguous share over the phase's CTAs, or
-// (lm_head) a share of whole tiles.
+// This CTA's share of a GEMM phase: units [u, u1) -- (tile, k-chunk) units, cut on whole tiles
+// for lm_head, or 16-feature units (column-owned) -- walked as segments, each one accumulator:
+// features [col0, col0 + n) x chunks [kc0, kc1).  A column-owned share wider than 256 features
+// is walked in equal passes.
 // (Unit counts stay below 2^31 / SMs for every supported shape: 32-bit products suffice.)
-__device__ __forceinline__ void gemm_range(const GemmPh &g, int64_t &u0, int64_t &u1) {
-    const int c = blockIdx.x;
-    if (c >= g.Gp) {
-        u0 = u1 = 0;
-        return;
+struct Seg {
+    int t, col0, n, kc0, kc1;
+    int cps;  // chunks per weight ring slot
+    __device__ __forceinline__ int entries() const { return (kc1 - kc0 + cps - 1) / cps; }
+};
+struct SegWalk {
+    int u, u1, pass;
+    __device__ __forceinline__ SegWalk(const GemmPh &g) {
+        const int c = blockIdx.x;
+        u = u1 = pass = 0;
+        if (c >= g.Gp) return;
+        if (g.own) {
+            u = c * g.T / g.Gp;
+            u1 = (c + 1) * g.T / g.Gp;
+            const int np = ((u1 - u) * kOwnCols + kTileN - 1) / kTileN;
+            pass = (u1 - u + np - 1) / np;
+        } else if (g.whole) {
+            u = c * g.T / g.Gp * g.kch;
+            u1 = (c + 1) * g.T / g.Gp * g.kch;
+        } else {
+            const int U = g.T * g.kch;
+            u = c * U / g.Gp;
+            u1 = (c + 1) * U / g.Gp;
+        }
     }
-    if (g.whole) {
-        u0 = (int64_t)(c * g.T / g.Gp) * g.kch;
-        u1 = (int64_t)((c + 1) * g.T / g.Gp) * g.kch;
-    } else {
-        const int U = g.T * g.kch;
-        u0 = c * U / g.Gp;
-        u1 = (c + 1) * U / g.Gp;
+    __device__ __forceinline__ bool next(const GemmPh &g, Seg &s) {
+        if (u >= u1) return false;
+        if (g.own) {
+            const int nu = min(pass, u1 - u);
+            s.t = 0;
+            s.col0 = u * kOwnCols;
+            s.n = nu * kOwnCols;
+            s.kc0 = 0;
+            s.kc1 = g.kch;
+            u += nu;
+        } else {
+            s.t = u / g.kch;
+            const int e = min(u1, (s.t + 1) * g.kch);
+            s.col0 = s.t * kTileN;
+            s.n = min(kTileN, g.N - s.col0);
+            s.kc0 = u - s.t * g.kch;
+            s.kc1 = s.kc0 + e - u;
+            u = e;
+        }
+        s.cps = s.n > 128 ? 1 : s.n > 64 ? 2 : s.n > 32 ? 4 : s.n > 16 ? 8 : 16;  // (a power of two)
+        return true;
     }
-}
+};
 // CTA owning unit u when U units are cut into Gp equal contiguous ranges.
 __device__ __forceinline__ int unit_owner(int u, int U, int Gp) {
     int c = u * Gp / U;
@@ -407,23 +463,29 @@ __device__ __forceinline__ void mega_w_producer(const MegaParams &p, MegaSmem &S
     uint32_t wi = 0;
     bool ok = true;
     auto acquire = [&](uint32_t i) -> bool {
-        return i < nws || mwait(&S.wempty[i % nws], ((i / nws) & 1) ^ 1, err, ab, lim);
+        return i < nws || mwait_warp(&S.wempty[i % nws], ((i / nws) & 1) ^ 1, err, ab, lim);
     };
     for (int l = 0; l <= p.layers && ok; ++l) {
         for (int gp = 0; gp < 4 && ok; ++gp) {
             if (l == p.layers && gp > 0) break;
             const int k = kGemmPhases[gp];
             const GemmPh g = gemm_phase(p, l, k);
-            int64_t u0, u1;
-            gemm_range(g, u0, u1);
-            for (int64_t u = u0; u < u1; ++u, ++wi) {
-                if (!acquire(wi)) { ok = false; break; }
-                const int s = (int)(wi % nws);
-                const int t = (int)(u / g.kch), kc = (int)(u - (int64_t)t * g.kch);
-                const uint32_t bytes = (uint32_t)tile_rows(g, t) * 128;
-                mbar_arrive_expect_tx(&S.wfull[s], bytes);
-                bulk_load(sW + (size_t)s * kSlotBytes, g.w + wblk_off(g.N, g.K, t, kc), bytes, &S.wfull[s], pol);
-                if (k == kPhGU && l == min(2, p.layers - 1) && u - u0 < 12) MEGA_DETAIL(16 + (int)(u - u0));
+            SegWalk walk(g);
+            Seg sg;
+            int nth = 0;
+            while (ok && walk.next(g, sg)) {
+                const uint32_t cb = (uint32_t)sg.n * 128;  // a chunk's bytes
+                for (int kc = sg.kc0; kc < sg.kc1; kc += sg.cps, ++wi, ++nth) {
+                    if (!acquire(wi)) { ok = false; break; }
+                    const int s = (int)(wi % nws), m = min(sg.cps, sg.kc1 - kc);
+                    if (elect_one()) {
+                        mbar_arrive_expect_tx(&S.wfull[s], (uint32_t)m * cb);
+                        for (int j = 0; j < m; ++j)
+                            bulk_load(sW + (size_t)s * kSlotBytes + (size_t)j * cb, g.w + wblk_off(g.N, sg.col0, kc + j),
+                                      cb, &S.wfull[s], pol);
+                    }
+                    if (k == kPhGU && l == min(2, p.layers - 1) && nth < 12) MEGA_DETAIL(16 + nth);
+                }
             }
             MEGA_STAMP(1 + kPhasesPerLayer * l + k, 2);
             if (k == 0 && l < p.layers && ok) {
@@ -448,7 +510,7 @@ __device__ __forceinline__ void mega_w_producer(const MegaParams &p, MegaSmem &S
                                 if (j >= (w ? nbb : ua.nb)) continue;
                                 if (kv == 0 && u.last && j == u.nb - 1 && !finq_seen) {
                                     const int fq = 1 + kPhasesPerLayer * l + kPhFinQ;
-                                    if (!spin_counter(&p.cnt[fq * kCntStride], phase_target(p, S, fq), err, ab, lim)) {
+                                    if (!spin_counter_warp(&p.cnt[fq * kCntStride], phase_target(p, S, fq), err, ab, lim)) {
                                         ok = false;
                                         break;
                                     }
@@ -459,7 +521,8 @@ __device__ __forceinline__ void mega_w_producer(const MegaParams &p, MegaSmem &S
                                 const int nj = min(kKVPos, u.n - j * kKVPos);
                                 if (!acquire(wi)) { ok = false; break; }
                                 const int s = (int)(wi % nws);
-                                if (kv == 0) {
+                                if (!elect_one()) {
+                                } else if (kv == 0) {
                                     const uint32_t kb = (uint32_t)(((nj + 7) & ~7) * 128);
                                     mbar_arrive_expect_tx(&S.wfull[s], p.hd > 64 ? 2 * kb : kb);
                                     bulk_load(sW + (size_t)s * kSlotBytes, blk, kb, &S.wfull[s], pol);
@@ -495,8 +558,9 @@ __device__ __forceinline__ void mega_x_producer(const MegaParams &p, MegaSmem &S
     const uint64_t lim = S.wait_ns;
     int *err = &p.c.v->err;
     const uint64_t pol = l2_policy_evict_last();
-    const int NX = S.nx, R16 = S.rows16, nxl = S.nx_lg;
-    const uint32_t stage = (uint32_t)R16 * 256;  // hi + lo parts of the live rows' groups
+    const int NX = S.nx, R16 = S.rows16, nxl = S.nx_lg, gx = S.xgroup;
+    const uint32_t chunk = (uint32_t)R16 * 256;  // hi + lo parts of the live rows' groups
+    const uint32_t stage = (uint32_t)gx * chunk;
     const int64_t chunk_stride = (int64_t)p.rows_cap16 * 256;
     uint32_t xi = 0;
     bool ok = true;
@@ -505,21 +569,26 @@ __device__ __forceinline__ void mega_x_producer(const MegaParams &p, MegaSmem &S
             if (l == p.layers && gp > 0) break;
             const int k = kGemmPhases[gp];
             const GemmPh g = gemm_phase(p, l, k);
-            int64_t u0, u1;
-            gemm_range(g, u0, u1);
-            if (u0 >= u1) continue;
-            // the phase this operand comes from (the one before it): FIN_D of l-1 / embedding,
-            // ATT, FIN_O, FIN_GU
-            const int dep = (l == p.layers || k == 0) ? kPhasesPerLayer * l : 1 + kPhasesPerLayer * l + k - 1;
-            if (!spin_counter(&p.cnt[dep * kCntStride], phase_target(p, S, dep), err, ab, lim)) { ok = false; break; }
+            SegWalk walk(g);
+            if (walk.u >= walk.u1) continue;
+            // the phase this operand comes from: FIN_D of l-1 / embedding, ATT, FIN_O, GU
+            const int dep = (l == p.layers || k == kPhQKV) ? kPhasesPerLayer * l
+                                                           : 1 + kPhasesPerLayer * l + (k == kPhGU ? kPhFinO : k - 1);
+            if (!spin_counter_warp(&p.cnt[dep * kCntStride], phase_target(p, S, dep), err, ab, lim)) { ok = false; break; }
             MEGA_STAMP(1 + kPhasesPerLayer * l + k, 1);
             fence_proxy_async_global();
-            for (int64_t u = u0; u < u1; ++u, ++xi) {
-                const int s = (int)(xi & (uint32_t)(NX - 1));
-                if (xi >= (uint32_t)NX && !mwait(&S.xempty[s], ((xi >> nxl) & 1) ^ 1, err, ab, lim)) { ok = false; break; }
-                const int kc = (int)(u % g.kch);
-                mbar_arrive_expect_tx(&S.xfull[s], stage);
-                bulk_load(sX + (size_t)s * stage, g.x + kc * chunk_stride, stage, &S.xfull[s], pol);
+            Seg sg;
+            while (ok && walk.next(g, sg)) {
+                for (int kc = sg.kc0; kc < sg.kc1; kc += gx, ++xi) {
+                    const int s = (int)(xi & (uint32_t)(NX - 1)), m = min(gx, sg.kc1 - kc);
+                    if (xi >= (uint32_t)NX && !mwait_warp(&S.xempty[s], ((xi >> nxl) & 1) ^ 1, err, ab, lim)) { ok = false; break; }
+                    if (elect_one()) {
+                        mbar_arrive_expect_tx(&S.xfull[s], (uint32_t)m * chunk);
+                        for (int j = 0; j < m; ++j)
+                            bulk_load(sX + (size_t)s * stage + (size_t)j * chunk, g.x + (kc + j) * chunk_stride, chunk,
+                                      &S.xfull[s], pol);
+                    }
+                }
             }
         }
     }
@@ -537,8 +606,8 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
     volatile int *ab = &S.abort;
     const uint64_t lim = S.wait_ns;
     int *err = &p.c.v->err;
-    const int NX = S.nx, R16 = S.rows16, nxl = S.nx_lg;
-    const uint32_t stage = (uint32_t)R16 * 256;
+    const int NX = S.nx, R16 = S.rows16, nxl = S.nx_lg, gx = S.xgroup;
+    const uint32_t chunk = (uint32_t)R16 * 256, stage = (uint32_t)gx * chunk;
     // at most 64 live rows: one MMA per k-step over the stacked hi / lo groups (M = 2 R16
     // rounded up to 64 or 128: the rows past the stage only feed accumulator rows nobody
     // reads); more: the hi and the lo groups as two 128-row operands into one accumulator
@@ -548,46 +617,63 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
     bool ok = true;
     constexpr uint32_t nws = kWSlots;
     auto wslot = [&](uint32_t i) -> uint32_t { return smem_u32(sW + (size_t)(i % nws) * kSlotBytes); };
-    auto wwait = [&](uint32_t i) -> bool { return mwait(&S.wfull[i % nws], (i / nws) & 1, err, ab, lim); };
-    auto gemm = [&](const GemmPh &g, int64_t u0, int64_t u1, bool det) {
-        const int64_t ub = u0;
-        for (int64_t u = u0; u < u1 && ok;) {
-            const int t = (int)(u / g.kch);
-            const int64_t e = min(u1, (int64_t)(t + 1) * g.kch);
-            const int a = tseg & 1;  // tiles alternate between two accumulators (epilogue overlaps)
+    auto wwait = [&](uint32_t i) -> bool { return mwait_warp(&S.wfull[i % nws], (i / nws) & 1, err, ab, lim); };
+    auto gemm = [&](const GemmPh &g, bool det) {
+        SegWalk walk(g);
+        Seg sg;
+        int nth = 0;  // ring entry of the phase
+        while (ok && walk.next(g, sg)) {
+            const int a = tseg & 1;  // segments alternate between two accumulators (epilogue overlaps)
             const int use_a = a ? use1 : use0;
-            if (use_a >= 1 && !mwait(&S.acc_empty[a], (use_a - 1) & 1, err, ab, lim)) { ok = false; break; }
+            if (use_a >= 1 && !mwait_warp(&S.acc_empty[a], (use_a - 1) & 1, err, ab, lim)) { ok = false; break; }
             tc_fence_after();
             const uint32_t d = tmem + (uint32_t)(a * kTileN);
-            const uint32_t idg = idesc_bf16_f32(R16 <= 32 ? 64u : 128u, (uint32_t)tile_rows(g, t));
-            bool first = true;
-            for (; u < e; ++u, ++wi, ++xi) {
+            const uint32_t idg = idesc_bf16_f32(R16 <= 32 ? 64u : 128u, (uint32_t)sg.n);
+            const uint32_t cb = (uint32_t)sg.n * 128;
+            // chunks go in groups that stay within one weight slot and one activation stage, so a
+            // group's MMAs issue back to back: one pair of waits and commits per group
+            const int grp = min(sg.cps, gx);
+            int wj = 0, xj = 0;  // chunk within the weight slot / the activation stage
+            for (int kc = sg.kc0; kc < sg.kc1; kc += grp) {
+                const bool dj = det && wj == 0 && nth < 12;
+                if (wj == 0 && !wwait(wi)) { ok = false; break; }
+                if (dj) MEGA_DETAIL(28 + nth);
                 const int xs = (int)(xi & (uint32_t)(NX - 1));
-                const bool dj = det && u - ub < 12;
-                if (!wwait(wi)) { ok = false; break; }
-                if (dj) MEGA_DETAIL(28 + (int)(u - ub));
-                if (!mwait(&S.xfull[xs], (xi >> nxl) & 1, err, ab, lim)) { ok = false; break; }
-                if (dj) MEGA_DETAIL(40 + (int)(u - ub));
+                if (xj == 0 && !mwait_warp(&S.xfull[xs], (xi >> nxl) & 1, err, ab, lim)) { ok = false; break; }
+                if (dj) MEGA_DETAIL(40 + nth);
                 tc_fence_after();
-                const uint32_t aw = wslot(wi), ax = smem_u32(sX + (size_t)xs * stage);
+                const int m = min(grp, sg.kc1 - kc);
+                const uint32_t aw = wslot(wi) + (uint32_t)wj * cb;
+                const uint32_t ax = smem_u32(sX) + (uint32_t)xs * stage + (uint32_t)xj * chunk;
+                const bool end = kc + m == sg.kc1;
+                const bool wlast = end || wj + grp == sg.cps, xlast = end || xj + grp == gx;
+                if (elect_one()) {
+                    for (int j = 0; j < m; ++j) {
 #pragma unroll
-                for (int kk = 0; kk < 4; ++kk) {
-                    const uint64_t bd = sdesc_kmajor_sw128(aw + kk * 32);
-                    const uint32_t acc = (first && kk == 0) ? 0u : 1u;
-                    if (stacked) {
-                        tc_mma_bf16(d, sdesc_kmajor_sw128(ax + kk * 32), bd, idg, acc);
-                    } else {
-                        tc_mma_bf16(d, sdesc_kmajor_sw128(ax + kk * 32, 2048), bd, idg, acc);
-                        tc_mma_bf16(d, sdesc_kmajor_sw128(ax + kLoOff + kk * 32, 2048), bd, idg, 1u);
+                        for (int kk = 0; kk < 4; ++kk) {
+                            const uint64_t bd = sdesc_kmajor_sw128(aw + j * cb + kk * 32);
+                            const uint32_t acc = (kc == sg.kc0 && j == 0 && kk == 0) ? 0u : 1u;
+                            if (stacked) {
+                                tc_mma_bf16(d, sdesc_kmajor_sw128(ax + j * chunk + kk * 32), bd, idg, acc);
+                            } else {
+                                tc_mma_bf16(d, sdesc_kmajor_sw128(ax + j * chunk + kk * 32, 2048), bd, idg, acc);
+                                tc_mma_bf16(d, sdesc_kmajor_sw128(ax + j * chunk + kLoOff + kk * 32, 2048), bd, idg, 1u);
+                            }
+                        }
                     }
+                    if (xlast) tc_commit(&S.xempty[xs]);
+                    if (wlast) tc_commit(&S.wempty[wi % nws]);
                 }
-                first = false;
-                tc_commit(&S.wempty[wi % nws]);
-                tc_commit(&S.xempty[xs]);
-                if (dj) MEGA_DETAIL(52 + (int)(u - ub));
+                __syncwarp();
+                if (wlast && dj) MEGA_DETAIL(52 + nth);
+                wj = wlast ? 0 : wj + grp;
+                xj = xlast ? 0 : xj + grp;
+                wi += wlast ? 1 : 0;
+                nth += wlast ? 1 : 0;
+                xi += xlast ? 1 : 0;
             }
             if (!ok) break;
-            tc_commit(&S.acc_full[a]);
+            if (elect_one()) tc_commit(&S.acc_full[a]);
             if (a) ++use1; else ++use0;
             ++tseg;
         }
@@ -609,7 +695,7 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
                     for (int x = 0; x < 2; ++x) {
                         if (j >= (x ? nbb : nba)) continue;
                         if (!wwait(wi)) return false;
-                        mbar_arrive(&S.kvready[(gi + i + x) & 1][wi % nws]);
+                        if (elect_one()) mbar_arrive(&S.kvready[(gi + i + x) & 1][wi % nws]);
                         ++wi;
                     }
         }
@@ -621,9 +707,7 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
             if (l == p.layers && gp > 0) break;
             const int k = kGemmPhases[gp];
             const GemmPh g = gemm_phase(p, l, k);
-            int64_t u0, u1;
-            gemm_range(g, u0, u1);
-            gemm(g, u0, u1, k == kPhGU && l == min(2, p.layers - 1));
+            gemm(g, k == kPhGU && l == min(2, p.layers - 1));
             MEGA_STAMP(1 + kPhasesPerLayer * l + k, 3);
             if (k == 0 && l < p.layers && ok) {
                 int64_t a0, a1;
@@ -634,7 +718,7 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
         }
     }
     // every MMA issued has retired before tensor memory is released
-    tc_commit(&S.drain);
+    if (elect_one()) tc_commit(&S.drain);
     mbar_wait(&S.drain, 0, err);
 }
 
@@ -646,6 +730,12 @@ __device__ __forceinline__ void store_hilo(uint8_t *base, int64_t off, float v) 
     *reinterpret_cast<uint16_t *>(base + off + kLoOff) = l;
 }
 
+
+// Eight bf16 values as one 16-byte granule.
+__device__ __forceinline__ uint4 pack8(const uint16_t (&v)[8]) {
+    return make_uint4((uint32_t)v[0] | ((uint32_t)v[1] << 16), (uint32_t)v[2] | ((uint32_t)v[3] << 16),
+                      (uint32_t)v[4] | ((uint32_t)v[5] << 16), (uint32_t)v[6] | ((uint32_t)v[7] << 16));
+}
 
 __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, uint8_t *sW, uint8_t *sQ, uint8_t *sP,
                                              uint32_t tmem) {
@@ -672,6 +762,10 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
     const int my_row = R16 <= 32   ? ((lane & 0x18) == 0 ? quarter * 8 + lane : 1 << 20)
                        : pair      ? ((lane & 8) == 0 ? quarter * 16 + 8 * (lane >> 4) + (lane & 7) : 1 << 20)
                                    : quarter * 32 + lane;
+    // the same for both lanes of a pair (lanes i and i ^ 8), past the batch for lanes of no row
+    const int my_row_any = R16 <= 32 ? ((lane & 16) == 0 ? quarter * 8 + (lane & 7) : 1 << 20)
+                           : pair    ? quarter * 16 + 8 * (lane >> 4) + (lane & 7)
+                                     : quarter * 32 + lane;
     const bool quarter_live = (R16 <= 32 ? quarter * 8 : pair ? quarter * 16 : quarter * 32) < R;
     uint32_t wring = 0;  // W ring entries of the phases before the current one (the producer's count)
     uint32_t kvpar = 0;  // per ring slot (bit s): parity of this warp group's next kvready wait
@@ -713,14 +807,15 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
         named_bar_sync(1, kMegaCThreads);
     };
     // this CTA's partial tiles: row my_row, columns [128 half, +128) of the tile
-    auto gemm_epi = [&](const GemmPh &g, int64_t u0, int64_t u1) {
-        for (int64_t u = u0; u < u1;) {
-            const int t = (int)(u / g.kch);
-            u = min(u1, (int64_t)(t + 1) * g.kch);
-            const int a = tseg & 1;
+    auto gemm_epi = [&](const GemmPh &g) {
+        SegWalk walk(g);
+        Seg sg;
+        while (walk.next(g, sg)) {
+            wring += (uint32_t)sg.entries();
+            const int t = sg.t, a = tseg & 1;
             mwait(&S.acc_full[a], (a ? cuse1 : cuse0) & 1, err, ab, lim);
             tc_fence_after();
-            const int rows_t = tile_rows(g, t);
+            const int rows_t = sg.n;
             if (quarter_live && half * 128 < rows_t) {
                 float *dst = p.gpart + ((int64_t)(cta + t) * p.rows_cap + (my_row < R ? my_row : 0)) * kTileN + half * 128;
 #pragma unroll 1
@@ -815,13 +910,10 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
 
     for (int l = 0; l < p.layers; ++l) {
         const int base = 1 + kPhasesPerLayer * l;
-        int64_t u0, u1;
         const GemmPh gq = gemm_phase(p, l, kPhQKV), go = gemm_phase(p, l, kPhO), gu = gemm_phase(p, l, kPhGU),
                      gdn = gemm_phase(p, l, kPhDown);
         // ------------------------------------------------------------ QKV
-        gemm_range(gq, u0, u1);
-        wring += (uint32_t)(u1 - u0);
-        gemm_epi(gq, u0, u1);
+        gemm_epi(gq);
         arrive(base + kPhQKV, false);
         // ------------------------------------------------------------ q, k, v (once per row)
         {
@@ -1235,9 +1327,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
 #undef DETAIL
         }
         // ------------------------------------------------------------ O projection
-        gemm_range(go, u0, u1);
-        wring += (uint32_t)(u1 - u0);
-        gemm_epi(go, u0, u1);
+        gemm_epi(go);
         arrive(base + kPhO, false);
         // ------------------------------------------------------------ residual, MLP norm input
         wait_phase(base + kPhO);
@@ -1247,78 +1337,59 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
         arrive(base + kPhFinO, true);
         if (l == min(2, p.layers - 1) && ctid == 0) MEGA_DETAIL(12);
         // ------------------------------------------------------------ gate / up
-        gemm_range(gu, u0, u1);
-        wring += (uint32_t)(u1 - u0);
-        gemm_epi(gu, u0, u1);
-        arrive(base + kPhGU, false);
-        // ------------------------------------------------------------ SwiGLU
+        // h = silu(r g) * (r u) straight from the accumulator: this CTA's features hold the whole
+        // K, in 16-feature units of 8 gate then 8 up features (the two warp halves take alternate
+        // pairs of units).  The row's 1/rms is read while the MMAs run.
         {
-            wait_phase(base + kPhGU);
-            const int fb = p.F / 128;
-            // unit = (row, 128 features of h) = one 256-row tile of the gate/up outputs; lane:
-            // 4 features, gate at tile column c, up at c + 64 (c = 4 lane, or 128 + 4 lane - 64
-            // for the tile's second 64 features).  A warp takes two units per pass with every
-            // partial load in flight before the sums (in CTA order).
-            const int c0 = (lane < 16) ? 4 * lane : 128 + 4 * lane - 64;
-            for (int u = gw; u < R * fb; u += 2 * nw) {
-                float4 gs[2], us[2];
-                int rr[2], tt[2];
-                float sq[2];  // the rows' sum-of-squares partials, loaded with the gate / up partials
+            wait_phase(base + kPhFinO);
+            load_rstd(p.ssqM);
+            const float rs = my_row_any < R ? S.rstd[my_row_any] : 0.f;
+            SegWalk walk(gu);
+            Seg sg;
+            while (walk.next(gu, sg)) {
+                wring += (uint32_t)sg.entries();
+                const int a = tseg & 1, nu = sg.n / kOwnCols;
+                mwait(&S.acc_full[a], (a ? cuse1 : cuse0) & 1, err, ab, lim);
+                tc_fence_after();
+                if (quarter_live) {
+#pragma unroll 1
+                    for (int un = 2 * half; un < nu; un += 4) {
+                        float v[32];
+                        tmem_ld_32x32b_x32(tmem + lane_base + (uint32_t)(a * kTileN + un * kOwnCols), v);
+                        if (pair) {  // hi + lo accumulators; then each lane of the pair keeps one unit
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const int uq = u + q * nw;
-                    gs[q] = us[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    rr[q] = -1;
-                    tt[q] = 0;
-                    sq[q] = 0.f;
-                    if (uq >= R * fb) continue;
-                    const int r = uq / fb, t = uq - r * fb;
-                    rr[q] = r;
-                    tt[q] = t;
-                    sq[q] = lane < d / 64 ? __ldcg(&p.ssqM[(int64_t)lane * p.rows_cap + r]) : 0.f;
-                    int ca, cb;
-                    tile_ctas(gu, t, ca, cb);
-                    for (int cq = ca; cq <= cb; cq += 4) {
-                        float4 a4[4], b4[4];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const bool ok = cq + k <= cb;
-                            const float *src = p.gpart + ((int64_t)(cq + k + t) * p.rows_cap + r) * kTileN + c0;
-                            a4[k] = ok ? __ldcg(reinterpret_cast<const float4 *>(src)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                            b4[k] = ok ? __ldcg(reinterpret_cast<const float4 *>(src + 64)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                            for (int e = 0; e < 32; ++e) v[e] += __shfl_xor_sync(0xffffffffu, v[e], 8);
                         }
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            gs[q].x += a4[k].x; gs[q].y += a4[k].y; gs[q].z += a4[k].z; gs[q].w += a4[k].w;
-                            us[q].x += b4[k].x; us[q].y += b4[k].y; us[q].z += b4[k].z; us[q].w += b4[k].w;
+                        for (int q = 0; q < 2; ++q) {
+                            if (pair ? q > 0 : false) break;
+                            const bool second = pair ? (lane & 8) != 0 : q == 1;
+                            if (my_row_any < R && un + (second ? 1 : 0) < nu) {
+                                uint16_t hh[8], hl[8];
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) {
+                                    const float gv = (second ? v[16 + e] : v[e]) * rs;
+                                    const float uv = (second ? v[24 + e] : v[8 + e]) * rs;
+                                    split_bf16(gv / (1.0f + expf(-gv)) * uv, hh[e], hl[e]);
+                                }
+                                const int f = sg.col0 / 2 + (un + (second ? 1 : 0)) * 8;
+                                const int64_t off = xblk_off(my_row_any, f, R16c);
+                                *reinterpret_cast<uint4 *>(p.hm + off) = pack8(hh);
+                                *reinterpret_cast<uint4 *>(p.hm + off + kLoOff) = pack8(hl);
+                            }
                         }
                     }
                 }
-                float rsq[2];
-#pragma unroll
-                for (int q = 0; q < 2; ++q) rsq[q] = rsqrtf(warp_sum(sq[q]) / (float)d + p.eps);
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    if (rr[q] < 0) continue;
-                    const float rs = rsq[q];
-                    const float gv[4] = {gs[q].x * rs, gs[q].y * rs, gs[q].z * rs, gs[q].w * rs};
-                    const float uv[4] = {us[q].x * rs, us[q].y * rs, us[q].z * rs, us[q].w * rs};
-                    uint16_t hh[4], hl[4];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) split_bf16(gv[e] / (1.0f + expf(-gv[e])) * uv[e], hh[e], hl[e]);
-                    const int64_t off = xblk_off(rr[q], tt[q] * 128 + 4 * lane, R16c);
-                    *reinterpret_cast<uint2 *>(p.hm + off) =
-                        make_uint2((uint32_t)hh[0] | ((uint32_t)hh[1] << 16), (uint32_t)hh[2] | ((uint32_t)hh[3] << 16));
-                    *reinterpret_cast<uint2 *>(p.hm + off + kLoOff) =
-                        make_uint2((uint32_t)hl[0] | ((uint32_t)hl[1] << 16), (uint32_t)hl[2] | ((uint32_t)hl[3] << 16));
-                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&S.acc_empty[a]);
+                if (a) ++cuse1; else ++cuse0;
+                ++tseg;
             }
-            arrive(base + kPhFinGU, true);
+            arrive(base + kPhGU, true);
         }
         // ------------------------------------------------------------ down
-        gemm_range(gdn, u0, u1);
-        wring += (uint32_t)(u1 - u0);
-        gemm_epi(gdn, u0, u1);
+        gemm_epi(gdn);
         arrive(base + kPhDown, false);
         // ------------------------------------------------------------ residual, next norm input
         wait_phase(base + kPhDown);
@@ -1338,20 +1409,20 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
         wait_phase(kPhasesPerLayer * p.layers);
         load_rstd(p.ssqA);
         const GemmPh g = gemm_phase(p, p.layers, 0);
-        int64_t u0, u1;
-        gemm_range(g, u0, u1);
         const bool act = my_row < R;
         const float rs = act ? S.rstd[my_row] : 0.f;
         const uint64_t seed = act ? __ldg(&p.c.row_seed[my_row]) : 0ull;
         const int nparts = 2 * g.T;
         float best = -INFINITY;  // running over this thread's tiles (its row and half)
         int bi = 0x7fffffff;
-        for (int64_t u = u0; u < u1; u += g.kch) {
-            const int t = (int)(u / g.kch);
+        SegWalk walk(g);
+        Seg sg;
+        while (walk.next(g, sg)) {
+            const int t = sg.t;
             const int a = tseg & 1;
             mwait(&S.acc_full[a], (a ? cuse1 : cuse0) & 1, err, ab, lim);
             tc_fence_after();
-            if (quarter_live && half * 128 < tile_rows(g, t)) {
+            if (quarter_live && half * 128 < sg.n) {
                 const int n0 = t * kTileN + half * 128;
                 float *dst = p.logits + (int64_t)(act ? my_row : 0) * p.V + n0;
                 const float best0 = best;  // the maximum over this thread's earlier tiles
@@ -1446,9 +1517,11 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
         const int rows = max(0, min(live, p.rows_cap));
         S.rows = rows;
         S.rows16 = max(16, (rows + 15) & ~15);
-        // X stages: the largest power of two (at most kMaxXStages) that fits after the W slots
+        // X stages of up to 16 KB: 4, 2 or 1 k-chunks each (fewer waits and commits per MMA), and
+        // the largest power of two of them (at most kMaxXStages) that fits after the W slots
         {
-            const int fit = min(kMaxXStages, (kRingBytes - kWSlots * kSlotBytes) / (S.rows16 * 256));
+            S.xgroup = S.rows16 <= 16 ? 4 : S.rows16 <= 32 ? 2 : 1;
+            const int fit = min(kMaxXStages, (kRingBytes - kWSlots * kSlotBytes) / (S.rows16 * 256 * S.xgroup));
             int lg = 0;
             while ((2 << lg) <= fit) ++lg;
             S.nx = 1 << lg;
@@ -1461,6 +1534,8 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
         const int64_t wl = p.c.kc->wait_ns;
         S.wait_ns = wl > 0 ? (uint64_t)wl : kWaitLimitNs;
         S.stall_idx = p.c.kc->stall_plus1 - 1;
+        // gate / up and its SwiGLU are one phase on the second of their two counters
+        if (S.stall_idx > 0 && (S.stall_idx - 1) % kPhasesPerLayer == kPhGU - 1) ++S.stall_idx;
         S.p_headroom = p.c.kc->eager_softmax ? 0.f : kSoftmaxHeadroom;
         S.abort = (*(volatile int *)&V->err & ERR_WAIT_TIMEOUT) != 0;
         S.last_flag = 0;
@@ -1481,11 +1556,11 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
     if (run) {
         if (warp == 0) {
             fill_att_blocks(p, S, lane);
-            if (lane == 0) mega_w_producer(p, S, sW);
+            mega_w_producer(p, S, sW);
         } else if (warp == 1) {
-            if (lane == 0) mega_mma(p, S, sW, sX, sQ, sP, tmem);
+            mega_mma(p, S, sW, sX, sQ, sP, tmem);
         } else if (warp == 2) {
-            if (lane == 0) mega_x_producer(p, S, sX);
+            mega_x_producer(p, S, sX);
         } else {
             mega_compute(p, S, sW, sQ, sP, tmem);
         }
@@ -1505,17 +1580,16 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
 }
 
 // ------------------------------------------------------------------------------ layout kernels
-// Row-major W [N][K] (bf16) -> blocked tiles of 256 rows (the last may have fewer): block
-// (t, kc) holds rows [256 t, ..) x columns [64 kc, +64), 16-byte granule j of row r stored at
-// granule j ^ (r % 8).  N must be a multiple of 128 and K of 64.
+// Row-major W [N][K] (bf16) -> chunk-major blocks: k-chunk kc holds its 64 columns of every row
+// (128 bytes a row), 16-byte granule j of row r stored at granule j ^ (r % 8), so any run of rows
+// of a chunk that starts at a multiple of 8 is one contiguous piece.  K must be a multiple of 64.
 static __global__ void block_weights_kernel(const uint16_t *src, uint8_t *dst, int N, int K) {
     const int gpr = K / 8;
     const int64_t total = (int64_t)N * gpr;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int n = (int)(e / gpr), j = (int)(e - (int64_t)n * gpr);
-        const int t = n / kTileN, r = n - t * kTileN;
         const uint4 v = *reinterpret_cast<const uint4 *>(src + (int64_t)n * K + (int64_t)j * 8);
-        *reinterpret_cast<uint4 *>(dst + wblk_off(N, K, t, j >> 3) + (int64_t)r * 128 + (((j & 7) ^ (r & 7)) << 4)) = v;
+        *reinterpret_cast<uint4 *>(dst + wblk_off(N, n, j >> 3) + (((j & 7) ^ (n & 7)) << 4)) = v;
     }
 }
 

@@ -1,5 +1,5 @@
-// Host engine behind include/sara.h: device memory layout, weight packing (pre-swizzled
-// 16 KB tiles), the step graph (a conditional WHILE loop whose body is controller ->
+// Host engine behind include/sara.h: device memory layout, weight packing (pre-swizzled,
+// chunk-major), the step graph (a conditional WHILE loop whose body is controller ->
 // [round start: prefill + prompt-KV fan-out] -> persistent decode-step kernel ->
 // sampling/bookkeeping), and the C ABI.
 #include <cuda.h>
@@ -65,7 +65,7 @@ struct sara_handle {
     bool use_graph = true, use_pdl = true;
     std::string err;
     DeviceBuf mem;
-    // weights: embedding row-major, projections as pre-swizzled 16 KB tiles (all layers
+    // weights: embedding row-major, projections chunk-major, pre-swizzled (all layers
     // of one kind contiguous), norms [layers][d]
     uint16_t *embed = nullptr, *final_norm = nullptr, *norm_attn = nullptr, *norm_mlp = nullptr;
     uint8_t *wb_qkv = nullptr, *wb_o = nullptr, *wb_gu = nullptr, *wb_down = nullptr, *wb_lm = nullptr;
@@ -489,7 +489,7 @@ void run_host_loop(sara_handle &h, int schedule) {
 
 // ------------------------------------------------------------------------ weights
 
-// Copy a row-major bf16 matrix [N][K] (host or device) into blocked 16 KB tiles at dst,
+// Copy a row-major bf16 matrix [N][K] (host or device) into chunk-major blocks at dst,
 // through the device staging buffer tmp.
 void block_matrix(cudaStream_t s, const void *src, bool on_device, uint16_t *tmp, uint8_t *dst, int N, int K) {
     CK(cudaMemcpyAsync(tmp, src, (size_t)N * K * 2, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
@@ -541,11 +541,11 @@ void load_weights(sara_handle &h, const sara_weights *w) {
             launch(s, false, dim3(1024), dim3(256), 0, block_weights_kernel, (const uint16_t *)tmp,
                    h.wb_qkv + l * h.ls_qkv, nqkv, d);
             block_matrix(s, w->wo[l], dev, tmp, h.wb_o + l * h.ls_o, d, H * hd);
-            // gate/up interleaved in blocks of 64 rows: [g 0..63, u 0..63, g 64..127, u 64..127, ...]
-            CK(cudaMemcpy2DAsync(tmp, (size_t)128 * d * 2, w->wgate[l], (size_t)64 * d * 2, (size_t)64 * d * 2, F / 64,
-                                 kind, s));
-            CK(cudaMemcpy2DAsync(tmp + (size_t)64 * d, (size_t)128 * d * 2, w->wup[l], (size_t)64 * d * 2,
-                                 (size_t)64 * d * 2, F / 64, kind, s));
+            // gate/up interleaved in blocks of 8 rows: [g 0..7, u 0..7, g 8..15, u 8..15, ...]
+            CK(cudaMemcpy2DAsync(tmp, (size_t)16 * d * 2, w->wgate[l], (size_t)8 * d * 2, (size_t)8 * d * 2, F / 8, kind,
+                                 s));
+            CK(cudaMemcpy2DAsync(tmp + (size_t)8 * d, (size_t)16 * d * 2, w->wup[l], (size_t)8 * d * 2,
+                                 (size_t)8 * d * 2, F / 8, kind, s));
             launch(s, false, dim3(1024), dim3(256), 0, block_weights_kernel, (const uint16_t *)tmp,
                    h.wb_gu + l * h.ls_gu, 2 * F, d);
             block_matrix(s, w->wdown[l], dev, tmp, h.wb_down + l * h.ls_down, d, F);
@@ -590,7 +590,7 @@ void alloc_decode(sara_handle &h) {
     h.ssqA = h.mem.alloc<float>((size_t)(d / 64) * S);
     h.ssqM = h.mem.alloc<float>((size_t)(d / 64) * S);
     // partial tiles: one segment per (CTA, tile) pair of a phase, at most CTAs + tiles - 1
-    const int tmax = std::max({nqkv, d, 2 * F}) / kTileN + 1;
+    const int tmax = std::max(nqkv, d) / kTileN + 1;
     h.gpart = h.mem.alloc<float>((size_t)(h.sms + tmax) * S * kTileN, false);
     h.qkv16 = h.mem.alloc<uint16_t>((size_t)S * nqkv, false);
     // the QKV and O projections are spread over few CTAs (each about one ring of weights)
@@ -1009,10 +1009,10 @@ void print_stamps(sara_handle &h, int rows, int ctx) {
     };
     const int NPH = 1 + kPhasesPerLayer * L + 1;
     std::vector<double> done(NPH);
-    for (int ph = 0; ph < NPH; ++ph) done[ph] = stat(ph, 0, true);
+    for (int ph = 0; ph < NPH; ++ph) done[ph] = std::max(stat(ph, 0, true), ph ? done[ph - 1] : 0.0);
     fprintf(stderr, "rows %d ctx %d: start->embed done %.2f us, lm_head done at %.2f us\n", rows, ctx, done[0],
             done[NPH - 1]);
-    const char *names[kPhasesPerLayer] = {"QKV", "FIN_Q", "ATT", "O", "FIN_O", "GU", "FIN_GU", "DOWN", "FIN_D"};
+    const char *names[kPhasesPerLayer] = {"QKV", "FIN_Q", "ATT", "O", "FIN_O", "-", "GU", "DOWN", "FIN_D"};
     const int l0 = L > 4 ? 2 : 0, l1 = L > 4 ? L - 2 : L;
     for (int k = 0; k < kPhasesPerLayer; ++k) {
         double span = 0, obs = 0, wahead = 0, mma = 0;

@@ -31,7 +31,7 @@ enum EpiKind : int {
     EPI_F32 = 0,     // Y fp32 [rows][ld]
     EPI_QKV = 1,     // RMSNorm scale, RoPE on q/k, q -> q_out (fp16), k/v -> KV cache (fp16)
     EPI_RESID = 2,   // x += Y; xg = x * g_next as a bf16 hi/lo pair; per-tile sum of squares of x
-    EPI_SWIGLU = 3,  // RMSNorm scale; tile = 64 gate rows + 64 up rows -> h = silu(g) * u (hi/lo)
+    EPI_SWIGLU = 3,  // RMSNorm scale; rows alternate 8 gate, 8 up -> h = silu(g) * u (hi/lo)
 };
 
 constexpr int kGemmThreads = 192;
@@ -50,7 +50,7 @@ struct GemmParams {
     const int *rows_dev;       // device count of valid rows (nullptr -> rows_fixed)
     int rows_fixed;
     int decode;                // 1: a single row tile, weights prefetched before the PDL wait
-    const uint8_t *w_blk;      // non-null: W stored as pre-swizzled 256-row tiles (bulk copies, wblk128_off)
+    const uint8_t *w_blk;      // non-null: W stored chunk-major, pre-swizzled (bulk copies, wblk128_off)
     int has_lo;                // 1: the activation's lo part (second tensor map) is multiplied too
     unsigned long long *ws_acc;  // [gridDim.x][kTileR * kTileM] fixed-point tile sums, zero between launches
     int *ws_cnt;               // [tiles] arrival counters, zero between launches
@@ -113,13 +113,10 @@ __device__ __forceinline__ int cta_of_unit(int64_t u, int64_t U, int G) {
 #endif
 __device__ __forceinline__ int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
 
-// Byte offset of the 128 x 64 weight sub-tile (m_tile, kc) of a weight [Nout][K] stored as
-// pre-swizzled tiles of 256 rows (the last may have 128): tile t = m_tile / 2 holds, for
-// each k-chunk, its rows at a 128-byte pitch, so the two 128-row halves are 16 KB apart.
-__device__ __forceinline__ int64_t wblk128_off(int Nout, int K, int m_tile, int kc) {
-    const int t = m_tile >> 1;
-    const int rows = min(256, Nout - 256 * t);
-    return (int64_t)t * 256 * K * 2 + (int64_t)kc * rows * 128 + (m_tile & 1) * 16384;
+// Byte offset of the 128 x 64 weight sub-tile (m_tile, kc) of a weight [Nout][K] stored
+// chunk-major and pre-swizzled: chunk kc holds its 64 columns of every row, 128 bytes a row.
+__device__ __forceinline__ int64_t wblk128_off(int Nout, int m_tile, int kc) {
+    return ((int64_t)kc * Nout + m_tile * 128) * 128;
 }
 
 
@@ -193,12 +190,12 @@ __device__ __forceinline__ void gemm_epilogue_chunk(const GemmParams &p, GemmSme
                 }
             }
         } else if constexpr (EPI == EPI_SWIGLU) {
-            if (mrow < 64) {
-                const int f = m_tile * 64 + mrow;
+            if ((mrow & 8) == 0) {  // rows alternate 8 gate, 8 up
+                const int f = m_tile * 64 + (mrow >> 4) * 8 + (mrow & 7);
 #pragma unroll
                 for (int c = 0; c < 32; ++c) {
                     if (c < ncols) {
-                        const float g = v[c], u = S.xch[(mrow + 64) * kEpiLd + c];
+                        const float g = v[c], u = S.xch[(mrow + 8) * kEpiLd + c];
                         const float h = g / (1.0f + expf(-g)) * u;
                         uint16_t hi, lo;
                         split_bf16(h, hi, lo);
@@ -281,7 +278,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
                     const int m_tile = tile % m_tiles;
                     mbar_expect_tx(&S.full[i], (uint32_t)kWStageBytes);
                     if (p.w_blk)
-                        bulk_load(sW + i * kWStageBytes, p.w_blk + wblk128_off(m_tiles * kTileM, kch * kTileK, m_tile, kc),
+                        bulk_load(sW + i * kWStageBytes, p.w_blk + wblk128_off(m_tiles * kTileM, m_tile, kc),
                                   kWStageBytes, &S.full[i], l2_policy_evict_first());
                     else
                         tma_load_2d(sW + i * kWStageBytes, &tmW, &S.full[i], kc * kTileK, m_tile * kTileM,
@@ -309,7 +306,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
                     mbar_arrive_expect_tx(&S.full[s], (uint32_t)kWStageBytes + xbytes);
                     if (p.w_blk)
                         bulk_load(sW + (size_t)s * kWStageBytes,
-                                  p.w_blk + wblk128_off(m_tiles * kTileM, kch * kTileK, m_tile, kc), kWStageBytes,
+                                  p.w_blk + wblk128_off(m_tiles * kTileM, m_tile, kc), kWStageBytes,
                                   &S.full[s], pol_w);
                     else
                         tma_load_2d(sW + (size_t)s * kWStageBytes, &tmW, &S.full[s], kc * kTileK, m_tile * kTileM,
