@@ -62,7 +62,6 @@ namespace sara {
 constexpr int kMegaThreads = 352;
 constexpr int kMegaCThreads = 256;  // compute warps 3..10
 constexpr int kWSlots = 4;  // weight / KV ring entries (a power of two: slot = index & 3)
-constexpr int kDetailRows = 16;  // profiling builds: rows of 4 detail stamps per CTA
 constexpr int kSlotBytes = 32768;
 constexpr int kRingBytes = 4 * 32768 + 65536;  // W slots, then the X stages
 constexpr int kMaxXStages = 8;
@@ -74,7 +73,6 @@ constexpr int kPhasesPerLayer = 9;
 constexpr int kMaxCtaBlocks = 256;    // attention KV block ids a CTA keeps in shared memory
 // phases of a layer (counter index 1 + 9 l + phase)
 enum : int { kPhQKV = 0, kPhFinQ = 1, kPhAtt = 2, kPhO = 3, kPhFinO = 4, kPhGU = 6, kPhDown = 7, kPhFinD = 8 };
-__device__ constexpr int kGemmPhases[4] = {kPhQKV, kPhO, kPhGU, kPhDown};
 constexpr int kSmallPhaseUnits = 2;   // QKV / O: units per participating CTA
 constexpr int kCntStride = 16;        // phase counters 128 bytes apart (one L2 line each)
 constexpr uint32_t kTmemCols = 512;
@@ -127,24 +125,21 @@ struct MegaParams {
     do {                                                                                                  \
         if (p.stamps) p.stamps[((size_t)blockIdx.x * p.n_stamp_ph + (ph)) * 4 + (kind)] = globaltimer_ns(); \
     } while (0)
-// Detail stamps of one layer (layer 2): the attention and first finalize phases (first unit
-// of each CTA, ids 0-15) and the first 12 units of the gate / up GEMM (ids 16-63: W copy
-// issued, W slot full and X stage full as seen by the MMA issuer, MMAs committed); the last
-// kDetailRows phase slots of the same array (the one before them holds the kernel start).
-#define MEGA_DETAIL(i)                                                                                    \
-    do {                                                                                                  \
-        if (p.stamps)                                                                                     \
-            p.stamps[((size_t)blockIdx.x * p.n_stamp_ph + p.n_stamp_ph - kDetailRows + ((i) >> 2)) * 4 + \
-                     ((i) & 3)] = globaltimer_ns();                                                       \
-    } while (0)
 #else
 #define MEGA_STAMP(ph, kind) \
     do {                     \
     } while (0)
-#define MEGA_DETAIL(i) \
-    do {               \
-    } while (0)
 #endif
+
+// A GEMM phase and this CTA's share of it (see SegWalk), fixed for a launch.
+struct GemmPlan {
+    const uint8_t *w, *x;  // blocked weights of layer 0, pair-blocked operand
+    int64_t ls;            // bytes of a layer's weights
+    int N, kch;            // output features, 64-column chunks of K
+    int t, kc, units;      // first tile (16-feature unit) and chunk, units of this CTA
+    int pass;              // column-owned: 16-feature units per pass; 0: split-K
+};
+constexpr int kPlanTiles = 32;  // contributor table entries per phase (wider phases compute them)
 
 struct MegaSmem {
     uint64_t wfull[kWSlots], wempty[kWSlots];
@@ -160,7 +155,10 @@ struct MegaSmem {
     int abort;
     int last_flag;
     int rows, rows16, nx, nx_lg, xgroup, n_items, att_span;  // nx = 2^nx_lg X stages of xgroup chunks
+    GemmPlan plan[5];           // this CTA's share of each GEMM phase (the same for every layer)
+    int2 tile_cta[3][kPlanTiles];  // first and last contributor of the tiles of q/k/v, O, down
     float rstd[128];
+    int rowpos[128];            // position of each live row
     // KV block ids: of this CTA's attention blocks (unit i's block j at ablk[aoff[i] + j]), and
     // of each row's current position (ablk_ok = 0: too many to hold, looked up in the table)
     int ablk[kMaxCtaBlocks];
@@ -184,9 +182,9 @@ constexpr size_t kMegaSmemBytes =
 // multiplies hi and lo parts at once (rows16 <= 64); with a 2048-byte group stride the hi
 // (lo) groups alone form a 128-row operand.
 constexpr int kLoOff = 1024;
-__host__ __device__ __forceinline__ int64_t xblk_off(int r, int k, int rows16) {
+__host__ __device__ __forceinline__ uint32_t xblk_off(int r, int k, int rows16) {
     const int chunk = k >> 6, col = k & 63;
-    return ((int64_t)chunk * 2 * rows16 + 16 * (r >> 3) + (r & 7)) * 128 +
+    return (uint32_t)(chunk * 2 * rows16 + 16 * (r >> 3) + (r & 7)) * 128 +
            ((((col >> 3) ^ (r & 7)) << 4) | ((col & 7) << 1));
 }
 // Byte offsets of K(pp, d) and V(pp, d) inside one 128-position KV block.
@@ -197,13 +195,19 @@ __host__ __device__ __forceinline__ int kv_v_off(int pp, int d) {
     const int c = pp & 63;
     return 32768 + (pp >> 6) * 16384 + d * 128 + ((((c >> 3) ^ (d & 7)) << 4) | ((c & 7) << 1));
 }
+// Order of a head's rows in the q/k/v weights: 16-row units of 8 dims of the first half and
+// their rotation partners, the same dims of the second half.  Row of dim dd.
+__host__ __device__ __forceinline__ int qkv_row(int dd, int half_hd) {
+    const int i = dd < half_hd ? dd : dd - half_hd;
+    return (i >> 3) * 16 + (i & 7) + (dd < half_hd ? 0 : 8);
+}
 // Byte offset of features col0.. (a multiple of 8) of k-chunk kc of a blocked weight matrix [N][K].
 __device__ __forceinline__ int64_t wblk_off(int N, int col0, int kc) { return ((int64_t)kc * N + col0) * 128; }
 
 // ------------------------------------------------------------------------------ waits
-// Bounded mbarrier wait that also gives up (returning false) once the CTA is aborting.
-__device__ __forceinline__ bool mwait(uint64_t *bar, uint32_t parity, int *err, volatile int *abort, uint64_t limit) {
-    if (mbar_try_wait(bar, parity)) return true;
+// The slow paths of the waits are functions of their own: inlined at every wait they made a third
+// of the kernel's code, which does not fit the instruction cache as it is.
+__device__ __noinline__ bool mwait_slow(uint32_t bar, uint32_t parity, int *err, volatile int *abort, uint64_t limit) {
     const uint64_t t0 = globaltimer_ns();
     for (uint32_t it = 1;; ++it) {
         if (mbar_try_wait(bar, parity)) return true;
@@ -217,17 +221,23 @@ __device__ __forceinline__ bool mwait(uint64_t *bar, uint32_t parity, int *err, 
         }
     }
 }
-
+// Bounded mbarrier wait that also gives up (returning false) once the CTA is aborting.
+__device__ __forceinline__ bool mwait(uint64_t *bar, uint32_t parity, int *err, volatile int *abort, uint64_t limit) {
+    const uint32_t b = smem_u32(bar);
+    if (mbar_try_wait(b, parity)) return true;
+    return mwait_slow(b, parity, err, abort, limit);
+}
 // The same for a converged warp: one answer for all of its lanes.
 __device__ __forceinline__ bool mwait_warp(uint64_t *bar, uint32_t parity, int *err, volatile int *abort, uint64_t limit) {
-    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    return __all_sync(0xffffffffu, mwait(bar, parity, err, abort, limit));
+    const uint32_t b = smem_u32(bar);
+    if (__all_sync(0xffffffffu, mbar_try_wait(b, parity))) return true;
+    return __all_sync(0xffffffffu, mwait_slow(b, parity, err, abort, limit));
 }
 
 // Spin until a phase counter reaches `target` (acquire loads);
 // bounded, gives up on abort or once another CTA reported a timeout.
-__device__ __forceinline__ bool spin_counter(const unsigned long long *cnt, unsigned long long target, int *err,
-                                             volatile int *abort, uint64_t limit) {
+__device__ __noinline__ bool spin_counter(const unsigned long long *cnt, unsigned long long target, int *err,
+                                          volatile int *abort, uint64_t limit) {
     if (ld_acquire_u64(cnt) >= target) return true;
     const uint64_t t0 = globaltimer_ns();
     for (uint32_t it = 1;; ++it) {
@@ -247,7 +257,6 @@ __device__ __forceinline__ bool spin_counter(const unsigned long long *cnt, unsi
         }
     }
 }
-
 // The same for a converged warp: one lane polls.
 __device__ __forceinline__ bool spin_counter_warp(const unsigned long long *cnt, unsigned long long target, int *err,
                                                   volatile int *abort, uint64_t limit) {
@@ -263,97 +272,92 @@ __device__ __forceinline__ unsigned long long phase_target(const MegaParams &p, 
 }
 
 // ------------------------------------------------------------------------------ phases
-// A GEMM phase: N output features, K inputs; unit widths below.  Two ways to split the work:
-//   K-split (own = false): (256-feature tile, 64-column chunk) units in equal contiguous ranges
-//     over the CTAs; each CTA stores its fp32 partial tiles and a finalisation phase sums them.
-//   column-owned (own = true): 16-feature units in equal contiguous ranges, each with the whole
-//     K, so that the CTA's epilogue applies the nonlinearity itself and no partials and no
+// GEMM phases: N output features, K inputs.  Two ways to split the work:
+//   split-K: (256-feature tile, 64-column chunk) units in equal contiguous ranges over the CTAs
+//     (lm_head: on whole tiles); each CTA stores its fp32 partial tiles and a finalisation phase
+//     sums them.
+//   column-owned (gate / up): 16-feature units in equal contiguous ranges, each with the whole K,
+//     so that the CTA's epilogue applies the nonlinearity itself and no partials and no
 //     finalisation phase are needed.  More activation traffic (every CTA reads the whole
 //     operand) and fewer weight rows per MMA, but one phase barrier and one L2 round trip less.
-struct GemmPh {
-    const uint8_t *w;
-    int N, K, kch, T, Gp;
-    const uint8_t *x;  // pair-blocked operand
-    bool whole;  // whole tiles per CTA (lm_head: the argmax of a tile is finished in one CTA)
-    bool own;    // column-owned
-};
+enum : int { kGQKV = 0, kGO = 1, kGDown = 2, kGGU = 3, kGLM = 4 };  // plan index
 constexpr int kOwnCols = 16;  // features per unit of a column-owned phase
+constexpr int kOwnUnits = kTileN / kOwnCols;  // units of a pass at most
 
-// GEMM phase k (kPhQKV, kPhO, kPhGU, kPhDown) of layer l; l == layers: lm_head.
-__device__ __forceinline__ GemmPh gemm_phase(const MegaParams &p, int l, int k) {
-    GemmPh g;
-    g.whole = false;
-    g.own = false;
-    g.Gp = gridDim.x;
-    if (l == p.layers) {
-        g.w = p.w_lm; g.N = p.V; g.K = p.d; g.x = p.xg; g.whole = true;
-    } else if (k == kPhQKV) {
-        g.w = p.w_qkv + l * p.ls_qkv; g.N = p.nqkv; g.K = p.d; g.x = p.xg; g.Gp = p.gp_qkv;
-    } else if (k == kPhO) {
-        g.w = p.w_o + l * p.ls_o; g.N = p.d; g.K = p.H * p.hd; g.x = p.att; g.Gp = p.gp_o;
-    } else if (k == kPhGU) {
-        g.w = p.w_gu + l * p.ls_gu; g.N = 2 * p.F; g.K = p.d; g.x = p.xg; g.own = true;
+// Geometry of a phase for CTA c of G: filled into plan[which] once per launch.
+// (Unit counts stay below 2^31 / SMs for every supported shape: 32-bit products suffice.)
+__device__ __noinline__ void make_plan(const MegaParams &p, GemmPlan &g, int which, int c, int G) {
+    int K = p.d, Gp = G;
+    g.x = p.xg;
+    g.pass = 0;
+    if (which == kGQKV) {
+        g.w = p.w_qkv; g.ls = p.ls_qkv; g.N = p.nqkv; Gp = p.gp_qkv;
+    } else if (which == kGO) {
+        g.w = p.w_o; g.ls = p.ls_o; g.N = p.d; K = p.H * p.hd; g.x = p.att; Gp = p.gp_o;
+    } else if (which == kGDown) {
+        g.w = p.w_down; g.ls = p.ls_down; g.N = p.d; K = p.F; g.x = p.hm;
+    } else if (which == kGGU) {
+        g.w = p.w_gu; g.ls = p.ls_gu; g.N = 2 * p.F;
     } else {
-        g.w = p.w_down + l * p.ls_down; g.N = p.d; g.K = p.F; g.x = p.hm;
+        g.w = p.w_lm; g.ls = 0; g.N = p.V;
     }
-    g.kch = g.K / 64;
-    g.T = g.own ? g.N / kOwnCols : (g.N + kTileN - 1) / kTileN;
+    g.kch = K / 64;
+    g.t = g.kc = g.units = 0;
     // at most one CTA per unit (tile for lm_head), so every participating CTA holds a
     // non-empty range and the CTAs between a tile's first and last owner all contributed
-    g.Gp = min(g.Gp, g.whole || g.own ? g.T : g.T * g.kch);
-    return g;
+    if (which == kGGU) {
+        const int U = g.N / kOwnCols;
+        Gp = min(Gp, U);
+        if (c < Gp) {
+            g.t = c * U / Gp;
+            g.units = (c + 1) * U / Gp - g.t;
+            const int np = (g.units + kOwnUnits - 1) / kOwnUnits;  // equal passes
+            g.pass = (g.units + np - 1) / np;
+        }
+    } else {
+        const int T = (g.N + kTileN - 1) / kTileN;
+        const int U = which == kGLM ? T : T * g.kch, m = which == kGLM ? g.kch : 1;
+        Gp = min(Gp, U);
+        if (c < Gp) {
+            const int u0 = c * U / Gp * m;
+            g.units = (c + 1) * U / Gp * m - u0;
+            g.t = u0 / g.kch;
+            g.kc = u0 - g.t * g.kch;
+        }
+    }
 }
 
-// This CTA's share of a GEMM phase: units [u, u1) -- (tile, k-chunk) units, cut on whole tiles
-// for lm_head, or 16-feature units (column-owned) -- walked as segments, each one accumulator:
-// features [col0, col0 + n) x chunks [kc0, kc1).  A column-owned share wider than 256 features
-// is walked in equal passes.
-// (Unit counts stay below 2^31 / SMs for every supported shape: 32-bit products suffice.)
+// A CTA's share of a phase walked as segments, each one accumulator: features [col0, col0 + n) x
+// chunks [kc0, kc1), in weight ring slots of cps chunks each.
 struct Seg {
-    int t, col0, n, kc0, kc1;
-    int cps;  // chunks per weight ring slot
+    int t, col0, n, kc0, kc1, cps;
     __device__ __forceinline__ int entries() const { return (kc1 - kc0 + cps - 1) / cps; }
 };
 struct SegWalk {
-    int u, u1, pass;
-    __device__ __forceinline__ SegWalk(const GemmPh &g) {
-        const int c = blockIdx.x;
-        u = u1 = pass = 0;
-        if (c >= g.Gp) return;
-        if (g.own) {
-            u = c * g.T / g.Gp;
-            u1 = (c + 1) * g.T / g.Gp;
-            const int np = ((u1 - u) * kOwnCols + kTileN - 1) / kTileN;
-            pass = (u1 - u + np - 1) / np;
-        } else if (g.whole) {
-            u = c * g.T / g.Gp * g.kch;
-            u1 = (c + 1) * g.T / g.Gp * g.kch;
-        } else {
-            const int U = g.T * g.kch;
-            u = c * U / g.Gp;
-            u1 = (c + 1) * U / g.Gp;
-        }
-    }
-    __device__ __forceinline__ bool next(const GemmPh &g, Seg &s) {
-        if (u >= u1) return false;
-        if (g.own) {
-            const int nu = min(pass, u1 - u);
-            s.t = 0;
-            s.col0 = u * kOwnCols;
+    int t, kc, left;
+    __device__ __forceinline__ SegWalk(const GemmPlan &g) : t(g.t), kc(g.kc), left(g.units) {}
+    __device__ __forceinline__ bool next(const GemmPlan &g, Seg &s) {
+        if (left <= 0) return false;
+        s.t = t;
+        if (g.pass > 0) {
+            const int nu = min(g.pass, left);
+            s.col0 = t * kOwnCols;
             s.n = nu * kOwnCols;
             s.kc0 = 0;
             s.kc1 = g.kch;
-            u += nu;
+            t += nu;
+            left -= nu;
         } else {
-            s.t = u / g.kch;
-            const int e = min(u1, (s.t + 1) * g.kch);
-            s.col0 = s.t * kTileN;
+            const int m = min(left, g.kch - kc);
+            s.col0 = t * kTileN;
             s.n = min(kTileN, g.N - s.col0);
-            s.kc0 = u - s.t * g.kch;
-            s.kc1 = s.kc0 + e - u;
-            u = e;
+            s.kc0 = kc;
+            s.kc1 = kc + m;
+            ++t;
+            kc = 0;
+            left -= m;
         }
-        s.cps = s.n > 128 ? 1 : s.n > 64 ? 2 : s.n > 32 ? 4 : s.n > 16 ? 8 : 16;  // (a power of two)
+        s.cps = 1 << (s.n > 128 ? 0 : s.n > 64 ? 1 : s.n > 32 ? 2 : s.n > 16 ? 3 : 4);
         return true;
     }
 };
@@ -364,24 +368,24 @@ __device__ __forceinline__ int unit_owner(int u, int U, int Gp) {
     while (c > 0 && c * U / Gp > u) --c;
     return c;
 }
-// First and last CTA holding a partial of tile t.  CTA c's partial of tile t is segment
-// c + t of the partial buffer (distinct for every (c, t) of a phase: ranges are ordered).
-__device__ __forceinline__ void tile_ctas(const GemmPh &g, int t, int &ca, int &cb) {
-    const int U = g.T * g.kch;
-    ca = unit_owner(t * g.kch, U, g.Gp);
-    cb = unit_owner((t + 1) * g.kch - 1, U, g.Gp);
+// First and last CTA holding a partial of tile t of a split-K phase.  CTA c's partial of tile t is
+// segment c + t of the partial buffer (distinct for every (c, t) of a phase: ranges are ordered).
+__device__ __noinline__ int2 tile_ctas(const MegaParams &p, const GemmPlan &g, int which, int t, int G) {
+    const int U = (g.N + kTileN - 1) / kTileN * g.kch;
+    const int Gp = min(which == kGQKV ? p.gp_qkv : which == kGO ? p.gp_o : G, U);
+    return make_int2(unit_owner(t * g.kch, U, Gp), unit_owner((t + 1) * g.kch - 1, U, Gp));
 }
 
 // Attention unit: one split of one row for one kv head.  Split sp covers the `span` KV
 // blocks from block sp * span on: positions [p0, p0 + n) of the row's ctx, in nb blocks.
 struct AttUnit {
     int item, kvh, row, sp, ctx, p0, n, nb, nsplit, slot;
-    bool last;
+    int last;
 };
-__device__ __forceinline__ AttUnit att_unit(const MegaParams &p, int64_t a, int span) {
+__device__ __noinline__ AttUnit att_unit(const MegaParams &p, int a, int span) {
     AttUnit u;
-    u.item = (int)(a / p.KVH);
-    u.kvh = (int)(a - (int64_t)u.item * p.KVH);
+    u.item = a / p.KVH;
+    u.kvh = a - u.item * p.KVH;
     const int2 it = __ldg(&p.c.att_items[u.item]);
     u.row = it.x;
     u.sp = it.y;
@@ -397,7 +401,7 @@ __device__ __forceinline__ AttUnit att_unit(const MegaParams &p, int64_t a, int 
 // Attention units in equal contiguous ranges, counted from the last CTA down: the QKV
 // projection runs on the first CTAs, so a small unit count lands on CTAs that are free
 // to prefetch during it.
-__device__ __forceinline__ void att_range(const MegaParams &p, int n_items, int64_t &a0, int64_t &a1) {
+__device__ __forceinline__ void att_range(const MegaParams &p, int n_items, int &a0, int &a1) {
     const int NU = n_items * p.KVH, G = (int)gridDim.x, v = G - 1 - (int)blockIdx.x;
     a0 = v * NU / G;
     a1 = (v + 1) * NU / G;
@@ -417,9 +421,9 @@ __device__ __forceinline__ uint8_t *kv_block(const MegaParams &p, const MegaSmem
 // The KV block ids of this CTA's attention units (one warp, lane i: unit a0 + i), read once
 // per launch from the block table into shared memory for the W producer.
 __device__ __forceinline__ void fill_att_blocks(const MegaParams &p, MegaSmem &S, int lane) {
-    int64_t a0, a1;
+    int a0, a1;
     att_range(p, S.n_items, a0, a1);
-    const int nu = (int)(a1 - a0);
+    const int nu = a1 - a0;
     bool ok = nu <= 32;
     int nb = 0, off = 0;
     AttUnit u{};
@@ -453,7 +457,15 @@ __device__ __forceinline__ void fill_att_blocks(const MegaParams &p, MegaSmem &S
     __syncwarp();
 }
 
+// Counter of a GEMM phase of layer l.
+__device__ __forceinline__ int gemm_counter(int gk, int l) {
+    return 1 + kPhasesPerLayer * l + (gk == kGQKV ? kPhQKV : gk == kGO ? kPhO : gk == kGGU ? kPhGU : kPhDown);
+}
+
 // ------------------------------------------------------------------------------ W producer
+// GEMM phases in launch order: q/k/v, O, gate / up, down of every layer, then lm_head.
+__device__ __forceinline__ int gemm_kind(int i) { return i == 0 ? kGQKV : i == 1 ? kGO : i == 2 ? kGGU : kGDown; }
+
 __device__ __forceinline__ void mega_w_producer(const MegaParams &p, MegaSmem &S, uint8_t *sW) {
     volatile int *ab = &S.abort;
     const uint64_t lim = S.wait_ns;
@@ -465,83 +477,78 @@ __device__ __forceinline__ void mega_w_producer(const MegaParams &p, MegaSmem &S
     auto acquire = [&](uint32_t i) -> bool {
         return i < nws || mwait_warp(&S.wempty[i % nws], ((i / nws) & 1) ^ 1, err, ab, lim);
     };
-    for (int l = 0; l <= p.layers && ok; ++l) {
-        for (int gp = 0; gp < 4 && ok; ++gp) {
-            if (l == p.layers && gp > 0) break;
-            const int k = kGemmPhases[gp];
-            const GemmPh g = gemm_phase(p, l, k);
-            SegWalk walk(g);
-            Seg sg;
-            int nth = 0;
-            while (ok && walk.next(g, sg)) {
-                const uint32_t cb = (uint32_t)sg.n * 128;  // a chunk's bytes
-                for (int kc = sg.kc0; kc < sg.kc1; kc += sg.cps, ++wi, ++nth) {
-                    if (!acquire(wi)) { ok = false; break; }
-                    const int s = (int)(wi % nws), m = min(sg.cps, sg.kc1 - kc);
-                    if (elect_one()) {
-                        mbar_arrive_expect_tx(&S.wfull[s], (uint32_t)m * cb);
-                        for (int j = 0; j < m; ++j)
-                            bulk_load(sW + (size_t)s * kSlotBytes + (size_t)j * cb, g.w + wblk_off(g.N, sg.col0, kc + j),
-                                      cb, &S.wfull[s], pol);
-                    }
-                    if (k == kPhGU && l == min(2, p.layers - 1) && nth < 12) MEGA_DETAIL(16 + nth);
+    int a0, a1;
+    att_range(p, S.n_items, a0, a1);
+#pragma unroll 1
+    for (int i = 0; i <= 4 * p.layers && ok; ++i) {
+        const int l = i >> 2, gk = i == 4 * p.layers ? kGLM : gemm_kind(i & 3);
+        const GemmPlan &g = S.plan[gk];
+        const uint8_t *w = g.w + l * g.ls;
+        const int64_t rowb = (int64_t)g.N * 128;  // bytes of a chunk
+        SegWalk walk(g);
+        Seg sg;
+#pragma unroll 1
+        while (ok && walk.next(g, sg)) {
+            const uint32_t cb = (uint32_t)sg.n * 128;  // a chunk's bytes
+            const uint8_t *src = w + sg.kc0 * rowb + (int64_t)sg.col0 * 128;
+#pragma unroll 1
+            for (int kc = sg.kc0; kc < sg.kc1; kc += sg.cps, ++wi) {
+                if (!acquire(wi)) { ok = false; break; }
+                const int s = (int)(wi % nws), m = min(sg.cps, sg.kc1 - kc);
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(&S.wfull[s], (uint32_t)m * cb);
+#pragma unroll 1
+                    for (int j = 0; j < m; ++j, src += rowb)
+                        bulk_load(sW + (size_t)s * kSlotBytes + (size_t)j * cb, src, cb, &S.wfull[s], pol);
                 }
+                src = w + (kc + m) * rowb + (int64_t)sg.col0 * 128;
             }
-            MEGA_STAMP(1 + kPhasesPerLayer * l + k, 2);
-            if (k == 0 && l < p.layers && ok) {
-                // the attention phase's KV blocks follow the QKV weights in ring order: unit
-                // pairs (one unit per compute warp group), block by block, the K of the pair's
-                // units, then their V^T; each one ring entry (K: d < 64 | d >= 64 halves, V^T:
-                // positions < 64 | >= 64).  The block holding a row's new position is copied
-                // once the q / k / v phase has appended it to the cache.
-                int64_t a0, a1;
-                att_range(p, S.n_items, a0, a1);
-                const int span = S.att_span;
-                bool finq_seen = false;
-                for (int64_t a = a0; a < a1 && ok; a += 2) {
-                    const bool two = a + 1 < a1;
-                    const AttUnit ua = att_unit(p, a, span);
-                    const AttUnit ub = two ? att_unit(p, a + 1, span) : ua;
-                    const int nbb = two ? ub.nb : 0;
-                    for (int j = 0; j < max(ua.nb, nbb) && ok; ++j) {
-                        for (int kv = 0; kv < 2 && ok; ++kv) {
-                            for (int w = 0; w < 2 && ok; ++w) {
-                                const AttUnit &u = w ? ub : ua;
-                                if (j >= (w ? nbb : ua.nb)) continue;
-                                if (kv == 0 && u.last && j == u.nb - 1 && !finq_seen) {
-                                    const int fq = 1 + kPhasesPerLayer * l + kPhFinQ;
-                                    if (!spin_counter_warp(&p.cnt[fq * kCntStride], phase_target(p, S, fq), err, ab, lim)) {
-                                        ok = false;
-                                        break;
-                                    }
-                                    fence_proxy_async_global();
-                                    finq_seen = true;
-                                }
-                                const uint8_t *blk = kv_block(p, S, l, u, (int)(a - a0) + w, j);
-                                const int nj = min(kKVPos, u.n - j * kKVPos);
-                                if (!acquire(wi)) { ok = false; break; }
-                                const int s = (int)(wi % nws);
-                                if (!elect_one()) {
-                                } else if (kv == 0) {
-                                    const uint32_t kb = (uint32_t)(((nj + 7) & ~7) * 128);
-                                    mbar_arrive_expect_tx(&S.wfull[s], p.hd > 64 ? 2 * kb : kb);
-                                    bulk_load(sW + (size_t)s * kSlotBytes, blk, kb, &S.wfull[s], pol);
-                                    if (p.hd > 64)
-                                        bulk_load(sW + (size_t)s * kSlotBytes + 16384, blk + 16384, kb, &S.wfull[s], pol);
-                                } else {
-                                    const uint32_t vb = (uint32_t)(p.hd * 128);
-                                    mbar_arrive_expect_tx(&S.wfull[s], nj > 64 ? 2 * vb : vb);
-                                    bulk_load(sW + (size_t)s * kSlotBytes, blk + 32768, vb, &S.wfull[s], pol);
-                                    if (nj > 64)
-                                        bulk_load(sW + (size_t)s * kSlotBytes + 16384, blk + 49152, vb, &S.wfull[s], pol);
-                                }
-                                ++wi;
-                            }
+        }
+        MEGA_STAMP(gk == kGLM ? 1 + kPhasesPerLayer * l : gemm_counter(gk, l), 2);
+        if (gk == kGQKV && ok) {
+            // the attention phase's KV blocks follow the QKV weights in ring order: unit
+            // pairs (one unit per compute warp group), block by block, the K of the pair's
+            // units, then their V^T; each one ring entry (K: d < 64 | d >= 64 halves, V^T:
+            // positions < 64 | >= 64).  The block holding a row's new position is copied
+            // once the q / k / v phase has appended it to the cache.
+            const int span = S.att_span;
+            bool finq_seen = false;
+#pragma unroll 1
+            for (int a = a0; a < a1 && ok; a += 2) {
+                const bool two = a + 1 < a1;
+                const AttUnit ua = att_unit(p, a, span);
+                const AttUnit ub = two ? att_unit(p, a + 1, span) : ua;
+                const int nbb = two ? ub.nb : 0, nbm = max(ua.nb, nbb);
+#pragma unroll 1
+                for (int q = 0; q < 4 * nbm && ok; ++q) {  // block q / 4, K or V^T, unit a or a + 1
+                    const int j = q >> 2, kv = (q >> 1) & 1, x = q & 1;
+                    if (j >= (x ? nbb : ua.nb)) continue;
+                    const int n = x ? ub.n : ua.n;
+                    if (kv == 0 && (x ? ub.last : ua.last) && j == (x ? nbb : ua.nb) - 1 && !finq_seen) {
+                        const int fq = 1 + kPhasesPerLayer * l + kPhFinQ;
+                        if (!spin_counter_warp(&p.cnt[fq * kCntStride], phase_target(p, S, fq), err, ab, lim)) {
+                            ok = false;
+                            break;
                         }
+                        fence_proxy_async_global();
+                        finq_seen = true;
                     }
+                    const uint8_t *blk = kv_block(p, S, l, x ? ub : ua, a - a0 + x, j) + kv * 32768;
+                    const int nj = min(kKVPos, n - j * kKVPos);
+                    if (!acquire(wi)) { ok = false; break; }
+                    const int s = (int)(wi % nws);
+                    // K: rows = positions, halves of the dims; V^T: rows = dims, halves of the positions
+                    const uint32_t hb = kv == 0 ? (uint32_t)(((nj + 7) & ~7) * 128) : (uint32_t)(p.hd * 128);
+                    const bool both = kv == 0 ? p.hd > 64 : nj > 64;
+                    if (elect_one()) {
+                        mbar_arrive_expect_tx(&S.wfull[s], both ? 2 * hb : hb);
+                        bulk_load(sW + (size_t)s * kSlotBytes, blk, hb, &S.wfull[s], pol);
+                        if (both) bulk_load(sW + (size_t)s * kSlotBytes + 16384, blk + 16384, hb, &S.wfull[s], pol);
+                    }
+                    ++wi;
                 }
-                MEGA_STAMP(1 + kPhasesPerLayer * l + kPhAtt, 2);
             }
+            MEGA_STAMP(1 + kPhasesPerLayer * l + kPhAtt, 2);
         }
     }
     if (!ok) {  // every copy already issued lands before the CTA exits
@@ -564,31 +571,32 @@ __device__ __forceinline__ void mega_x_producer(const MegaParams &p, MegaSmem &S
     const int64_t chunk_stride = (int64_t)p.rows_cap16 * 256;
     uint32_t xi = 0;
     bool ok = true;
-    for (int l = 0; l <= p.layers && ok; ++l) {
-        for (int gp = 0; gp < 4 && ok; ++gp) {
-            if (l == p.layers && gp > 0) break;
-            const int k = kGemmPhases[gp];
-            const GemmPh g = gemm_phase(p, l, k);
-            SegWalk walk(g);
-            if (walk.u >= walk.u1) continue;
-            // the phase this operand comes from: FIN_D of l-1 / embedding, ATT, FIN_O, GU
-            const int dep = (l == p.layers || k == kPhQKV) ? kPhasesPerLayer * l
-                                                           : 1 + kPhasesPerLayer * l + (k == kPhGU ? kPhFinO : k - 1);
-            if (!spin_counter_warp(&p.cnt[dep * kCntStride], phase_target(p, S, dep), err, ab, lim)) { ok = false; break; }
-            MEGA_STAMP(1 + kPhasesPerLayer * l + k, 1);
-            fence_proxy_async_global();
-            Seg sg;
-            while (ok && walk.next(g, sg)) {
-                for (int kc = sg.kc0; kc < sg.kc1; kc += gx, ++xi) {
-                    const int s = (int)(xi & (uint32_t)(NX - 1)), m = min(gx, sg.kc1 - kc);
-                    if (xi >= (uint32_t)NX && !mwait_warp(&S.xempty[s], ((xi >> nxl) & 1) ^ 1, err, ab, lim)) { ok = false; break; }
-                    if (elect_one()) {
-                        mbar_arrive_expect_tx(&S.xfull[s], (uint32_t)m * chunk);
-                        for (int j = 0; j < m; ++j)
-                            bulk_load(sX + (size_t)s * stage + (size_t)j * chunk, g.x + (kc + j) * chunk_stride, chunk,
-                                      &S.xfull[s], pol);
-                    }
+#pragma unroll 1
+    for (int i = 0; i <= 4 * p.layers && ok; ++i) {
+        const int l = i >> 2, gk = i == 4 * p.layers ? kGLM : gemm_kind(i & 3);
+        const GemmPlan &g = S.plan[gk];
+        SegWalk walk(g);
+        if (walk.left <= 0) continue;
+        // the phase this operand comes from: FIN_D of l-1 / embedding, ATT, FIN_O, GU
+        const int dep = kPhasesPerLayer * l + (gk == kGO ? 1 + kPhAtt : gk == kGGU ? 1 + kPhFinO : gk == kGDown ? 1 + kPhGU : 0);
+        if (!spin_counter_warp(&p.cnt[dep * kCntStride], phase_target(p, S, dep), err, ab, lim)) { ok = false; break; }
+        MEGA_STAMP(gk == kGLM ? 1 + kPhasesPerLayer * l : gemm_counter(gk, l), 1);
+        fence_proxy_async_global();
+        Seg sg;
+#pragma unroll 1
+        while (ok && walk.next(g, sg)) {
+            const uint8_t *src = g.x + sg.kc0 * chunk_stride;
+#pragma unroll 1
+            for (int kc = sg.kc0; kc < sg.kc1; kc += gx, ++xi) {
+                const int s = (int)(xi & (uint32_t)(NX - 1)), m = min(gx, sg.kc1 - kc);
+                if (xi >= (uint32_t)NX && !mwait_warp(&S.xempty[s], ((xi >> nxl) & 1) ^ 1, err, ab, lim)) { ok = false; break; }
+                if (elect_one()) {
+                    mbar_arrive_expect_tx(&S.xfull[s], (uint32_t)m * chunk);
+#pragma unroll 1
+                    for (int j = 0; j < m; ++j)
+                        bulk_load(sX + (size_t)s * stage + (size_t)j * chunk, src + j * chunk_stride, chunk, &S.xfull[s], pol);
                 }
+                src += gx * chunk_stride;
             }
         }
     }
@@ -601,8 +609,7 @@ __device__ __forceinline__ void mega_x_producer(const MegaParams &p, MegaSmem &S
 }
 
 // ------------------------------------------------------------------------------ MMA issuer
-__device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8_t *sW, uint8_t *sX, uint8_t *sQ,
-                                         uint8_t *sP, uint32_t tmem) {
+__device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8_t *sW, uint8_t *sX, uint32_t tmem) {
     volatile int *ab = &S.abort;
     const uint64_t lim = S.wait_ns;
     int *err = &p.c.v->err;
@@ -612,109 +619,95 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
     // rounded up to 64 or 128: the rows past the stage only feed accumulator rows nobody
     // reads); more: the hi and the lo groups as two 128-row operands into one accumulator
     const bool stacked = R16 <= 64;
+    const uint32_t sbo = stacked ? 1024u : 2048u;
     uint32_t wi = 0, xi = 0;
-    int use0 = 0, use1 = 0, tseg = 0;  // accumulator buffer uses, GEMM tiles so far
+    uint32_t use[2] = {0, 0};  // accumulator buffer uses
+    uint32_t tseg = 0;         // segments so far
     bool ok = true;
     constexpr uint32_t nws = kWSlots;
-    auto wslot = [&](uint32_t i) -> uint32_t { return smem_u32(sW + (size_t)(i % nws) * kSlotBytes); };
-    auto wwait = [&](uint32_t i) -> bool { return mwait_warp(&S.wfull[i % nws], (i / nws) & 1, err, ab, lim); };
-    auto gemm = [&](const GemmPh &g, bool det) {
+    int a0, a1;
+    att_range(p, S.n_items, a0, a1);
+    int gi = 0;  // attention units so far (unit i of a phase runs on group (gi + i) & 1)
+#pragma unroll 1
+    for (int i = 0; i <= 4 * p.layers && ok; ++i) {
+        const int gk = i == 4 * p.layers ? kGLM : gemm_kind(i & 3);
+        const GemmPlan &g = S.plan[gk];
         SegWalk walk(g);
         Seg sg;
-        int nth = 0;  // ring entry of the phase
+#pragma unroll 1
         while (ok && walk.next(g, sg)) {
-            const int a = tseg & 1;  // segments alternate between two accumulators (epilogue overlaps)
-            const int use_a = a ? use1 : use0;
+            const uint32_t a = tseg & 1;  // segments alternate between two accumulators (epilogue overlaps)
+            const uint32_t use_a = a ? use[1] : use[0];
             if (use_a >= 1 && !mwait_warp(&S.acc_empty[a], (use_a - 1) & 1, err, ab, lim)) { ok = false; break; }
             tc_fence_after();
-            const uint32_t d = tmem + (uint32_t)(a * kTileN);
+            const uint32_t d = tmem + a * kTileN;
             const uint32_t idg = idesc_bf16_f32(R16 <= 32 ? 64u : 128u, (uint32_t)sg.n);
             const uint32_t cb = (uint32_t)sg.n * 128;
             // chunks go in groups that stay within one weight slot and one activation stage, so a
             // group's MMAs issue back to back: one pair of waits and commits per group
             const int grp = min(sg.cps, gx);
             int wj = 0, xj = 0;  // chunk within the weight slot / the activation stage
+#pragma unroll 1
             for (int kc = sg.kc0; kc < sg.kc1; kc += grp) {
-                const bool dj = det && wj == 0 && nth < 12;
-                if (wj == 0 && !wwait(wi)) { ok = false; break; }
-                if (dj) MEGA_DETAIL(28 + nth);
+                if (wj == 0 && !mwait_warp(&S.wfull[wi % nws], (wi / nws) & 1, err, ab, lim)) { ok = false; break; }
                 const int xs = (int)(xi & (uint32_t)(NX - 1));
                 if (xj == 0 && !mwait_warp(&S.xfull[xs], (xi >> nxl) & 1, err, ab, lim)) { ok = false; break; }
-                if (dj) MEGA_DETAIL(40 + nth);
                 tc_fence_after();
                 const int m = min(grp, sg.kc1 - kc);
-                const uint32_t aw = wslot(wi) + (uint32_t)wj * cb;
-                const uint32_t ax = smem_u32(sX) + (uint32_t)xs * stage + (uint32_t)xj * chunk;
                 const bool end = kc + m == sg.kc1;
                 const bool wlast = end || wj + grp == sg.cps, xlast = end || xj + grp == gx;
                 if (elect_one()) {
-                    for (int j = 0; j < m; ++j) {
+                    uint32_t aw = smem_u32(sW) + (wi % nws) * kSlotBytes + (uint32_t)wj * cb;
+                    uint32_t ax = smem_u32(sX) + (uint32_t)xs * stage + (uint32_t)xj * chunk;
+                    uint32_t acc = kc == sg.kc0 ? 0u : 1u;
+#pragma unroll 1
+                    for (int j = 0; j < m; ++j, aw += cb, ax += chunk) {
 #pragma unroll
                         for (int kk = 0; kk < 4; ++kk) {
-                            const uint64_t bd = sdesc_kmajor_sw128(aw + j * cb + kk * 32);
-                            const uint32_t acc = (kc == sg.kc0 && j == 0 && kk == 0) ? 0u : 1u;
-                            if (stacked) {
-                                tc_mma_bf16(d, sdesc_kmajor_sw128(ax + j * chunk + kk * 32), bd, idg, acc);
-                            } else {
-                                tc_mma_bf16(d, sdesc_kmajor_sw128(ax + j * chunk + kk * 32, 2048), bd, idg, acc);
-                                tc_mma_bf16(d, sdesc_kmajor_sw128(ax + j * chunk + kLoOff + kk * 32, 2048), bd, idg, 1u);
-                            }
+                            const uint64_t bd = sdesc_kmajor_sw128(aw + kk * 32);
+                            tc_mma_bf16(d, sdesc_kmajor_sw128(ax + kk * 32, sbo), bd, idg, acc);
+                            acc = 1u;
+                            if (!stacked) tc_mma_bf16(d, sdesc_kmajor_sw128(ax + kLoOff + kk * 32, sbo), bd, idg, 1u);
                         }
                     }
                     if (xlast) tc_commit(&S.xempty[xs]);
                     if (wlast) tc_commit(&S.wempty[wi % nws]);
+                    if (end) tc_commit(&S.acc_full[a]);
                 }
                 __syncwarp();
-                if (wlast && dj) MEGA_DETAIL(52 + nth);
                 wj = wlast ? 0 : wj + grp;
                 xj = xlast ? 0 : xj + grp;
                 wi += wlast ? 1 : 0;
-                nth += wlast ? 1 : 0;
                 xi += xlast ? 1 : 0;
             }
-            if (!ok) break;
-            if (elect_one()) tc_commit(&S.acc_full[a]);
-            if (a) ++use1; else ++use0;
+            if (a) ++use[1]; else ++use[0];
             ++tseg;
         }
-    };
-    // The attention phase's ring entries (its KV tiles) are read and released by the compute
-    // warp groups.  The issuer is the ring's one in-order observer: it waits for each entry to
-    // land and hands it to the group that runs its unit (an arrival on kvready[group][slot]).
-    // A group's consecutive uses of a slot are then at most one barrier phase apart (the slot
-    // is refilled only after the group released its previous tile there), which a group
-    // waiting on the shared wfull barriers directly could not rely on.
-    int gi = 0;  // attention units so far (unit i of a phase runs on group (gi + i) & 1)
-    auto att_fwd = [&](int64_t a0, int64_t a1) -> bool {
-        const int n = (int)(a1 - a0), span = S.att_span;
-        for (int i = 0; i < n; i += 2) {
-            const bool two = i + 1 < n;
-            const int nba = att_unit(p, a0 + i, span).nb, nbb = two ? att_unit(p, a0 + i + 1, span).nb : 0;
-            for (int j = 0; j < max(nba, nbb); ++j)
-                for (int kv = 0; kv < 2; ++kv)
-                    for (int x = 0; x < 2; ++x) {
-                        if (j >= (x ? nbb : nba)) continue;
-                        if (!wwait(wi)) return false;
-                        if (elect_one()) mbar_arrive(&S.kvready[(gi + i + x) & 1][wi % nws]);
-                        ++wi;
-                    }
-        }
-        gi += n;
-        return true;
-    };
-    for (int l = 0; l <= p.layers && ok; ++l) {
-        for (int gp = 0; gp < 4 && ok; ++gp) {
-            if (l == p.layers && gp > 0) break;
-            const int k = kGemmPhases[gp];
-            const GemmPh g = gemm_phase(p, l, k);
-            gemm(g, k == kPhGU && l == min(2, p.layers - 1));
-            MEGA_STAMP(1 + kPhasesPerLayer * l + k, 3);
-            if (k == 0 && l < p.layers && ok) {
-                int64_t a0, a1;
-                att_range(p, S.n_items, a0, a1);
-                if (!att_fwd(a0, a1)) ok = false;
-                MEGA_STAMP(1 + kPhasesPerLayer * l + kPhAtt, 3);
+        MEGA_STAMP(gk == kGLM ? 1 + kPhasesPerLayer * (i >> 2) : gemm_counter(gk, i >> 2), 3);
+        if (gk == kGQKV && ok) {
+            // The attention phase's ring entries (its KV tiles) are read and released by the compute
+            // warp groups.  The issuer is the ring's one in-order observer: it waits for each entry to
+            // land and hands it to the group that runs its unit (an arrival on kvready[group][slot]).
+            // A group's consecutive uses of a slot are then at most one barrier phase apart (the slot
+            // is refilled only after the group released its previous tile there), which a group
+            // waiting on the shared wfull barriers directly could not rely on.
+            const int n = a1 - a0, span = S.att_span;
+#pragma unroll 1
+            for (int u = 0; u < n && ok; u += 2) {
+                const bool two = u + 1 < n;
+                const int nba = att_unit(p, a0 + u, span).nb, nbb = two ? att_unit(p, a0 + u + 1, span).nb : 0;
+                const int nbm = max(nba, nbb);
+#pragma unroll 1
+                for (int q = 0; q < 4 * nbm; ++q) {  // the W producer's order
+                    const int j = q >> 2, x = q & 1;
+                    if (j >= (x ? nbb : nba)) continue;
+                    if (!mwait_warp(&S.wfull[wi % nws], (wi / nws) & 1, err, ab, lim)) { ok = false; break; }
+                    if (elect_one()) mbar_arrive(&S.kvready[(gi + u + x) & 1][wi % nws]);
+                    ++wi;
+                }
             }
+            gi += n;
+            MEGA_STAMP(1 + kPhasesPerLayer * (i >> 2) + kPhAtt, 3);
         }
     }
     // every MMA issued has retired before tensor memory is released
@@ -723,22 +716,21 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
 }
 
 // ------------------------------------------------------------------------------ compute
-__device__ __forceinline__ void store_hilo(uint8_t *base, int64_t off, float v) {
-    uint16_t h, l;
-    split_bf16(v, h, l);
-    *reinterpret_cast<uint16_t *>(base + off) = h;
-    *reinterpret_cast<uint16_t *>(base + off + kLoOff) = l;
-}
-
-
-// Eight bf16 values as one 16-byte granule.
+// Eight / four bf16 values as one 16- / 8-byte store.
 __device__ __forceinline__ uint4 pack8(const uint16_t (&v)[8]) {
     return make_uint4((uint32_t)v[0] | ((uint32_t)v[1] << 16), (uint32_t)v[2] | ((uint32_t)v[3] << 16),
                       (uint32_t)v[4] | ((uint32_t)v[5] << 16), (uint32_t)v[6] | ((uint32_t)v[7] << 16));
 }
+__device__ __forceinline__ uint2 pack4(const uint16_t (&v)[4]) {
+    return make_uint2((uint32_t)v[0] | ((uint32_t)v[1] << 16), (uint32_t)v[2] | ((uint32_t)v[3] << 16));
+}
 
-__device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, uint8_t *sW, uint8_t *sQ, uint8_t *sP,
-                                             uint32_t tmem) {
+// The compute warps' code runs once per layer and is far larger than the instruction caches'
+// first levels, so its size is time: each step exists once (the layer loop is unrolled over
+// nothing, the three residual finalisations and the three split-K epilogues share their code),
+// divisions by launch constants are done once (GemmPlan, tile_cta), and batches of loads are
+// spread over the lanes instead of being unrolled further.
+__device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, uint8_t *sW, uint8_t *sQ, uint32_t tmem) {
     volatile int *ab = &S.abort;
     const uint64_t lim = S.wait_ns;
     int *err = &p.c.v->err;
@@ -754,18 +746,15 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
     // GEMM accumulator lane -> activation row.  Stacked operand (at most 64 live rows): operand
     // row m holds the hi (lo) part of row 8 (m / 16) + m % 8 for m % 16 < 8 (>= 8); M = 128
     // puts operand row m in lane m, M = 64 (at most 32 rows) in lane 32 (m / 16) + m % 16.
-    // The hi and lo accumulators of a row are lanes i and i ^ 8 of one warp (pair sum by a
-    // shuffle; the hi lane stores).  Otherwise (M = 128, hi and lo accumulated together) row
-    // i is lane i.
+    // The hi and lo accumulators of a row are lanes i and i ^ 8 of one warp: after adding them
+    // with a shuffle each lane of the pair finishes half of the columns.  Otherwise (M = 128,
+    // hi and lo accumulated together) row i is lane i.  Lanes of no row: past the batch.
     const int R16 = S.rows16;
-    const bool pair = R16 <= 64;
-    const int my_row = R16 <= 32   ? ((lane & 0x18) == 0 ? quarter * 8 + lane : 1 << 20)
-                       : pair      ? ((lane & 8) == 0 ? quarter * 16 + 8 * (lane >> 4) + (lane & 7) : 1 << 20)
-                                   : quarter * 32 + lane;
-    // the same for both lanes of a pair (lanes i and i ^ 8), past the batch for lanes of no row
-    const int my_row_any = R16 <= 32 ? ((lane & 16) == 0 ? quarter * 8 + (lane & 7) : 1 << 20)
-                           : pair    ? quarter * 16 + 8 * (lane >> 4) + (lane & 7)
-                                     : quarter * 32 + lane;
+    const bool pair = R16 <= 64, second = pair && (lane & 8) != 0;
+    const int my_row = R16 <= 32 ? ((lane & 16) == 0 ? quarter * 8 + (lane & 7) : 1 << 20)
+                       : pair    ? quarter * 16 + 8 * (lane >> 4) + (lane & 7)
+                                 : quarter * 32 + lane;
+    const bool act = my_row < R;
     const bool quarter_live = (R16 <= 32 ? quarter * 8 : pair ? quarter * 16 : quarter * 32) < R;
     uint32_t wring = 0;  // W ring entries of the phases before the current one (the producer's count)
     uint32_t kvpar = 0;  // per ring slot (bit s): parity of this warp group's next kvready wait
@@ -774,8 +763,22 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
         mwait(&S.kvready[half][sl], (kvpar >> sl) & 1u, err, ab, lim);
         kvpar ^= 1u << sl;
     };
-    int gi = 0, cuse0 = 0, cuse1 = 0, tseg = 0;  // accumulator buffer uses, GEMM tiles so far
-
+    int gi = 0;             // attention units so far
+    uint32_t cuse = 0;      // bit a: parity of accumulator a's next use
+    uint32_t tseg = 0;      // GEMM segments so far
+    auto acc_wait = [&]() -> uint32_t {  // the next segment's accumulator, its MMAs done
+        const uint32_t a = tseg & 1;
+        mwait(&S.acc_full[a], (cuse >> a) & 1u, err, ab, lim);
+        tc_fence_after();
+        return a;
+    };
+    auto acc_release = [&](uint32_t a) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&S.acc_empty[a]);
+        cuse ^= 1u << a;
+        ++tseg;
+    };
     // phase arrival: the CTA's writes of this phase (made visible to thread 0 by the barrier)
     // are released to the other CTAs with the counter increment
     // (x_operand: this phase wrote a GEMM operand that bulk copies of other CTAs will read)
@@ -794,219 +797,216 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
         }
         named_bar_sync(1, kMegaCThreads);
     };
+    // 1/rms of every row from its d / 64 (at most 32) partial sums of squares: a warp per row,
+    // a lane per partial
     auto load_rstd = [&](const float *ssq) {
-        if (ctid < R) {  // every partial load in flight at once (d <= 2048: at most 32)
-            float v[32];
-#pragma unroll
-            for (int t = 0; t < 32; ++t) v[t] = t < d / 64 ? __ldcg(&ssq[(int64_t)t * p.rows_cap + ctid]) : 0.f;
-            float s = 0.f;
-#pragma unroll
-            for (int t = 0; t < 32; ++t) s += v[t];
-            S.rstd[ctid] = rsqrtf(s / (float)d + p.eps);
+        for (int r = cw; r < R; r += 8) {
+            const float s = warp_sum(lane < d / 64 ? __ldcg(&ssq[lane * p.rows_cap + r]) : 0.f);
+            if (lane == 0) S.rstd[r] = rsqrtf(s / (float)d + p.eps);
         }
         named_bar_sync(1, kMegaCThreads);
     };
-    // this CTA's partial tiles: row my_row, columns [128 half, +128) of the tile
-    auto gemm_epi = [&](const GemmPh &g) {
-        SegWalk walk(g);
-        Seg sg;
-        while (walk.next(g, sg)) {
-            wring += (uint32_t)sg.entries();
-            const int t = sg.t, a = tseg & 1;
-            mwait(&S.acc_full[a], (a ? cuse1 : cuse0) & 1, err, ab, lim);
-            tc_fence_after();
-            const int rows_t = sg.n;
-            if (quarter_live && half * 128 < rows_t) {
-                float *dst = p.gpart + ((int64_t)(cta + t) * p.rows_cap + (my_row < R ? my_row : 0)) * kTileN + half * 128;
-#pragma unroll 1
-                for (int cc = 0; cc < 4; ++cc) {
-                    float v[32];
-                    tmem_ld_32x32b_x32(tmem + lane_base + (uint32_t)(a * kTileN + half * 128 + cc * 32), v);
-                    if (pair) {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] += __shfl_xor_sync(0xffffffffu, v[e], 8);
-                    }
-                    if (my_row < R) {
-                        float4 *q = reinterpret_cast<float4 *>(dst + cc * 32);
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) q[e] = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
-                    }
-                }
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&S.acc_empty[a]);
-            if (a) ++cuse1; else ++cuse0;
-            ++tseg;
-        }
+    // contributors of tile t of split-K phase `which`
+    auto contributors = [&](int which, int t) -> int2 {
+        return t < kPlanTiles ? S.tile_cta[which][t] : tile_ctas(p, S.plan[which], which, t, G);
     };
-    // x += (sum of g's partials); x_g = x * gn (blocked hi/lo); per (row, 128-feature
-    // block) sum of squares of x.  g == nullptr: x as it is (embedding).
-    auto fin_resid = [&](const GemmPh *g, const uint16_t *gn, float *ssq) {
-        // unit = (row, 64 features): lane = 2 features; up to 32 contributors' loads in
-        // flight per round, summed in CTA order.  Sums of squares per 128 features: the two
-        // 64-feature halves of a block are adjacent units of the same warp pass
-        const int d64 = d / 64;
-        for (int u = gw; u < R * d64; u += nw) {
-            const int r = u / d64, h64 = u - r * d64;
-            const int f = h64 * 64 + lane * 2;
-            // the norm weights load with the residual and the partials (a layer's norm is not
-            // in L1, and after the residual's store the load could not move ahead of it)
-            const uint32_t gb = __ldg(reinterpret_cast<const unsigned int *>(gn + f));
-            float2 x = __ldcg(reinterpret_cast<const float2 *>(p.x + (int64_t)r * d + f));
-            if (g) {
-                const int gt = f / kTileN, col = f - gt * kTileN;
-                int ca, cb;
-                tile_ctas(*g, gt, ca, cb);
-                float2 s = make_float2(0.f, 0.f);
-                for (int c0 = ca; c0 <= cb; c0 += 32) {
-                    float2 v[32];
+    // Four columns' sum of a tile's partials for one row: lanes 0-15 and 16-31 of a warp take
+    // alternate contributors (up to 16 loads in flight each), then add up.  `off`: row and column
+    // inside a segment, in floats.
+    auto part_sum = [&](int2 ct, int t, int off) -> float4 {
+        const int64_t seg = (int64_t)p.rows_cap * kTileN;
+        const float *src = p.gpart + (int64_t)(ct.x + (lane >> 4) + t) * seg + off;
+        int n = (ct.y - ct.x - (lane >> 4) + 2) >> 1;  // contributors of this half
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+        while (__any_sync(0xffffffffu, n > 0)) {
+            float4 v[16];
 #pragma unroll
-                    for (int k = 0; k < 32; ++k)
-                        v[k] = c0 + k <= cb ? __ldcg(reinterpret_cast<const float2 *>(
-                                                  p.gpart + ((int64_t)(c0 + k + gt) * p.rows_cap + r) * kTileN + col))
-                                            : make_float2(0.f, 0.f);
-#pragma unroll
-                    for (int k = 0; k < 32; ++k) {
-                        s.x += v[k].x; s.y += v[k].y;
-                    }
-                }
-                x.x += s.x; x.y += s.y;
-                *reinterpret_cast<float2 *>(p.x + (int64_t)r * d + f) = x;
+            for (int k = 0; k < 16; ++k) {
+                v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (k < n) v[k] = __ldcg(reinterpret_cast<const float4 *>(src));
+                src += 2 * seg;
             }
-            uint16_t h0, l0, h1, l1;
-            split_bf16(x.x * bf16_to_f32(gb & 0xffff), h0, l0);
-            split_bf16(x.y * bf16_to_f32(gb >> 16), h1, l1);
-            const int64_t off = xblk_off(r, f, R16c);
-            *reinterpret_cast<uint32_t *>(p.xg + off) = (uint32_t)h0 | ((uint32_t)h1 << 16);
-            *reinterpret_cast<uint32_t *>(p.xg + off + kLoOff) = (uint32_t)l0 | ((uint32_t)l1 << 16);
-            const float sq = warp_sum(x.x * x.x + x.y * x.y);
-            if (lane == 0) ssq[(int64_t)h64 * p.rows_cap + r] = sq;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) { s.x += v[k].x; s.y += v[k].y; s.z += v[k].z; s.w += v[k].w; }
+            n -= 16;
         }
+        s.x += __shfl_xor_sync(0xffffffffu, s.x, 16);
+        s.y += __shfl_xor_sync(0xffffffffu, s.y, 16);
+        s.z += __shfl_xor_sync(0xffffffffu, s.z, 16);
+        s.w += __shfl_xor_sync(0xffffffffu, s.w, 16);
+        return s;
     };
 
     // the KV block of each row's current position (its k, v are appended there every layer)
     if (ctid < R) {
         const int pos = __ldg(&p.c.row_pos[ctid]);
+        S.rowpos[ctid] = pos;
         S.rowblk[ctid] = __ldg(&p.c.blk_tab[(int64_t)__ldg(&p.c.row_slot[ctid]) * p.c.nblk_max + pos / kKVPos]);
     }
 
-    // ---------------------------------------------------------------- embedding
-    // (same (row, 64-feature) units and lanes as the finalisation that reads them back)
-    for (int u = gw; u < R * (d / 64); u += nw) {
-        const int r = u / (d / 64), h64 = u - r * (d / 64);
-        int tok = p.c.row_tok[r];
-        if (tok < 0 || tok >= p.V) {
-            if (lane == 0) report_error(err, ERR_BOUNDS);
-            tok = 0;
-        }
-        const int f = h64 * 64 + lane * 2;
-        const uint32_t e = *reinterpret_cast<const uint32_t *>(p.embed + (int64_t)tok * d + f);
-        *reinterpret_cast<float2 *>(p.x + (int64_t)r * d + f) = make_float2(bf16_to_f32(e & 0xffff), bf16_to_f32(e >> 16));
-    }
-    __syncwarp();
-    fin_resid(nullptr, p.attn_norm, p.ssqA);
-    arrive(0, true);
-
-    for (int l = 0; l < p.layers; ++l) {
+    // Steps 3 l + k of layer l: k = 0: residual and attention norm input (embedding, or the
+    // previous layer's down projection), then the q/k/v GEMM; 1: q, k, v and attention, then the
+    // O GEMM; 2: residual and MLP norm input, gate / up, then the down GEMM.  Step 3 L ends with
+    // the final norm input.
+#pragma unroll 1
+    for (int step = 0, l = 0, k = 0;; ++step) {
         const int base = 1 + kPhasesPerLayer * l;
-        const GemmPh gq = gemm_phase(p, l, kPhQKV), go = gemm_phase(p, l, kPhO), gu = gemm_phase(p, l, kPhGU),
-                     gdn = gemm_phase(p, l, kPhDown);
-        // ------------------------------------------------------------ QKV
-        gemm_epi(gq);
-        arrive(base + kPhQKV, false);
-        // ------------------------------------------------------------ q, k, v (once per row)
-        {
-            // unit = (row, head, 64 dims): the head's QKV partials summed in CTA order, times
-            // 1/rms; RoPE on q and k; q pre-scaled by log2(e)/sqrt(hd) for the exp2 softmax;
-            // fp16 q, k, v for the attention phase; k and v appended to the KV cache at the
-            // row's position
+        if (k != 1) {
+            // ---------------------------------------------------- residual, next norm input
+            // x += sum of the GEMM's partials (x = E[tok] at the start); x_g = x * gn as a blocked
+            // hi/lo pair; per (row, 64 features) sum of squares.  Unit = (row, 64 features): lane
+            // % 16 = 4 features; the two halves of the warp split the contributors, then the first
+            // stores x and the hi parts, the second the lo parts.
+            const int which = k == 0 ? kGDown : kGO;
+            const uint16_t *gn = k == 2 ? p.mlp_norm + l * d : l < p.layers ? p.attn_norm + l * d : p.final_norm;
+            float *ssq = k == 2 ? p.ssqM : p.ssqA;
+            if (step > 0) wait_phase(k == 2 ? base + kPhO : base - kPhasesPerLayer + kPhDown);
+            const int d64 = d / 64;
+#pragma unroll 1
+            for (int u = gw; u < R * d64; u += nw) {
+                const int r = u / d64, h64 = u - r * d64;
+                const int f = h64 * 64 + (lane & 15) * 4;
+                // the norm weights load with the residual and the partials
+                const uint2 gb = __ldg(reinterpret_cast<const uint2 *>(gn + f));
+                float4 x;
+                float *xp = p.x + r * d + f;
+                if (step == 0) {
+                    int tok = p.c.row_tok[r];
+                    if (tok < 0 || tok >= p.V) {
+                        if (lane == 0) report_error(err, ERR_BOUNDS);
+                        tok = 0;
+                    }
+                    const uint2 e = __ldg(reinterpret_cast<const uint2 *>(p.embed + (int64_t)tok * d + f));
+                    x = make_float4(bf16_to_f32(e.x & 0xffff), bf16_to_f32(e.x >> 16), bf16_to_f32(e.y & 0xffff),
+                                    bf16_to_f32(e.y >> 16));
+                } else {
+                    x = __ldcg(reinterpret_cast<const float4 *>(xp));
+                    const int t = f / kTileN;
+                    const float4 s = part_sum(contributors(which, t), t, r * kTileN + f - t * kTileN);
+                    x.x += s.x; x.y += s.y; x.z += s.z; x.w += s.w;
+                }
+                uint16_t h[4], lo[4];
+                split_bf16(x.x * bf16_to_f32(gb.x & 0xffff), h[0], lo[0]);
+                split_bf16(x.y * bf16_to_f32(gb.x >> 16), h[1], lo[1]);
+                split_bf16(x.z * bf16_to_f32(gb.y & 0xffff), h[2], lo[2]);
+                split_bf16(x.w * bf16_to_f32(gb.y >> 16), h[3], lo[3]);
+                uint8_t *dst = p.xg + xblk_off(r, f, R16c);
+                float sq = 0.f;
+                if (lane < 16) {
+                    *reinterpret_cast<float4 *>(xp) = x;
+                    *reinterpret_cast<uint2 *>(dst) = pack4(h);
+                    sq = (x.x * x.x + x.y * x.y) + (x.z * x.z + x.w * x.w);
+                } else {
+                    *reinterpret_cast<uint2 *>(dst + kLoOff) = pack4(lo);
+                }
+                sq = warp_sum(sq);
+                if (lane == 0) ssq[h64 * p.rows_cap + r] = sq;
+            }
+            arrive(k == 2 ? base + kPhFinO : base - 1, true);
+            if (l == p.layers) break;
+            if (k == 2) {
+                // ------------------------------------------------ gate / up with SwiGLU
+                // h = silu(r g) * (r u) straight from the accumulator: this CTA's features hold the
+                // whole K, in 16-feature units of 8 gate then 8 up features.  The two warp halves
+                // take alternate pairs of units; each lane of a pair finishes one unit of its row.
+                // The row's 1/rms is read while the MMAs run.
+                wait_phase(base + kPhFinO);
+                load_rstd(p.ssqM);
+                const float rs = act ? S.rstd[my_row] : 0.f;
+                const GemmPlan &g = S.plan[kGGU];
+                SegWalk walk(g);
+                Seg sg;
+#pragma unroll 1
+                while (walk.next(g, sg)) {
+                    wring += (uint32_t)sg.entries();
+                    const uint32_t a = acc_wait();
+                    const int nu = sg.n / kOwnCols;
+                    if (quarter_live) {
+#pragma unroll 1
+                        for (int un = 2 * half; un < nu; un += 4) {
+                            float v[32];
+                            tmem_ld_32x32b_x32(tmem + lane_base + a * kTileN + un * kOwnCols, v);
+                            if (pair) {
+#pragma unroll
+                                for (int e = 0; e < 32; ++e) v[e] += __shfl_xor_sync(0xffffffffu, v[e], 8);
+                            }
+#pragma unroll 1
+                            for (int q = second ? 1 : 0; q < (pair && !second ? 1 : 2); ++q) {
+                                if (!act || un + q >= nu) continue;
+                                uint16_t hh[8], hl[8];
+#pragma unroll
+                                for (int e = 0; e < 8; ++e) {
+                                    const float gv = (q ? v[16 + e] : v[e]) * rs;
+                                    const float uv = (q ? v[24 + e] : v[8 + e]) * rs;
+                                    split_bf16(gv / (1.0f + expf(-gv)) * uv, hh[e], hl[e]);
+                                }
+                                uint8_t *dst = p.hm + xblk_off(my_row, sg.col0 / 2 + (un + q) * 8, R16c);
+                                *reinterpret_cast<uint4 *>(dst) = pack8(hh);
+                                *reinterpret_cast<uint4 *>(dst + kLoOff) = pack8(hl);
+                            }
+                        }
+                    }
+                    acc_release(a);
+                }
+                arrive(base + kPhGU, true);
+            }
+        } else {
+            // -------------------------------------------------------- q, k, v (once per row)
+            // The head's QKV partials summed, times 1/rms; RoPE on q and k; q pre-scaled by
+            // log2(e)/sqrt(hd) for the exp2 softmax; fp16 q, k, v for the attention phase; k and v
+            // appended to the KV cache at the row's position.  Unit = (row, 64 weight rows): a
+            // head's weight rows come in 16s, 8 dims and their rotation partners, so lane % 16
+            // holds 4 dims and lane ^ 2 their partners; the warp's halves split the contributors.
             wait_phase(base + kPhQKV);
-            const int nh = p.H + 2 * p.KVH, dpu = min(hd, 64), upr = hd / dpu;
-            for (int u = gw; u < R * nh * upr; u += nw) {
-                const int r = u / (nh * upr), rem = u - r * nh * upr;
-                // lanes past the unit's dims (head dim 32) repeat lane 0's loads and store nothing:
-                // every lane takes part in the row's sum-of-squares reduction
-                const bool live = 2 * lane < dpu;
-                const int head = rem / upr, d0 = (rem - head * upr) * dpu + (live ? 2 * lane : 0);
-                const bool isq = head < p.H, isk = !isq && head < p.H + p.KVH;
-                const int half_hd = hd >> 1;
-                const int pd0 = d0 < half_hd ? d0 + half_hd : d0 - half_hd;
-                const int f0 = head * hd + d0, t = f0 / kTileN;
-                const int col = f0 - t * kTileN, pcol = head * hd + pd0 - t * kTileN;
-                int ca, cb;
-                tile_ctas(gq, t, ca, cb);
-                // the row's sum-of-squares partials and rotation factors load with the first
-                // batch of QKV partials
-                const float sq = lane < d / 64 ? __ldcg(&p.ssqA[(int64_t)lane * p.rows_cap + r]) : 0.f;
-                const int pos = __ldg(&p.c.row_pos[r]);
-                float2 c0r = make_float2(1.f, 0.f), c1r = c0r;
+            const int n64 = p.nqkv / 64, half_hd = hd >> 1;
+#pragma unroll 1
+            for (int u = gw; u < R * n64; u += nw) {
+                const int r = u / n64, n0 = (u - r * n64) * 64 + (lane & 15) * 4;
+                const int head = n0 / hd, j = n0 - head * hd;
+                const bool isq = head < p.H, isk = !isq && head < p.H + p.KVH, hi = (j & 8) != 0;
+                const int fr = (j >> 4) * 8 + (j & 7), d0 = hi ? fr + half_hd : fr;
+                // the row's sum-of-squares partials and rotation factors load with the QKV partials
+                const float sq = lane < d / 64 ? __ldcg(&p.ssqA[lane * p.rows_cap + r]) : 0.f;
+                const int pos = S.rowpos[r];
+                float4 c0 = make_float4(1.f, 0.f, 1.f, 0.f), c1 = c0;  // (cos, sin) of two dims each
                 if (isq || isk) {
-                    const int fr = d0 < half_hd ? d0 : pd0;
-                    c0r = __ldg(&p.rope[(int64_t)pos * half_hd + fr]);
-                    c1r = __ldg(&p.rope[(int64_t)pos * half_hd + fr + 1]);
+                    const float4 *rp = reinterpret_cast<const float4 *>(p.rope + (int64_t)pos * half_hd + fr);
+                    c0 = __ldg(rp);
+                    c1 = __ldg(rp + 1);
                 }
-                float2 x = make_float2(0.f, 0.f), xp = x;
-                for (int c0 = ca; c0 <= cb; c0 += 16) {  // 16 contributors' loads in flight, CTA order
-                    float2 a[16], b2[16];
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        const bool ok = c0 + k <= cb;
-                        const float *src = p.gpart + ((int64_t)(c0 + k + t) * p.rows_cap + r) * kTileN;
-                        a[k] = ok ? __ldcg(reinterpret_cast<const float2 *>(src + col)) : make_float2(0.f, 0.f);
-                        b2[k] = (ok && !(head >= p.H + p.KVH)) ? __ldcg(reinterpret_cast<const float2 *>(src + pcol))
-                                                               : make_float2(0.f, 0.f);
-                    }
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) {
-                        x.x += a[k].x; x.y += a[k].y;
-                        xp.x += b2[k].x; xp.y += b2[k].y;
-                    }
-                }
+                const int t = n0 / kTileN;
+                const float4 x = part_sum(contributors(kGQKV, t), t, r * kTileN + n0 - t * kTileN);
                 const float rs = rsqrtf(warp_sum(sq) / (float)d + p.eps) * (isq ? p.scale_log2 : 1.f);
-                if (!live) continue;
-                float y0 = x.x, y1 = x.y;
-                if (isq || isk) {  // rotate the pairs (i, i + hd/2)
-                    if (d0 < half_hd) {
-                        y0 = x.x * c0r.x - xp.x * c0r.y;
-                        y1 = x.y * c1r.x - xp.y * c1r.y;
-                    } else {
-                        y0 = x.x * c0r.x + xp.x * c0r.y;
-                        y1 = x.y * c1r.x + xp.y * c1r.y;
-                    }
-                }
-                const uint16_t h0 = f32_to_f16_sat(y0 * rs), h1 = f32_to_f16_sat(y1 * rs);
-                *reinterpret_cast<uint32_t *>(p.qkv16 + (int64_t)r * p.nqkv + head * hd + d0) =
-                    (uint32_t)h0 | ((uint32_t)h1 << 16);
-                if (!isq) {  // the new position's k / v into the cache (blocked layout)
-                    const int kvh = head - p.H - (isk ? 0 : p.KVH);
-                    uint8_t *blk = kv_addr(p, l, S.rowblk[r], kvh);
-                    const int pp = pos % kKVPos;
+                float4 o;
+                o.x = __shfl_xor_sync(0xffffffffu, x.x, 2);
+                o.y = __shfl_xor_sync(0xffffffffu, x.y, 2);
+                o.z = __shfl_xor_sync(0xffffffffu, x.z, 2);
+                o.w = __shfl_xor_sync(0xffffffffu, x.w, 2);
+                const float sg = hi ? 1.f : -1.f;  // rotate the pairs (i, i + hd/2); identity for v
+                const uint16_t h[4] = {f32_to_f16_sat((x.x * c0.x + sg * (o.x * c0.y)) * rs),
+                                       f32_to_f16_sat((x.y * c0.z + sg * (o.y * c0.w)) * rs),
+                                       f32_to_f16_sat((x.z * c1.x + sg * (o.z * c1.y)) * rs),
+                                       f32_to_f16_sat((x.w * c1.z + sg * (o.w * c1.w)) * rs)};
+                const int pp = pos % kKVPos;
+                if (lane < 16) {
+                    *reinterpret_cast<uint2 *>(p.qkv16 + r * p.nqkv + head * hd + d0) = pack4(h);
+                } else if (!isq) {  // the new position's k / v into the cache (blocked layout)
+                    uint8_t *blk = kv_addr(p, l, S.rowblk[r], head - p.H - (isk ? 0 : p.KVH));
                     if (isk) {
-                        *reinterpret_cast<uint32_t *>(blk + kv_k_off(pp, d0)) = (uint32_t)h0 | ((uint32_t)h1 << 16);
+                        *reinterpret_cast<uint2 *>(blk + kv_k_off(pp, d0)) = pack4(h);
                     } else {
-                        *reinterpret_cast<uint16_t *>(blk + kv_v_off(pp, d0)) = h0;
-                        *reinterpret_cast<uint16_t *>(blk + kv_v_off(pp, d0 + 1)) = h1;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) *reinterpret_cast<uint16_t *>(blk + kv_v_off(pp, d0 + e)) = h[e];
                     }
                 }
             }
             arrive(base + kPhFinQ, false);
-        }
-        // ------------------------------------------------------------ attention
-        {
-            int64_t a0, a1;
+            // -------------------------------------------------------- attention
+            int a0, a1;
             att_range(p, S.n_items, a0, a1);
-            const int n = (int)(a1 - a0);
+            const int n = a1 - a0;
             wait_phase(base + kPhFinQ);
-            const bool det_layer = l == min(2, p.layers - 1);
-            if (det_layer && ctid == 0) MEGA_DETAIL(13);
-            if (det_layer && ctid == 0) MEGA_DETAIL(14);
-#define DETAIL(i)                                       \
-    do {                                                \
-        if (det_layer && ctid == 0 && i_unit == 0) MEGA_DETAIL(i); \
-    } while (0)
-            int i_unit = 0;
-            DETAIL(0);
             // units alternate between the two warp groups: group h (warps 3..6 / 7..10, named
             // barrier 2 + h) runs the units (gi + i) & 1 == h, each unit: q in registers, then
             // per KV block scores -> probabilities against the running max -> output sum
@@ -1022,26 +1022,24 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
             uint8_t *pbufs = sQ + half * 2 * kAttPBytes;  // this group's two P buffers
             const int g8 = lane >> 2, t4 = lane & 3;     // mma fragment row / column pair
             const int kst = hd >> 4;                      // k-steps of q.k (16 dims each)
+#pragma unroll 1
             for (int ip = 0; ip < n; ip += 2) {
                 const bool two = ip + 1 < n;
-                const AttUnit ua = att_unit(p, a0 + ip, span);
-                const int nba = ua.nb, nbb = two ? att_unit(p, a0 + ip + 1, span).nb : 0;
                 const int x = ((gi + ip) & 1) == half ? 0 : 1;  // our unit of the pair
+                const AttUnit u = att_unit(p, a0 + ip + (two ? x : 0), span);
+                const int nbo = two ? att_unit(p, a0 + ip + (x ^ 1), span).nb : 0;  // the other unit's blocks
                 const uint32_t w0 = wpair;
-                wpair += 2u * (uint32_t)(nba + nbb);
+                wpair += 2u * (uint32_t)(u.nb + nbo);
                 if (x == 1 && !two) continue;
-                const int i = ip + x;
-                const AttUnit u = x ? att_unit(p, a0 + i, span) : ua;
-                const int jm = min(nba, nbb);
+                const int jm = min(u.nb, nbo);
                 auto ent = [&](int j, int kv) -> uint32_t {
                     return j < jm ? w0 + 4u * j + 2u * kv + x : w0 + 4u * jm + 2u * (j - jm) + kv;
                 };
-                if (half == 0) { i_unit = i; DETAIL(1); }
                 // ---- q of the unit's heads as mma B fragments (q^T: k = dim, n = head g8)
                 uint32_t qf[8][2];
                 {
                     const bool hv = g8 < Gq;
-                    const uint16_t *qh = p.qkv16 + (int64_t)u.row * p.nqkv + (u.kvh * Gq + (hv ? g8 : 0)) * hd + 2 * t4;
+                    const uint16_t *qh = p.qkv16 + u.row * p.nqkv + (u.kvh * Gq + (hv ? g8 : 0)) * hd + 2 * t4;
 #pragma unroll
                     for (int ks = 0; ks < 8; ++ks) {
                         const bool ok = hv && ks < kst;
@@ -1059,12 +1057,12 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                 for (int m = 0; m < 2; ++m)
 #pragma unroll
                     for (int q = 0; q < 4; ++q) o[m][q] = 0.f;
+#pragma unroll 1
                 for (int jb = 0; jb < u.nb; ++jb) {
                     const int nj = min(kKVPos, u.n - jb * kKVPos);
                     const uint32_t ek = ent(jb, 0), ev = ent(jb, 1);
                     kv_wait(ek);
-                    if (half == 0 && jb == 0) DETAIL(2);
-                    const uint32_t kbase = smem_u32(sW + (size_t)(ek % kWSlots) * kSlotBytes);
+                    const uint32_t kbase = smem_u32(sW) + (ek % kWSlots) * kSlotBytes;
                     float sc[2][4];
 #pragma unroll
                     for (int m = 0; m < 2; ++m) {
@@ -1072,13 +1070,14 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                         for (int q = 0; q < 4; ++q) sc[m][q] = 0.f;
                         const int pb0 = 32 * hq + 16 * m;
                         if (pb0 < nj) {  // rows past the copied ones are never read
-                            const int pr = pb0 + (lane & 7) + ((lane >> 3) & 1) * 8;  // ldmatrix row of this lane
+                            const int pr = pb0 + (lane & 15);  // ldmatrix row of this lane
+                            const uint32_t krow = kbase + pr * 128;
+                            const int sw = pr & 7, lh = lane >> 4;
 #pragma unroll
                             for (int ks = 0; ks < 8; ++ks) {
                                 if (ks < kst) {
-                                    const int dim = 16 * ks + (lane >> 4) * 8;
                                     uint32_t a[4];
-                                    ldsm_x4(kbase + (dim >> 6) * 16384 + pr * 128 + ((((dim & 63) >> 3) ^ (pr & 7)) << 4), a);
+                                    ldsm_x4(krow + (ks >> 2) * 16384 + ((((2 * ks & 7) + lh) ^ sw) << 4), a);
                                     mma_f16_16816(sc[m], a, qf[ks][0], qf[ks][1]);
                                 }
                             }
@@ -1086,67 +1085,58 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                     }
                     // scores: sc[m][q] = s(position 32 hq + 16 m + g8 + 8 (q >> 1), head 2 t4 + (q & 1))
                     uint8_t *pbuf = pbufs + (jb & 1) * kAttPBytes;
-                    auto put_p = [&](float (&e)[2][4]) {
-#pragma unroll
-                        for (int m = 0; m < 2; ++m)
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const int pos = 32 * hq + 16 * m + g8 + 8 * (q >> 1);
-                                *reinterpret_cast<uint16_t *>(pbuf + (2 * t4 + (q & 1)) * kAttPRow + 2 * pos) =
-                                    f32_to_f16_sat(e[m][q]);
-                            }
-                    };
                     float e[2][4];
                     bool rebase = jb == 0;
-                    if (!rebase) {
+#pragma unroll 1
+                    for (;;) {
+                        const bool rb = rebase;
+                        if (rb) {  // the block's maximum per head joins the running max
+                            float mx[2] = {-INFINITY, -INFINITY};
+#pragma unroll
+                            for (int m = 0; m < 2; ++m)
+#pragma unroll
+                                for (int q = 0; q < 4; ++q)
+                                    if (32 * hq + 16 * m + g8 + 8 * (q >> 1) < nj) mx[q & 1] = fmaxf(mx[q & 1], sc[m][q]);
+#pragma unroll
+                            for (int kk = 0; kk < 2; ++kk)
+#pragma unroll
+                                for (int o2 = 4; o2 < 32; o2 <<= 1)
+                                    mx[kk] = fmaxf(mx[kk], __shfl_xor_sync(0xffffffffu, mx[kk], o2));
+                            if (g8 == 0) {
+                                S.red[half][hq][2 * t4] = mx[0];
+                                S.red[half][hq][2 * t4 + 1] = mx[1];
+                            }
+                            named_bar_sync(hb, 128);
+#pragma unroll
+                            for (int kk = 0; kk < 2; ++kk) {
+                                const int h = 2 * t4 + kk;
+                                const float mnew = fmaxf(mrun[kk], fmaxf(fmaxf(S.red[half][0][h], S.red[half][1][h]),
+                                                                         fmaxf(S.red[half][2][h], S.red[half][3][h])));
+                                const float alpha = exp2f(mrun[kk] - mnew);  // 0 on the first block
+                                mrun[kk] = mnew;
+                                lthr[kk] *= alpha;
+#pragma unroll
+                                for (int m = 0; m < 2; ++m) {
+                                    o[m][kk] *= alpha;
+                                    o[m][kk + 2] *= alpha;
+                                }
+                            }
+                        }
                         bool over = false;
 #pragma unroll
                         for (int m = 0; m < 2; ++m)
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
-                                const bool valid = 32 * hq + 16 * m + g8 + 8 * (q >> 1) < nj;
-                                e[m][q] = valid ? exp2f(sc[m][q] - mrun[q & 1]) : 0.f;
-                                over |= valid && sc[m][q] - mrun[q & 1] > S.p_headroom;
+                                const int pos = 32 * hq + 16 * m + g8 + 8 * (q >> 1);
+                                const bool valid = pos < nj;
+                                const float s = sc[m][q] - mrun[q & 1];
+                                e[m][q] = valid ? exp2f(s) : 0.f;
+                                over |= valid && s > S.p_headroom;
+                                *reinterpret_cast<uint16_t *>(pbuf + (2 * t4 + (q & 1)) * kAttPRow + 2 * pos) =
+                                    f32_to_f16_sat(e[m][q]);
                             }
-                        put_p(e);
-                        rebase = named_bar_any(hb, 128, over);
-                    }
-                    if (rebase) {  // the block's maximum per head joins the running max
-                        float mx[2] = {-INFINITY, -INFINITY};
-#pragma unroll
-                        for (int m = 0; m < 2; ++m)
-#pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                if (32 * hq + 16 * m + g8 + 8 * (q >> 1) < nj) mx[q & 1] = fmaxf(mx[q & 1], sc[m][q]);
-#pragma unroll
-                        for (int k = 0; k < 2; ++k)
-#pragma unroll
-                            for (int o2 = 4; o2 < 32; o2 <<= 1) mx[k] = fmaxf(mx[k], __shfl_xor_sync(0xffffffffu, mx[k], o2));
-                        if (g8 == 0) {
-                            S.red[half][hq][2 * t4] = mx[0];
-                            S.red[half][hq][2 * t4 + 1] = mx[1];
-                        }
-                        named_bar_sync(hb, 128);
-                        float alpha[2];
-#pragma unroll
-                        for (int k = 0; k < 2; ++k) {
-                            const int h = 2 * t4 + k;
-                            const float mnew = fmaxf(mrun[k], fmaxf(fmaxf(S.red[half][0][h], S.red[half][1][h]),
-                                                                    fmaxf(S.red[half][2][h], S.red[half][3][h])));
-                            alpha[k] = exp2f(mrun[k] - mnew);  // 0 on the first block
-                            mrun[k] = mnew;
-                            lthr[k] *= alpha[k];
-                        }
-#pragma unroll
-                        for (int m = 0; m < 2; ++m)
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                o[m][q] *= alpha[q & 1];
-                                const bool valid = 32 * hq + 16 * m + g8 + 8 * (q >> 1) < nj;
-                                e[m][q] = valid ? exp2f(sc[m][q] - mrun[q & 1]) : 0.f;
-                            }
-                        put_p(e);
-                        named_bar_sync(hb, 128);
+                        rebase = named_bar_any(hb, 128, over) && !rb;
+                        if (!rebase) break;
                     }
                     // every warp has read the K block: its ring slot goes back to the producer
                     if (ht == 0) mbar_arrive(&S.wempty[ek % kWSlots]);
@@ -1154,27 +1144,26 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                     for (int m = 0; m < 2; ++m)
 #pragma unroll
                         for (int q = 0; q < 4; ++q) lthr[q & 1] += e[m][q];
-                    if (half == 0 && jb == 0) DETAIL(3);
                     // ---- O^T += V^T P^T over the block's positions (k-steps of 16)
                     kv_wait(ev);
-                    const uint32_t vbase = smem_u32(sW + (size_t)(ev % kWSlots) * kSlotBytes);
-                    const uint32_t pbase = smem_u32(pbuf);
+                    const uint32_t vbase = smem_u32(sW) + (ev % kWSlots) * kSlotBytes;
+                    const uint32_t pbase = smem_u32(pbuf) + (lane & 7) * kAttPRow + 16 * (lane >> 3);
                     const int kpv = (nj + 15) >> 4;
 #pragma unroll
                     for (int ks = 0; ks < 8; ks += 2) {
                         if (ks < kpv) {
                             uint32_t bq[4];  // P^T fragments of k-steps ks, ks + 1 (rows: heads 0..7)
-                            ldsm_x4(pbase + (lane & 7) * kAttPRow + (16 * ks + 8 * (lane >> 3)) * 2, bq);
+                            ldsm_x4(pbase + 32 * ks, bq);
 #pragma unroll
                             for (int m = 0; m < 2; ++m) {
-                                const int dr = 16 * (hq + 4 * m) + (lane & 7) + ((lane >> 3) & 1) * 8;  // V^T row (dim)
                                 if (16 * (hq + 4 * m) < hd) {
+                                    const int dr = 16 * (hq + 4 * m) + (lane & 15);  // V^T row (dim)
 #pragma unroll
                                     for (int kk = 0; kk < 2; ++kk) {
                                         if (ks + kk < kpv) {
-                                            const int pos = 16 * (ks + kk) + (lane >> 4) * 8;
+                                            const int gr = 2 * ((ks + kk) & 3) + (lane >> 4);
                                             uint32_t a[4];
-                                            ldsm_x4(vbase + (pos >> 6) * 16384 + dr * 128 + ((((pos & 63) >> 3) ^ (dr & 7)) << 4), a);
+                                            ldsm_x4(vbase + (ks >> 2) * 16384 + dr * 128 + ((gr ^ (dr & 7)) << 4), a);
                                             mma_f16_16816(o[m], a, bq[2 * kk], bq[2 * kk + 1]);
                                         }
                                     }
@@ -1185,94 +1174,96 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                     named_bar_sync(hb, 128);  // every warp has read the V^T block
                     if (ht == 0) mbar_arrive(&S.wempty[ev % kWSlots]);
                 }
-                if (half == 0) DETAIL(4);
                 // ---- row sums: heads 2 t4, 2 t4 + 1 over the warp (lanes of equal t4), then
                 // over the group's warps
                 float lrun[2];
-                {
 #pragma unroll
-                    for (int k = 0; k < 2; ++k)
+                for (int kk = 0; kk < 2; ++kk)
 #pragma unroll
-                        for (int o2 = 4; o2 < 32; o2 <<= 1) lthr[k] += __shfl_xor_sync(0xffffffffu, lthr[k], o2);
-                    if (g8 == 0) {
-                        S.red2[half][hq][2 * t4] = lthr[0];
-                        S.red2[half][hq][2 * t4 + 1] = lthr[1];
-                    }
-                    named_bar_sync(hb, 128);
+                    for (int o2 = 4; o2 < 32; o2 <<= 1) lthr[kk] += __shfl_xor_sync(0xffffffffu, lthr[kk], o2);
+                if (g8 == 0) {
+                    S.red2[half][hq][2 * t4] = lthr[0];
+                    S.red2[half][hq][2 * t4 + 1] = lthr[1];
+                }
+                named_bar_sync(hb, 128);
 #pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        const int h = 2 * t4 + k;
-                        lrun[k] = (S.red2[half][0][h] + S.red2[half][1][h]) + (S.red2[half][2][h] + S.red2[half][3][h]);
-                    }
+                for (int kk = 0; kk < 2; ++kk) {
+                    const int h = 2 * t4 + kk;
+                    lrun[kk] = (S.red2[half][0][h] + S.red2[half][1][h]) + (S.red2[half][2][h] + S.red2[half][3][h]);
                 }
                 // ---- output (single split) or partial + split merge.  o[m][q]: O^T(dim
                 // 16 (hq + 4 m) + g8 + 8 (q >> 1), head 2 t4 + (q & 1))
-                {
-                    const int dd = quarter * 32 + lane;  // output dim of this thread in the merge
-                    if (u.nsplit == 1) {
+                const bool single = u.nsplit == 1;
+                float *mine = p.part + ((int64_t)u.item * p.KVH + u.kvh) * Gq * (hd + 2);
 #pragma unroll
-                        for (int m = 0; m < 2; ++m)
+                for (int m = 0; m < 2; ++m)
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const int dim = 16 * (hq + 4 * m) + g8 + 8 * (q >> 1), h = 2 * t4 + (q & 1);
-                                if (dim < hd && h < Gq)
-                                    store_hilo(p.att, xblk_off(u.row, (u.kvh * Gq + h) * hd + dim, R16c),
-                                               o[m][q] / lrun[q & 1]);
-                            }
-                    } else {
-                        float *mine = p.part + ((int64_t)u.item * p.KVH + u.kvh) * Gq * (hd + 2);
-#pragma unroll
-                        for (int m = 0; m < 2; ++m)
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const int dim = 16 * (hq + 4 * m) + g8 + 8 * (q >> 1), h = 2 * t4 + (q & 1);
-                                if (dim < hd && h < Gq) mine[h * (hd + 2) + 2 + dim] = o[m][q];
-                            }
-                        if (hq == 0 && g8 == 0) {
-#pragma unroll
-                            for (int k = 0; k < 2; ++k) {
-                                const int h = 2 * t4 + k;
-                                if (h < Gq) {
-                                    mine[h * (hd + 2)] = mrun[k];
-                                    mine[h * (hd + 2) + 1] = lrun[k];
-                                }
+                    for (int q = 0; q < 4; ++q) {
+                        const int dim = 16 * (hq + 4 * m) + g8 + 8 * (q >> 1), h = 2 * t4 + (q & 1);
+                        if (dim < hd && h < Gq) {
+                            if (single) {
+                                uint16_t hv, lv;
+                                split_bf16(o[m][q] / lrun[q & 1], hv, lv);
+                                uint8_t *dst = p.att + xblk_off(u.row, (u.kvh * Gq + h) * hd + dim, R16c);
+                                *reinterpret_cast<uint16_t *>(dst) = hv;
+                                *reinterpret_cast<uint16_t *>(dst + kLoOff) = lv;
+                            } else {
+                                mine[h * (hd + 2) + 2 + dim] = o[m][q];
                             }
                         }
-                        named_bar_sync(hb, 128);
-                        if (half == 0) DETAIL(5);
-                        if (ht == 0) {  // one acquire-release count: publishes this split, sees the others
-                            const int old = atom_add_acq_rel_gpu(&p.att_cnt[u.row * p.KVH + u.kvh], 1);
-                            S.last_flag2[half] = old == u.nsplit - 1;
-                            if (S.last_flag2[half]) p.att_cnt[u.row * p.KVH + u.kvh] = 0;
+                    }
+                if (single) continue;
+                if (hq == 0 && g8 == 0) {
+#pragma unroll
+                    for (int kk = 0; kk < 2; ++kk) {
+                        const int h = 2 * t4 + kk;
+                        if (h < Gq) {
+                            mine[h * (hd + 2)] = mrun[kk];
+                            mine[h * (hd + 2) + 1] = lrun[kk];
                         }
-                        named_bar_sync(hb, 128);
-                        if (half == 0) DETAIL(6);
-                        if (S.last_flag2[half]) {  // merge the row's splits in split order
-                            const int ns = min(u.nsplit, kMegaMaxSplits);
-                            const int64_t sp_stride = (int64_t)p.KVH * Gq * (hd + 2);
-                            const float *pbase = p.part + ((int64_t)__ldg(&p.c.row_item0[u.row]) * p.KVH + u.kvh) * Gq * (hd + 2);
-                            // the first four splits' outputs (thread dd: dim dd of every head) load
-                            // together with the split weights' inputs: one round trip for both
-                            const float *src = pbase + 2 + dd;
-                            float vpre[4][8];
+                    }
+                }
+                named_bar_sync(hb, 128);
+                if (ht == 0) {  // one acquire-release count: publishes this split, sees the others
+                    const int old = atom_add_acq_rel_gpu(&p.att_cnt[u.row * p.KVH + u.kvh], 1);
+                    S.last_flag2[half] = old == u.nsplit - 1;
+                    if (S.last_flag2[half]) p.att_cnt[u.row * p.KVH + u.kvh] = 0;
+                }
+                named_bar_sync(hb, 128);
+                if (S.last_flag2[half]) {  // merge the row's splits in split order
+                    const int ns = min(u.nsplit, kMegaMaxSplits);
+                    const int dd = quarter * 32 + lane;  // output dim of this thread
+                    const int sp_stride = p.KVH * Gq * (hd + 2), hs = hd + 2;
+                    const float *pb = p.part + ((int64_t)__ldg(&p.c.row_item0[u.row]) * p.KVH + u.kvh) * Gq * hs;
+                    float acc[8];
 #pragma unroll
-                            for (int q = 0; q < 4; ++q)
+                    for (int g = 0; g < 8; ++g) acc[g] = 0.f;
+#pragma unroll 1
+                    for (int s0 = 0; s0 < ns; s0 += 4) {
+                        // four splits' outputs in flight (thread dd: dim dd of every head); the first
+                        // four load together with the split weights' inputs: one round trip for both
+                        const float *src = pb + s0 * sp_stride + 2 + dd;
+                        float v[4][8];
 #pragma unroll
-                                for (int g = 0; g < 8; ++g)
-                                    vpre[q][g] = (dd < hd && g < Gq && q < ns) ? __ldcg(src + q * sp_stride + g * (hd + 2)) : 0.f;
-                            // split weights 2^(m_s - M) and the total weight L per head (warp hq: heads hq, hq + 4)
+                        for (int q = 0; q < 4; ++q, src += sp_stride)
+#pragma unroll
+                            for (int g = 0; g < 8; ++g)
+                                v[q][g] = (dd < hd && g < Gq && s0 + q < ns) ? __ldcg(src + g * hs) : 0.f;
+                        if (s0 == 0) {
+                            // split weights 2^(m_s - M), total weight L per head (warp hq: heads hq, hq + 4)
+#pragma unroll 1
                             for (int g = hq; g < Gq; g += 4) {
                                 float ms[3], ls[3];
                                 float Mx = -INFINITY;
 #pragma unroll
                                 for (int q = 0; q < 3; ++q) {
                                     const int sp = lane + 32 * q;
-                                    ms[q] = sp < ns ? __ldcg(pbase + sp * sp_stride + g * (hd + 2)) : -INFINITY;
-                                    ls[q] = sp < ns ? __ldcg(pbase + sp * sp_stride + g * (hd + 2) + 1) : 0.f;
+                                    ms[q] = sp < ns ? __ldcg(pb + sp * sp_stride + g * hs) : -INFINITY;
+                                    ls[q] = sp < ns ? __ldcg(pb + sp * sp_stride + g * hs + 1) : 0.f;
                                     Mx = fmaxf(Mx, ms[q]);
                                 }
 #pragma unroll
-                                for (int o = 16; o > 0; o >>= 1) Mx = fmaxf(Mx, __shfl_xor_sync(0xffffffffu, Mx, o));
+                                for (int o2 = 16; o2 > 0; o2 >>= 1) Mx = fmaxf(Mx, __shfl_xor_sync(0xffffffffu, Mx, o2));
                                 float L = 0.f;
 #pragma unroll
                                 for (int q = 0; q < 3; ++q) {
@@ -1285,208 +1276,164 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                                 if (lane == 0) S.ml[half][g] = L;
                             }
                             named_bar_sync(hb, 128);
-                            if (dd < hd) {  // thread dd: output dim dd of every head
-                                float acc[8];
-#pragma unroll
-                                for (int g = 0; g < 8; ++g) acc[g] = 0.f;
-#pragma unroll
-                                for (int q = 0; q < 4; ++q)
-#pragma unroll
-                                    for (int g = 0; g < 8; ++g) acc[g] += (g < Gq && q < ns ? S.mw[half][g][q] : 0.f) * vpre[q][g];
-                                for (int s0 = 4; s0 < ns; s0 += 4) {  // the rest, four splits' loads in flight
-                                    float v[4][8];
-#pragma unroll
-                                    for (int q = 0; q < 4; ++q)
-#pragma unroll
-                                        for (int g = 0; g < 8; ++g)
-                                            v[q][g] = (g < Gq && s0 + q < ns) ? __ldcg(src + (s0 + q) * sp_stride + g * (hd + 2)) : 0.f;
-#pragma unroll
-                                    for (int q = 0; q < 4; ++q)
-#pragma unroll
-                                        for (int g = 0; g < 8; ++g)
-                                            acc[g] += (g < Gq && s0 + q < ns ? S.mw[half][g][s0 + q] : 0.f) * v[q][g];
-                                }
-#pragma unroll
-                                for (int g = 0; g < 8; ++g)
-                                    if (g < Gq)
-                                        store_hilo(p.att, xblk_off(u.row, (u.kvh * Gq + g) * hd + dd, R16c),
-                                                   acc[g] / S.ml[half][g]);
-                            }
                         }
-                        named_bar_sync(hb, 128);
-                        if (half == 0) DETAIL(7);
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+#pragma unroll
+                            for (int g = 0; g < 8; ++g)
+                                if (g < Gq && s0 + q < ns) acc[g] += S.mw[half][g][s0 + q] * v[q][g];
+                    }
+                    if (dd < hd) {
+#pragma unroll
+                        for (int g = 0; g < 8; ++g)
+                            if (g < Gq) {
+                                uint16_t hv, lv;
+                                split_bf16(acc[g] / S.ml[half][g], hv, lv);
+                                uint8_t *dst = p.att + xblk_off(u.row, (u.kvh * Gq + g) * hd + dd, R16c);
+                                *reinterpret_cast<uint16_t *>(dst) = hv;
+                                *reinterpret_cast<uint16_t *>(dst + kLoOff) = lv;
+                            }
                     }
                 }
+                named_bar_sync(hb, 128);
             }
             wring = wpair;
             gi += n;
-            i_unit = 0;
-            DETAIL(8);
             arrive(base + kPhAtt, true);
-            DETAIL(9);
-#undef DETAIL
         }
-        // ------------------------------------------------------------ O projection
-        gemm_epi(go);
-        arrive(base + kPhO, false);
-        // ------------------------------------------------------------ residual, MLP norm input
-        wait_phase(base + kPhO);
-        if (l == min(2, p.layers - 1) && ctid == 0) MEGA_DETAIL(10);
-        fin_resid(&go, p.mlp_norm + (int64_t)l * d, p.ssqM);
-        if (l == min(2, p.layers - 1) && ctid == 0) MEGA_DETAIL(11);
-        arrive(base + kPhFinO, true);
-        if (l == min(2, p.layers - 1) && ctid == 0) MEGA_DETAIL(12);
-        // ------------------------------------------------------------ gate / up
-        // h = silu(r g) * (r u) straight from the accumulator: this CTA's features hold the whole
-        // K, in 16-feature units of 8 gate then 8 up features (the two warp halves take alternate
-        // pairs of units).  The row's 1/rms is read while the MMAs run.
+        // ---------------------------------------------------------------- split-K GEMM
+        // this CTA's partial tiles: row my_row, columns [128 half, +128) of the tile
         {
-            wait_phase(base + kPhFinO);
-            load_rstd(p.ssqM);
-            const float rs = my_row_any < R ? S.rstd[my_row_any] : 0.f;
-            SegWalk walk(gu);
+            const GemmPlan &g = S.plan[k];
+            SegWalk walk(g);
             Seg sg;
-            while (walk.next(gu, sg)) {
-                wring += (uint32_t)sg.entries();
-                const int a = tseg & 1, nu = sg.n / kOwnCols;
-                mwait(&S.acc_full[a], (a ? cuse1 : cuse0) & 1, err, ab, lim);
-                tc_fence_after();
-                if (quarter_live) {
 #pragma unroll 1
-                    for (int un = 2 * half; un < nu; un += 4) {
+            while (walk.next(g, sg)) {
+                wring += (uint32_t)sg.entries();
+                const uint32_t a = acc_wait();
+                if (quarter_live && half * 128 < sg.n) {
+                    float *dst = p.gpart + ((cta + sg.t) * p.rows_cap + (act ? my_row : 0)) * kTileN + half * 128;
+#pragma unroll 1
+                    for (int cc = 0; cc < 4; ++cc) {
                         float v[32];
-                        tmem_ld_32x32b_x32(tmem + lane_base + (uint32_t)(a * kTileN + un * kOwnCols), v);
-                        if (pair) {  // hi + lo accumulators; then each lane of the pair keeps one unit
+                        tmem_ld_32x32b_x32(tmem + lane_base + a * kTileN + half * 128 + cc * 32, v);
+                        if (pair) {
 #pragma unroll
                             for (int e = 0; e < 32; ++e) v[e] += __shfl_xor_sync(0xffffffffu, v[e], 8);
                         }
+#pragma unroll 1
+                        for (int q = second ? 1 : 0; q < (pair && !second ? 1 : 2); ++q) {  // 16 columns each
+                            if (!act) continue;
+                            float4 *o = reinterpret_cast<float4 *>(dst + cc * 32 + q * 16);
 #pragma unroll
-                        for (int q = 0; q < 2; ++q) {
-                            if (pair ? q > 0 : false) break;
-                            const bool second = pair ? (lane & 8) != 0 : q == 1;
-                            if (my_row_any < R && un + (second ? 1 : 0) < nu) {
-                                uint16_t hh[8], hl[8];
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) {
-                                    const float gv = (second ? v[16 + e] : v[e]) * rs;
-                                    const float uv = (second ? v[24 + e] : v[8 + e]) * rs;
-                                    split_bf16(gv / (1.0f + expf(-gv)) * uv, hh[e], hl[e]);
-                                }
-                                const int f = sg.col0 / 2 + (un + (second ? 1 : 0)) * 8;
-                                const int64_t off = xblk_off(my_row_any, f, R16c);
-                                *reinterpret_cast<uint4 *>(p.hm + off) = pack8(hh);
-                                *reinterpret_cast<uint4 *>(p.hm + off + kLoOff) = pack8(hl);
-                            }
+                            for (int e = 0; e < 4; ++e)
+                                o[e] = q ? make_float4(v[16 + 4 * e], v[17 + 4 * e], v[18 + 4 * e], v[19 + 4 * e])
+                                         : make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
                         }
                     }
                 }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&S.acc_empty[a]);
-                if (a) ++cuse1; else ++cuse0;
-                ++tseg;
+                acc_release(a);
             }
-            arrive(base + kPhGU, true);
+            arrive(base + (k == 0 ? kPhQKV : k == 1 ? kPhO : kPhDown), false);
         }
-        // ------------------------------------------------------------ down
-        gemm_epi(gdn);
-        arrive(base + kPhDown, false);
-        // ------------------------------------------------------------ residual, next norm input
-        wait_phase(base + kPhDown);
-        fin_resid(&gdn, (l + 1 < p.layers) ? p.attn_norm + (int64_t)(l + 1) * d : p.final_norm, p.ssqA);
-        arrive(base + kPhFinD, true);
+        if (++k == 3) {
+            k = 0;
+            ++l;
+        }
     }
 
     // ---------------------------------------------------------------- lm_head + Gumbel-max
     // logits = (x_g W_lm^T) / rms(x) for the live rows, fused with the temperature-1 sampler:
-    // each thread scans its row's 128 columns of a tile in increasing token order, adds the
+    // each thread scans its columns of a tile in increasing token order, adds the
     // Gumbel noise g(row key, token) and keeps the first maximum of logit + g; the per (row,
     // tile, half) maxima go to the bookkeeping kernel, which takes the row's argmax (ties to
     // the lowest token id).  Products and sums are rounded separately (no contraction), as
     // the sampler on stored logits would do them.  The logits themselves are written only
     // when requested (teacher forcing).
-    {
-        wait_phase(kPhasesPerLayer * p.layers);
-        load_rstd(p.ssqA);
-        const GemmPh g = gemm_phase(p, p.layers, 0);
-        const bool act = my_row < R;
-        const float rs = act ? S.rstd[my_row] : 0.f;
-        const uint64_t seed = act ? __ldg(&p.c.row_seed[my_row]) : 0ull;
-        const int nparts = 2 * g.T;
-        float best = -INFINITY;  // running over this thread's tiles (its row and half)
-        int bi = 0x7fffffff;
-        SegWalk walk(g);
-        Seg sg;
-        while (walk.next(g, sg)) {
-            const int t = sg.t;
-            const int a = tseg & 1;
-            mwait(&S.acc_full[a], (a ? cuse1 : cuse0) & 1, err, ab, lim);
-            tc_fence_after();
-            if (quarter_live && half * 128 < sg.n) {
-                const int n0 = t * kTileN + half * 128;
-                float *dst = p.logits + (int64_t)(act ? my_row : 0) * p.V + n0;
-                const float best0 = best;  // the maximum over this thread's earlier tiles
+    wait_phase(kPhasesPerLayer * p.layers);
+    load_rstd(p.ssqA);
+    const GemmPlan &g = S.plan[kGLM];
+    const float rs = act ? S.rstd[my_row] : 0.f;
+    const uint64_t seed = act ? __ldg(&p.c.row_seed[my_row]) : 0ull;
+    const int nparts = 2 * ((g.N + kTileN - 1) / kTileN);
+    float best = -INFINITY;  // running over this thread's tiles (its row and columns)
+    int bi = 0x7fffffff;
+    SegWalk walk(g);
+    Seg sg;
 #pragma unroll 1
-                for (int cc = 0; cc < 4; ++cc) {
-                    float v[32];
-                    tmem_ld_32x32b_x32(tmem + lane_base + (uint32_t)(a * kTileN + half * 128 + cc * 32), v);
-                    if (pair) {
+    while (walk.next(g, sg)) {
+        const uint32_t a = acc_wait();
+        if (quarter_live && half * 128 < sg.n) {
+            const float best0 = best;  // the maximum over this thread's earlier tiles
+#pragma unroll 1
+            for (int cc = 0; cc < 4; ++cc) {
+                float v[32];
+                tmem_ld_32x32b_x32(tmem + lane_base + a * kTileN + half * 128 + cc * 32, v);
+                if (pair) {
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] += __shfl_xor_sync(0xffffffffu, v[e], 8);
-                    }
-                    if (act) {
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = __fmul_rn(v[e], rs);
-                        if (p.write_logits) {
-                            float4 *q = reinterpret_cast<float4 *>(dst + cc * 32);
-#pragma unroll
-                            for (int e = 0; e < 8; ++e) q[e] = make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
-                        }
-                        // Only tokens whose noise could lift them over the best so far are
-                        // evaluated exactly: g(u) increases with u = (top 24 hash bits + 0.5) / 2^24,
-                        // so v_e + g(u_e) > best needs u_e > exp(-exp(-(best - max_e v_e))); the
-                        // cut is taken 1e-3 lower in g and 4 codes lower in the 24-bit u, far
-                        // beyond the rounding of the float evaluation, so no candidate is lost.
-                        // `best` runs over all of this thread's tiles: a (tile, half) whose
-                        // tokens cannot beat an earlier tile's maximum reports -inf, which the
-                        // row's argmax ignores (ties go to the lower token id either way).
-                        float vmax = v[0];
-#pragma unroll
-                        for (int e = 1; e < 32; ++e) vmax = fmaxf(vmax, v[e]);
-                        const float ureq = expf(-expf(-(best - vmax - 1e-3f)));  // 0 while best = -inf
-                        const float cut = ureq * 16777216.0f - 4.0f;
-                        const uint32_t thr = cut > 0.f ? (uint32_t)cut : 0u;
-                        const int nb = n0 + cc * 32;
-                        uint32_t cand = 0;
-#pragma unroll
-                        for (int e = 0; e < 32; ++e)
-                            cand |= (uint32_t)((uint32_t)(splitmix_at(seed, (uint64_t)(nb + e) + 1) >> 40) >= thr) << e;
-                        while (cand) {  // candidates in increasing token order: the first maximum is kept
-                            const int e = __ffs(cand) - 1;
-                            cand &= cand - 1;
-                            float ve = v[0];
-#pragma unroll
-                            for (int k = 1; k < 32; ++k) ve = (k == e) ? v[k] : ve;
-                            const float z = __fadd_rn(ve, gumbel_from_hash(splitmix_at(seed, (uint64_t)(nb + e) + 1)));
-                            if (z > best) { best = z; bi = nb + e; }
-                        }
-                    }
+                    for (int e = 0; e < 32; ++e) v[e] += __shfl_xor_sync(0xffffffffu, v[e], 8);
                 }
-                if (act) {  // this (tile, half)'s maximum if it beats the earlier tiles, else -inf
-                    const bool won = best > best0;
-                    p.c.arg_val[(int64_t)my_row * nparts + 2 * t + half] = won ? best : -INFINITY;
-                    p.c.arg_idx[(int64_t)my_row * nparts + 2 * t + half] = won ? bi : 0x7fffffff;
+                // 16 columns at a time; each lane of a pair takes one half of the 32
+#pragma unroll 1
+                for (int q = second ? 1 : 0; q < (pair && !second ? 1 : 2); ++q) {
+                    if (!act) continue;
+                    float z[16];
+#pragma unroll
+                    for (int e = 0; e < 16; ++e) z[e] = __fmul_rn(q ? v[16 + e] : v[e], rs);
+                    const int nb = sg.col0 + half * 128 + cc * 32 + q * 16;
+                    if (p.write_logits) {
+                        float4 *o = reinterpret_cast<float4 *>(p.logits + (int64_t)my_row * p.V + nb);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) o[e] = make_float4(z[4 * e], z[4 * e + 1], z[4 * e + 2], z[4 * e + 3]);
+                    }
+                    // Only tokens whose noise could lift them over the best so far are
+                    // evaluated exactly: g(u) increases with u = (top 24 hash bits + 0.5) / 2^24,
+                    // so z_e + g(u_e) > best needs u_e > exp(-exp(-(best - max_e z_e))); the
+                    // cut is taken 1e-3 lower in g and 4 codes lower in the 24-bit u, far
+                    // beyond the rounding of the float evaluation, so no candidate is lost.
+                    // `best` runs over all of this thread's tiles: a (tile, half) whose
+                    // tokens cannot beat an earlier tile's maximum reports -inf, which the
+                    // row's argmax ignores (ties go to the lower token id either way).
+                    float vmax = z[0];
+#pragma unroll
+                    for (int e = 1; e < 16; ++e) vmax = fmaxf(vmax, z[e]);
+                    const float ureq = expf(-expf(-(best - vmax - 1e-3f)));  // 0 while best = -inf
+                    const float cut = ureq * 16777216.0f - 4.0f;
+                    const uint32_t thr = cut > 0.f ? (uint32_t)cut : 0u;
+                    uint32_t cand = 0;
+#pragma unroll
+                    for (int e = 0; e < 16; ++e)
+                        cand |= (uint32_t)((uint32_t)(splitmix_at(seed, (uint64_t)(nb + e) + 1) >> 40) >= thr) << e;
+#pragma unroll 1
+                    while (cand) {  // candidates in increasing token order: the first maximum is kept
+                        const int e = __ffs(cand) - 1;
+                        cand &= cand - 1;
+                        float ze = z[0];
+#pragma unroll
+                        for (int i = 1; i < 16; ++i) ze = (i == e) ? z[i] : ze;
+                        const float zg = __fadd_rn(ze, gumbel_from_hash(splitmix_at(seed, (uint64_t)(nb + e) + 1)));
+                        if (zg > best) { best = zg; bi = nb + e; }
+                    }
                 }
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&S.acc_empty[a]);
-            if (a) ++cuse1; else ++cuse0;
-            ++tseg;
+            // this (tile, half)'s maximum if it beats the earlier tiles, else -inf; the lanes of a
+            // pair hold disjoint columns (ties to the lower id)
+            float wv = best > best0 ? best : -INFINITY;
+            int wi = best > best0 ? bi : 0x7fffffff;
+            if (pair) {
+                const float ov = __shfl_xor_sync(0xffffffffu, wv, 8);
+                const int oi = __shfl_xor_sync(0xffffffffu, wi, 8);
+                if (ov > wv || (ov == wv && oi < wi)) { wv = ov; wi = oi; }
+            }
+            if (act && !second) {
+                p.c.arg_val[my_row * nparts + 2 * sg.t + half] = wv;
+                p.c.arg_idx[my_row * nparts + 2 * sg.t + half] = wi;
+            }
         }
-        named_bar_sync(1, kMegaCThreads);
-        if (ctid == 0) MEGA_STAMP(1 + kPhasesPerLayer * p.layers, 0);
+        acc_release(a);
     }
+    named_bar_sync(1, kMegaCThreads);
+    if (ctid == 0) MEGA_STAMP(1 + kPhasesPerLayer * p.layers, 0);
 }
 
 // ------------------------------------------------------------------------------ kernel
@@ -1541,8 +1488,17 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
         S.last_flag = 0;
         fence_mbar_init();
     }
-    if (threadIdx.x == 0) MEGA_STAMP(p.n_stamp_ph - kDetailRows - 1, 0);  // kernel start
+    if (threadIdx.x == 0) MEGA_STAMP(p.n_stamp_ph - 1, 0);  // kernel start
     const uint64_t t_start = globaltimer_ns();
+    // the launch's GEMM shares and the contributors of the split-K tiles
+    if (threadIdx.x >= 32 * 3 && threadIdx.x < 32 * 3 + 5)
+        make_plan(p, S.plan[threadIdx.x - 96], threadIdx.x - 96, blockIdx.x, gridDim.x);
+    if (threadIdx.x >= 128 && threadIdx.x < 128 + 3 * kPlanTiles) {
+        const int which = (threadIdx.x - 128) / kPlanTiles, t = (threadIdx.x - 128) % kPlanTiles;
+        GemmPlan g;
+        make_plan(p, g, which, 0, gridDim.x);
+        if (t < (g.N + kTileN - 1) / kTileN) S.tile_cta[which][t] = tile_ctas(p, g, which, t, gridDim.x);
+    }
     if (warp == 1) {
         tmem_alloc(&S.tmem_base, kTmemCols);
         tmem_relinquish();
@@ -1558,11 +1514,11 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
             fill_att_blocks(p, S, lane);
             mega_w_producer(p, S, sW);
         } else if (warp == 1) {
-            mega_mma(p, S, sW, sX, sQ, sP, tmem);
+            mega_mma(p, S, sW, sX, tmem);
         } else if (warp == 2) {
             mega_x_producer(p, S, sX);
         } else {
-            mega_compute(p, S, sW, sQ, sP, tmem);
+            mega_compute(p, S, sW, sQ, tmem);
         }
     }
     tc_fence_before();
@@ -1580,15 +1536,27 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
 }
 
 // ------------------------------------------------------------------------------ layout kernels
-// Row-major W [N][K] (bf16) -> chunk-major blocks: k-chunk kc holds its 64 columns of every row
-// (128 bytes a row), 16-byte granule j of row r stored at granule j ^ (r % 8), so any run of rows
-// of a chunk that starts at a multiple of 8 is one contiguous piece.  K must be a multiple of 64.
-static __global__ void block_weights_kernel(const uint16_t *src, uint8_t *dst, int N, int K) {
+// Rows of a source matrix in the blocked matrix that it is a part of.
+enum : int {
+    kRowsPlain = 0,  // row + row0
+    kRowsHead = 1,   // q, k, v: each head's rows in qkv_row order, + row0
+    kRowsAlt = 2,    // gate, up: alternate blocks of 8 rows (row0 = 0: gate, 8: up)
+};
+// Row-major W [n_src][K] (bf16, 16-byte aligned) into chunk-major blocks of a matrix of N rows:
+// k-chunk kc holds its 64 columns of every row (128 bytes a row), 16-byte granule j of row r stored
+// at granule j ^ (r % 8), so any run of rows of a chunk that starts at a multiple of 8 is one
+// contiguous piece.  K must be a multiple of 64.
+static __global__ void block_weights_kernel(const uint16_t *src, uint8_t *dst, int n_src, int K, int N, int rows, int row0,
+                                            int head_dim) {
     const int gpr = K / 8;
-    const int64_t total = (int64_t)N * gpr;
+    const int64_t total = (int64_t)n_src * gpr;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int n = (int)(e / gpr), j = (int)(e - (int64_t)n * gpr);
+        int n = (int)(e / gpr);
+        const int j = (int)(e - (int64_t)n * gpr);
         const uint4 v = *reinterpret_cast<const uint4 *>(src + (int64_t)n * K + (int64_t)j * 8);
+        if (rows == kRowsHead) n = n / head_dim * head_dim + qkv_row(n % head_dim, head_dim / 2);
+        else if (rows == kRowsAlt) n = (n >> 3) * 16 + (n & 7);
+        n += row0;
         *reinterpret_cast<uint4 *>(dst + wblk_off(N, n, j >> 3) + (((j & 7) ^ (n & 7)) << 4)) = v;
     }
 }

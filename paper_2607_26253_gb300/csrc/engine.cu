@@ -372,7 +372,7 @@ MegaParams mega_params(const sara_handle &h) {
     p.cnt = h.phase_cnt;
     p.epoch = h.phase_cnt + (size_t)h.n_phase_cnt * kCntStride;
     p.stamps = h.stamps;
-    p.n_stamp_ph = h.n_phase_cnt + 1 + kDetailRows;  // phases, kernel start, detail stamps
+    p.n_stamp_ph = h.n_phase_cnt + 1;  // phases, kernel start
     p.ktime = &h.vars->kt0;
     return p;
 }
@@ -489,11 +489,17 @@ void run_host_loop(sara_handle &h, int schedule) {
 
 // ------------------------------------------------------------------------ weights
 
-// Copy a row-major bf16 matrix [N][K] (host or device) into chunk-major blocks at dst,
-// through the device staging buffer tmp.
-void block_matrix(cudaStream_t s, const void *src, bool on_device, uint16_t *tmp, uint8_t *dst, int N, int K) {
-    CK(cudaMemcpyAsync(tmp, src, (size_t)N * K * 2, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
-    launch(s, false, dim3(1024), dim3(256), 0, block_weights_kernel, (const uint16_t *)tmp, dst, N, K);
+// A row-major bf16 matrix [n_src][K] (host or device) into chunk-major blocks at dst (a matrix of
+// N rows; rows, row0: see block_weights_kernel).  Host and misaligned sources go through the
+// device staging buffer tmp.
+void block_matrix(cudaStream_t s, const void *src, bool on_device, uint16_t *tmp, uint8_t *dst, int n_src, int K, int N,
+                  int rows = kRowsPlain, int row0 = 0, int head_dim = 0) {
+    if (!on_device || (reinterpret_cast<uintptr_t>(src) & 15)) {
+        CK(cudaMemcpyAsync(tmp, src, (size_t)n_src * K * 2, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
+        src = tmp;
+    }
+    launch(s, false, dim3(1024), dim3(256), 0, block_weights_kernel, static_cast<const uint16_t *>(src), dst, n_src, K, N,
+           rows, row0, head_dim);
 }
 
 void load_weights(sara_handle &h, const sara_weights *w) {
@@ -526,29 +532,22 @@ void load_weights(sara_handle &h, const sara_weights *w) {
     CK(cudaMemcpyAsync(h.embed, w->embed, (size_t)V * d * 2, kind, s));
     CK(cudaMemcpyAsync(h.final_norm, w->final_norm, (size_t)d * 2, kind, s));
     // staging buffer for one row-major matrix, freed when loading is done
-    const size_t stage = std::max({(size_t)V * d, (size_t)nqkv * d, (size_t)2 * F * d, (size_t)d * H * hd});
+    const size_t stage = std::max({(size_t)V * d, (size_t)H * hd * d, (size_t)F * d});
     uint16_t *tmp = nullptr;
     if (cudaMalloc(&tmp, stage * 2) != cudaSuccess) throw SaraError(SARA_ENOMEM, "cudaMalloc of the weight staging buffer failed");
     try {
-        block_matrix(s, w->lm_head, dev, tmp, h.wb_lm, V, d);
+        block_matrix(s, w->lm_head, dev, tmp, h.wb_lm, V, d, V);
         for (int l = 0; l < L; ++l) {
             CK(cudaMemcpyAsync(h.norm_attn + (size_t)l * d, w->attn_norm[l], (size_t)d * 2, kind, s));
             CK(cudaMemcpyAsync(h.norm_mlp + (size_t)l * d, w->mlp_norm[l], (size_t)d * 2, kind, s));
-            // fused q|k|v rows
-            CK(cudaMemcpyAsync(tmp, w->wq[l], (size_t)H * hd * d * 2, kind, s));
-            CK(cudaMemcpyAsync(tmp + (size_t)H * hd * d, w->wk[l], (size_t)KVH * hd * d * 2, kind, s));
-            CK(cudaMemcpyAsync(tmp + (size_t)(H + KVH) * hd * d, w->wv[l], (size_t)KVH * hd * d * 2, kind, s));
-            launch(s, false, dim3(1024), dim3(256), 0, block_weights_kernel, (const uint16_t *)tmp,
-                   h.wb_qkv + l * h.ls_qkv, nqkv, d);
-            block_matrix(s, w->wo[l], dev, tmp, h.wb_o + l * h.ls_o, d, H * hd);
-            // gate/up interleaved in blocks of 8 rows: [g 0..7, u 0..7, g 8..15, u 8..15, ...]
-            CK(cudaMemcpy2DAsync(tmp, (size_t)16 * d * 2, w->wgate[l], (size_t)8 * d * 2, (size_t)8 * d * 2, F / 8, kind,
-                                 s));
-            CK(cudaMemcpy2DAsync(tmp + (size_t)8 * d, (size_t)16 * d * 2, w->wup[l], (size_t)8 * d * 2,
-                                 (size_t)8 * d * 2, F / 8, kind, s));
-            launch(s, false, dim3(1024), dim3(256), 0, block_weights_kernel, (const uint16_t *)tmp,
-                   h.wb_gu + l * h.ls_gu, 2 * F, d);
-            block_matrix(s, w->wdown[l], dev, tmp, h.wb_down + l * h.ls_down, d, F);
+            uint8_t *qkv = h.wb_qkv + l * h.ls_qkv, *gu = h.wb_gu + l * h.ls_gu;
+            block_matrix(s, w->wq[l], dev, tmp, qkv, H * hd, d, nqkv, kRowsHead, 0, hd);
+            block_matrix(s, w->wk[l], dev, tmp, qkv, KVH * hd, d, nqkv, kRowsHead, H * hd, hd);
+            block_matrix(s, w->wv[l], dev, tmp, qkv, KVH * hd, d, nqkv, kRowsHead, (H + KVH) * hd, hd);
+            block_matrix(s, w->wo[l], dev, tmp, h.wb_o + l * h.ls_o, d, H * hd, d);
+            block_matrix(s, w->wgate[l], dev, tmp, gu, F, d, 2 * F, kRowsAlt, 0);
+            block_matrix(s, w->wup[l], dev, tmp, gu, F, d, 2 * F, kRowsAlt, 8);
+            block_matrix(s, w->wdown[l], dev, tmp, h.wb_down + l * h.ls_down, d, F, d);
         }
         CK(cudaStreamSynchronize(s));
     } catch (...) {
@@ -993,12 +992,12 @@ void teacher_impl(sara_handle &h, int n, int Lp, const int32_t *prompts, int T, 
 // arrived) to this one's, the median delay until CTAs observed the dependency, and how far
 // ahead of the previous phase's completion the W producer had issued this phase's copies.
 void print_stamps(sara_handle &h, int rows, int ctx) {
-    const int NP = h.n_phase_cnt + 1 + kDetailRows, G = h.sms, L = h.cfg.layers;
+    const int NP = h.n_phase_cnt + 1, G = h.sms, L = h.cfg.layers;
     std::vector<uint64_t> st((size_t)G * NP * 4);
     CK(cudaMemcpy(st.data(), h.stamps, st.size() * 8, cudaMemcpyDeviceToHost));
     auto at = [&](int c, int ph, int k) { return st[((size_t)c * NP + ph) * 4 + k]; };
     uint64_t t0 = ~0ull;
-    for (int c = 0; c < G; ++c) t0 = std::min(t0, at(c, NP - kDetailRows - 1, 0));
+    for (int c = 0; c < G; ++c) t0 = std::min(t0, at(c, NP - 1, 0));
     auto stat = [&](int ph, int k, bool mx) {
         std::vector<double> v;
         for (int c = 0; c < G; ++c)
@@ -1029,41 +1028,6 @@ void print_stamps(sara_handle &h, int rows, int ctx) {
                 span / n, obs / n, wahead / n, mma / n);
     }
     fprintf(stderr, "  LM     span %7.2f us\n", done[NPH - 1] - done[NPH - 2]);
-    // detail stamps (layer 2): median over CTAs relative to the QKV phase's completion
-    const int lq = std::min(2, L - 1);
-    const double ref = done[1 + kPhasesPerLayer * lq];
-    const char *dn[15] = {"att start", "q built", "S ready", "P ready", "O ready", "partial out", "split count",
-                          "merged", "units done", "att arrived", "fin_o start", "fin_o work", "fin_o arrived",
-                          "att dep seen", "att rstd"};
-    for (int i = 0; i < 15; ++i) {
-        std::vector<double> v;
-        for (int c = 0; c < G; ++c) {
-            const uint64_t x = at(c, NP - kDetailRows + i / 4, i % 4);
-            if (x >= t0) v.push_back((double)(x - t0) * 1e-3 - ref);
-        }
-        std::sort(v.begin(), v.end());
-        if (!v.empty())
-            fprintf(stderr, "    %-14s n=%3zu  med %+7.2f  max %+7.2f us\n", dn[i], v.size(), v[v.size() / 2], v.back());
-    }
-    // gate / up units of layer 2 (medians over CTAs, relative to FIN_O's completion)
-    const double ref_fo = done[1 + kPhasesPerLayer * lq + kPhFinO];
-    fprintf(stderr, "    GU unit: W issued / W full / X full / MMA committed (us after FIN_O)\n");
-    for (int j = 0; j < 12; ++j) {
-        double med[4];
-        int nn = 0;
-        for (int kind = 0; kind < 4; ++kind) {
-            std::vector<double> v;
-            const int i = 16 + 12 * kind + j;
-            for (int c = 0; c < G; ++c) {
-                const uint64_t x = at(c, NP - kDetailRows + i / 4, i % 4);
-                if (x >= t0) v.push_back((double)(x - t0) * 1e-3 - ref_fo);
-            }
-            std::sort(v.begin(), v.end());
-            med[kind] = v.empty() ? 0.0 : v[v.size() / 2];
-            nn = std::max(nn, (int)v.size());
-        }
-        fprintf(stderr, "      %2d n=%3d  %+7.2f %+7.2f %+7.2f %+7.2f\n", j, nn, med[0], med[1], med[2], med[3]);
-    }
 }
 #endif
 
@@ -1129,7 +1093,7 @@ void profile_impl(sara_handle &h, int which, int rows, int ctx, int iters, doubl
     CK(cudaMemcpyAsync(c.seq_len, len.data(), rows * 4, cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(c.seq_uid, uid.data(), rows * 8, cudaMemcpyHostToDevice, s));
 #ifdef SARA_STAMPS
-    const size_t nst = (size_t)h.sms * (h.n_phase_cnt + 1 + kDetailRows) * 4;
+    const size_t nst = (size_t)h.sms * (h.n_phase_cnt + 1) * 4;
     if (!h.stamps) h.stamps = h.mem.alloc<uint64_t>(nst);
 #endif
     CK(cudaStreamSynchronize(s));

@@ -159,10 +159,12 @@ __device__ __forceinline__ void gemm_epilogue_chunk(const GemmParams &p, GemmSme
         for (int c = 0; c < 32; ++c) S.xch[mrow * kEpiLd + c] = v[c];
         named_bar_sync(1, 128);
         if constexpr (EPI == EPI_QKV) {
+            // a head's rows: 16-row units of 8 dims of the first half and their rotation partners
             const int hd = p.head_dim, half = hd >> 1;
-            const int head = n / hd, i = n - head * hd;
-            const int partner = (i < half) ? mrow + half : mrow - half;
-            const int fi = (i < half) ? i : i - half;
+            const int head = n / hd, u = n - head * hd;
+            const int partner = mrow ^ 8;
+            const int fi = (u >> 4) * 8 + (u & 7);
+            const int i = (u & 8) ? fi + half : fi;
             const int nq = p.n_heads, nkv = p.n_kv;
             const bool rot = head < nq + nkv;  // q or k: rotate the pair (i, i + hd/2)
             float2 cs[32];
@@ -179,7 +181,7 @@ __device__ __forceinline__ void gemm_epilogue_chunk(const GemmParams &p, GemmSme
                         y = (i < half) ? (y * cs[c].x - o * cs[c].y) : (y * cs[c].x + o * cs[c].y);
                     }
                     if (head < nq) {
-                        p.q_out[(int64_t)r * (nq * hd) + n] = f32_to_f16_sat(y);
+                        p.q_out[(int64_t)r * (nq * hd) + head * hd + i] = f32_to_f16_sat(y);
                     } else {
                         const int isv = head >= nq + nkv;
                         const int kvh = head - nq - isv * nkv;
