@@ -73,6 +73,10 @@ constexpr int kPhasesPerLayer = 9;
 constexpr int kMaxCtaBlocks = 256;    // attention KV block ids a CTA keeps in shared memory
 // phases of a layer (counter index 1 + 9 l + phase)
 enum : int { kPhQKV = 0, kPhFinQ = 1, kPhAtt = 2, kPhO = 3, kPhFinO = 4, kPhGU = 6, kPhDown = 7, kPhFinD = 8 };
+// Up to this many live rows the q/k/v and O projections are column-owned on warp-level MMAs
+// (small_k), with their operand in fragment order.
+constexpr int kSmallRows = 8;
+constexpr int kSmallUnits = 2;  // 16-feature units a pass of small_k takes
 constexpr int kSmallPhaseUnits = 2;   // QKV / O: units per participating CTA
 constexpr int kCntStride = 16;        // phase counters 128 bytes apart (one L2 line each)
 constexpr uint32_t kTmemCols = 512;
@@ -157,6 +161,7 @@ struct MegaSmem {
     int rows, rows16, nx, nx_lg, xgroup, n_items, att_span;  // nx = 2^nx_lg X stages of xgroup chunks
     GemmPlan plan[5];           // this CTA's share of each GEMM phase (the same for every layer)
     int2 tile_cta[3][kPlanTiles];  // first and last contributor of the tiles of q/k/v, O, down
+    int small;                  // at most kSmallRows live rows
     float rstd[128];
     int rowpos[128];            // position of each live row
     // KV block ids: of this CTA's attention blocks (unit i's block j at ablk[aoff[i] + j]), and
@@ -186,6 +191,16 @@ __host__ __device__ __forceinline__ uint32_t xblk_off(int r, int k, int rows16) 
     const int chunk = k >> 6, col = k & 63;
     return (uint32_t)(chunk * 2 * rows16 + 16 * (r >> 3) + (r & 7)) * 128 +
            ((((col >> 3) ^ (r & 7)) << 4) | ((col & 7) << 1));
+}
+// Fragment-order activation (the operand of small_k): per 32-wide k-block and 8-row tile, the hi
+// then the lo part, each 32 lanes x 16 bytes: what lane 4 g + t of a warp needs of row g as
+// m16n8k16 B fragments of the block's two k-steps, so a warp reads a (block, tile, part) with one
+// coalesced 16-byte load per lane, straight into its registers.  Byte offset of the hi part of
+// element (r, k); the lo part sits kFragLo after it.
+constexpr int kFragLo = 512;
+__host__ __device__ __forceinline__ uint32_t frag_off(int r, int k, int rows16) {
+    return (uint32_t)((k >> 5) * (rows16 >> 3) + (r >> 3)) * 1024 + ((r & 7) * 4 + ((k & 7) >> 1)) * 16 +
+           ((k >> 3) & 3) * 4 + (k & 1) * 2;
 }
 // Byte offsets of K(pp, d) and V(pp, d) inside one 128-position KV block.
 __host__ __device__ __forceinline__ int kv_k_off(int pp, int d) {
@@ -276,8 +291,9 @@ __device__ __forceinline__ unsigned long long phase_target(const MegaParams &p, 
 //   split-K: (256-feature tile, 64-column chunk) units in equal contiguous ranges over the CTAs
 //     (lm_head: on whole tiles); each CTA stores its fp32 partial tiles and a finalisation phase
 //     sums them.
-//   column-owned (gate / up): 16-feature units in equal contiguous ranges, each with the whole K,
-//     so that the CTA's epilogue applies the nonlinearity itself and no partials and no
+//   column-owned (gate / up; q/k/v and O at few live rows): 16-feature units in equal contiguous
+//     ranges, each with the whole K, so that the CTA's epilogue applies what follows (SwiGLU;
+//     RoPE and the cache append; residual and norm input) itself and no partials and no
 //     finalisation phase are needed.  More activation traffic (every CTA reads the whole
 //     operand) and fewer weight rows per MMA, but one phase barrier and one L2 round trip less.
 enum : int { kGQKV = 0, kGO = 1, kGDown = 2, kGGU = 3, kGLM = 4 };  // plan index
@@ -286,7 +302,7 @@ constexpr int kOwnUnits = kTileN / kOwnCols;  // units of a pass at most
 
 // Geometry of a phase for CTA c of G: filled into plan[which] once per launch.
 // (Unit counts stay below 2^31 / SMs for every supported shape: 32-bit products suffice.)
-__device__ __noinline__ void make_plan(const MegaParams &p, GemmPlan &g, int which, int c, int G) {
+__device__ __noinline__ void make_plan(const MegaParams &p, GemmPlan &g, int which, int c, int G, bool small) {
     int K = p.d, Gp = G;
     g.x = p.xg;
     g.pass = 0;
@@ -305,13 +321,18 @@ __device__ __noinline__ void make_plan(const MegaParams &p, GemmPlan &g, int whi
     g.t = g.kc = g.units = 0;
     // at most one CTA per unit (tile for lm_head), so every participating CTA holds a
     // non-empty range and the CTAs between a tile's first and last owner all contributed
-    if (which == kGGU) {
-        const int U = g.N / kOwnCols;
-        Gp = min(Gp, U);
+    const bool sm = small && (which == kGQKV || which == kGO);
+    if (which == kGGU || sm) {
+        const int U = g.N / kOwnCols, most = sm ? kSmallUnits : kOwnUnits;
+        Gp = min(G, U);
+        if (sm) {  // equal shares: a pass of small_k costs about the same for one unit or two
+            const int per = (U + Gp - 1) / Gp;
+            Gp = (U + per - 1) / per;
+        }
         if (c < Gp) {
             g.t = c * U / Gp;
             g.units = (c + 1) * U / Gp - g.t;
-            const int np = (g.units + kOwnUnits - 1) / kOwnUnits;  // equal passes
+            const int np = (g.units + most - 1) / most;  // equal passes
             g.pass = (g.units + np - 1) / np;
         }
     } else {
@@ -576,7 +597,7 @@ __device__ __forceinline__ void mega_x_producer(const MegaParams &p, MegaSmem &S
         const int l = i >> 2, gk = i == 4 * p.layers ? kGLM : gemm_kind(i & 3);
         const GemmPlan &g = S.plan[gk];
         SegWalk walk(g);
-        if (walk.left <= 0) continue;
+        if (walk.left <= 0 || (S.small && (gk == kGQKV || gk == kGO))) continue;  // (small_k loads its own)
         // the phase this operand comes from: FIN_D of l-1 / embedding, ATT, FIN_O, GU
         const int dep = kPhasesPerLayer * l + (gk == kGO ? 1 + kPhAtt : gk == kGGU ? 1 + kPhFinO : gk == kGDown ? 1 + kPhGU : 0);
         if (!spin_counter_warp(&p.cnt[dep * kCntStride], phase_target(p, S, dep), err, ab, lim)) { ok = false; break; }
@@ -634,8 +655,20 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
         const GemmPlan &g = S.plan[gk];
         SegWalk walk(g);
         Seg sg;
+        const bool fwd = S.small && (gk == kGQKV || gk == kGO);
 #pragma unroll 1
         while (ok && walk.next(g, sg)) {
+            if (fwd) {  // small_k's weights: handed over to both compute groups as they land (see below)
+#pragma unroll 1
+                for (int e = sg.entries(); e > 0; --e, ++wi) {
+                    if (!mwait_warp(&S.wfull[wi % nws], (wi / nws) & 1, err, ab, lim)) { ok = false; break; }
+                    if (elect_one()) {
+                        mbar_arrive(&S.kvready[0][wi % nws]);
+                        mbar_arrive(&S.kvready[1][wi % nws]);
+                    }
+                }
+                continue;
+            }
             const uint32_t a = tseg & 1;  // segments alternate between two accumulators (epilogue overlaps)
             const uint32_t use_a = a ? use[1] : use[0];
             if (use_a >= 1 && !mwait_warp(&S.acc_empty[a], (use_a - 1) & 1, err, ab, lim)) { ok = false; break; }
@@ -725,12 +758,95 @@ __device__ __forceinline__ uint2 pack4(const uint16_t (&v)[4]) {
     return make_uint2((uint32_t)v[0] | ((uint32_t)v[1] << 16), (uint32_t)v[2] | ((uint32_t)v[3] << 16));
 }
 
+// Column-owned projection of up to 8 rows on warp-level MMAs: sum_k W[c][k] X[r][k] for the
+// segment's one or two 16-feature units, the whole K split over the eight compute warps by
+// 32-wide k-blocks (block kb on warp kb % 8).  X comes straight from global memory in fragment
+// order (six blocks' loads in flight at once), W from the ring's slots, which the issuer hands
+// over; the per-warp sums go to red[warp][unit][feature][row rotated by feature].
+// Against the split-K tcgen05 phase plus its finalisation phase this is one phase barrier and
+// two L2 round trips less (q/k/v at one row: 7.3 -> 5.0 us per layer, O: 6.8 -> 4.5); every CTA
+// reads the whole operand, so above 8 rows the gain is gone (26 rows: 16.5 -> 14.2 us for both,
+// but as much lost to the larger code of the other phases).
+template <typename KvWait>
+__device__ __forceinline__ void small_k(MegaSmem &S, const uint8_t *sW, float *red, const uint8_t *X, int rows16, int kch,
+                                        const Seg &sg, uint32_t wring, int cw, int lane, KvWait &&kv_wait) {
+    constexpr int B = 6;  // k-blocks per batch
+    const int mt = sg.n / kOwnCols, E = sg.entries(), lgc = __ffs(sg.cps) - 1;
+    const uint32_t kbs = (uint32_t)(rows16 >> 3) * 1024;  // bytes of a k-block
+    float acc[kSmallUnits][4];
+#pragma unroll
+    for (int m = 0; m < kSmallUnits; ++m)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[m][q] = 0.f;
+    const int arow = lane & 15;  // ldmatrix row of this lane
+#pragma unroll 1
+    for (int e0 = 0; e0 < E; e0 += kWSlots) {  // as many slots as the ring holds
+        const int e1 = min(E, e0 + kWSlots);
+        const int kb1 = min(2 * kch, 2 * sg.cps * e1);
+        int seen = e0;  // slots handed over so far
+#pragma unroll 1
+        for (int kb0 = 2 * sg.cps * e0 + cw; kb0 < kb1; kb0 += 8 * B) {
+            uint4 xh[B], xl[B];
+            const uint8_t *src = X + kb0 * kbs + lane * 16;
+#pragma unroll
+            for (int b = 0; b < B; ++b, src += 8 * kbs) {
+                xh[b] = xl[b] = make_uint4(0, 0, 0, 0);
+                if (kb0 + 8 * b < kb1) {
+                    xh[b] = __ldcg(reinterpret_cast<const uint4 *>(src));
+                    xl[b] = __ldcg(reinterpret_cast<const uint4 *>(src + kFragLo));
+                }
+            }
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                const int kb = kb0 + 8 * b;
+                if (kb < kb1) {
+                    const int e = (kb >> 1) >> lgc;
+#pragma unroll 1
+                    for (; seen <= e; ++seen) kv_wait(wring + seen);
+                    const uint32_t wb = smem_u32(sW) + ((wring + e) % kWSlots) * kSlotBytes +
+                                        (uint32_t)(((kb >> 1) - (e << lgc)) * sg.n * 128 + arow * 128);
+#pragma unroll
+                    for (int ks = 0; ks < 2; ++ks) {
+                        const int gran = ((kb & 1) * 2 + ks) * 2 + (lane >> 4);
+#pragma unroll
+                        for (int m = 0; m < kSmallUnits; ++m) {
+                            if (m < mt) {
+                                uint32_t a[4];
+                                ldsm_x4(wb + m * kOwnCols * 128 + ((gran ^ (arow & 7)) << 4), a);
+                                mma_bf16_16816(acc[m], a, ks ? xh[b].z : xh[b].x, ks ? xh[b].w : xh[b].y);
+                                mma_bf16_16816(acc[m], a, ks ? xl[b].z : xl[b].x, ks ? xl[b].w : xl[b].y);
+                            }
+                        }
+                    }
+                }
+            }
+        }
+#pragma unroll 1
+        for (; seen < e1; ++seen) kv_wait(wring + seen);  // (every thread follows every hand-over)
+        if (e1 < E) {
+            named_bar_sync(1, kMegaCThreads);
+            if (cw == 0 && lane == 0)
+                for (int e = e0; e < e1; ++e) mbar_arrive(&S.wempty[(wring + e) % kWSlots]);
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < kSmallUnits; ++m)
+        if (m < mt) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int c = (lane >> 2) + 8 * (q >> 1), r = 2 * (lane & 3) + (q & 1);
+                red[((cw * kSmallUnits + m) * kOwnCols + c) * 8 + ((r + c) & 7)] = acc[m][q];
+            }
+        }
+}
+
 // The compute warps' code runs once per layer and is far larger than the instruction caches'
 // first levels, so its size is time: each step exists once (the layer loop is unrolled over
 // nothing, the three residual finalisations and the three split-K epilogues share their code),
 // divisions by launch constants are done once (GemmPlan, tile_cta), and batches of loads are
 // spread over the lanes instead of being unrolled further.
-__device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, uint8_t *sW, uint8_t *sQ, uint32_t tmem) {
+__device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, uint8_t *sW, uint8_t *sX, uint8_t *sQ,
+                                             uint32_t tmem) {
     volatile int *ab = &S.abort;
     const uint64_t lim = S.wait_ns;
     int *err = &p.c.v->err;
@@ -740,6 +856,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
     const int half = cw >> 2;                    // warps 3..6 -> 0, 7..10 -> 1
     const int G = gridDim.x, cta = blockIdx.x;
     const int R = S.rows, R16c = p.rows_cap16;
+    const bool small = S.small != 0;
     const int d = p.d, hd = p.hd, Gq = p.Gq;
     const int gw = cta * 8 + cw, nw = G * 8;
     const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
@@ -797,14 +914,18 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
         }
         named_bar_sync(1, kMegaCThreads);
     };
-    // 1/rms of every row from its d / 64 (at most 32) partial sums of squares: a warp per row,
-    // a lane per partial
-    auto load_rstd = [&](const float *ssq) {
+    // 1/rms of every row from its np (at most 128) partial sums of squares: a warp per row, a
+    // lane per partial
+    auto load_rstd = [&](const float *ssq, int np) {
+#pragma unroll 1
         for (int r = cw; r < R; r += 8) {
-            const float s = warp_sum(lane < d / 64 ? __ldcg(&ssq[lane * p.rows_cap + r]) : 0.f);
+            float s = 0.f;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (lane + 32 * q < np) s += __ldcg(&ssq[(lane + 32 * q) * p.rows_cap + r]);
+            s = warp_sum(s);
             if (lane == 0) S.rstd[r] = rsqrtf(s / (float)d + p.eps);
         }
-        named_bar_sync(1, kMegaCThreads);
     };
     // contributors of tile t of split-K phase `which`
     auto contributors = [&](int which, int t) -> int2 {
@@ -838,6 +959,10 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
         return s;
     };
 
+    // the attention output's layout: the O projection's operand
+    auto att_off = [&](int r, int kk) -> uint32_t { return small ? frag_off(r, kk, R16c) : xblk_off(r, kk, R16c); };
+    const int lo_off = small ? kFragLo : kLoOff;
+
     // the KV block of each row's current position (its k, v are appended there every layer)
     if (ctid < R) {
         const int pos = __ldg(&p.c.row_pos[ctid]);
@@ -852,7 +977,8 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
 #pragma unroll 1
     for (int step = 0, l = 0, k = 0;; ++step) {
         const int base = 1 + kPhasesPerLayer * l;
-        if (k != 1) {
+        const bool fin = k == 0 || (k == 2 && !small);
+        if (fin) {
             // ---------------------------------------------------- residual, next norm input
             // x += sum of the GEMM's partials (x = E[tok] at the start); x_g = x * gn as a blocked
             // hi/lo pair; per (row, 64 features) sum of squares.  Unit = (row, 64 features): lane
@@ -891,28 +1017,35 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                 split_bf16(x.y * bf16_to_f32(gb.x >> 16), h[1], lo[1]);
                 split_bf16(x.z * bf16_to_f32(gb.y & 0xffff), h[2], lo[2]);
                 split_bf16(x.w * bf16_to_f32(gb.y >> 16), h[3], lo[3]);
-                uint8_t *dst = p.xg + xblk_off(r, f, R16c);
                 float sq = 0.f;
                 if (lane < 16) {
                     *reinterpret_cast<float4 *>(xp) = x;
-                    *reinterpret_cast<uint2 *>(dst) = pack4(h);
                     sq = (x.x * x.x + x.y * x.y) + (x.z * x.z + x.w * x.w);
+                }
+                const uint2 w = lane < 16 ? pack4(h) : pack4(lo);
+                if (small && l < p.layers) {  // small_k's operand
+                    uint8_t *dst = p.xg + frag_off(r, f, R16c) + (lane < 16 ? 0 : kFragLo);
+                    *reinterpret_cast<uint32_t *>(dst) = w.x;
+                    *reinterpret_cast<uint32_t *>(dst + 16) = w.y;
                 } else {
-                    *reinterpret_cast<uint2 *>(dst + kLoOff) = pack4(lo);
+                    *reinterpret_cast<uint2 *>(p.xg + xblk_off(r, f, R16c) + (lane < 16 ? 0 : kLoOff)) = w;
                 }
                 sq = warp_sum(sq);
                 if (lane == 0) ssq[h64 * p.rows_cap + r] = sq;
             }
             arrive(k == 2 ? base + kPhFinO : base - 1, true);
             if (l == p.layers) break;
-            if (k == 2) {
+        }
+        if (k == 2) {
+            {
                 // ------------------------------------------------ gate / up with SwiGLU
                 // h = silu(r g) * (r u) straight from the accumulator: this CTA's features hold the
                 // whole K, in 16-feature units of 8 gate then 8 up features.  The two warp halves
                 // take alternate pairs of units; each lane of a pair finishes one unit of its row.
                 // The row's 1/rms is read while the MMAs run.
                 wait_phase(base + kPhFinO);
-                load_rstd(p.ssqM);
+                load_rstd(p.ssqM, small ? d / kOwnCols : d / 64);
+                named_bar_sync(1, kMegaCThreads);
                 const float rs = act ? S.rstd[my_row] : 0.f;
                 const GemmPlan &g = S.plan[kGGU];
                 SegWalk walk(g);
@@ -951,7 +1084,8 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                 }
                 arrive(base + kPhGU, true);
             }
-        } else {
+        } else if (k == 1) {
+          if (!small) {
             // -------------------------------------------------------- q, k, v (once per row)
             // The head's QKV partials summed, times 1/rms; RoPE on q and k; q pre-scaled by
             // log2(e)/sqrt(hd) for the exp2 softmax; fp16 q, k, v for the attention phase; k and v
@@ -1002,6 +1136,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                 }
             }
             arrive(base + kPhFinQ, false);
+          }
             // -------------------------------------------------------- attention
             int a0, a1;
             att_range(p, S.n_items, a0, a1);
@@ -1204,9 +1339,9 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                             if (single) {
                                 uint16_t hv, lv;
                                 split_bf16(o[m][q] / lrun[q & 1], hv, lv);
-                                uint8_t *dst = p.att + xblk_off(u.row, (u.kvh * Gq + h) * hd + dim, R16c);
+                                uint8_t *dst = p.att + att_off(u.row, (u.kvh * Gq + h) * hd + dim);
                                 *reinterpret_cast<uint16_t *>(dst) = hv;
-                                *reinterpret_cast<uint16_t *>(dst + kLoOff) = lv;
+                                *reinterpret_cast<uint16_t *>(dst + lo_off) = lv;
                             } else {
                                 mine[h * (hd + 2) + 2 + dim] = o[m][q];
                             }
@@ -1289,9 +1424,9 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                             if (g < Gq) {
                                 uint16_t hv, lv;
                                 split_bf16(acc[g] / S.ml[half][g], hv, lv);
-                                uint8_t *dst = p.att + xblk_off(u.row, (u.kvh * Gq + g) * hd + dd, R16c);
+                                uint8_t *dst = p.att + att_off(u.row, (u.kvh * Gq + g) * hd + dd);
                                 *reinterpret_cast<uint16_t *>(dst) = hv;
-                                *reinterpret_cast<uint16_t *>(dst + kLoOff) = lv;
+                                *reinterpret_cast<uint16_t *>(dst + lo_off) = lv;
                             }
                     }
                 }
@@ -1301,6 +1436,85 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
             gi += n;
             arrive(base + kPhAtt, true);
         }
+        if (small && k != 2) {
+            // ------------------------------------------------ column-owned q/k/v or O projection
+            // Each CTA's few features hold the whole K, so what follows the sums is applied at
+            // once.  Thread: feature c = ctid % 16 of its (unit, row) elements.
+            //   q/k/v: RMSNorm scale, RoPE (a unit is 8 dims of a head and their rotation
+            //     partners), fp16, cache append.
+            //   O: x += sum, the MLP norm's input, sums of squares (one partial per 16 features).
+            wait_phase(k == 0 ? base - 1 : base + kPhAtt);
+            const GemmPlan &g = S.plan[k];
+            const uint8_t *X = k == 0 ? p.xg : p.att;
+            float *red = reinterpret_cast<float *>(sX);  // no copy targets the X stages during these phases
+            const int half_hd = hd >> 1, c = ctid & 15, r = (ctid >> 4) & 7, m = ctid >> 7;
+            SegWalk walk(g);
+            Seg sg;
+#pragma unroll 1
+            while (walk.next(g, sg)) {
+                const bool live = r < R && m * kOwnCols < sg.n;  // this thread's element (unit m, feature c, row r)
+                const int n0 = sg.col0 + m * kOwnCols, head = n0 / hd;
+                const bool rot = head < p.H + p.KVH;
+                float2 pre = make_float2(1.f, 0.f);  // (cos, sin) or (residual, norm weight), in flight with the operand
+                if (live) {
+                    if (k != 0) {
+                        pre.x = __ldcg(p.x + r * d + n0 + c);
+                        pre.y = bf16_to_f32(__ldg(p.mlp_norm + l * d + n0 + c));
+                    } else if (rot) {
+                        pre = __ldg(&p.rope[S.rowpos[r] * half_hd + (n0 - head * hd) / 2 + (c & 7)]);
+                    }
+                }
+                if (k == 0) load_rstd(p.ssqA, d / 64);
+                small_k(S, sW, red, X, R16c, g.kch, sg, wring, cw, lane, kv_wait);
+                named_bar_sync(1, kMegaCThreads);
+                const int E = sg.entries();
+                if (ctid == 0)  // the slots not yet returned
+                    for (int e = (E - 1) / kWSlots * kWSlots; e < E; ++e) mbar_arrive(&S.wempty[(wring + e) % kWSlots]);
+                wring += (uint32_t)E;
+                float v = 0.f;
+                if (live) {
+#pragma unroll
+                    for (int w = 0; w < 8; ++w) v += red[((w * kSmallUnits + m) * kOwnCols + c) * 8 + ((r + c) & 7)];
+                }
+                uint32_t w0, w1;  // what this lane keeps and what its neighbour lane ^ 1 takes
+                float sq = 0.f;
+                if (k == 0) {
+                    const float vp = __shfl_xor_sync(0xffffffffu, v, 8);
+                    const float y = v * pre.x + (c < 8 ? -1.f : 1.f) * (vp * pre.y);
+                    w0 = w1 = f32_to_f16_sat(y * ((live ? S.rstd[r] : 0.f) * (head < p.H ? p.scale_log2 : 1.f)));
+                } else {
+                    const float x = pre.x + v;
+                    if (live) p.x[r * d + n0 + c] = x;
+                    uint16_t h, lo;
+                    split_bf16(x * pre.y, h, lo);
+                    w0 = (c & 1) ? lo : h;  // even lanes store both hi parts, odd lanes both lo parts
+                    w1 = (c & 1) ? h : lo;
+                    sq = live ? x * x : 0.f;
+#pragma unroll
+                    for (int o = 1; o < 16; o <<= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+                }
+                const uint32_t wn = __shfl_xor_sync(0xffffffffu, w1, 1);
+                const uint32_t pk = (c & 1) ? wn | (w0 << 16) : w0 | (wn << 16);  // features c & ~1, c | 1
+                if (live && k == 0) {
+                    const int dim = (n0 - head * hd) / 2 + (c & 7) + (c < 8 ? 0 : half_hd);
+                    if ((c & 1) == 0) *reinterpret_cast<uint32_t *>(p.qkv16 + r * p.nqkv + head * hd + dim) = pk;
+                    if (head >= p.H) {  // the new position's k / v into the cache (blocked layout)
+                        uint8_t *blk = kv_addr(p, l, S.rowblk[r], head - p.H - (rot ? 0 : p.KVH));
+                        const int pp = S.rowpos[r] % kKVPos;
+                        if (!rot) *reinterpret_cast<uint16_t *>(blk + kv_v_off(pp, dim)) = (uint16_t)w0;
+                        else if ((c & 1) == 0) *reinterpret_cast<uint32_t *>(blk + kv_k_off(pp, dim)) = pk;
+                    }
+                } else if (live) {
+                    *reinterpret_cast<uint32_t *>(p.xg + xblk_off(r, (n0 + c) & ~1, R16c) + ((c & 1) ? kLoOff : 0)) = pk;
+                    if (c == 0) p.ssqM[n0 / kOwnCols * p.rows_cap + r] = sq;
+                }
+                named_bar_sync(1, kMegaCThreads);  // red is free again
+            }
+            fence_proxy_async_smem();  // (its room is a target of bulk copies again)
+            arrive(base + (k == 0 ? kPhFinQ : kPhFinO), k == 1);
+            // (the split-K phase's counter keeps step: a later launch with more rows waits on it)
+            if (ctid == 0) atomicAdd(&p.cnt[(base + (k == 0 ? kPhQKV : kPhO)) * kCntStride], 1ull);
+        } else {
         // ---------------------------------------------------------------- split-K GEMM
         // this CTA's partial tiles: row my_row, columns [128 half, +128) of the tile
         {
@@ -1336,6 +1550,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
             }
             arrive(base + (k == 0 ? kPhQKV : k == 1 ? kPhO : kPhDown), false);
         }
+        }
         if (++k == 3) {
             k = 0;
             ++l;
@@ -1351,7 +1566,8 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
     // the sampler on stored logits would do them.  The logits themselves are written only
     // when requested (teacher forcing).
     wait_phase(kPhasesPerLayer * p.layers);
-    load_rstd(p.ssqA);
+    load_rstd(p.ssqA, d / 64);
+    named_bar_sync(1, kMegaCThreads);
     const GemmPlan &g = S.plan[kGLM];
     const float rs = act ? S.rstd[my_row] : 0.f;
     const uint64_t seed = act ? __ldg(&p.c.row_seed[my_row]) : 0ull;
@@ -1464,6 +1680,7 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
         const int rows = max(0, min(live, p.rows_cap));
         S.rows = rows;
         S.rows16 = max(16, (rows + 15) & ~15);
+        S.small = live <= kSmallRows;
         // X stages of up to 16 KB: 4, 2 or 1 k-chunks each (fewer waits and commits per MMA), and
         // the largest power of two of them (at most kMaxXStages) that fits after the W slots
         {
@@ -1481,8 +1698,11 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
         const int64_t wl = p.c.kc->wait_ns;
         S.wait_ns = wl > 0 ? (uint64_t)wl : kWaitLimitNs;
         S.stall_idx = p.c.kc->stall_plus1 - 1;
-        // gate / up and its SwiGLU are one phase on the second of their two counters
-        if (S.stall_idx > 0 && (S.stall_idx - 1) % kPhasesPerLayer == kPhGU - 1) ++S.stall_idx;
+        // phases that finalise their own sums count on the second of their two counters
+        if (S.stall_idx > 0) {
+            const int ph = (S.stall_idx - 1) % kPhasesPerLayer;
+            if (ph == kPhGU - 1 || (S.small && (ph == kPhQKV || ph == kPhO))) ++S.stall_idx;
+        }
         S.p_headroom = p.c.kc->eager_softmax ? 0.f : kSoftmaxHeadroom;
         S.abort = (*(volatile int *)&V->err & ERR_WAIT_TIMEOUT) != 0;
         S.last_flag = 0;
@@ -1490,13 +1710,14 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
     }
     if (threadIdx.x == 0) MEGA_STAMP(p.n_stamp_ph - 1, 0);  // kernel start
     const uint64_t t_start = globaltimer_ns();
+    const bool small = *(volatile int *)&V->live <= kSmallRows;
     // the launch's GEMM shares and the contributors of the split-K tiles
     if (threadIdx.x >= 32 * 3 && threadIdx.x < 32 * 3 + 5)
-        make_plan(p, S.plan[threadIdx.x - 96], threadIdx.x - 96, blockIdx.x, gridDim.x);
+        make_plan(p, S.plan[threadIdx.x - 96], threadIdx.x - 96, blockIdx.x, gridDim.x, small);
     if (threadIdx.x >= 128 && threadIdx.x < 128 + 3 * kPlanTiles) {
         const int which = (threadIdx.x - 128) / kPlanTiles, t = (threadIdx.x - 128) % kPlanTiles;
         GemmPlan g;
-        make_plan(p, g, which, 0, gridDim.x);
+        make_plan(p, g, which, 0, gridDim.x, false);
         if (t < (g.N + kTileN - 1) / kTileN) S.tile_cta[which][t] = tile_ctas(p, g, which, t, gridDim.x);
     }
     if (warp == 1) {
@@ -1518,7 +1739,7 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
         } else if (warp == 2) {
             mega_x_producer(p, S, sX);
         } else {
-            mega_compute(p, S, sW, sQ, tmem);
+            mega_compute(p, S, sW, sX, sQ, tmem);
         }
     }
     tc_fence_before();

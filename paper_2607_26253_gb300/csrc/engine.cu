@@ -587,7 +587,7 @@ void alloc_decode(sara_handle &h) {
     h.att = h.mem.alloc<uint8_t>(R16 * Hhd * 4);
     h.hm = h.mem.alloc<uint8_t>(R16 * F * 4);
     h.ssqA = h.mem.alloc<float>((size_t)(d / 64) * S);
-    h.ssqM = h.mem.alloc<float>((size_t)(d / 64) * S);
+    h.ssqM = h.mem.alloc<float>((size_t)(d / kOwnCols) * S);
     // partial tiles: one segment per (CTA, tile) pair of a phase, at most CTAs + tiles - 1
     const int tmax = std::max(nqkv, d) / kTileN + 1;
     h.gpart = h.mem.alloc<float>((size_t)(h.sms + tmax) * S * kTileN, false);
