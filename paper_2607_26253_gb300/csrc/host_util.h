@@ -55,4 +55,21 @@ inline CUtensorMap make_tmap_bf16(const void *base, int inner, int outer, int bo
     return tm;
 }
 
+// Launch with thread-block clusters of `cluster` CTAs along x.
+template <typename Kern, typename... Args>
+inline void launch_cluster(cudaStream_t s, dim3 grid, dim3 block, size_t smem, unsigned cluster, Kern kern, Args... args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = cluster;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    CK(cudaLaunchKernelEx(&cfg, kern, args...));
+}
+
 }  // namespace sara

@@ -192,8 +192,8 @@ int sara_sample(const float *logits, int32_t R, int32_t V, uint64_t sample_seed,
                 int32_t *token, void *stream) {
     if (!logits || !uid || !t || !token || R < 1 || V < 1) return SARA_EINVAL;
     return op_guard([&] {
-        sample_rows_kernel<<<R, 256, 0, static_cast<cudaStream_t>(stream)>>>(logits, V, sample_seed, uid, t, token);
-        CK(cudaGetLastError());
+        launch_cluster(static_cast<cudaStream_t>(stream), dim3((unsigned)R * kSampleCtas), dim3(256), 0, kSampleCtas,
+                       sample_rows_kernel, logits, (int)V, sample_seed, uid, t, (int *)token);
     });
 }
 

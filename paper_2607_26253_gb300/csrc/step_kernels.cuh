@@ -288,18 +288,66 @@ static __global__ void __launch_bounds__(kCtlThreads, 1) teacher_setup_kernel(St
     }
 }
 
-// Gumbel-max over given fp32 logits (kernel-level entry point): one CTA per row.
+// Gumbel-max over given fp32 logits (kernel-level entry point): one cluster of kSampleCtas CTAs per
+// row, each a contiguous share of the vocabulary, the row's maximum joined through distributed
+// shared memory.  Bound by instruction issue (a 64-bit hash per token), so the noise's logarithms
+// are taken only for tokens that could beat the warp's best so far (g(u) increases with the
+// hash's top 24 bits; see the lm_head phase for the cut).  64 rows x 151,936, whole call: 37 us;
+// 277 us with one CTA per row (64 of 152 SMs) and the noise of every token.
+constexpr int kSampleCtas = 8;
 static __global__ void __launch_bounds__(256) sample_rows_kernel(const float *logits, int V, uint64_t sample_seed,
-                                                                 const int64_t *uid, const int *t, int *token) {
+                                                                 const int64_t *uid, const int32_t *t, int *token) {
     __shared__ float sv[8];
     __shared__ int si[8];
-    const int r = blockIdx.x;
+    __shared__ uint32_t cv[kSampleCtas], ci[kSampleCtas];  // (rank 0) the cluster's maxima
+    const int r = blockIdx.x / kSampleCtas, rank = (int)cluster_rank();
     const uint64_t rs = sampler_row_seed(sample_seed, uid[r], t[r]);
-    float best = -INFINITY;
+    const float *row = logits + (int64_t)r * V;
+    const int per = ((V + kSampleCtas - 1) / kSampleCtas + 3) & ~3;
+    const int v1 = min(V, (rank + 1) * per);
+    const bool vec = (reinterpret_cast<uintptr_t>(row) & 15) == 0;
+    float best = -INFINITY, wbest = -INFINITY;  // this thread's, and the warp's as of the last step
     int bi = 0x7fffffff;
-    for (int v = threadIdx.x; v < V; v += blockDim.x) {
-        const float z = logits[(int64_t)r * V + v] + gumbel_from_hash(splitmix_at(rs, (uint64_t)v + 1));
-        if (z > best) { best = z; bi = v; }
+#pragma unroll 1
+    for (int b = rank * per; b < v1; b += 2048) {
+        float z[8];  // tokens b + 4 tid .. and b + 1024 + 4 tid ..
+        uint32_t cand = 0;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int v = b + q * 1024 + (int)threadIdx.x * 4;
+            if (vec && v + 3 < v1) {
+                const float4 x = __ldg(reinterpret_cast<const float4 *>(row + v));
+                z[4 * q] = x.x; z[4 * q + 1] = x.y; z[4 * q + 2] = x.z; z[4 * q + 3] = x.w;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) z[4 * q + e] = v + e < v1 ? __ldg(row + v + e) : -INFINITY;
+            }
+        }
+        float vmax = z[0];
+#pragma unroll
+        for (int e = 1; e < 8; ++e) vmax = fmaxf(vmax, z[e]);
+        const float ureq = expf(-expf(-(wbest - vmax - 1e-3f)));  // 0 while wbest = -inf; NaN: every token
+        const float cut = ureq * 16777216.0f - 4.0f;
+        const uint32_t thr = cut > 0.f ? (uint32_t)cut : 0u;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int v = b + (e >> 2) * 1024 + (int)threadIdx.x * 4 + (e & 3);
+            cand |= (uint32_t)(v < v1 && (uint32_t)(splitmix_at(rs, (uint64_t)v + 1) >> 40) >= thr) << e;
+        }
+#pragma unroll 1
+        while (cand) {  // in increasing token order: the first maximum is kept
+            const int e = __ffs(cand) - 1;
+            cand &= cand - 1;
+            float ze = z[0];
+#pragma unroll
+            for (int i = 1; i < 8; ++i) ze = (i == e) ? z[i] : ze;
+            const int v = b + (e >> 2) * 1024 + (int)threadIdx.x * 4 + (e & 3);
+            ze = __fadd_rn(ze, gumbel_from_hash(splitmix_at(rs, (uint64_t)v + 1)));
+            if (ze > best) { best = ze; bi = v; }
+        }
+        wbest = best;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) wbest = fmaxf(wbest, __shfl_xor_sync(0xffffffffu, wbest, o));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -312,6 +360,17 @@ static __global__ void __launch_bounds__(256) sample_rows_kernel(const float *lo
     if (threadIdx.x == 0) {
         for (int w = 1; w < 8; ++w)
             if (sv[w] > best || (sv[w] == best && si[w] < bi)) { best = sv[w]; bi = si[w]; }
+        st_cluster_u32(cluster_addr(&cv[rank], 0), __float_as_uint(best));
+        st_cluster_u32(cluster_addr(&ci[rank], 0), (uint32_t)bi);
+    }
+    cluster_sync();
+    if (rank == 0 && threadIdx.x == 0) {
+        best = -INFINITY;
+        bi = 0x7fffffff;
+        for (int w = 0; w < kSampleCtas; ++w) {
+            const float ov = __uint_as_float(cv[w]);
+            if (ov > best || (ov == best && (int)ci[w] < bi)) { best = ov; bi = (int)ci[w]; }
+        }
         token[r] = bi;
     }
 }
