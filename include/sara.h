@@ -270,20 +270,20 @@ SARA_API void sara_destroy(sara_handle *h);
 
 /* ---------------------------------------------------------------------------------------
  * Kernel-level entry points (device pointers, the caller's stream), for unit parity tests
- * of the building blocks.  The GEMM and the attention launch the kernels the step's prefill
- * of fresh prompts runs; the sampler is a one-CTA-per-row form of the decode step's
- * Gumbel-max.  The decode step itself runs its projections, attention and logits inside one
+ * of the building blocks and for callers that want the operations by themselves; the sampler
+ * draws by the decode step's rule.  The decode step itself runs its projections, attention and logits inside one
  * persistent kernel, which is tested end to end through sara_teacher_force.
  * ------------------------------------------------------------------------------------- */
 
 /*
- * Y[r][n] = sum_c X[r][c] * W[n][c] for r < R, n < Nout (the prefill projection GEMM:
- * tcgen05 MMA with the accumulator in tensor memory, TMA-fed, stream-K over the weight).
+ * Y[r][n] = sum_c X[r][c] * W[n][c] for r < R, n < Nout (a projection of up to 128 rows:
+ * tcgen05 MMA with the accumulator in tensor memory, TMA-fed, few tiles split over K within a
+ * thread-block cluster).
  * X: [R][K] bf16, W: [Nout][K] bf16, Y: [R][Nout] fp32, all device, 16-byte aligned.
  * Shapes: 1 <= R <= 128, Nout % 128 == 0, K % 64 == 0, K >= 64.
  * workspace: device scratch of at least sara_gemm_workspace_bytes(R, Nout, K) bytes, all zero
- * on first use (the kernel leaves it zero again): per-CTA fixed-point tile sums and per-tile
- * arrival counters of the stream-K split.  Calls sharing a workspace must not overlap.
+ * on first use and left zero (part of the call's contract; the present kernel keeps its partial
+ * sums on chip).  Calls sharing a workspace must not overlap.
  */
 SARA_API size_t sara_gemm_workspace_bytes(int32_t R, int32_t Nout, int32_t K);
 SARA_API int sara_gemm_bf16(const uint16_t *X, const uint16_t *W, float *Y, int32_t R,
@@ -295,14 +295,8 @@ SARA_API int sara_gemm_bf16(const uint16_t *X, const uint16_t *W, float *Y, int3
  * example code running inside a host framework whose memory pool has already reserved the
  * GPU (a raw cudaMalloc there fails or fragments the pool), or a plugin whose interface only
  * hands over inputs and outputs.  The paper has no counterpart; this is a library service.
- * It allocates nothing: the stream-K scratch is a fixed array inside the library
- * (8 MiB of tile sums for at most 64 CTAs + 8 KiB of tile counters), which every GPU that
- * loads the library holds until the process exits.  The first call on a device looks up
- * the array's device address (cudaGetSymbolAddress); make that first call before any
- * stream capture.  Every call shares the array: each call clears what it needs before its
- * kernel, and calls whose work overlaps on the GPU (several streams or threads) race and
- * must be serialised by the caller.  Shapes as sara_gemm_bf16, plus Nout <= 262,144
- * (SARA_EINVAL beyond).  X, W, Y device pointers; work is issued on `stream`.
+ * It needs no scratch and allocates nothing; calls may overlap.  Shapes as sara_gemm_bf16, plus
+ * Nout <= 262,144 (SARA_EINVAL beyond).  X, W, Y device pointers; work is issued on `stream`.
  */
 SARA_API int sara_gemm_bf16_static(const uint16_t *X, const uint16_t *W, float *Y, int32_t R,
                                    int32_t Nout, int32_t K, void *stream);

@@ -1,21 +1,35 @@
-// Kernel-level entry points of include/sara.h on caller-provided device buffers: the
-// prefill's projection GEMM and attention kernels, and a one-CTA-per-row Gumbel-max sampler
-// (the decode step's sampling rule).
+// Kernel-level entry points of include/sara.h on caller-provided device buffers: the projection
+// GEMM of up to 128 rows, attention of single query rows, and the Gumbel-max sampler.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <string>
 #include <vector>
 
 #include "../../include/sara.h"
 #include "attention.cuh"
-#include "gemm_tc.cuh"
+#include "gemm_rows.cuh"
 #include "host_util.h"
 #include "step_kernels.cuh"
 
 using namespace sara;
+
+namespace sara {
+int gemm_rows_sms() {
+    constexpr int kMaxDevices = 64;
+    static std::atomic<int> known[kMaxDevices];  // SMs of devices whose kernel attribute is set, 0: not yet
+    int dev = 0, sms = 0;
+    CK(cudaGetDevice(&dev));
+    if (dev >= 0 && dev < kMaxDevices && (sms = known[dev].load(std::memory_order_acquire)) > 0) return sms;
+    CK(cudaFuncSetAttribute(gemm_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 + kRowsRing));
+    CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    if (dev >= 0 && dev < kMaxDevices) known[dev].store(sms, std::memory_order_release);
+    return sms;
+}
+}  // namespace sara
 
 namespace {
 
@@ -28,13 +42,14 @@ int sm_count() {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// The workspace of the GEMM's contract (the kernel no longer uses it; sizes unchanged).
 struct GemmWs {
     size_t part_bytes, cnt_bytes;
 };
 GemmWs gemm_ws_layout(int Nout, int sms) {
     GemmWs w;
-    w.part_bytes = align_up((size_t)sms * kTileR * kTileM * sizeof(unsigned long long), 256);
-    w.cnt_bytes = align_up((size_t)(Nout / kTileM) * sizeof(int), 256);
+    w.part_bytes = align_up((size_t)sms * kRowsMax * kRowsTileM * sizeof(unsigned long long), 256);
+    w.cnt_bytes = align_up((size_t)(Nout / kRowsTileM) * sizeof(int), 256);
     return w;
 }
 
@@ -82,30 +97,24 @@ size_t sara_gemm_workspace_bytes(int32_t R, int32_t Nout, int32_t K) {
 int sara_gemm_bf16(const uint16_t *X, const uint16_t *W, float *Y, int32_t R, int32_t Nout, int32_t K, void *workspace,
                    size_t workspace_bytes, void *stream) {
     if (!X || !W || !Y || !workspace) return SARA_EINVAL;
-    if (R < 1 || R > kTileR || Nout < kTileM || Nout % kTileM || K < kTileK || K % kTileK) return SARA_EINVAL;
+    if (R < 1 || R > kRowsMax || Nout < kRowsTileM || Nout % kRowsTileM || K < kRowsTileK || K % kRowsTileK) return SARA_EINVAL;
     if ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(W)) & 15) return SARA_EINVAL;
     return op_guard([&] {
-        const int sms = sm_count();
+        const int sms = gemm_rows_sms();
         const GemmWs w = gemm_ws_layout(Nout, sms);
         if (workspace_bytes < w.part_bytes + w.cnt_bytes) throw SaraError(SARA_EINVAL, "workspace too small");
-        CK(cudaFuncSetAttribute(gemm_tc_kernel<EPI_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmemBytes));
-        const CUtensorMap tw = make_tmap_bf16(W, K, Nout, kTileK, kTileM);
-        const CUtensorMap tx = make_tmap_bf16(X, K, R, kTileK, kXBoxRows);
-        GemmParams p{};
-        p.m_tiles = Nout / kTileM;
-        p.k_chunks = K / kTileK;
-        p.rows_cap = R;
-        p.rows_dev = nullptr;
-        p.rows_fixed = R;
-        p.decode = 1;
-        p.ws_acc = reinterpret_cast<unsigned long long *>(workspace);
-        p.ws_cnt = reinterpret_cast<int *>(reinterpret_cast<uint8_t *>(workspace) + w.part_bytes);
-        p.err = nullptr;
-        p.y_f32 = Y;
-        p.ld = Nout;
-        gemm_tc_kernel<EPI_F32><<<sms, kGemmThreads, kGemmSmemBytes, static_cast<cudaStream_t>(stream)>>>(tw, tx, tx, p);
-        CK(cudaGetLastError());
+        launch_gemm_rows(static_cast<cudaStream_t>(stream), sms, X, W, Y, R, Nout, K);
     });
+}
+
+int sara_gemm_bf16_static(const uint16_t *X, const uint16_t *W, float *Y, int32_t R, int32_t Nout, int32_t K,
+                          void *stream) {
+    constexpr int kStaticMaxNout = 262144;
+    if (!X || !W || !Y) return SARA_EINVAL;
+    if (R < 1 || R > kRowsMax || Nout < kRowsTileM || Nout % kRowsTileM || K < kRowsTileK || K % kRowsTileK) return SARA_EINVAL;
+    if (Nout > kStaticMaxNout) return SARA_EINVAL;
+    if ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(W)) & 15) return SARA_EINVAL;
+    return op_guard([&] { launch_gemm_rows(static_cast<cudaStream_t>(stream), gemm_rows_sms(), X, W, Y, R, Nout, K); });
 }
 
 size_t sara_attention_workspace_bytes(int32_t b, int32_t n_heads, int32_t head_dim, int32_t max_ctx) {

@@ -318,8 +318,7 @@ def gemm_bf16(X, W, workspace=None):
 
 
 def gemm_bf16_static(X, W, out=None):
-    """Y = X @ W^T like gemm_bf16, through the entry point that allocates nothing (its scratch
-    is a fixed array inside the library).  X [R, K], W [N, K] torch bf16 CUDA; `out` [R, N]
+    """Y = X @ W^T like gemm_bf16, through the entry point that needs no scratch.  X [R, K], W [N, K] torch bf16 CUDA; `out` [R, N]
     fp32 CUDA may be passed so the call itself allocates nothing."""
     import torch
     R, K = X.shape
