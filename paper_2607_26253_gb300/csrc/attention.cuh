@@ -1,7 +1,7 @@
 // Grouped-query attention with one query per row over that row's KV history:
 //     out[r, h] = softmax(q[r, h] . K[0..ctx_r)^T / sqrt(hd)) V[0..ctx_r),  ctx_r = pos_r + 1
-// Used for decode (row = live rollout, KV = its slot) and for prefill (row = one prompt
-// token, KV = the prompt's slot, causal by construction).
+// The attention entry point's path for operands that are not 16-byte aligned (attn_split.cuh
+// serves the others).
 //
 // q and the KV cache are fp16; the output is a bf16 hi/lo pair (the next GEMM's operand).
 //

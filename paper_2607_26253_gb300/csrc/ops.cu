@@ -11,6 +11,7 @@
 
 #include "../../include/sara.h"
 #include "attention.cuh"
+#include "attn_split.cuh"
 #include "gemm_rows.cuh"
 #include "host_util.h"
 #include "step_kernels.cuh"
@@ -138,6 +139,33 @@ int sara_attention_decode(const uint16_t *q, const uint16_t *kv, int64_t kv_stri
         if (workspace_bytes < sara_attention_workspace_bytes(b, n_heads, head_dim, max_ctx))
             throw SaraError(SARA_EINVAL, "workspace too small");
         cudaStream_t s = static_cast<cudaStream_t>(stream);
+        const int G = n_heads / n_kv_heads;
+        if (G != 1 && G != 2 && G != 4 && G != 6 && G != 8) throw SaraError(SARA_EINVAL, "query group must be 1, 2, 4, 6 or 8");
+        const int sms = sm_count();
+        // 16-byte loads of K, V and q rows (head dims below 128 may come less aligned); the grid's
+        // z and y dimensions hold 65,535 rows and KV heads
+        const bool wide = ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(kv)) & 15) == 0 && kv_stride % 8 == 0;
+        if (wide && b <= 65535 && n_kv_heads <= 65535) {
+            AttnSplitParams a{};
+            a.q = q;
+            a.kv = kv;
+            a.ctx = ctx;
+            a.out = out;
+            a.bad = reinterpret_cast<int *>(workspace);  // (b ints: far below the workspace's size)
+            a.kv_stride = kv_stride;
+            a.H = n_heads;
+            a.KVH = n_kv_heads;
+            a.cap = cap;
+            a.max_ctx = max_ctx;
+            a.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)head_dim));
+            launch_attn_split(s, sms, b, head_dim, a);
+            std::vector<int> bad(b);
+            CK(cudaMemcpyAsync(bad.data(), a.bad, b * sizeof(int), cudaMemcpyDeviceToHost, s));
+            CK(cudaStreamSynchronize(s));
+            for (int i = 0; i < b; ++i)
+                if (bad[i]) throw SaraError(SARA_EINVAL, "ctx out of range");
+            return;
+        }
         const size_t splits = (size_t)(max_ctx + 127) / 128;
         const size_t items_cap = (size_t)b * splits;
         uint8_t *ws = reinterpret_cast<uint8_t *>(workspace);
@@ -185,10 +213,8 @@ int sara_attention_decode(const uint16_t *q, const uint16_t *kv, int64_t kv_stri
         a.part = part;
         a.cnt = cnt;
         a.err = nullptr;
-        const int sms = sm_count();
+        CK(cudaMemsetAsync(cnt, 0, (size_t)b * n_heads * sizeof(int), s));
         dim3 grid(std::max(1, sms * 4 / n_kv_heads), n_kv_heads);
-        const int G = n_heads / n_kv_heads;
-        if (G != 1 && G != 2 && G != 4 && G != 6 && G != 8) throw SaraError(SARA_EINVAL, "query group must be 1, 2, 4, 6 or 8");
         if (head_dim == 32) launch_g<32>(grid, G, s, a);
         else if (head_dim == 64) launch_g<64>(grid, G, s, a);
         else launch_g<128>(grid, G, s, a);

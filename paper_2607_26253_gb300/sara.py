@@ -337,7 +337,7 @@ def attention_decode(q, kv, ctx, n_kv_heads: int, cap: int, max_ctx: int | None 
     max_ctx = int(ctx.max().item()) if max_ctx is None else max_ctx
     out = torch.empty(q.shape, dtype=torch.bfloat16, device=q.device)
     nbytes = load().sara_attention_workspace_bytes(b, H, hd, max_ctx)
-    ws = torch.zeros(nbytes, dtype=torch.uint8, device=q.device)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device=q.device)  # (nothing in it is read before it is written)
     _check(load().sara_attention_decode(q.data_ptr(), kv.data_ptr(), kv.stride(0), ctx.data_ptr(), out.data_ptr(),
                                         b, H, n_kv_heads, hd, cap, max_ctx, ws.data_ptr(), ws.numel(),
                                         torch.cuda.current_stream().cuda_stream))

@@ -1,5 +1,5 @@
 """Edges of the kernel-level row operations: the sampler's cluster shares and unaligned rows, the projection GEMM's K
-splits and tile walks."""
+splits and tile walks, the attention's position shares, alignment and refusals."""
 import numpy as np
 import pytest
 
@@ -64,3 +64,74 @@ def test_gemm_splits_and_tile_walks(pkg, R, N, K, static):
     # fp32 accumulation of exact bf16 products: |error| <= K 2^-23 sum |x w|
     bound = K * 2.0 ** -23 * (np.abs(xf) @ np.abs(wf).T) + 1e-6
     assert (np.abs(Y - xf @ wf.T) <= bound).all()
+
+
+def _attention_ref(q, kv, ctx, n_kv):
+    b, H, hd = q.shape
+    out = np.zeros((b, H, hd))
+    for i in range(b):
+        for h in range(H):
+            K, V = kv[i, 0, h // (H // n_kv), :ctx[i]], kv[i, 1, h // (H // n_kv), :ctx[i]]
+            s = K @ q[i, h] / np.sqrt(hd)
+            p = np.exp(s - s.max())
+            out[i, h] = (p / p.sum()) @ V
+    return out
+
+
+def _attention_case(rng, H, KVH, hd, ctxs):
+    b, cap = len(ctxs), max(ctxs) + 3
+    return (rng.standard_normal((b, H, hd)).astype(np.float16), rng.standard_normal((b, 2, KVH, cap, hd)).astype(np.float16),
+            np.array(ctxs, np.int32), cap)
+
+
+def _check_attention(out, q, kv, ctx, KVH):
+    import torch
+    got = synth.bf16_bits_to_f32(out.view(torch.int16).cpu().numpy().view(np.uint16)).astype(np.float64)
+    want = _attention_ref(q.astype(np.float64), kv.astype(np.float64), ctx, KVH)
+    # the bf16 rounding of the output (2^-9 relative) dominates
+    assert np.all(np.abs(got - want) <= 2.0 ** -8 * np.abs(want) + 1e-3)
+
+
+# positions around a warp's step of 16 and the CTAs' shares of a row; every group size and head dim; one row and many
+@pytest.mark.parametrize("H,KVH,hd,ctxs", [(6, 1, 128, [1]), (8, 1, 64, [15, 16, 17]), (2, 1, 32, [63, 64, 65, 129]),
+                                          (4, 4, 128, [512, 1, 513]), (8, 2, 32, [2048, 7]),
+                                          (12, 2, 128, list(range(1, 101))), (16, 2, 64, [12288])])
+def test_attention_edges(pkg, H, KVH, hd, ctxs):
+    q, kv, ctx, cap = _attention_case(np.random.default_rng(H + hd), H, KVH, hd, ctxs)
+    out = pkg.attention_decode(_dev(q), _dev(kv), _dev(ctx), KVH, cap, max_ctx=max(ctxs))
+    _check_attention(out, q, kv, ctx, KVH)
+
+
+def test_attention_unaligned_operands(pkg):
+    # q and K / V that start 8 bytes off a 16-byte boundary (head dim 64): accepted as ever
+    import torch
+    q, kv, ctx, cap = _attention_case(np.random.default_rng(1), 8, 2, 64, [100, 300])
+
+    def off(a):
+        buf = torch.zeros(a.size + 4, dtype=torch.float16, device="cuda")
+        buf[4:] = _dev(a).reshape(-1)
+        return buf[4:].view(a.shape)
+
+    _check_attention(pkg.attention_decode(off(q), off(kv), _dev(ctx), 2, cap), q, kv, ctx, 2)
+
+
+def test_attention_infinite_value(pkg):
+    # an infinite V element reaches the result with its sign, beside exact values in the other dims
+    q, kv, ctx, cap = _attention_case(np.random.default_rng(2), 12, 2, 128, [40, 300])
+    kv[0, 1, 0, 7, 5], kv[1, 1, 1, 250, 90] = np.inf, -np.inf
+    out = pkg.attention_decode(_dev(q), _dev(kv), _dev(ctx), 2, cap).float().cpu().numpy()
+    assert np.all(out[0, :6, 5] == np.inf) and np.all(out[1, 6:, 90] == -np.inf)
+    mask = np.isfinite(out)
+    assert mask.sum() == out.size - 12
+    kv[~np.isfinite(kv)] = 0
+    want = _attention_ref(q.astype(np.float64), kv.astype(np.float64), ctx, 2)
+    assert np.all(np.abs(out - want)[mask] <= 2.0 ** -8 * np.abs(want)[mask] + 2e-3)
+
+
+@pytest.mark.parametrize("bad", [0, -1, 301])
+def test_attention_context_out_of_range_refused(pkg, bad):
+    q, kv, ctx, cap = _attention_case(np.random.default_rng(3), 4, 2, 32, [300, 20, 5])
+    ctx[1] = bad
+    with pytest.raises(pkg.SaraError) as e:
+        pkg.attention_decode(_dev(q), _dev(kv), _dev(ctx), 2, cap, max_ctx=300)
+    assert e.value.code == pkg.SARA_EINVAL
