@@ -301,8 +301,6 @@ static __device__ void ctl_round_setup(const StepConst &K, StepVars &V, const St
         c.pre_slot[r] = c.fresh_pslot[f];
         c.pre_pos[r] = t;
         c.pre_tok[r] = c.p_tok[(int64_t)q * Lp + t];
-        c.pre_items[r] = make_int2(r, 0);
-        c.pre_item0[r] = r;
     }
     if (threadIdx.x == 0) {
         V.live = R;
@@ -675,8 +673,6 @@ static __device__ void ctl_async_join(const StepConst &K, StepVars &V, const Ste
         c.pre_slot[r] = c.fresh_pslot[f];
         c.pre_pos[r] = t;
         c.pre_tok[r] = c.p_tok[(int64_t)c.act_tmp[f] * Lp + t];
-        c.pre_items[r] = make_int2(r, 0);
-        c.pre_item0[r] = r;
     }
     __syncthreads();
     const int live = live0 + R;

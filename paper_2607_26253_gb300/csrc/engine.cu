@@ -20,6 +20,7 @@
 #include "decode_step.cuh"
 #include "gemm_tc.cuh"
 #include "host_util.h"
+#include "prefill_attn.cuh"
 #include "step_kernels.cuh"
 
 using namespace sara;
@@ -132,6 +133,15 @@ namespace {
 thread_local std::string g_create_error;
 
 // ------------------------------------------------------------------------ launches
+// f(kernel, threads) for the prefill attention kernel of a head dim and query group.
+template <typename F>
+void with_prefill_attn(int hd, int G, F f) {
+    const bool two = G % 2 == 0;  // heads per CTA
+    if (hd == 32) two ? f(prefill_attn_kernel<32, 2>, 256) : f(prefill_attn_kernel<32, 1>, 128);
+    else if (hd == 64) two ? f(prefill_attn_kernel<64, 2>, 256) : f(prefill_attn_kernel<64, 1>, 128);
+    else two ? f(prefill_attn_kernel<128, 2>, 256) : f(prefill_attn_kernel<128, 1>, 128);
+}
+
 void set_kernel_attrs() {
     static bool done = false;
     if (done) return;
@@ -139,6 +149,11 @@ void set_kernel_attrs() {
     CK(cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmemBytes));
     CK(cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmemBytes));
     CK(cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmemBytes));
+    for (int hd : {32, 64, 128})
+        for (int G : {1, 2})
+            with_prefill_attn(hd, G, [&](auto kern, int) {
+                CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)prefill_attn_smem(hd)));
+            });
     CK(cudaFuncSetAttribute(decode_step_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMegaSmemBytes));
     done = true;
 }
@@ -187,29 +202,6 @@ void launch_gemm(cudaStream_t s, bool pdl, int grid, const CUtensorMap &tw, cons
     grid = gemm_grid(grid, p.m_tiles, p.decode != 0);
     p.has_lo = 1;
     launch(s, pdl, dim3(grid), dim3(kGemmThreads), kGemmSmemBytes, gemm_tc_kernel<EPI>, tw, tx, tx_lo, p);
-}
-
-template <int HD>
-void launch_attention_hd(cudaStream_t s, bool pdl, dim3 grid, int G, const AttnParams &p) {
-    switch (G) {
-        case 1: launch(s, pdl, grid, dim3(kAttnThreads), 0, attn_rows_kernel<HD, 1>, p); break;
-        case 2: launch(s, pdl, grid, dim3(kAttnThreads), 0, attn_rows_kernel<HD, 2>, p); break;
-        case 4: launch(s, pdl, grid, dim3(kAttnThreads), 0, attn_rows_kernel<HD, 4>, p); break;
-        case 6: launch(s, pdl, grid, dim3(kAttnThreads), 0, attn_rows_kernel<HD, 6>, p); break;
-        case 8: launch(s, pdl, grid, dim3(kAttnThreads), 0, attn_rows_kernel<HD, 8>, p); break;
-        default: throw SaraError(SARA_EINVAL, "n_heads / n_kv_heads must be 1, 2, 4, 6 or 8");
-    }
-}
-
-void launch_attention(cudaStream_t s, bool pdl, int sms, int hd, const AttnParams &p) {
-    dim3 grid(std::max(1, (sms * 4) / std::max(1, p.n_kv)), p.n_kv);
-    const int G = p.n_heads / p.n_kv;
-    switch (hd) {
-        case 32: launch_attention_hd<32>(s, pdl, grid, G, p); break;
-        case 64: launch_attention_hd<64>(s, pdl, grid, G, p); break;
-        case 128: launch_attention_hd<128>(s, pdl, grid, G, p); break;
-        default: throw SaraError(SARA_EINVAL, "head_dim must be 32, 64 or 128");
-    }
 }
 
 GemmParams gemm_base(const sara_handle &h, int m_tiles, int k_chunks, const Acts &A, const int *rows_dev) {
@@ -261,27 +253,22 @@ void enqueue_prefill_kernel(sara_handle &h, cudaStream_t s, int which, int l, bo
             break;
         }
         case K_ATTN: {
-            AttnParams a{};
+            PrefillAttnParams a{};
             a.q = A.q;
             a.out = A.att;
             a.out_lo = A.att_lo;
             a.kv = kv_l;
             a.slot_stride = h.kv_pr_slot;
             a.cap = h.cap_p;
+            a.H = H;
+            a.KVH = KVH;
             a.row_slot = c.pre_slot;
-            a.row_pos = c.pre_pos;
-            a.items = c.pre_items;
-            a.n_items_dev = &h.vars->pre_rows;
-            a.row_item0 = c.pre_item0;
-            a.n_heads = H;
-            a.n_kv = KVH;
-            a.chunk = h.cap_p;  // one split per row
+            a.rows = rows_dev;
+            a.Lp = &h.kc->Lp;
             a.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)hd));
-            a.part = h.attn_part;
-            a.cnt = h.attn_cnt;
-            a.err = &h.vars->err;
-            a.stamps = h.stamps;
-            launch_attention(s, pdl, h.sms, hd, a);
+            with_prefill_attn(hd, H / KVH, [&](auto kern, int threads) {
+                launch(s, pdl, dim3(h.sms * 2), dim3(threads), prefill_attn_smem(hd), kern, a);
+            });
             break;
         }
         case K_OPROJ: {
@@ -727,8 +714,6 @@ void create_impl(sara_handle &h, const sara_model_cfg *cfgp, const sara_weights 
         c.pre_slot = h.mem.alloc<int32_t>(h.pre_cap);
         c.pre_pos = h.mem.alloc<int32_t>(h.pre_cap);
         c.pre_tok = h.mem.alloc<int32_t>(h.pre_cap);
-        c.pre_item0 = h.mem.alloc<int32_t>(h.pre_cap);
-        c.pre_items = h.mem.alloc<int2>(h.pre_cap);
         c.max_seqs = S;
         h.gen_tok = h.mem.alloc<int32_t>((size_t)P * K * m.max_gen_len, false);
         c.gen_tok = h.gen_tok;

@@ -267,8 +267,6 @@ static __global__ void __launch_bounds__(kCtlThreads, 1) teacher_setup_kernel(St
         c.pre_slot[r] = f;
         c.pre_pos[r] = t;
         c.pre_tok[r] = c.p_tok[(int64_t)f * Lp + t];
-        c.pre_items[r] = make_int2(r, 0);
-        c.pre_item0[r] = r;
     }
     if (threadIdx.x == 0) {
         StepVars z;

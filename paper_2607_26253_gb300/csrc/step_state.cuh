@@ -108,8 +108,7 @@ struct StepPtrs {
     int2 *att_items;
     int32_t *sampled;          // [max_seqs] token drawn for each row
     // prefill rows of the round
-    int32_t *pre_slot, *pre_pos, *pre_tok, *pre_item0;
-    int2 *pre_items;
+    int32_t *pre_slot, *pre_pos, *pre_tok;
     // outputs
     int32_t *gen_tok;          // [P][k][max_gen]
     // teacher forcing
