@@ -749,15 +749,6 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
 }
 
 // ------------------------------------------------------------------------------ compute
-// Eight / four bf16 values as one 16- / 8-byte store.
-__device__ __forceinline__ uint4 pack8(const uint16_t (&v)[8]) {
-    return make_uint4((uint32_t)v[0] | ((uint32_t)v[1] << 16), (uint32_t)v[2] | ((uint32_t)v[3] << 16),
-                      (uint32_t)v[4] | ((uint32_t)v[5] << 16), (uint32_t)v[6] | ((uint32_t)v[7] << 16));
-}
-__device__ __forceinline__ uint2 pack4(const uint16_t (&v)[4]) {
-    return make_uint2((uint32_t)v[0] | ((uint32_t)v[1] << 16), (uint32_t)v[2] | ((uint32_t)v[3] << 16));
-}
-
 // Column-owned projection of up to 8 rows on warp-level MMAs: sum_k W[c][k] X[r][k] for the
 // segment's one or two 16-feature units, the whole K split over the eight compute warps by
 // 32-wide k-blocks (block kb on warp kb % 8).  X comes straight from global memory in fragment

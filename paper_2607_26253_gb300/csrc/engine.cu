@@ -21,6 +21,7 @@
 #include "gemm_tc.cuh"
 #include "host_util.h"
 #include "prefill_attn.cuh"
+#include "prefill_gemm.cuh"
 #include "step_kernels.cuh"
 
 using namespace sara;
@@ -53,7 +54,8 @@ struct Acts {  // activation buffers of the prefill rows (row-major, TMA operand
     uint16_t *xg = nullptr, *xg_lo = nullptr, *q = nullptr, *att = nullptr, *att_lo = nullptr, *h = nullptr,
              *h_lo = nullptr;
     float *ssq_a = nullptr, *ssq_m = nullptr;
-    CUtensorMap tm_xg{}, tm_xg_lo{}, tm_att{}, tm_att_lo{}, tm_h{}, tm_h_lo{};
+    CUtensorMap tm_xg{}, tm_xg_lo{}, tm_att{}, tm_att_lo{}, tm_h{}, tm_h_lo{};  // boxes of kXBoxRows rows
+    CUtensorMap big_xg{}, big_xg_lo{}, big_att{}, big_att_lo{}, big_h{}, big_h_lo{};  // of kBigRows rows
 };
 
 }  // namespace
@@ -91,6 +93,7 @@ struct sara_handle {
     // workspaces
     unsigned long long *gemm_acc = nullptr;
     int *gemm_cnt = nullptr;
+    float *big_part = nullptr;  // partial tiles of the many-row prefill GEMM, two per SM
     float *attn_part = nullptr;
     int *attn_cnt = nullptr;
     float *lm_val = nullptr;
@@ -115,7 +118,7 @@ struct sara_handle {
     // graph
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr;
+    cudaStream_t cap_stream = nullptr, cap_stream2 = nullptr, cap_stream3 = nullptr;
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
 
     ~sara_handle() {
@@ -123,6 +126,7 @@ struct sara_handle {
         if (graph) cudaGraphDestroy(graph);
         if (cap_stream) cudaStreamDestroy(cap_stream);
         if (cap_stream2) cudaStreamDestroy(cap_stream2);
+        if (cap_stream3) cudaStreamDestroy(cap_stream3);
         if (ev0) cudaEventDestroy(ev0);
         if (ev1) cudaEventDestroy(ev1);
     }
@@ -145,10 +149,12 @@ void with_prefill_attn(int hd, int G, F f) {
 void set_kernel_attrs() {
     static bool done = false;
     if (done) return;
-    CK(cudaFuncSetAttribute(gemm_tc_kernel<EPI_F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmemBytes));
     CK(cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmemBytes));
     CK(cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmemBytes));
     CK(cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGemmSmemBytes));
+    CK(cudaFuncSetAttribute(prefill_gemm_kernel<EPI_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigSmemBytes));
+    CK(cudaFuncSetAttribute(prefill_gemm_kernel<EPI_RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigSmemBytes));
+    CK(cudaFuncSetAttribute(prefill_gemm_kernel<EPI_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBigSmemBytes));
     for (int hd : {32, 64, 128})
         for (int G : {1, 2})
             with_prefill_attn(hd, G, [&](auto kern, int) {
@@ -186,22 +192,15 @@ void launch(cudaStream_t s, bool pdl, dim3 grid, dim3 block, size_t smem, Kern k
     launch_ex(s, pdl, false, grid, block, smem, kern, args...);
 }
 
-// Grid of a decode GEMM: one whole tile per CTA when the tile count nearly fills the SMs
-// (no split reduction at all), else one CTA per SM with the stream-K split.
-int gemm_grid(int sms, int tiles, bool decode) {
-#ifdef SARA_STAMPS
-    if (const char *e = getenv("SARA_GEMM_GRID")) return std::max(1, std::min(sms, atoi(e)));  // profiling sweeps
-#endif
-    if (decode && tiles <= sms && tiles * 20 >= sms * 17) return tiles;
-    return sms;
-}
-
+// One prefill projection: the many-row kernel (tensor maps of kBigRows rows) or the few-row one.
 template <int EPI>
-void launch_gemm(cudaStream_t s, bool pdl, int grid, const CUtensorMap &tw, const CUtensorMap &tx,
-                 const CUtensorMap &tx_lo, GemmParams p) {
-    grid = gemm_grid(grid, p.m_tiles, p.decode != 0);
-    p.has_lo = 1;
-    launch(s, pdl, dim3(grid), dim3(kGemmThreads), kGemmSmemBytes, gemm_tc_kernel<EPI>, tw, tx, tx_lo, p);
+void launch_gemm(const sara_handle &h, cudaStream_t s, bool pdl, bool big, const CUtensorMap &tx, const CUtensorMap &tx_lo,
+                 GemmParams p) {
+    if (big)
+        launch(s, pdl, dim3(h.sms), dim3(kBigThreads), kBigSmemBytes, prefill_gemm_kernel<EPI>, tx, tx_lo, p,
+               p.m_tiles * kTileM, h.big_part);
+    else
+        launch(s, pdl, dim3(h.sms), dim3(kGemmThreads), kGemmSmemBytes, gemm_tc_kernel<EPI>, tx, tx_lo, p);
 }
 
 GemmParams gemm_base(const sara_handle &h, int m_tiles, int k_chunks, const Acts &A, const int *rows_dev) {
@@ -210,7 +209,6 @@ GemmParams gemm_base(const sara_handle &h, int m_tiles, int k_chunks, const Acts
     p.k_chunks = k_chunks;
     p.rows_cap = A.rows_cap;
     p.rows_dev = rows_dev;
-    p.decode = 0;
     p.ws_acc = h.gemm_acc;
     p.ws_cnt = h.gemm_cnt;
     p.err = &h.vars->err;
@@ -225,13 +223,12 @@ enum Kern { K_QKV = 1, K_ATTN = 2, K_OPROJ = 3, K_GATEUP = 4, K_DOWN = 5 };
 
 // Launch one projection / attention kernel of layer l over the prefill rows (one row per
 // fresh prompt token, KV = the prompt slots).  Weights are read from the blocked tiles.
-void enqueue_prefill_kernel(sara_handle &h, cudaStream_t s, int which, int l, bool pdl) {
+void enqueue_prefill_kernel(sara_handle &h, cudaStream_t s, int which, int l, bool pdl, bool big) {
     const sara_model_cfg &m = h.cfg;
     const StepPtrs &c = h.ptrs;
     Acts &A = h.pre;
     const int *rows_dev = &h.vars->pre_rows;
     const int d = m.d_model, H = m.n_heads, KVH = m.n_kv_heads, hd = m.head_dim, F = m.ffn;
-    const int G = h.sms;
     const bool last = l == m.layers - 1;
     uint16_t *kv_l = h.kv_pr + l * h.kv_pr_layer;
     switch (which) {
@@ -249,7 +246,7 @@ void enqueue_prefill_kernel(sara_handle &h, cudaStream_t s, int which, int l, bo
             p.kv = kv_l;
             p.kv_slot_stride = h.kv_pr_slot;
             p.kv_cap = h.cap_p;
-            launch_gemm<EPI_QKV>(s, pdl, G, A.tm_xg, A.tm_xg, A.tm_xg_lo, p);
+            launch_gemm<EPI_QKV>(h, s, pdl, big, big ? A.big_xg : A.tm_xg, big ? A.big_xg_lo : A.tm_xg_lo, p);
             break;
         }
         case K_ATTN: {
@@ -280,7 +277,7 @@ void enqueue_prefill_kernel(sara_handle &h, cudaStream_t s, int which, int l, bo
             p.g_next = h.norm_mlp + (size_t)l * d;
             p.ssq_out = A.ssq_m;
             p.ld = d;
-            launch_gemm<EPI_RESID>(s, pdl, G, A.tm_att, A.tm_att, A.tm_att_lo, p);
+            launch_gemm<EPI_RESID>(h, s, pdl, big, big ? A.big_att : A.tm_att, big ? A.big_att_lo : A.tm_att_lo, p);
             break;
         }
         case K_GATEUP: {
@@ -290,7 +287,7 @@ void enqueue_prefill_kernel(sara_handle &h, cudaStream_t s, int which, int l, bo
             p.h_out = A.h;
             p.h_lo = A.h_lo;
             p.ld = F;
-            launch_gemm<EPI_SWIGLU>(s, pdl, G, A.tm_xg, A.tm_xg, A.tm_xg_lo, p);
+            launch_gemm<EPI_SWIGLU>(h, s, pdl, big, big ? A.big_xg : A.tm_xg, big ? A.big_xg_lo : A.tm_xg_lo, p);
             break;
         }
         case K_DOWN: {
@@ -302,7 +299,7 @@ void enqueue_prefill_kernel(sara_handle &h, cudaStream_t s, int which, int l, bo
             p.g_next = last ? h.final_norm : h.norm_attn + (size_t)(l + 1) * d;
             p.ssq_out = A.ssq_a;
             p.ld = d;
-            launch_gemm<EPI_RESID>(s, pdl, G, A.tm_h, A.tm_h, A.tm_h_lo, p);
+            launch_gemm<EPI_RESID>(h, s, pdl, big, big ? A.big_h : A.tm_h, big ? A.big_h_lo : A.tm_h_lo, p);
             break;
         }
         default: throw SaraError(SARA_EINVAL, "unknown kernel id");
@@ -376,21 +373,26 @@ void enqueue_decode_step(sara_handle &h, cudaStream_t s, bool write_logits = fal
 
 // Prefill of the fresh prompts of a round: embedding, every layer up to the last layer's
 // K/V (the prompt's last hidden state is not needed: its last token is the rollouts' first
-// decode row).
-void enqueue_prefill(sara_handle &h, cudaStream_t s, bool pdl) {
-    const sara_model_cfg &m = h.cfg;
-    const StepPtrs &c = h.ptrs;
+// decode row).  The layers run the many-row or the few-row GEMM (see kPrefillFewRows).
+int few_rows(const sara_handle &h) {
+    const int K = std::max({h.cfg.d_model, h.cfg.n_heads * h.cfg.head_dim, h.cfg.ffn});
+    return K / 64 > kPrefillFewChunks ? kPrefillFewRows : 0;
+}
+void enqueue_prefill_embed(sara_handle &h, cudaStream_t s) {
     Acts &A = h.pre;
-    launch(s, false, dim3(A.rows_cap), dim3(128), 0, embed_kernel, (const uint16_t *)h.embed,
-           (const uint16_t *)h.norm_attn, (const int *)&h.vars->pre_rows, (const int *)c.pre_tok, m.d_model,
-           A.rows_cap, m.vocab, A.x_f32, A.xg, A.xg_lo, A.ssq_a, &h.vars->err);
+    launch(s, false, dim3((A.rows_cap + 7) / 8), dim3(256), 0, embed_kernel, (const uint16_t *)h.embed,
+           (const uint16_t *)h.norm_attn, (const int *)&h.vars->pre_rows, (const int *)h.ptrs.pre_tok, h.cfg.d_model,
+           A.rows_cap, h.cfg.vocab, A.x_f32, A.xg, A.xg_lo, A.ssq_a, &h.vars->err);
+}
+void enqueue_prefill_layers(sara_handle &h, cudaStream_t s, bool pdl, bool big) {
+    const sara_model_cfg &m = h.cfg;
     for (int l = 0; l < m.layers; ++l) {
-        enqueue_prefill_kernel(h, s, K_QKV, l, pdl);
+        enqueue_prefill_kernel(h, s, K_QKV, l, pdl, big);
         if (l == m.layers - 1) break;
-        enqueue_prefill_kernel(h, s, K_ATTN, l, pdl);
-        enqueue_prefill_kernel(h, s, K_OPROJ, l, pdl);
-        enqueue_prefill_kernel(h, s, K_GATEUP, l, pdl);
-        enqueue_prefill_kernel(h, s, K_DOWN, l, pdl);
+        enqueue_prefill_kernel(h, s, K_ATTN, l, pdl, big);
+        enqueue_prefill_kernel(h, s, K_OPROJ, l, pdl, big);
+        enqueue_prefill_kernel(h, s, K_GATEUP, l, pdl, big);
+        enqueue_prefill_kernel(h, s, K_DOWN, l, pdl, big);
     }
 }
 
@@ -402,6 +404,37 @@ void enqueue_prompt_blocks(sara_handle &h, cudaStream_t s, bool pdl, const StepP
 
 
 // ------------------------------------------------------------------------ graph
+// More than `few` prefill rows: the condition of the prefill's two GEMM variants.
+__global__ void prefill_route_kernel(cudaGraphConditionalHandle many, const int *rows, int few) {
+    cudaGraphSetConditional(many, *rows > few ? 1u : 0u);
+}
+
+// Adds IF(hc) {fills[0]} (ELSE {fills[1]}) to the graph that stream cs captures; the branches are
+// captured on `inner`.
+void add_if(cudaStream_t cs, cudaStream_t inner, cudaGraphConditionalHandle hc,
+            const std::vector<std::function<void(cudaStream_t)>> &fills) {
+    cudaStreamCaptureStatus st;
+    cudaGraph_t capg;
+    const cudaGraphNode_t *deps = nullptr;
+    size_t ndeps = 0;
+    CK(cudaStreamGetCaptureInfo(cs, &st, nullptr, &capg, &deps, nullptr, &ndeps));
+    std::vector<cudaGraphNode_t> dv(deps, deps + ndeps);
+    cudaGraphNodeParams ip{};
+    ip.type = cudaGraphNodeTypeConditional;
+    ip.conditional.handle = hc;
+    ip.conditional.type = cudaGraphCondTypeIf;
+    ip.conditional.size = (unsigned)fills.size();
+    cudaGraphNode_t inode;
+    CK(cudaGraphAddNode(&inode, capg, dv.data(), nullptr, dv.size(), &ip));
+    CK(cudaStreamUpdateCaptureDependencies(cs, &inode, nullptr, 1, cudaStreamSetCaptureDependencies));
+    for (size_t i = 0; i < fills.size(); ++i) {
+        cudaGraph_t body = ip.conditional.phGraph_out[i], done;
+        CK(cudaStreamBeginCaptureToGraph(inner, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
+        fills[i](inner);
+        CK(cudaStreamEndCapture(inner, &done));
+    }
+}
+
 void build_graph(sara_handle &h) {
     const bool pdl = h.use_pdl;
     CK(cudaGraphCreate(&h.graph, 0));
@@ -423,30 +456,20 @@ void build_graph(sara_handle &h) {
     CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
     launch(cs, false, dim3(1), dim3(kCtlThreads), 0, ctl_kernel, h.ptrs, hs, h.has_model ? 3 : 1);
     if (h.has_model) {
-        // IF(fresh prompts) { prefill }, then IF(new rollouts) { KV blocks of the new rollouts }
-        auto add_if = [&](cudaGraphConditionalHandle hc, const std::function<void(cudaStream_t)> &fill) {
-            cudaStreamCaptureStatus st;
-            cudaGraph_t capg;
-            const cudaGraphNode_t *deps = nullptr;
-            size_t ndeps = 0;
-            CK(cudaStreamGetCaptureInfo(cs, &st, nullptr, &capg, &deps, nullptr, &ndeps));
-            std::vector<cudaGraphNode_t> dv(deps, deps + ndeps);
-            cudaGraphNodeParams ip{};
-            ip.type = cudaGraphNodeTypeConditional;
-            ip.conditional.handle = hc;
-            ip.conditional.type = cudaGraphCondTypeIf;
-            ip.conditional.size = 1;
-            cudaGraphNode_t inode;
-            CK(cudaGraphAddNode(&inode, capg, dv.data(), nullptr, dv.size(), &ip));
-            CK(cudaStreamUpdateCaptureDependencies(cs, &inode, nullptr, 1, cudaStreamSetCaptureDependencies));
-            cudaGraph_t ibody = ip.conditional.phGraph_out[0];
-            CK(cudaStreamBeginCaptureToGraph(h.cap_stream2, ibody, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
-            fill(h.cap_stream2);
-            cudaGraph_t ib2;
-            CK(cudaStreamEndCapture(h.cap_stream2, &ib2));
-        };
-        add_if(hs.h[2], [&](cudaStream_t st) { enqueue_prefill(h, st, pdl); });
-        add_if(hs.h[1], [&](cudaStream_t st) { enqueue_prompt_blocks(h, st, pdl, h.ptrs); });
+        // IF(fresh prompts) { embedding; IF(many rows) {layers} ELSE {layers} }, then
+        // IF(new rollouts) { KV blocks of the new rollouts }
+        add_if(cs, h.cap_stream2, hs.h[2], {[&](cudaStream_t st) {
+            enqueue_prefill_embed(h, st);
+            cudaStreamCaptureStatus cst;
+            cudaGraph_t pg;
+            CK(cudaStreamGetCaptureInfo(st, &cst, nullptr, &pg, nullptr, nullptr, nullptr));
+            cudaGraphConditionalHandle hr;
+            CK(cudaGraphConditionalHandleCreate(&hr, pg, 0, cudaGraphCondAssignDefault));
+            launch(st, false, dim3(1), dim3(1), 0, prefill_route_kernel, hr, (const int *)&h.vars->pre_rows, few_rows(h));
+            add_if(st, h.cap_stream3, hr, {[&](cudaStream_t s3) { enqueue_prefill_layers(h, s3, pdl, true); },
+                                           [&](cudaStream_t s3) { enqueue_prefill_layers(h, s3, pdl, false); }});
+        }});
+        add_if(cs, h.cap_stream2, hs.h[1], {[&](cudaStream_t st) { enqueue_prompt_blocks(h, st, pdl, h.ptrs); }});
         enqueue_decode_step(h, cs);
     }
     cudaGraph_t b2;
@@ -467,7 +490,10 @@ void run_host_loop(sara_handle &h, int schedule) {
         if (!h.has_model) continue;
         const bool joins = schedule != 0 ? v.n_new > 0 : (v.round_steps == 0 && v.live > 0);
         if (joins) {
-            if (v.n_fresh > 0) enqueue_prefill(h, s, h.use_pdl);
+            if (v.n_fresh > 0) {
+                enqueue_prefill_embed(h, s);
+                enqueue_prefill_layers(h, s, h.use_pdl, v.pre_rows > few_rows(h));
+            }
             enqueue_prompt_blocks(h, s, h.use_pdl, h.ptrs);
         }
         enqueue_decode_step(h, s);
@@ -608,6 +634,13 @@ void make_tensor_maps(sara_handle &h) {
     const sara_model_cfg &m = h.cfg;
     const int d = m.d_model, H = m.n_heads, hd = m.head_dim, F = m.ffn;
     Acts *A = &h.pre;
+    auto big = [&](const uint16_t *x, int K) { return make_tmap_bf16(x, K, A->rows_cap, kTileK, kBigRows); };
+    A->big_xg = big(A->xg, d);
+    A->big_xg_lo = big(A->xg_lo, d);
+    A->big_att = big(A->att, H * hd);
+    A->big_att_lo = big(A->att_lo, H * hd);
+    A->big_h = big(A->h, F);
+    A->big_h_lo = big(A->h_lo, F);
     A->tm_xg = make_tmap_bf16(A->xg, d, A->rows_cap, kTileK, kXBoxRows);
     A->tm_xg_lo = make_tmap_bf16(A->xg_lo, d, A->rows_cap, kTileK, kXBoxRows);
     A->tm_att = make_tmap_bf16(A->att, H * hd, A->rows_cap, kTileK, kXBoxRows);
@@ -658,6 +691,7 @@ void create_impl(sara_handle &h, const sara_model_cfg *cfgp, const sara_weights 
     set_kernel_attrs();
     CK(cudaStreamCreateWithFlags(&h.cap_stream, cudaStreamNonBlocking));
     CK(cudaStreamCreateWithFlags(&h.cap_stream2, cudaStreamNonBlocking));
+    CK(cudaStreamCreateWithFlags(&h.cap_stream3, cudaStreamNonBlocking));
     CK(cudaEventCreate(&h.ev0));
     CK(cudaEventCreate(&h.ev1));
 
@@ -750,6 +784,7 @@ void create_impl(sara_handle &h, const sara_model_cfg *cfgp, const sara_weights 
         alloc_acts(h, h.pre, h.pre_cap);
         alloc_decode(h);
         // GEMM stream-K workspace: one fixed-point tile sum per CTA + per-tile counters (zeroed)
+        h.big_part = h.mem.alloc<float>((size_t)2 * h.sms * kBigPartFloats, false);
         h.gemm_acc = h.mem.alloc<unsigned long long>((size_t)h.sms * kTileR * kTileM);
         const int max_m = std::max({(m.n_heads + 2 * KVH) * hd, d, 2 * m.ffn, m.vocab}) / 128;
         h.gemm_cnt = h.mem.alloc<int>((size_t)max_m * ((h.pre_cap + kTileR - 1) / kTileR + 1));
@@ -950,7 +985,8 @@ void teacher_impl(sara_handle &h, int n, int Lp, const int32_t *prompts, int T, 
     try {
         reset_decode_state(h, s);
         launch(s, false, dim3(1), dim3(kCtlThreads), 0, teacher_setup_kernel, c, n, (const int64_t *)h.uid_dev);
-        enqueue_prefill(h, s, false);
+        enqueue_prefill_embed(h, s);
+        enqueue_prefill_layers(h, s, h.use_pdl, n * (Lp - 1) > few_rows(h));
         enqueue_prompt_blocks(h, s, false, c);
         for (int step = 0; step < T; ++step) {
             enqueue_decode_step(h, s, true);

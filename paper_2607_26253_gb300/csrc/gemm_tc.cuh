@@ -1,13 +1,14 @@
-// Projection GEMM of the prefill path on sm_103a:
+// Projection GEMM of a prefill of few rows (see kPrefillFewRows):
 //     Y[r][n] = sum_c X[r][c] * W[n][c]        (X: activations, W: a linear layer's weight)
 // computed "swap-AB" on the 5th-generation tensor core: the weight tile is the MMA's A
 // operand (M = 128 output features), the activation rows are B (N = rows rounded up to
 // 16, <= 128), the fp32 accumulator lives in tensor memory.  Activations arrive as a bf16
 // pair hi + lo (hi = bf16(x), lo = bf16(x - hi)); both are multiplied with the same weight
 // tile into the same accumulator, so the product keeps ~16 mantissa bits of x at the cost of
-// one extra MMA per weight tile (the GEMM is weight-bandwidth bound).  Operands are staged in shared
-// memory by TMA (128-byte swizzle) through a multi-stage mbarrier pipeline; one elected
-// thread issues tcgen05.mma; four epilogue warps read the accumulator with tcgen05.ld.
+// one extra MMA per weight tile (the GEMM is weight-bandwidth bound).  Weights come as bulk copies
+// of pre-swizzled blocks, activations by TMA (128-byte swizzle), through a multi-stage mbarrier
+// pipeline; one elected thread issues tcgen05.mma; four epilogue warps read the accumulator with
+// tcgen05.ld.
 //
 // Work split: stream-K.  The (tile, k-chunk) units of the whole GEMM are cut into
 // gridDim.x equal contiguous ranges, so every SM streams the same number of weight bytes.
@@ -18,17 +19,12 @@
 //
 // Warp roles (192 threads): warp 0 = TMA producer, warp 1 = MMA issuer + tensor-memory
 // owner, warps 2..5 = epilogue (warp w reads tensor-memory lanes 32*(w%4) .. +31).
-//
-// In decode mode (one row tile) the producer streams the first pipeline stages of weights
-// before waiting on the preceding grid (programmatic dependent launch), so weight reads
-// overlap the previous kernel's tail.
 #pragma once
 #include "device_common.cuh"
 
 namespace sara {
 
 enum EpiKind : int {
-    EPI_F32 = 0,     // Y fp32 [rows][ld]
     EPI_QKV = 1,     // RMSNorm scale, RoPE on q/k, q -> q_out (fp16), k/v -> KV cache (fp16)
     EPI_RESID = 2,   // x += Y; xg = x * g_next as a bf16 hi/lo pair; per-tile sum of squares of x
     EPI_SWIGLU = 3,  // RMSNorm scale; rows alternate 8 gate, 8 up -> h = silu(g) * u (hi/lo)
@@ -47,16 +43,13 @@ constexpr int kEpiLd = 33;                          // padded fp32 row of the ex
 struct GemmParams {
     int m_tiles, k_chunks;
     int rows_cap;              // rows of the activation tensor map
-    const int *rows_dev;       // device count of valid rows (nullptr -> rows_fixed)
-    int rows_fixed;
-    int decode;                // 1: a single row tile, weights prefetched before the PDL wait
-    const uint8_t *w_blk;      // non-null: W stored chunk-major, pre-swizzled (bulk copies, wblk128_off)
-    int has_lo;                // 1: the activation's lo part (second tensor map) is multiplied too
+    const int *rows_dev;       // device count of valid rows
+    const uint8_t *w_blk;      // W stored chunk-major, pre-swizzled (bulk copies, wblk128_off)
     unsigned long long *ws_acc;  // [gridDim.x][kTileR * kTileM] fixed-point tile sums, zero between launches
     int *ws_cnt;               // [tiles] arrival counters, zero between launches
     int *err;
     // outputs / epilogue inputs
-    float *y_f32; int ld;      // EPI_F32 output; row stride
+    int ld;                    // row stride of the outputs
     const float *ssq;          // [ssq_tiles][rows_cap] per-128-feature partial sums of x^2
     int ssq_tiles; float inv_dim; float eps;
     uint16_t *q_out;           // EPI_QKV: [rows][n_heads * head_dim] fp16
@@ -125,11 +118,7 @@ __device__ __forceinline__ void gemm_epilogue_chunk(const GemmParams &p, GemmSme
                                                     int r_base, int c0, int rows_in_tile, int mrow, int etid) {
     const int n = m_tile * kTileM + mrow;  // output feature
     const int ncols = min(32, rows_in_tile - c0);
-    if constexpr (EPI == EPI_F32) {
-#pragma unroll
-        for (int c = 0; c < 32; ++c)
-            if (c < ncols) p.y_f32[(int64_t)(r_base + c0 + c) * p.ld + n] = v[c];
-    } else {
+    {
         if constexpr (EPI == EPI_QKV || EPI == EPI_SWIGLU) {
 #pragma unroll
             for (int c = 0; c < 32; ++c) v[c] *= S.inv_rms[c0 + c];
@@ -221,8 +210,7 @@ __device__ __forceinline__ void gemm_epilogue_chunk(const GemmParams &p, GemmSme
 
 template <int EPI>
 __global__ void __launch_bounds__(kGemmThreads, 1)
-gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX,
-               const __grid_constant__ CUtensorMap tmXlo, GemmParams p) {
+gemm_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmXlo, GemmParams p) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t *sW = base;
@@ -242,9 +230,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         S.epi_abort = 0;
         S.skip = (p.err != nullptr) && (*(volatile int *)p.err != 0);
         fence_mbar_init();
-        if (!p.w_blk) prefetch_tensormap(&tmW);
         prefetch_tensormap(&tmX);
-        if (p.has_lo) prefetch_tensormap(&tmXlo);
+        prefetch_tensormap(&tmXlo);
     }
     if (warp == 1) { tmem_alloc(&S.tmem_base, 256); tmem_relinquish(); }
     tc_fence_before();
@@ -257,42 +244,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     pdl_allow_dependents();
 
     const int m_tiles = p.m_tiles, kch = p.k_chunks;
-    // In decode mode the row count does not change the partition (one row tile).
-    int rows = 0, r_tiles = 1;
-    if (!p.decode) {
-        pdl_wait_prior_grids();
-        rows = p.rows_dev ? min(*p.rows_dev, p.rows_cap) : p.rows_fixed;
-        r_tiles = (rows + kTileR - 1) / kTileR;
-    }
+    pdl_wait_prior_grids();
+    const int rows = min(*p.rows_dev, p.rows_cap), r_tiles = (rows + kTileR - 1) / kTileR;
     const int64_t U = (int64_t)m_tiles * r_tiles * kch;
     const int64_t u0 = S.skip ? 0 : unit_begin(cta, U, G);
     const int64_t u1 = S.skip ? 0 : unit_begin(cta + 1, U, G);
 
     if (warp == 0) {
         // ------------------------------------------------------------ TMA producer
-        if (p.decode) {
-            if (lane == 0) {
-                // weights of the first stages before the dependency wait
-                const int64_t n_pre = min64(kGemmStages, u1 - u0);
-                for (int64_t i = 0; i < n_pre; ++i) {
-                    const int64_t u = u0 + i;
-                    const int tile = (int)(u / kch), kc = (int)(u % kch);
-                    const int m_tile = tile % m_tiles;
-                    mbar_expect_tx(&S.full[i], (uint32_t)kWStageBytes);
-                    if (p.w_blk)
-                        bulk_load(sW + i * kWStageBytes, p.w_blk + wblk128_off(m_tiles * kTileM, m_tile, kc),
-                                  kWStageBytes, &S.full[i], l2_policy_evict_first());
-                    else
-                        tma_load_2d(sW + i * kWStageBytes, &tmW, &S.full[i], kc * kTileK, m_tile * kTileM,
-                                    l2_policy_evict_first());
-                }
-            }
-            pdl_wait_prior_grids();
-            rows = p.rows_dev ? min(*p.rows_dev, p.rows_cap) : p.rows_fixed;
-        }
         if (lane == 0) {
             const uint64_t pol_w = l2_policy_evict_first(), pol_x = l2_policy_evict_last();
-            const int64_t n_pre = p.decode ? min64(kGemmStages, u1 - u0) : 0;
             int64_t i = 0;
             for (int64_t u = u0; u < u1; ++u, ++i) {
                 const int s = (int)(i % kGemmStages);
@@ -303,24 +264,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
                 const int m_tile = tile % m_tiles, r_tile = tile / m_tiles;
                 const int rin = min(kTileR, max(rows - r_tile * kTileR, 0));
                 const int nbox = max(1, (rin + kXBoxRows - 1) / kXBoxRows);
-                const uint32_t xbytes = (uint32_t)(nbox * kXBoxRows * kTileK * 2) * (p.has_lo ? 2u : 1u);
-                if (i >= n_pre) {
-                    mbar_arrive_expect_tx(&S.full[s], (uint32_t)kWStageBytes + xbytes);
-                    if (p.w_blk)
-                        bulk_load(sW + (size_t)s * kWStageBytes,
-                                  p.w_blk + wblk128_off(m_tiles * kTileM, m_tile, kc), kWStageBytes,
-                                  &S.full[s], pol_w);
-                    else
-                        tma_load_2d(sW + (size_t)s * kWStageBytes, &tmW, &S.full[s], kc * kTileK, m_tile * kTileM,
-                                    pol_w);
-                } else {
-                    mbar_arrive_expect_tx(&S.full[s], xbytes);
-                }
+                const uint32_t xbytes = (uint32_t)(nbox * kXBoxRows * kTileK * 2) * 2u;
+                mbar_arrive_expect_tx(&S.full[s], (uint32_t)kWStageBytes + xbytes);
+                bulk_load(sW + (size_t)s * kWStageBytes, p.w_blk + wblk128_off(m_tiles * kTileM, m_tile, kc), kWStageBytes,
+                          &S.full[s], pol_w);
                 for (int b = 0; b < nbox; ++b) {
                     tma_load_2d(sX + (size_t)s * kXStageBytes + b * kXBoxRows * kTileK * 2, &tmX, &S.full[s],
                                 kc * kTileK, r_tile * kTileR + b * kXBoxRows, pol_x);
-                    if (p.has_lo)
-                        tma_load_2d(sXlo + (size_t)s * kXStageBytes + b * kXBoxRows * kTileK * 2, &tmXlo, &S.full[s],
+                    tma_load_2d(sXlo + (size_t)s * kXStageBytes + b * kXBoxRows * kTileK * 2, &tmXlo, &S.full[s],
                                     kc * kTileK, r_tile * kTileR + b * kXBoxRows, pol_x);
                 }
             }
@@ -335,10 +286,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
-        if (p.decode) {
-            pdl_wait_prior_grids();
-            rows = p.rows_dev ? min(*p.rows_dev, p.rows_cap) : p.rows_fixed;
-        }
         if (lane == 0) {
             int64_t i = 0;
             int seg = 0;
@@ -373,7 +320,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
                     for (int kk = 0; kk < kTileK / 16; ++kk) {
                         const uint64_t adesc = sdesc_kmajor_sw128(aw + kk * 32);
                         tc_mma_bf16(d, adesc, sdesc_kmajor_sw128(ax + kk * 32), idesc, (first && kk == 0) ? 0u : 1u);
-                        if (p.has_lo) tc_mma_bf16(d, adesc, sdesc_kmajor_sw128(axl + kk * 32), idesc, 1u);
+                        tc_mma_bf16(d, adesc, sdesc_kmajor_sw128(axl + kk * 32), idesc, 1u);
                     }
                     first = false;
                     tc_commit(&S.empty[s]);
@@ -388,15 +335,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         }
     } else {
         // ------------------------------------------------------------ epilogue (warps 2..5)
-        pdl_wait_prior_grids();
-        if (p.decode) rows = p.rows_dev ? min(*p.rows_dev, p.rows_cap) : p.rows_fixed;
         const int quarter = warp & 3;
         const int mrow = quarter * 32 + lane;
         const int etid = threadIdx.x - 64;  // 0..127
         const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
-        // Per-row values (1/rms, position, KV slot) staged once per tile: in
-        // decode mode every tile has the same rows, so they are loaded once, while the
-        // mainloop streams weights.
+        // Per-row values (1/rms, position, KV slot) staged once per row tile.
         int staged_rbase = -1;
         auto stage_rows = [&](int r_base, int rin) {
             if constexpr (EPI == EPI_QKV || EPI == EPI_SWIGLU) {
@@ -423,10 +366,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
                 named_bar_sync(1, 128);
             }
         };
-        if (p.decode && u0 < u1) {
-            stage_rows(0, min(kTileR, rows));
-            staged_rbase = 0;
-        }
         int seg = 0;
         for (int64_t u = u0; u < u1; ++seg) {
             const int tile = (int)(u / kch);

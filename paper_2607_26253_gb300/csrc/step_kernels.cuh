@@ -9,35 +9,41 @@
 namespace sara {
 
 // x_f32[r] = E[tok[r]]; xg[r] = x * g as a bf16 hi/lo pair; ssq[t][r] = sum over features
-// [128t, 128t+128) of x^2.  One CTA (128 threads) per row; rows >= *rows_dev exit.
-static __global__ void __launch_bounds__(128) embed_kernel(const uint16_t *E, const uint16_t *g, const int *rows_dev,
+// [128t, 128t+128) of x^2.  One warp per row, four features a lane, so that a 128-feature sum is one
+// warp reduction; bound by its stores (10 bytes a feature: 16,320 x 1,536 77 -> 42 us against a CTA
+// per row with two barriers per 128 features).
+static __global__ void __launch_bounds__(256) embed_kernel(const uint16_t *E, const uint16_t *g, const int *rows_dev,
                                                            const int *row_tok, int d, int rows_cap, int vocab,
                                                            float *x_f32, uint16_t *xg, uint16_t *xg_lo, float *ssq,
                                                            int *err) {
     pdl_wait_prior_grids();
     pdl_allow_dependents();
-    const int rows = min(*rows_dev, rows_cap);
-    __shared__ float red[4];
-    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
+    const int rows = min(*rows_dev, rows_cap), lane = threadIdx.x & 31;
+    for (int r = blockIdx.x * 8 + (threadIdx.x >> 5); r < rows; r += gridDim.x * 8) {
         int tok = row_tok[r];
         if (tok < 0 || tok >= vocab) {  // token ids come from the caller: never read outside E
-            if (threadIdx.x == 0) report_error(err, ERR_BOUNDS);
+            if (lane == 0) report_error(err, ERR_BOUNDS);
             tok = 0;
         }
         const uint16_t *er = E + (int64_t)tok * d;
+#pragma unroll 4
         for (int t = 0; t < d / 128; ++t) {
-            const int f = t * 128 + threadIdx.x;
-            const float x = bf16_to_f32(er[f]);
-            x_f32[(int64_t)r * d + f] = x;
-            uint16_t hi, lo;
-            split_bf16(x * bf16_to_f32(g[f]), hi, lo);
-            xg[(int64_t)r * d + f] = hi;
-            xg_lo[(int64_t)r * d + f] = lo;
-            const float s = warp_sum(x * x);
-            if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-            __syncthreads();
-            if (threadIdx.x == 0) ssq[(int64_t)t * rows_cap + r] = red[0] + red[1] + red[2] + red[3];
-            __syncthreads();
+            const int f = t * 128 + lane * 4;
+            const uint2 e = __ldg(reinterpret_cast<const uint2 *>(er + f));
+            const uint2 w = __ldg(reinterpret_cast<const uint2 *>(g + f));
+            const float4 x = make_float4(bf16_to_f32(e.x & 0xffff), bf16_to_f32(e.x >> 16), bf16_to_f32(e.y & 0xffff),
+                                         bf16_to_f32(e.y >> 16));
+            uint16_t hi[4], lo[4];
+            split_bf16(x.x * bf16_to_f32(w.x & 0xffff), hi[0], lo[0]);
+            split_bf16(x.y * bf16_to_f32(w.x >> 16), hi[1], lo[1]);
+            split_bf16(x.z * bf16_to_f32(w.y & 0xffff), hi[2], lo[2]);
+            split_bf16(x.w * bf16_to_f32(w.y >> 16), hi[3], lo[3]);
+            const int64_t o = (int64_t)r * d + f;
+            *reinterpret_cast<float4 *>(x_f32 + o) = x;
+            *reinterpret_cast<uint2 *>(xg + o) = pack4(hi);
+            *reinterpret_cast<uint2 *>(xg_lo + o) = pack4(lo);
+            const float s = warp_sum((x.x * x.x + x.y * x.y) + (x.z * x.z + x.w * x.w));
+            if (lane == 0) ssq[(int64_t)t * rows_cap + r] = s;
         }
     }
 }
