@@ -180,10 +180,10 @@ __device__ __forceinline__ uint64_t sampler_row_seed(uint64_t sample_seed, int64
 }
 
 // The step graph's conditions: h[0] loop, h[1] rollouts join (their KV set-up runs), h[2] fresh
-// prompts are prefilled first (-1: whenever rollouts join).  use_handles: bit 0 = h[0] exists,
-// bit 1 = h[1] and h[2] exist.
+// prompts are prefilled first (-1: whenever rollouts join), h[3] decode steps up to the next
+// boundary with work for the controller.  use_handles: bit 0 = h[0] exists, bit 1 = the others.
 struct CondHandles {
-    cudaGraphConditionalHandle h[3];
+    cudaGraphConditionalHandle h[4];
 };
 __device__ __forceinline__ void set_conds(const CondHandles &hs, int loop, int round_start, int use_handles,
                                           int prefill = -1) {
@@ -192,6 +192,7 @@ __device__ __forceinline__ void set_conds(const CondHandles &hs, int loop, int r
         if (use_handles & 2) {
             cudaGraphSetConditional(hs.h[1], round_start ? 1u : 0u);
             cudaGraphSetConditional(hs.h[2], (prefill < 0 ? round_start : prefill) ? 1u : 0u);
+            cudaGraphSetConditional(hs.h[3], loop ? 1u : 0u);
         }
     }
 }
@@ -732,7 +733,10 @@ static __device__ void ctl_async_step(const StepConst &K, StepVars &V, const Ste
     set_conds(hs, !done, !done && V.n_new > 0, use_handles, !done && V.n_fresh > 0);
 }
 
-// Per-iteration controller kernel of the step graph.
+// Controller kernel of the step graph: a round end and the next round's start, or a boundary of
+// the asynchronous schedule.  (The decode steps in between loop in the graph without it.)  Without
+// a policy every round's rollouts are finished at once, so the rounds loop in here: a graph
+// iteration per round cost as much as the round (97 rounds over 65,536 prompts: 1.6 ms).
 static __global__ void __launch_bounds__(kCtlThreads, 1)
 ctl_kernel(StepPtrs c, CondHandles hs, int use_handles) {
     __shared__ CtlShared sh;
@@ -780,10 +784,25 @@ ctl_kernel(StepPtrs c, CondHandles hs, int use_handles) {
         set_conds(hs, 0, 0, use_handles);
         return;
     }
-    ctl_round(K, V, c, sh);
-    __syncthreads();
-    if (V.err & (ERR_CAPACITY | ERR_BOUNDS)) { if (threadIdx.x == 0) V.done = 1; }
-    __syncthreads();
+    for (;;) {
+        ctl_round(K, V, c, sh);
+        __syncthreads();
+        if (V.err & (ERR_CAPACITY | ERR_BOUNDS)) { if (threadIdx.x == 0) V.done = 1; }
+        __syncthreads();
+        if (K.decode || V.done) break;
+        // the next iteration's bounds (as at the top of the kernel)
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            V.iters += 1;
+            if ((K.max_iters > 0 && V.iters > K.max_iters) || V.rounds_done > K.N + 1) {
+                report_error(&V.err, ERR_ITER_BOUND);
+                V.done = 1;
+                V.live = 0;
+            }
+        }
+        __syncthreads();
+        if (V.done) break;
+    }
     const int done = V.done;
     if (done) {
         // remaining active prompts end INCOMPLETE

@@ -364,11 +364,13 @@ MegaParams mega_params(const sara_handle &h) {
 // One decode step over the live rows: the persistent decode-step kernel (embedding, every
 // layer, lm_head with the fused Gumbel-max maxima) followed by the sampling finish and
 // bookkeeping kernel.  write_logits: also store the fp32 logits (teacher forcing).
-void enqueue_decode_step(sara_handle &h, cudaStream_t s, bool write_logits = false) {
+void enqueue_decode_step(sara_handle &h, cudaStream_t s, bool write_logits = false,
+                         const cudaGraphConditionalHandle *more = nullptr) {
     MegaParams mp = mega_params(h);
     mp.write_logits = write_logits ? 1 : 0;
     launch_ex(s, false, true, dim3(h.sms), dim3(kMegaThreads), kMegaSmemBytes, decode_step_kernel, mp);
-    launch(s, false, dim3(h.cfg.max_seqs), dim3(256), 0, sample_finish_kernel, h.ptrs, h.cfg.vocab);
+    launch(s, false, dim3(h.cfg.max_seqs), dim3(256), 0, sample_finish_kernel, h.ptrs, h.cfg.vocab,
+           more ? *more : cudaGraphConditionalHandle{}, more ? 1 : 0);
 }
 
 // Prefill of the fresh prompts of a round: embedding, every layer up to the last layer's
@@ -409,10 +411,10 @@ __global__ void prefill_route_kernel(cudaGraphConditionalHandle many, const int 
     cudaGraphSetConditional(many, *rows > few ? 1u : 0u);
 }
 
-// Adds IF(hc) {fills[0]} (ELSE {fills[1]}) to the graph that stream cs captures; the branches are
-// captured on `inner`.
-void add_if(cudaStream_t cs, cudaStream_t inner, cudaGraphConditionalHandle hc,
-            const std::vector<std::function<void(cudaStream_t)>> &fills) {
+// Adds IF(hc) {fills[0]} (ELSE {fills[1]}) or WHILE(hc) {fills[0]} to the graph that stream cs
+// captures; the branches are captured on `inner`.
+void add_cond(cudaStream_t cs, cudaStream_t inner, cudaGraphConditionalHandle hc, cudaGraphConditionalNodeType type,
+              const std::vector<std::function<void(cudaStream_t)>> &fills) {
     cudaStreamCaptureStatus st;
     cudaGraph_t capg;
     const cudaGraphNode_t *deps = nullptr;
@@ -422,7 +424,7 @@ void add_if(cudaStream_t cs, cudaStream_t inner, cudaGraphConditionalHandle hc,
     cudaGraphNodeParams ip{};
     ip.type = cudaGraphNodeTypeConditional;
     ip.conditional.handle = hc;
-    ip.conditional.type = cudaGraphCondTypeIf;
+    ip.conditional.type = type;
     ip.conditional.size = (unsigned)fills.size();
     cudaGraphNode_t inode;
     CK(cudaGraphAddNode(&inode, capg, dv.data(), nullptr, dv.size(), &ip));
@@ -451,14 +453,16 @@ void build_graph(sara_handle &h) {
     if (h.has_model) {
         CK(cudaGraphConditionalHandleCreate(&hs.h[1], body, 0, cudaGraphCondAssignDefault));
         CK(cudaGraphConditionalHandleCreate(&hs.h[2], body, 0, cudaGraphCondAssignDefault));
+        CK(cudaGraphConditionalHandleCreate(&hs.h[3], body, 0, cudaGraphCondAssignDefault));
     }
     cudaStream_t cs = h.cap_stream;
     CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
     launch(cs, false, dim3(1), dim3(kCtlThreads), 0, ctl_kernel, h.ptrs, hs, h.has_model ? 3 : 1);
     if (h.has_model) {
         // IF(fresh prompts) { embedding; IF(many rows) {layers} ELSE {layers} }, then
-        // IF(new rollouts) { KV blocks of the new rollouts }
-        add_if(cs, h.cap_stream2, hs.h[2], {[&](cudaStream_t st) {
+        // IF(new rollouts) { KV blocks of the new rollouts }, then WHILE(decode steps up to the next
+        // boundary with work for the controller) { decode step; bookkeeping }
+        add_cond(cs, h.cap_stream2, hs.h[2], cudaGraphCondTypeIf, {[&](cudaStream_t st) {
             enqueue_prefill_embed(h, st);
             cudaStreamCaptureStatus cst;
             cudaGraph_t pg;
@@ -466,11 +470,12 @@ void build_graph(sara_handle &h) {
             cudaGraphConditionalHandle hr;
             CK(cudaGraphConditionalHandleCreate(&hr, pg, 0, cudaGraphCondAssignDefault));
             launch(st, false, dim3(1), dim3(1), 0, prefill_route_kernel, hr, (const int *)&h.vars->pre_rows, few_rows(h));
-            add_if(st, h.cap_stream3, hr, {[&](cudaStream_t s3) { enqueue_prefill_layers(h, s3, pdl, true); },
+            add_cond(st, h.cap_stream3, hr, cudaGraphCondTypeIf, {[&](cudaStream_t s3) { enqueue_prefill_layers(h, s3, pdl, true); },
                                            [&](cudaStream_t s3) { enqueue_prefill_layers(h, s3, pdl, false); }});
         }});
-        add_if(cs, h.cap_stream2, hs.h[1], {[&](cudaStream_t st) { enqueue_prompt_blocks(h, st, pdl, h.ptrs); }});
-        enqueue_decode_step(h, cs);
+        add_cond(cs, h.cap_stream2, hs.h[1], cudaGraphCondTypeIf, {[&](cudaStream_t st) { enqueue_prompt_blocks(h, st, pdl, h.ptrs); }});
+        add_cond(cs, h.cap_stream2, hs.h[3], cudaGraphCondTypeWhile,
+                 {[&](cudaStream_t st) { enqueue_decode_step(h, st, false, &hs.h[3]); }});
     }
     cudaGraph_t b2;
     CK(cudaStreamEndCapture(cs, &b2));

@@ -75,7 +75,13 @@ __device__ __forceinline__ int scan256(int v, int &total, int *warp_tot) {
 // to its token (ties: lowest token id).  The last CTA to finish appends each row's token to
 // its rollout, retires rollouts that reached their length, compacts the live rows (order
 // kept) and writes the next step's rows and attention items.
-static __global__ void __launch_bounds__(256) sample_finish_kernel(StepPtrs c, int vocab) {
+//
+// use_more: the kernel ends a decode loop of the step graph and sets its condition: another step
+// follows unless the controller has work (a round's last rollout finished, or on the asynchronous
+// schedule a prompt's batch), an error was reported, or a bound is reached (the controller then
+// reports it).
+static __global__ void __launch_bounds__(256) sample_finish_kernel(StepPtrs c, int vocab, cudaGraphConditionalHandle more,
+                                                                   int use_more) {
     __shared__ float sv[8];
     __shared__ int si[8];
     __shared__ int s_last;
@@ -126,7 +132,10 @@ static __global__ void __launch_bounds__(256) sample_finish_kernel(StepPtrs c, i
         V.kt0 = ~0ull;
         V.kt1 = 0ull;
     }
-    if (live == 0) return;
+    if (live == 0) {
+        if (use_more && tid == 0) cudaGraphSetConditional(more, 0u);
+        return;
+    }
     const StepConst &K = *c.kc;
     const int Lp = K.Lp, B = K.attn_chunk;
     const int nsh = shared_blocks(Lp, B);
@@ -234,6 +243,19 @@ static __global__ void __launch_bounds__(256) sample_finish_kernel(StepPtrs c, i
         V.blk_top = top;
         V.blk_low = low;
         V.slot_top = stop;
+        if (use_more) {
+            bool next = out > 0 && *(volatile int *)&V.err == 0 &&
+                        (K.schedule != 0 ? V.n_dec == 0 && V.exec_steps <= (int64_t)K.N * K.max_gen + 1
+                                         : V.round_steps <= V.round_maxL);
+            if (next) {  // one more iteration of the loop
+                V.iters += 1;
+                if (K.max_iters > 0 && V.iters > K.max_iters) {
+                    report_error(&V.err, ERR_ITER_BOUND);
+                    next = false;
+                }
+            }
+            cudaGraphSetConditional(more, next ? 1u : 0u);
+        }
     }
 }
 
