@@ -887,6 +887,14 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
         cuse ^= 1u << a;
         ++tseg;
     };
+    // What the other lane of a pair holds of this lane's 16 of 32 columns (not a pair: nothing).
+    auto pair_part = [&](const float (&v)[32], float (&w)[16]) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const float t = __shfl_xor_sync(0xffffffffu, second ? v[e] : v[16 + e], 8);
+            w[e] = pair ? t : 0.f;
+        }
+    };
     // phase arrival: the CTA's writes of this phase (made visible to thread 0 by the barrier)
     // are released to the other CTAs with the counter increment
     // (x_operand: this phase wrote a GEMM operand that bulk copies of other CTAs will read)
@@ -1051,18 +1059,16 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                         for (int un = 2 * half; un < nu; un += 4) {
                             float v[32];
                             tmem_ld_32x32b_x32(tmem + lane_base + a * kTileN + un * kOwnCols, v);
-                            if (pair) {
-#pragma unroll
-                                for (int e = 0; e < 32; ++e) v[e] += __shfl_xor_sync(0xffffffffu, v[e], 8);
-                            }
+                            float w[16];
+                            pair_part(v, w);
 #pragma unroll 1
                             for (int q = second ? 1 : 0; q < (pair && !second ? 1 : 2); ++q) {
                                 if (!act || un + q >= nu) continue;
                                 uint16_t hh[8], hl[8];
 #pragma unroll
                                 for (int e = 0; e < 8; ++e) {
-                                    const float gv = (q ? v[16 + e] : v[e]) * rs;
-                                    const float uv = (q ? v[24 + e] : v[8 + e]) * rs;
+                                    const float gv = ((q ? v[16 + e] : v[e]) + w[e]) * rs;
+                                    const float uv = ((q ? v[24 + e] : v[8 + e]) + w[8 + e]) * rs;
                                     split_bf16(gv / (1.0f + expf(-gv)) * uv, hh[e], hl[e]);
                                 }
                                 uint8_t *dst = p.hm + xblk_off(my_row, sg.col0 / 2 + (un + q) * 8, R16c);
@@ -1522,18 +1528,20 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                     for (int cc = 0; cc < 4; ++cc) {
                         float v[32];
                         tmem_ld_32x32b_x32(tmem + lane_base + a * kTileN + half * 128 + cc * 32, v);
-                        if (pair) {
-#pragma unroll
-                            for (int e = 0; e < 32; ++e) v[e] += __shfl_xor_sync(0xffffffffu, v[e], 8);
-                        }
+                        float w[16];
+                        pair_part(v, w);
 #pragma unroll 1
                         for (int q = second ? 1 : 0; q < (pair && !second ? 1 : 2); ++q) {  // 16 columns each
                             if (!act) continue;
-                            float4 *o = reinterpret_cast<float4 *>(dst + cc * 32 + q * 16);
+                            float *o = dst + cc * 32 + q * 16;
 #pragma unroll
-                            for (int e = 0; e < 4; ++e)
-                                o[e] = q ? make_float4(v[16 + 4 * e], v[17 + 4 * e], v[18 + 4 * e], v[19 + 4 * e])
-                                         : make_float4(v[4 * e], v[4 * e + 1], v[4 * e + 2], v[4 * e + 3]);
+                            for (int e = 0; e < 16; ++e) w[e] += q ? v[16 + e] : v[e];
+                            st_global_v8(o, w);
+                            st_global_v8(o + 8, w + 8);
+                            if (!pair) {
+#pragma unroll
+                                for (int e = 0; e < 16; ++e) w[e] = 0.f;
+                            }
                         }
                     }
                 }
@@ -1576,17 +1584,15 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
             for (int cc = 0; cc < 4; ++cc) {
                 float v[32];
                 tmem_ld_32x32b_x32(tmem + lane_base + a * kTileN + half * 128 + cc * 32, v);
-                if (pair) {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) v[e] += __shfl_xor_sync(0xffffffffu, v[e], 8);
-                }
+                float w[16];
+                pair_part(v, w);
                 // 16 columns at a time; each lane of a pair takes one half of the 32
 #pragma unroll 1
                 for (int q = second ? 1 : 0; q < (pair && !second ? 1 : 2); ++q) {
                     if (!act) continue;
                     float z[16];
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) z[e] = __fmul_rn(q ? v[16 + e] : v[e], rs);
+                    for (int e = 0; e < 16; ++e) z[e] = __fmul_rn((q ? v[16 + e] : v[e]) + w[e], rs);
                     const int nb = sg.col0 + half * 128 + cc * 32 + q * 16;
                     if (p.write_logits) {
                         float4 *o = reinterpret_cast<float4 *>(p.logits + (int64_t)my_row * p.V + nb);
