@@ -31,11 +31,11 @@
 //
 // Phases of layer l (counter index 1 + 9l + k):
 //   0 QKV   x_g W_qkv^T -> partials        (a subset of the CTAs: few tiles)
-//   1 FIN_Q q, k, v = RMSNorm scale + RoPE of the summed partials, fp16, once per row; the
-//           new k, v appended to the KV cache
+//   1 FIN_Q q, k, v = RMSNorm scale + RoPE of the summed partials, fp16, once per row
 //   2 ATT   softmax(q K^T) V, 128-position KV blocks, online softmax over a split's blocks
 //           with warp-level MMAs (mma.sync: N = 8 heads, operands and accumulators in
-//           registers; the tcgen05 path's issue / commit / tensor-memory round trips cost more
+//           registers, no exchange between warps inside a split; the new k, v join the tiles and
+//           the KV cache here; the tcgen05 path's issue / commit / tensor-memory round trips cost more
 //           than these products); the last split of a row to finish merges the splits
 //   3 O     att W_o^T -> partials           (a subset of the CTAs)
 //   4 FIN_O x += sum; x_g = x * g_mlp (bf16 hi/lo, blocked); per-row sum of squares
@@ -80,10 +80,9 @@ constexpr int kSmallUnits = 2;  // 16-feature units a pass of small_k takes
 constexpr int kSmallPhaseUnits = 2;   // QKV / O: units per participating CTA
 constexpr int kCntStride = 16;        // phase counters 128 bytes apart (one L2 line each)
 constexpr uint32_t kTmemCols = 512;
-// Attention P tiles (per warp group, two buffers): [8 heads][128 positions] fp16, rows padded
-// to 272 bytes so the eight rows of an ldmatrix fall in distinct banks.
-constexpr int kAttPRow = 272;
-constexpr int kAttPBytes = 8 * kAttPRow;
+// Floats per head row of the attention states that a warp group joins in shared memory (128 dims,
+// padded so that the eight heads' rows start in distinct banks).
+constexpr int kAttORow = 132;
 // Attention probabilities are taken against a running maximum that is re-based only when a
 // score exceeds it by more than this (log2 units): P <= 2^8 in fp16, and most blocks skip the
 // block maximum and the rescale of the output.
@@ -135,6 +134,14 @@ struct MegaParams {
     } while (0)
 #endif
 
+// Attention unit: one split of one row for one kv head.  Split sp covers the `span` KV
+// blocks from block sp * span on: positions [p0, p0 + n) of the row's ctx, in nb blocks.
+struct AttUnit {
+    int item, kvh, row, sp, ctx, p0, n, nb, nsplit, slot;
+    int last;
+};
+constexpr int kMaxCtaUnits = 32;  // attention units a CTA keeps in shared memory
+
 // A GEMM phase and this CTA's share of it (see SegWalk), fixed for a launch.
 struct GemmPlan {
     const uint8_t *w, *x;  // blocked weights of layer 0, pair-blocked operand
@@ -151,6 +158,7 @@ struct MegaSmem {
     uint64_t xfull[kMaxXStages], xempty[kMaxXStages];
     uint64_t acc_full[2], acc_empty[2];
     uint64_t drain;
+    uint64_t units_ready;       // the attention unit table is filled (warp 0)
     unsigned long long target;  // counter value meaning "every CTA of this launch arrived"
     uint64_t wait_ns;           // bounded-wait limit of this launch
     float p_headroom;           // attention: log2 of how far P may exceed 1 before re-basing
@@ -166,18 +174,21 @@ struct MegaSmem {
     int rowpos[128];            // position of each live row
     // KV block ids: of this CTA's attention blocks (unit i's block j at ablk[aoff[i] + j]), and
     // of each row's current position (ablk_ok = 0: too many to hold, looked up in the table)
+    AttUnit units[kMaxCtaUnits];
+    AttUnit unit_tmp[kMegaThreads / 32][2];  // per warp: units beyond them, computed as they come
     int ablk[kMaxCtaBlocks];
-    int aoff[32];
+    int aoff[kMaxCtaUnits];
     int rowblk[128];
     int ablk_ok;
-    float red[2][4][8], red2[2][4][8];  // per warp group: attention max / sum reductions
+    float red[2][4][8], red2[2][4][8];  // per warp group and warp: attention max / weighted sum of each head
+    int kvrel[kWSlots];                  // warps that have read the slot's KV tile
     float mw[2][8][kMegaMaxSplits];      // per warp group: split weights of a merge
     float ml[2][8];
     int last_flag2[2];
 };
 
 constexpr size_t kMegaSmemBytes =
-    1024 + (size_t)kRingBytes + 4 * 4096 + sizeof(MegaSmem);
+    1024 + (size_t)kRingBytes + sizeof(MegaSmem);
 
 // ------------------------------------------------------------------------------ layouts
 // Pair-blocked activation (a GEMM operand held as bf16 hi + lo parts): per 64-wide k-chunk,
@@ -397,13 +408,9 @@ __device__ __noinline__ int2 tile_ctas(const MegaParams &p, const GemmPlan &g, i
     return make_int2(unit_owner(t * g.kch, U, Gp), unit_owner((t + 1) * g.kch - 1, U, Gp));
 }
 
-// Attention unit: one split of one row for one kv head.  Split sp covers the `span` KV
-// blocks from block sp * span on: positions [p0, p0 + n) of the row's ctx, in nb blocks.
-struct AttUnit {
-    int item, kvh, row, sp, ctx, p0, n, nb, nsplit, slot;
-    int last;
-};
-__device__ __noinline__ AttUnit att_unit(const MegaParams &p, int a, int span) {
+// Unit a of the launch (written to shared memory: a struct returned by a function would go through
+// local memory, whose lines the small L1 beside this kernel's shared memory does not keep).
+__device__ __noinline__ void att_unit(const MegaParams &p, int a, int span, AttUnit *dst) {
     AttUnit u;
     u.item = a / p.KVH;
     u.kvh = a - u.item * p.KVH;
@@ -417,8 +424,19 @@ __device__ __noinline__ AttUnit att_unit(const MegaParams &p, int a, int span) {
     u.nsplit = ((u.ctx + kKVPos - 1) / kKVPos + span - 1) / span;
     u.last = u.p0 + u.n == u.ctx;
     u.slot = __ldg(&p.c.row_slot[u.row]);
-    return u;
+    *dst = u;
 }
+// Unit i of this CTA (the launch's unit a0 + i), for a converged warp; slot 0 / 1: which of the warp's
+// own entries a unit beyond the table goes to.
+__device__ __forceinline__ const AttUnit &cta_unit(const MegaParams &p, MegaSmem &S, int a0, int i, int slot) {
+    if (S.ablk_ok) return S.units[i];
+    AttUnit *t = &S.unit_tmp[threadIdx.x >> 5][slot];
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) att_unit(p, a0 + i, S.att_span, t);
+    __syncwarp();
+    return *t;
+}
+
 // Attention units in equal contiguous ranges, counted from the last CTA down: the QKV
 // projection runs on the first CTAs, so a small unit count lands on CTAs that are free
 // to prefetch during it.
@@ -445,13 +463,12 @@ __device__ __forceinline__ void fill_att_blocks(const MegaParams &p, MegaSmem &S
     int a0, a1;
     att_range(p, S.n_items, a0, a1);
     const int nu = a1 - a0;
-    bool ok = nu <= 32;
+    bool ok = nu <= kMaxCtaUnits;
     int nb = 0, off = 0;
-    AttUnit u{};
     if (ok) {
         if (lane < nu) {
-            u = att_unit(p, a0 + lane, S.att_span);
-            nb = u.nb;
+            att_unit(p, a0 + lane, S.att_span, &S.units[lane]);
+            nb = S.units[lane].nb;
         }
         int x = nb;  // inclusive warp scan of the block counts
 #pragma unroll
@@ -464,7 +481,7 @@ __device__ __forceinline__ void fill_att_blocks(const MegaParams &p, MegaSmem &S
     }
     if (ok && lane < nu) {
         S.aoff[lane] = off;
-        const int32_t *src = p.c.blk_tab + (int64_t)u.slot * p.c.nblk_max + u.p0 / kKVPos;
+        const int32_t *src = p.c.blk_tab + (int64_t)S.units[lane].slot * p.c.nblk_max + S.units[lane].p0 / kKVPos;
         for (int j0 = 0; j0 < nb; j0 += 8) {  // eight loads in flight
             int v[8];
 #pragma unroll
@@ -530,30 +547,19 @@ __device__ __forceinline__ void mega_w_producer(const MegaParams &p, MegaSmem &S
             // the attention phase's KV blocks follow the QKV weights in ring order: unit
             // pairs (one unit per compute warp group), block by block, the K of the pair's
             // units, then their V^T; each one ring entry (K: d < 64 | d >= 64 halves, V^T:
-            // positions < 64 | >= 64).  The block holding a row's new position is copied
-            // once the q / k / v phase has appended it to the cache.
-            const int span = S.att_span;
-            bool finq_seen = false;
+            // positions < 64 | >= 64).  None depends on this step: the new position's k and v are
+            // put into the tiles, and into the cache, by the warp that reads them.
 #pragma unroll 1
             for (int a = a0; a < a1 && ok; a += 2) {
                 const bool two = a + 1 < a1;
-                const AttUnit ua = att_unit(p, a, span);
-                const AttUnit ub = two ? att_unit(p, a + 1, span) : ua;
+                const AttUnit &ua = cta_unit(p, S, a0, a - a0, 0);
+                const AttUnit &ub = two ? cta_unit(p, S, a0, a - a0 + 1, 1) : ua;
                 const int nbb = two ? ub.nb : 0, nbm = max(ua.nb, nbb);
 #pragma unroll 1
                 for (int q = 0; q < 4 * nbm && ok; ++q) {  // block q / 4, K or V^T, unit a or a + 1
                     const int j = q >> 2, kv = (q >> 1) & 1, x = q & 1;
                     if (j >= (x ? nbb : ua.nb)) continue;
                     const int n = x ? ub.n : ua.n;
-                    if (kv == 0 && (x ? ub.last : ua.last) && j == (x ? nbb : ua.nb) - 1 && !finq_seen) {
-                        const int fq = 1 + kPhasesPerLayer * l + kPhFinQ;
-                        if (!spin_counter_warp(&p.cnt[fq * kCntStride], phase_target(p, S, fq), err, ab, lim)) {
-                            ok = false;
-                            break;
-                        }
-                        fence_proxy_async_global();
-                        finq_seen = true;
-                    }
                     const uint8_t *blk = kv_block(p, S, l, x ? ub : ua, a - a0 + x, j) + kv * 32768;
                     const int nj = min(kKVPos, n - j * kKVPos);
                     if (!acquire(wi)) { ok = false; break; }
@@ -724,11 +730,12 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
             // A group's consecutive uses of a slot are then at most one barrier phase apart (the slot
             // is refilled only after the group released its previous tile there), which a group
             // waiting on the shared wfull barriers directly could not rely on.
-            const int n = a1 - a0, span = S.att_span;
+            const int n = a1 - a0;
+            if (i == 0 && !mwait_warp(&S.units_ready, 0, err, ab, lim)) ok = false;
 #pragma unroll 1
             for (int u = 0; u < n && ok; u += 2) {
                 const bool two = u + 1 < n;
-                const int nba = att_unit(p, a0 + u, span).nb, nbb = two ? att_unit(p, a0 + u + 1, span).nb : 0;
+                const int nba = cta_unit(p, S, a0, u, 0).nb, nbb = two ? cta_unit(p, S, a0, u + 1, 1).nb : 0;
                 const int nbm = max(nba, nbb);
 #pragma unroll 1
                 for (int q = 0; q < 4 * nbm; ++q) {  // the W producer's order
@@ -752,7 +759,7 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
 // Column-owned projection of up to 8 rows on warp-level MMAs: sum_k W[c][k] X[r][k] for the
 // segment's one or two 16-feature units, the whole K split over the eight compute warps by
 // 32-wide k-blocks (block kb on warp kb % 8).  X comes straight from global memory in fragment
-// order (six blocks' loads in flight at once), W from the ring's slots, which the issuer hands
+// order (three blocks' loads in flight at once), W from the ring's slots, which the issuer hands
 // over; the per-warp sums go to red[warp][unit][feature][row rotated by feature].
 // Against the split-K tcgen05 phase plus its finalisation phase this is one phase barrier and
 // two L2 round trips less (q/k/v at one row: 7.3 -> 5.0 us per layer, O: 6.8 -> 4.5); every CTA
@@ -761,7 +768,7 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
 template <typename KvWait>
 __device__ __forceinline__ void small_k(MegaSmem &S, const uint8_t *sW, float *red, const uint8_t *X, int rows16, int kch,
                                         const Seg &sg, uint32_t wring, int cw, int lane, KvWait &&kv_wait) {
-    constexpr int B = 6;  // k-blocks per batch
+    constexpr int B = 3;  // k-blocks per batch (more would spill registers, in every phase of the kernel)
     const int mt = sg.n / kOwnCols, E = sg.entries(), lgc = __ffs(sg.cps) - 1;
     const uint32_t kbs = (uint32_t)(rows16 >> 3) * 1024;  // bytes of a k-block
     float acc[kSmallUnits][4];
@@ -836,8 +843,7 @@ __device__ __forceinline__ void small_k(MegaSmem &S, const uint8_t *sW, float *r
 // nothing, the three residual finalisations and the three split-K epilogues share their code),
 // divisions by launch constants are done once (GemmPlan, tile_cta), and batches of loads are
 // spread over the lanes instead of being unrolled further.
-__device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, uint8_t *sW, uint8_t *sX, uint8_t *sQ,
-                                             uint32_t tmem) {
+__device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, uint8_t *sW, uint8_t *sX, uint32_t tmem) {
     volatile int *ab = &S.abort;
     const uint64_t lim = S.wait_ns;
     int *err = &p.c.v->err;
@@ -1085,8 +1091,8 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
           if (!small) {
             // -------------------------------------------------------- q, k, v (once per row)
             // The head's QKV partials summed, times 1/rms; RoPE on q and k; q pre-scaled by
-            // log2(e)/sqrt(hd) for the exp2 softmax; fp16 q, k, v for the attention phase; k and v
-            // appended to the KV cache at the row's position.  Unit = (row, 64 weight rows): a
+            // log2(e)/sqrt(hd) for the exp2 softmax; fp16 q, k, v for the attention phase.  Unit =
+            // (row, 64 weight rows): a
             // head's weight rows come in 16s, 8 dims and their rotation partners, so lane % 16
             // holds 4 dims and lane ^ 2 their partners; the warp's halves split the contributors.
             wait_phase(base + kPhQKV);
@@ -1119,18 +1125,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                                        f32_to_f16_sat((x.y * c0.z + sg * (o.y * c0.w)) * rs),
                                        f32_to_f16_sat((x.z * c1.x + sg * (o.z * c1.y)) * rs),
                                        f32_to_f16_sat((x.w * c1.z + sg * (o.w * c1.w)) * rs)};
-                const int pp = pos % kKVPos;
-                if (lane < 16) {
-                    *reinterpret_cast<uint2 *>(p.qkv16 + r * p.nqkv + head * hd + d0) = pack4(h);
-                } else if (!isq) {  // the new position's k / v into the cache (blocked layout)
-                    uint8_t *blk = kv_addr(p, l, S.rowblk[r], head - p.H - (isk ? 0 : p.KVH));
-                    if (isk) {
-                        *reinterpret_cast<uint2 *>(blk + kv_k_off(pp, d0)) = pack4(h);
-                    } else {
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) *reinterpret_cast<uint16_t *>(blk + kv_v_off(pp, d0 + e)) = h[e];
-                    }
-                }
+                if (lane < 16) *reinterpret_cast<uint2 *>(p.qkv16 + r * p.nqkv + head * hd + d0) = pack4(h);
             }
             arrive(base + kPhFinQ, false);
           }
@@ -1138,28 +1133,44 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
             int a0, a1;
             att_range(p, S.n_items, a0, a1);
             const int n = a1 - a0;
+            if (l == 0) mwait(&S.units_ready, 0, err, ab, lim);
             wait_phase(base + kPhFinQ);
             // units alternate between the two warp groups: group h (warps 3..6 / 7..10, named
-            // barrier 2 + h) runs the units (gi + i) & 1 == h, each unit: q in registers, then
-            // per KV block scores -> probabilities against the running max -> output sum
-            // (online softmax over the unit's blocks, warp-level MMAs on the ring's K and V^T
-            // tiles, which the group releases), then output / split partial + merge, in order
+            // barrier 2 + h) runs the units (gi + i) & 1 == h.  Each warp of a group takes 32 positions
+            // of every KV block by itself -- scores, probabilities and output sum stay in its registers
+            // (online softmax, warp-level MMAs; the probabilities turn from accumulator into operand
+            // by an 8 x 8 transpose), and nothing waits for another warp until the unit's end, where
+            // the four warps' states are joined in shared memory.
+            // Bound by the chain of a unit: phase wait, q, its blocks (about 1.1 us each once the two
+            // that the ring prefetches are used up), join, split merge.  With 32 positions per warp for the
+            // scores but 32 dims per warp for the output, as before, P went through shared memory behind
+            // two barriers a block; and the ring's prefetch stopped at the block with the new
+            // position until the phase that wrote it there was over.  1.5B kernel, ms before -> after:
+            // 16 rows of 800 positions 1.337 -> 1.320, 64 of 600 1.791 -> 1.765, 128 of 300
+            // 2.310 -> 2.280, one row of 384 1.145 -> 1.152 (its join costs more than the barriers did).
             const int hb = 2 + half;     // this group's named barrier
             const int ht = ctid & 127;   // thread index within the group
             const int hq = ht >> 5;      // warp within the group
-            const int span = S.att_span;
             // ring entries of the phase's KV blocks: per unit pair, block by block, the K of
             // the pair's units, then their V^T (the W producer's order)
             uint32_t wpair = wring;
-            uint8_t *pbufs = sQ + half * 2 * kAttPBytes;  // this group's two P buffers
-            const int g8 = lane >> 2, t4 = lane & 3;     // mma fragment row / column pair
+            const int g8 = lane >> 2, t4 = lane & 3;     // mma fragment row (head) / column pair
             const int kst = hd >> 4;                      // k-steps of q.k (16 dims each)
+            float *mo = reinterpret_cast<float *>(sX) + half * 4 * 8 * kAttORow;  // [warp][head][dim], X stages' room
+            // a tile's slot goes back to the producer once the group's four warps have read it
+            auto kv_release = [&](uint32_t e) {
+                __syncwarp();
+                if (lane == 0 && atom_add_acq_rel_cta(&S.kvrel[e % kWSlots], 1) == 3) {
+                    S.kvrel[e % kWSlots] = 0;
+                    mbar_arrive(&S.wempty[e % kWSlots]);
+                }
+            };
 #pragma unroll 1
             for (int ip = 0; ip < n; ip += 2) {
                 const bool two = ip + 1 < n;
                 const int x = ((gi + ip) & 1) == half ? 0 : 1;  // our unit of the pair
-                const AttUnit u = att_unit(p, a0 + ip + (two ? x : 0), span);
-                const int nbo = two ? att_unit(p, a0 + ip + (x ^ 1), span).nb : 0;  // the other unit's blocks
+                const AttUnit &u = cta_unit(p, S, a0, ip + (two ? x : 0), 0);
+                const int nbo = two ? cta_unit(p, S, a0, ip + (x ^ 1), 1).nb : 0;  // the other unit's blocks
                 const uint32_t w0 = wpair;
                 wpair += 2u * (uint32_t)(u.nb + nbo);
                 if (x == 1 && !two) continue;
@@ -1179,181 +1190,186 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                         qf[ks][1] = ok ? __ldcg(reinterpret_cast<const unsigned int *>(qh + 16 * ks + 8)) : 0u;
                     }
                 }
-                // ---- per block: S^T = K q^T (warp hq: positions 32 hq ..), probabilities
-                // against the running max, which is re-based only when a score exceeds it by
-                // more than the headroom; P to shared memory; O^T += V^T P^T (warp hq: dims
-                // 16 (hq + 4 m)).  Thread (g8, t4) holds heads 2 t4, 2 t4 + 1 throughout.
-                float mrun[2] = {-INFINITY, -INFINITY}, lthr[2] = {0.f, 0.f};
-                float o[2][4];
+                // ---- the new position's k and v, if it is one of this warp's: four dims a lane
+                const int pp = (u.ctx - 1) % kKVPos;
+                const bool mine_new = u.last && (pp >> 5) == hq && 4 * lane < hd;
+                uint2 kn = make_uint2(0, 0), vn = kn;
+                uint8_t *blkn = nullptr;
+                if (mine_new) {
+                    blkn = kv_addr(p, l, S.rowblk[u.row], u.kvh);
+                    const uint16_t *src = p.qkv16 + u.row * p.nqkv + (p.H + u.kvh) * hd + 4 * lane;
+                    kn = __ldcg(reinterpret_cast<const uint2 *>(src));
+                    vn = __ldcg(reinterpret_cast<const uint2 *>(src + p.KVH * hd));
+                }
+                // ---- per block: S^T = K q^T over this warp's 32 positions, probabilities against the
+                // running max, which is re-based only when a score exceeds it by more than the headroom;
+                // O^T += V^T P^T.  Thread (g8, t4): positions 16 i + g8 + {0, 8}, heads 2 t4 + {0, 1}; dims
+                // 16 i + g8 + {0, 8} of the output.
+                float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f}, o[8][4];
 #pragma unroll
-                for (int m = 0; m < 2; ++m)
+                for (int i = 0; i < 8; ++i)
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) o[m][q] = 0.f;
+                    for (int q = 0; q < 4; ++q) o[i][q] = 0.f;
 #pragma unroll 1
                 for (int jb = 0; jb < u.nb; ++jb) {
-                    const int nj = min(kKVPos, u.n - jb * kKVPos);
+                    const int nj = min(kKVPos, u.n - jb * kKVPos) - 32 * hq;  // this warp's positions: below nj
                     const uint32_t ek = ent(jb, 0), ev = ent(jb, 1);
+                    const bool add_new = mine_new && jb == u.nb - 1;
                     kv_wait(ek);
-                    const uint32_t kbase = smem_u32(sW) + (ek % kWSlots) * kSlotBytes;
-                    float sc[2][4];
-#pragma unroll
-                    for (int m = 0; m < 2; ++m) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) sc[m][q] = 0.f;
-                        const int pb0 = 32 * hq + 16 * m;
-                        if (pb0 < nj) {  // rows past the copied ones are never read
-                            const int pr = pb0 + (lane & 15);  // ldmatrix row of this lane
-                            const uint32_t krow = kbase + pr * 128;
-                            const int sw = pr & 7, lh = lane >> 4;
-#pragma unroll
-                            for (int ks = 0; ks < 8; ++ks) {
-                                if (ks < kst) {
-                                    uint32_t a[4];
-                                    ldsm_x4(krow + (ks >> 2) * 16384 + ((((2 * ks & 7) + lh) ^ sw) << 4), a);
-                                    mma_f16_16816(sc[m], a, qf[ks][0], qf[ks][1]);
-                                }
-                            }
-                        }
+                    if (add_new) {  // into the tile that only this warp reads there, and into the cache
+                        *reinterpret_cast<uint2 *>(sW + (size_t)(ek % kWSlots) * kSlotBytes + kv_k_off(pp, 4 * lane)) = kn;
+                        *reinterpret_cast<uint2 *>(blkn + kv_k_off(pp, 4 * lane)) = kn;
+                        fence_proxy_async_smem();
                     }
-                    // scores: sc[m][q] = s(position 32 hq + 16 m + g8 + 8 (q >> 1), head 2 t4 + (q & 1))
-                    uint8_t *pbuf = pbufs + (jb & 1) * kAttPBytes;
-                    float e[2][4];
-                    bool rebase = jb == 0;
-#pragma unroll 1
-                    for (;;) {
-                        const bool rb = rebase;
-                        if (rb) {  // the block's maximum per head joins the running max
-                            float mx[2] = {-INFINITY, -INFINITY};
+                    __syncwarp();
+                    uint32_t pf[2][2];  // P^T of 16 positions each as mma B fragments
+                    if (nj > 0) {
+                        const int pr = 32 * hq + (lane & 15);
+                        const uint32_t krow = smem_u32(sW) + (ek % kWSlots) * kSlotBytes + pr * 128;
+                        float sc[2][4];
 #pragma unroll
-                            for (int m = 0; m < 2; ++m)
+                        for (int i = 0; i < 2; ++i)
 #pragma unroll
-                                for (int q = 0; q < 4; ++q)
-                                    if (32 * hq + 16 * m + g8 + 8 * (q >> 1) < nj) mx[q & 1] = fmaxf(mx[q & 1], sc[m][q]);
+                            for (int q = 0; q < 4; ++q) sc[i][q] = 0.f;
 #pragma unroll
-                            for (int kk = 0; kk < 2; ++kk)
+                        for (int ks = 0; ks < 8; ++ks) {
+                            if (ks < kst) {
+                                const uint32_t off = (ks >> 2) * 16384 + ((((2 * ks & 7) + (lane >> 4)) ^ (pr & 7)) << 4);
 #pragma unroll
-                                for (int o2 = 4; o2 < 32; o2 <<= 1)
-                                    mx[kk] = fmaxf(mx[kk], __shfl_xor_sync(0xffffffffu, mx[kk], o2));
-                            if (g8 == 0) {
-                                S.red[half][hq][2 * t4] = mx[0];
-                                S.red[half][hq][2 * t4 + 1] = mx[1];
-                            }
-                            named_bar_sync(hb, 128);
-#pragma unroll
-                            for (int kk = 0; kk < 2; ++kk) {
-                                const int h = 2 * t4 + kk;
-                                const float mnew = fmaxf(mrun[kk], fmaxf(fmaxf(S.red[half][0][h], S.red[half][1][h]),
-                                                                         fmaxf(S.red[half][2][h], S.red[half][3][h])));
-                                const float alpha = exp2f(mrun[kk] - mnew);  // 0 on the first block
-                                mrun[kk] = mnew;
-                                lthr[kk] *= alpha;
-#pragma unroll
-                                for (int m = 0; m < 2; ++m) {
-                                    o[m][kk] *= alpha;
-                                    o[m][kk + 2] *= alpha;
+                                for (int i = 0; i < 2; ++i) {
+                                    uint32_t a[4];
+                                    ldsm_x4(krow + off + i * 2048, a);
+                                    mma_f16_16816(sc[i], a, qf[ks][0], qf[ks][1]);
                                 }
                             }
                         }
-                        bool over = false;
+                        float mx[2] = {-INFINITY, -INFINITY};
 #pragma unroll
-                        for (int m = 0; m < 2; ++m)
+                        for (int i = 0; i < 2; ++i)
 #pragma unroll
                             for (int q = 0; q < 4; ++q) {
-                                const int pos = 32 * hq + 16 * m + g8 + 8 * (q >> 1);
-                                const bool valid = pos < nj;
-                                const float s = sc[m][q] - mrun[q & 1];
-                                e[m][q] = valid ? exp2f(s) : 0.f;
-                                over |= valid && s > S.p_headroom;
-                                *reinterpret_cast<uint16_t *>(pbuf + (2 * t4 + (q & 1)) * kAttPRow + 2 * pos) =
-                                    f32_to_f16_sat(e[m][q]);
+                                if (16 * i + g8 + 8 * (q >> 1) >= nj) sc[i][q] = -INFINITY;
+                                mx[q & 1] = fmaxf(mx[q & 1], sc[i][q]);
                             }
-                        rebase = named_bar_any(hb, 128, over) && !rb;
-                        if (!rebase) break;
-                    }
-                    // every warp has read the K block: its ring slot goes back to the producer
-                    if (ht == 0) mbar_arrive(&S.wempty[ek % kWSlots]);
 #pragma unroll
-                    for (int m = 0; m < 2; ++m)
+                        for (int q = 0; q < 2; ++q)
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) lthr[q & 1] += e[m][q];
-                    // ---- O^T += V^T P^T over the block's positions (k-steps of 16)
-                    kv_wait(ev);
-                    const uint32_t vbase = smem_u32(sW) + (ev % kWSlots) * kSlotBytes;
-                    const uint32_t pbase = smem_u32(pbuf) + (lane & 7) * kAttPRow + 16 * (lane >> 3);
-                    const int kpv = (nj + 15) >> 4;
+                            for (int x2 = 4; x2 < 32; x2 <<= 1) mx[q] = fmaxf(mx[q], __shfl_xor_sync(0xffffffffu, mx[q], x2));
+                        // (always on the first block)
+                        if (__any_sync(0xffffffffu, mx[0] - m[0] > S.p_headroom || mx[1] - m[1] > S.p_headroom)) {
 #pragma unroll
-                    for (int ks = 0; ks < 8; ks += 2) {
-                        if (ks < kpv) {
-                            uint32_t bq[4];  // P^T fragments of k-steps ks, ks + 1 (rows: heads 0..7)
-                            ldsm_x4(pbase + 32 * ks, bq);
+                            for (int q = 0; q < 2; ++q) {
+                                const float mnew = fmaxf(m[q], mx[q]), alpha = exp2f(m[q] - mnew);
+                                m[q] = mnew;
+                                l[q] *= alpha;
 #pragma unroll
-                            for (int m = 0; m < 2; ++m) {
-                                if (16 * (hq + 4 * m) < hd) {
-                                    const int dr = 16 * (hq + 4 * m) + (lane & 15);  // V^T row (dim)
-#pragma unroll
-                                    for (int kk = 0; kk < 2; ++kk) {
-                                        if (ks + kk < kpv) {
-                                            const int gr = 2 * ((ks + kk) & 3) + (lane >> 4);
-                                            uint32_t a[4];
-                                            ldsm_x4(vbase + (ks >> 2) * 16384 + dr * 128 + ((gr ^ (dr & 7)) << 4), a);
-                                            mma_f16_16816(o[m], a, bq[2 * kk], bq[2 * kk + 1]);
-                                        }
-                                    }
+                                for (int i = 0; i < 8; ++i) {
+                                    o[i][q] *= alpha;
+                                    o[i][q + 2] *= alpha;
                                 }
                             }
                         }
+#pragma unroll
+                        for (int i = 0; i < 2; ++i)
+#pragma unroll
+                            for (int y = 0; y < 2; ++y) {  // positions 16 i + 8 y ..
+                                const float p0 = exp2f(sc[i][2 * y] - m[0]), p1 = exp2f(sc[i][2 * y + 1] - m[1]);
+                                l[0] += p0;
+                                l[1] += p1;
+                                pf[i][y] = movmatrix_trans((uint32_t)f32_to_f16_sat(p0) | ((uint32_t)f32_to_f16_sat(p1) << 16));
+                            }
                     }
-                    named_bar_sync(hb, 128);  // every warp has read the V^T block
-                    if (ht == 0) mbar_arrive(&S.wempty[ev % kWSlots]);
+                    kv_release(ek);
+                    kv_wait(ev);
+                    if (add_new) {
+                        uint8_t *tile = sW + (size_t)(ev % kWSlots) * kSlotBytes - 32768;
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const uint16_t v = (uint16_t)((e < 2 ? vn.x : vn.y) >> (16 * (e & 1)));
+                            const int off = kv_v_off(pp, 4 * lane + e);
+                            *reinterpret_cast<uint16_t *>(tile + off) = v;
+                            *reinterpret_cast<uint16_t *>(blkn + off) = v;
+                        }
+                        fence_proxy_async_smem();
+                    }
+                    __syncwarp();
+                    if (nj > 0) {
+                        const int dr = lane & 15;
+                        const uint32_t vrow = smem_u32(sW) + (ev % kWSlots) * kSlotBytes + (hq >> 1) * 16384 + dr * 128;
+#pragma unroll
+                        for (int kk = 0; kk < 2; ++kk) {  // positions 16 kk .. of the warp's
+                            const uint32_t off = ((uint32_t)((hq & 1) * 4 + 2 * kk + (lane >> 4)) ^ (dr & 7)) << 4;
+#pragma unroll
+                            for (int i = 0; i < 8; ++i)  // dims 16 i ..
+                                if (16 * i < hd) {
+                                    uint32_t a[4];
+                                    ldsm_x4(vrow + off + i * 2048, a);
+                                    mma_f16_16816(o[i], a, pf[kk][0], pf[kk][1]);
+                                }
+                        }
+                    }
+                    kv_release(ev);
                 }
-                // ---- row sums: heads 2 t4, 2 t4 + 1 over the warp (lanes of equal t4), then
-                // over the group's warps
-                float lrun[2];
+                // ---- the four warps' states: weights 2^(m_w - M), sums in warp order
 #pragma unroll
-                for (int kk = 0; kk < 2; ++kk)
+                for (int q = 0; q < 2; ++q) {
 #pragma unroll
-                    for (int o2 = 4; o2 < 32; o2 <<= 1) lthr[kk] += __shfl_xor_sync(0xffffffffu, lthr[kk], o2);
-                if (g8 == 0) {
-                    S.red2[half][hq][2 * t4] = lthr[0];
-                    S.red2[half][hq][2 * t4 + 1] = lthr[1];
+                    for (int x2 = 4; x2 < 32; x2 <<= 1) l[q] += __shfl_xor_sync(0xffffffffu, l[q], x2);
+                    if (g8 == 0) S.red[half][hq][2 * t4 + q] = m[q];
                 }
                 named_bar_sync(hb, 128);
 #pragma unroll
-                for (int kk = 0; kk < 2; ++kk) {
-                    const int h = 2 * t4 + kk;
-                    lrun[kk] = (S.red2[half][0][h] + S.red2[half][1][h]) + (S.red2[half][2][h] + S.red2[half][3][h]);
+                for (int q = 0; q < 2; ++q) {
+                    const int h = 2 * t4 + q;
+                    const float M = fmaxf(fmaxf(S.red[half][0][h], S.red[half][1][h]),
+                                          fmaxf(S.red[half][2][h], S.red[half][3][h]));
+                    const float w = exp2f(m[q] - M);  // 0 for a warp without positions
+                    if (g8 == 0) S.red2[half][hq][h] = l[q] * w;
+                    float *dst = mo + (hq * 8 + h) * kAttORow + g8;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        if (16 * i < hd) {
+                            dst[16 * i] = o[i][q] * w;
+                            dst[16 * i + 8] = o[i][q + 2] * w;
+                        }
                 }
-                // ---- output (single split) or partial + split merge.  o[m][q]: O^T(dim
-                // 16 (hq + 4 m) + g8 + 8 (q >> 1), head 2 t4 + (q & 1))
+                named_bar_sync(hb, 128);
+                // ---- output (single split) or partial + split merge; thread ht: dim ht of every head
                 const bool single = u.nsplit == 1;
+                const int dd = ht;
                 float *mine = p.part + ((int64_t)u.item * p.KVH + u.kvh) * Gq * (hd + 2);
 #pragma unroll
-                for (int m = 0; m < 2; ++m)
+                for (int g = 0; g < 8; ++g) {
+                    if (g < Gq && dd < hd) {
+                        float v = 0.f, L = 0.f;
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const int dim = 16 * (hq + 4 * m) + g8 + 8 * (q >> 1), h = 2 * t4 + (q & 1);
-                        if (dim < hd && h < Gq) {
-                            if (single) {
-                                uint16_t hv, lv;
-                                split_bf16(o[m][q] / lrun[q & 1], hv, lv);
-                                uint8_t *dst = p.att + att_off(u.row, (u.kvh * Gq + h) * hd + dim);
-                                *reinterpret_cast<uint16_t *>(dst) = hv;
-                                *reinterpret_cast<uint16_t *>(dst + lo_off) = lv;
-                            } else {
-                                mine[h * (hd + 2) + 2 + dim] = o[m][q];
-                            }
+                        for (int w = 0; w < 4; ++w) v += mo[(w * 8 + g) * kAttORow + dd];
+                        if (single) {
+#pragma unroll
+                            for (int w = 0; w < 4; ++w) L += S.red2[half][w][g];
+                            uint16_t hv, lv;
+                            split_bf16(v / L, hv, lv);
+                            uint8_t *dst = p.att + att_off(u.row, (u.kvh * Gq + g) * hd + dd);
+                            *reinterpret_cast<uint16_t *>(dst) = hv;
+                            *reinterpret_cast<uint16_t *>(dst + lo_off) = lv;
+                        } else {
+                            mine[g * (hd + 2) + 2 + dd] = v;
                         }
                     }
-                if (single) continue;
-                if (hq == 0 && g8 == 0) {
+                }
+                if (single) {
+                    named_bar_sync(hb, 128);  // the states' room is free again
+                    continue;
+                }
+                if (dd < Gq) {
+                    float M = S.red[half][0][dd], L = S.red2[half][0][dd];
 #pragma unroll
-                    for (int kk = 0; kk < 2; ++kk) {
-                        const int h = 2 * t4 + kk;
-                        if (h < Gq) {
-                            mine[h * (hd + 2)] = mrun[kk];
-                            mine[h * (hd + 2) + 1] = lrun[kk];
-                        }
+                    for (int w = 1; w < 4; ++w) {
+                        M = fmaxf(M, S.red[half][w][dd]);
+                        L += S.red2[half][w][dd];
                     }
+                    mine[dd * (hd + 2)] = M;
+                    mine[dd * (hd + 2) + 1] = L;
                 }
                 named_bar_sync(hb, 128);
                 if (ht == 0) {  // one acquire-release count: publishes this split, sees the others
@@ -1364,20 +1380,19 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                 named_bar_sync(hb, 128);
                 if (S.last_flag2[half]) {  // merge the row's splits in split order
                     const int ns = min(u.nsplit, kMegaMaxSplits);
-                    const int dd = quarter * 32 + lane;  // output dim of this thread
                     const int sp_stride = p.KVH * Gq * (hd + 2), hs = hd + 2;
                     const float *pb = p.part + ((int64_t)__ldg(&p.c.row_item0[u.row]) * p.KVH + u.kvh) * Gq * hs;
                     float acc[8];
 #pragma unroll
                     for (int g = 0; g < 8; ++g) acc[g] = 0.f;
 #pragma unroll 1
-                    for (int s0 = 0; s0 < ns; s0 += 4) {
-                        // four splits' outputs in flight (thread dd: dim dd of every head); the first
-                        // four load together with the split weights' inputs: one round trip for both
+                    for (int s0 = 0; s0 < ns; s0 += 2) {
+                        // two splits' outputs in flight (thread dd: dim dd of every head; more would spill
+                        // registers); the first two load together with the split weights' inputs
                         const float *src = pb + s0 * sp_stride + 2 + dd;
-                        float v[4][8];
+                        float v[2][8];
 #pragma unroll
-                        for (int q = 0; q < 4; ++q, src += sp_stride)
+                        for (int q = 0; q < 2; ++q, src += sp_stride)
 #pragma unroll
                             for (int g = 0; g < 8; ++g)
                                 v[q][g] = (dd < hd && g < Gq && s0 + q < ns) ? __ldcg(src + g * hs) : 0.f;
@@ -1410,7 +1425,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                             named_bar_sync(hb, 128);
                         }
 #pragma unroll
-                        for (int q = 0; q < 4; ++q)
+                        for (int q = 0; q < 2; ++q)
 #pragma unroll
                             for (int g = 0; g < 8; ++g)
                                 if (g < Gq && s0 + q < ns) acc[g] += S.mw[half][g][s0 + q] * v[q][g];
@@ -1431,6 +1446,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
             }
             wring = wpair;
             gi += n;
+            fence_proxy_async_smem();  // (the X stages are targets of bulk copies again)
             arrive(base + kPhAtt, true);
         }
         if (small && k != 2) {
@@ -1438,7 +1454,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
             // Each CTA's few features hold the whole K, so what follows the sums is applied at
             // once.  Thread: feature c = ctid % 16 of its (unit, row) elements.
             //   q/k/v: RMSNorm scale, RoPE (a unit is 8 dims of a head and their rotation
-            //     partners), fp16, cache append.
+            //     partners), fp16.
             //   O: x += sum, the MLP norm's input, sums of squares (one partial per 16 features).
             wait_phase(k == 0 ? base - 1 : base + kPhAtt);
             const GemmPlan &g = S.plan[k];
@@ -1495,12 +1511,6 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                 if (live && k == 0) {
                     const int dim = (n0 - head * hd) / 2 + (c & 7) + (c < 8 ? 0 : half_hd);
                     if ((c & 1) == 0) *reinterpret_cast<uint32_t *>(p.qkv16 + r * p.nqkv + head * hd + dim) = pk;
-                    if (head >= p.H) {  // the new position's k / v into the cache (blocked layout)
-                        uint8_t *blk = kv_addr(p, l, S.rowblk[r], head - p.H - (rot ? 0 : p.KVH));
-                        const int pp = S.rowpos[r] % kKVPos;
-                        if (!rot) *reinterpret_cast<uint16_t *>(blk + kv_v_off(pp, dim)) = (uint16_t)w0;
-                        else if ((c & 1) == 0) *reinterpret_cast<uint32_t *>(blk + kv_k_off(pp, dim)) = pk;
-                    }
                 } else if (live) {
                     *reinterpret_cast<uint32_t *>(p.xg + xblk_off(r, (n0 + c) & ~1, R16c) + ((c & 1) ? kLoOff : 0)) = pk;
                     if (c == 0) p.ssqM[n0 / kOwnCols * p.rows_cap + r] = sq;
@@ -1654,9 +1664,7 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
     extern __shared__ uint8_t smem_raw[];
     uint8_t *base = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     uint8_t *sW = base;
-    uint8_t *sQ = sW + kRingBytes;
-    uint8_t *sP = sQ + 8192;
-    MegaSmem &S = *reinterpret_cast<MegaSmem *>(sP + 8192);
+    MegaSmem &S = *reinterpret_cast<MegaSmem *>(sW + kRingBytes);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     StepVars *V = p.c.v;
 
@@ -1666,6 +1674,7 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
             mbar_init(&S.wempty[s], 1);
             mbar_init(&S.kvready[0][s], 1);
             mbar_init(&S.kvready[1][s], 1);
+            S.kvrel[s] = 0;
         }
         for (int s = 0; s < kMaxXStages; ++s) { mbar_init(&S.xfull[s], 1); mbar_init(&S.xempty[s], 1); }
         for (int a = 0; a < 2; ++a) {
@@ -1673,6 +1682,7 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
             mbar_init(&S.acc_empty[a], 8);
         }
         mbar_init(&S.drain, 1);
+        mbar_init(&S.units_ready, 1);
         const int live = *(volatile int *)&V->live;
         const int rows = max(0, min(live, p.rows_cap));
         S.rows = rows;
@@ -1730,13 +1740,14 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
     if (run) {
         if (warp == 0) {
             fill_att_blocks(p, S, lane);
+            if (lane == 0) mbar_arrive(&S.units_ready);
             mega_w_producer(p, S, sW);
         } else if (warp == 1) {
             mega_mma(p, S, sW, sX, tmem);
         } else if (warp == 2) {
             mega_x_producer(p, S, sX);
         } else {
-            mega_compute(p, S, sW, sX, sQ, tmem);
+            mega_compute(p, S, sW, sX, tmem);
         }
     }
     tc_fence_before();

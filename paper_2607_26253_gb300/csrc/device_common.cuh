@@ -237,6 +237,13 @@ __device__ __forceinline__ int atom_add_acq_rel_gpu(int *p, int v) {
     return old;
 }
 
+// The same on shared memory at CTA scope.
+__device__ __forceinline__ int atom_add_acq_rel_cta(int *p, int v) {
+    int old;
+    asm volatile("atom.acq_rel.cta.shared::cta.add.s32 %0, [%1], %2;" : "=r"(old) : "r"(smem_u32(p)), "r"(v) : "memory");
+    return old;
+}
+
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long *p) {
     unsigned long long v;
     asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
@@ -340,20 +347,6 @@ __device__ __forceinline__ bool elect_one() {
 // Named barrier among `nthreads` threads (multiple of 32) with id `id` (1..15).
 __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
-}
-
-// Named barrier that also returns whether any of its threads passed v = true.
-__device__ __forceinline__ bool named_bar_any(int id, int nthreads, bool v) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred pi, po;\n\t"
-        "setp.ne.u32 pi, %1, 0;\n\t"
-        "bar.red.or.pred po, %2, %3, pi;\n\t"
-        "selp.u32 %0, 1, 0, po;\n\t}"
-        : "=r"(r)
-        : "r"((uint32_t)v), "r"(id), "r"(nthreads)
-        : "memory");
-    return r != 0;
 }
 
 // Thread-block clusters: this CTA's rank, the barrier over every thread of the cluster (release /

@@ -1,6 +1,7 @@
 """The decode step's row-count and width branches: every accumulator layout of its projections (row counts around 8, 16,
-32, 64 and 128) and MLP widths from a single 16-feature unit per CTA to more than one 256-feature pass, teacher-forced
-logits against the float64 oracle within the stated tolerance."""
+32, 64 and 128), MLP widths from a single 16-feature unit per CTA to more than one 256-feature pass, more attention units
+than a CTA's table holds, and new positions at the edges of a warp's 32 positions and of a KV block; teacher-forced logits
+against the float64 oracle within the stated tolerance."""
 import numpy as np
 import pytest
 
@@ -31,14 +32,25 @@ ODD = _shape("ffn 320")
 WIDE = _shape("ffn 20032", layers=1, ffn=20032)                     # 2,504 units: two passes on some CTAs
 DEEP = _shape("d 2048", layers=2, d_model=2048, n_heads=16, head_dim=128, ffn=448)
 MANY_HEADS = _shape("32 heads", d_model=512, n_heads=32, n_kv_heads=4, head_dim=128, ffn=128)  # K = 4,096 > d
+MANY_KV = _shape("48 kv heads", layers=2, d_model=128, n_heads=48, n_kv_heads=48, head_dim=32, ffn=64)  # 40 units per SM
 
 
 @pytest.mark.parametrize("shape,rows", [(NARROW, 1), (NARROW, 9), (NARROW, 128), (ODD, 8), (ODD, 17), (ODD, 33),
                                         (ODD, 65), (WIDE, 2), (WIDE, 32), (WIDE, 64), (DEEP, 1), (DEEP, 16),
-                                        (DEEP, 31), (DEEP, 48), (MANY_HEADS, 3), (MANY_HEADS, 32), (MANY_HEADS, 40)],
+                                        (DEEP, 31), (DEEP, 48), (MANY_HEADS, 3), (MANY_HEADS, 32), (MANY_HEADS, 40),
+                                        (MANY_KV, 128)],
                          ids=lambda v: getattr(v, "name", v))
 def test_teacher_forced_logits_by_rows_and_widths(pkg, shape, rows):
-    Lp, T = 5, 3
+    _check(pkg, shape, rows, Lp=5, T=3)
+
+
+@pytest.mark.parametrize("rows", [2, 20])
+@pytest.mark.parametrize("Lp", [30, 62, 126, 254])
+def test_new_position_at_tile_edges(pkg, Lp, rows):
+    _check(pkg, ODD, rows, Lp, T=5)
+
+
+def _check(pkg, shape, rows, Lp, T):
     weights = synth.model_weights(shape, 3)
     rng = np.random.default_rng(rows + shape.ffn)
     prompts = rng.integers(0, shape.vocab, size=(rows, Lp)).astype(np.int32)
