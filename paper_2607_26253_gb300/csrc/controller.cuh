@@ -29,6 +29,7 @@ struct CtlShared {
     int bcast[8];
     int hist[2 * kMaxK + 2];
     unsigned pslot_used[256];  // bitmap of prompt slots (<= 8192)
+    int span[kAttCands + 1];
 };
 
 __device__ __forceinline__ int blk_excl_scan(int v, int &total, CtlShared &sh) {
@@ -67,6 +68,39 @@ __device__ __forceinline__ long long blk_sum64(long long v, CtlShared &sh) {
     for (int w = 0; w < 32; ++w) t += sh.warp_tot64[w];
     __syncthreads();
     return t;
+}
+
+// The attention span for n rows at row_pos (the whole block; sm: kAttCands + 1 words of shared memory): a warp
+// counts a candidate's units over the rows.
+static __device__ __noinline__ int att_span_rows(const int32_t *row_pos, int n, const StepConst &K, int *sm) {
+    const int tid = threadIdx.x, lane = tid & 31, B = K.attn_chunk;
+    if (tid == 0) sm[kAttCands] = 1;
+    __syncthreads();
+    int mx = 1;
+    for (int i = tid; i < n; i += blockDim.x) mx = max(mx, (row_pos[i] + B) / B);
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if (lane == 0 && mx > 1) atomicMax(&sm[kAttCands], mx);
+    __syncthreads();
+    mx = sm[kAttCands];
+    if (mx == 1) return 1;  // (every thread)
+    for (int k = tid >> 5; k < kAttCands; k += blockDim.x >> 5) {
+        const int s = (mx + att_cand_splits(k) - 1) / att_cand_splits(k);
+        int units = 0, blocks = 0;
+        for (int i = lane; i < n; i += 32) {
+            const int b = (row_pos[i] + B) / B;
+            blocks += b;
+            units += (b + s - 1) / s;
+        }
+        units = __reduce_add_sync(0xffffffffu, units);
+        blocks = __reduce_add_sync(0xffffffffu, blocks);
+        if (lane == 0)
+            sm[k] = __float_as_int(att_cost(s, (mx + s - 1) / s, units * K.att_kvh, blocks * K.att_kvh, K.att_ctas));
+    }
+    __syncthreads();
+    int best = 0;
+    for (int k = 1; k < kAttCands; ++k)
+        if (__int_as_float(sm[k]) < __int_as_float(sm[best])) best = k;
+    return (mx + att_cand_splits(best) - 1) / att_cand_splits(best);
 }
 
 __device__ __forceinline__ int blk_max(int v, CtlShared &sh) {
@@ -257,7 +291,7 @@ static __device__ void ctl_round_setup(const StepConst &K, StepVars &V, const St
     if (R > c.max_seqs) { if (threadIdx.x == 0) report_error(&V.err, ERR_CAPACITY); return; }
     // first decode step: input = last prompt token at position Lp - 1
     const int nblk = (Lp + K.attn_chunk - 1) / K.attn_chunk;
-    const int span = att_span_for((int64_t)R * nblk, K.att_slots, R);
+    const int span = att_span_uniform(R, nblk, K.att_kvh, K.att_ctas);
     const int nsplit = (nblk + span - 1) / span;
     int maxL = 0;
     for (int r = threadIdx.x; r < R; r += kCtlThreads) {
@@ -678,14 +712,7 @@ static __device__ void ctl_async_join(const StepConst &K, StepVars &V, const Ste
     __syncthreads();
     const int live = live0 + R;
     // attention items of every live row: splits of `span` KV blocks
-    int blocks = 0;
-    for (int base = 0; base < live; base += kCtlThreads) {
-        const int i = base + tid;
-        int tot;
-        blk_excl_scan(i < live ? (c.row_pos[i] + K.attn_chunk) / K.attn_chunk : 0, tot, sh);
-        blocks += tot;
-    }
-    const int span = att_span_for(blocks, K.att_slots, live);
+    const int span = att_span_rows(c.row_pos, live, K, sh.span);
     int items = 0;
     for (int base = 0; base < live; base += kCtlThreads) {
         const int i = base + tid;

@@ -623,12 +623,6 @@ void alloc_decode(sara_handle &h) {
 
 // Phase counters and split counters back to zero (start of every call: a step that failed
 // part-way may have left them anywhere).
-// Decode attention units run at once per kv head: one per compute warp group (two per SM).
-int att_slots(const sara_handle &h) {
-    const int kvh = h.has_model ? std::max(1, h.cfg.n_kv_heads) : 1;
-    return std::max(1, 2 * h.sms / kvh);
-}
-
 void reset_decode_state(sara_handle &h, cudaStream_t s) {
     const sara_model_cfg &m = h.cfg;
     CK(cudaMemsetAsync(h.phase_cnt, 0, ((size_t)h.n_phase_cnt + 1) * kCntStride * 8, s));
@@ -874,7 +868,8 @@ void collect_impl(sara_handle &h, const sara_prompts *pr, int64_t N, int32_t k, 
     K.teacher = 0;
     K.max_gen = m.max_gen_len;
     K.attn_chunk = kDecodeChunk;
-    K.att_slots = att_slots(h);
+    K.att_ctas = h.sms;
+    K.att_kvh = std::max(1, m.n_kv_heads);
     K.max_iters = h.max_iters;
     K.stall_plus1 = h.stall_idx + 1;
     K.wait_ns = (int64_t)h.wait_ns;
@@ -977,7 +972,7 @@ void teacher_impl(sara_handle &h, int n, int Lp, const int32_t *prompts, int T, 
     StepConst K{};
     K.P = n; K.Lp = Lp; K.k = 2; K.n0 = 1; K.commit_min = 2; K.a0 = 1; K.b0 = 1; K.B = n; K.N = n;
     K.tau_num = 0; K.tau_den = 1; K.sample_seed = sample_seed; K.decode = 1; K.teacher = 1; K.T_forced = T;
-    K.max_gen = m.max_gen_len; K.attn_chunk = kDecodeChunk; K.att_slots = att_slots(h);
+    K.max_gen = m.max_gen_len; K.attn_chunk = kDecodeChunk; K.att_ctas = h.sms; K.att_kvh = std::max(1, m.n_kv_heads);
     CK(cudaMemcpyAsync(h.kc, &K, sizeof(K), cudaMemcpyHostToDevice, s));
     CK(cudaMemcpyAsync(h.p_tok, prompts, (size_t)n * Lp * 4, kin, s));
     CK(cudaMemcpyAsync(h.forced, forced, (size_t)n * T * 4, kin, s));
@@ -1072,9 +1067,10 @@ void profile_impl(sara_handle &h, int which, int rows, int ctx, int iters, doubl
     StepConst K{};
     K.P = 1; K.Lp = ctx; K.k = 2; K.n0 = 1; K.commit_min = 2; K.a0 = 1; K.b0 = 1; K.B = 1; K.N = 1;
     K.tau_num = 0; K.tau_den = 1; K.decode = 1; K.max_gen = m.max_gen_len; K.attn_chunk = kDecodeChunk;
-    K.att_slots = att_slots(h);
+    K.att_ctas = h.sms;
+    K.att_kvh = m.n_kv_heads;
     const int nblk = (ctx + kDecodeChunk - 1) / kDecodeChunk;
-    const int span = att_span_for((int64_t)rows * nblk, K.att_slots, rows);
+    const int span = att_span_uniform(rows, nblk, K.att_kvh, K.att_ctas);
     const int nsplit = (nblk + span - 1) / span;
     std::vector<int> slot(rows), pos(rows, ctx - 1), tok(rows, 0), item0(rows), zero(rows, 0), len(rows, m.max_gen_len);
     std::vector<uint64_t> seed(rows);

@@ -82,6 +82,7 @@ __device__ __forceinline__ int scan256(int v, int &total, int *warp_tot) {
 // reports it).
 static __global__ void __launch_bounds__(256) sample_finish_kernel(StepPtrs c, int vocab, cudaGraphConditionalHandle more,
                                                                    int use_more) {
+    __shared__ int span_sm[kAttCands + 1];
     __shared__ float sv[8];
     __shared__ int si[8];
     __shared__ int s_last;
@@ -210,14 +211,7 @@ static __global__ void __launch_bounds__(256) sample_finish_kernel(StepPtrs c, i
         out += tot;
     }
     // attention items of the next step: splits of `span` KV blocks
-    int blocks = 0;
-    for (int base = 0; base < out; base += 256) {
-        const int i = base + tid;
-        int tot;
-        scan256(i < out ? (c.row_pos[i] + K.attn_chunk) / K.attn_chunk : 0, tot, warp_tot);
-        blocks += tot;
-    }
-    const int span = att_span_for(blocks, K.att_slots, out);
+    const int span = att_span_rows(c.row_pos, out, K, span_sm);
     int items = 0;
     for (int base = 0; base < out; base += 256) {
         const int i = base + tid;
@@ -266,7 +260,7 @@ static __global__ void __launch_bounds__(kCtlThreads, 1) teacher_setup_kernel(St
     StepVars &V = *c.v;
     const int Lp = K.Lp, Lpre = Lp - 1;
     const int nblk = (Lp + K.attn_chunk - 1) / K.attn_chunk;
-    const int span = att_span_for((int64_t)n * nblk, K.att_slots, n);
+    const int span = att_span_uniform(n, nblk, K.att_kvh, K.att_ctas);
     const int nsplit = (nblk + span - 1) / span;
     const int nsh = shared_blocks(Lp, K.attn_chunk);
     for (int i = threadIdx.x; i < c.n_priv; i += kCtlThreads) c.blk_free[i] = c.n_shared + c.n_priv - 1 - i;

@@ -22,7 +22,8 @@ struct StepConst {
     int32_t T_forced;     // teacher: generated tokens per rollout
     int32_t max_gen;      // stride of the generated-token output
     int32_t attn_chunk;   // decode attention: positions per KV block
-    int32_t att_slots;    // decode attention: units one step runs at once, per kv head
+    int32_t att_ctas;     // decode attention: CTAs that share a step's units
+    int32_t att_kvh;      // decode attention: kv heads
     int32_t max_iters;    // bound on the step loop's iterations (0: none beyond the round bounds)
     int32_t stall_plus1;  // test hook: 1 + the decode-step phase counter whose waits never
                           // complete (0: none)
@@ -65,18 +66,37 @@ struct StepVars {
     int64_t resv;
 };
 
-// KV blocks per decode attention split: the smallest span that leaves at most `slots` split
-// units per kv head when `blocks` blocks (summed over the `rows` rows) are to be covered, and
-// at least the rows' mean block count / kAttSplitsTarget, so that few long rows are not cut
-// into many one-block splits (each split adds partial stores and a share of the merge).
-constexpr int kAttSplitsTarget = 8;
-__host__ __device__ inline int att_span_for(int64_t blocks, int slots, int64_t rows) {
-    if (slots < 1) slots = 1;
-    if (rows < 1) rows = 1;
-    int64_t s = (blocks + slots - 1) / slots;
-    const int64_t by_len = (blocks + rows * kAttSplitsTarget - 1) / (rows * kAttSplitsTarget);
-    if (by_len > s) s = by_len;
-    return s < 1 ? 1 : (int)s;
+// KV blocks per decode attention split ("span").  A unit (one split of a row, for one kv head) is one
+// CTA's work, and units go to the CTAs in equal counts, so a launch lasts about as long as its busiest
+// CTA: its units' blocks, 0.7 blocks' time for each unit's ends, and, where rows are cut, a merge
+// of 2 blocks' time and 1/8 more for each split.  (1.5B kernel, a block about 1.1 us a layer: one row of
+// 500 positions 1.163 ms in four splits, 1.174 uncut, 1.203 in 3 + 1; 26 rows of 758 1.378 in halves,
+// 1.407 in thirds or uncut; 64 rows of 600 1.654 uncut, 1.745 in 3 + 2, and 1.765 with the
+// smallest span that two units per CTA had room for, as it was; 128 rows of 2000 3.236 uncut, 3.44 in
+// halves.)  The span taken is the one of least estimated time among those that cut the longest row
+// into 1 .. 8, 12, 16 .. 40 equal splits.
+constexpr int kAttCands = 16;
+__host__ __device__ inline int att_cand_splits(int k) { return k < 8 ? k + 1 : 4 * (k - 5); }
+// Estimated time, in 1/16 blocks: `units` units of all rows and kv heads, `blocks` blocks in them, at most
+// s blocks each and ns splits of a row.
+__host__ __device__ inline float att_cost(int s, int ns, int units, int blocks, int ctas) {
+    const int q = (units + ctas - 1) / ctas;  // units of the busiest CTA
+    const float load = (float)blocks / (float)units * (float)(16 * q);
+    return (load > (float)(16 * s) ? load : (float)(16 * s)) + (float)(11 * q + (ns > 1 ? 32 + 2 * ns : 0));
+}
+// The span for `rows` rows of nb blocks each.
+__host__ __device__ inline int att_span_uniform(int rows, int nb, int kvh, int ctas) {
+    int best = 1;
+    float least = 0.f;
+    for (int k = 0; k < kAttCands && rows > 0; ++k) {
+        const int n = att_cand_splits(k), s = (nb + n - 1) / n > 1 ? (nb + n - 1) / n : 1, ns = (nb + s - 1) / s;
+        const float t = att_cost(s, ns, rows * ns * kvh, rows * nb * kvh, ctas);
+        if (k == 0 || t < least) {
+            least = t;
+            best = s;
+        }
+    }
+    return best;
 }
 
 struct StepPtrs {

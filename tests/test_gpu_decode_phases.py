@@ -1,7 +1,7 @@
 """The decode step's row-count and width branches: every accumulator layout of its projections (row counts around 8, 16,
 32, 64 and 128), MLP widths from a single 16-feature unit per CTA to more than one 256-feature pass, more attention units
-than a CTA's table holds, and new positions at the edges of a warp's 32 positions and of a KV block; teacher-forced logits
-against the float64 oracle within the stated tolerance."""
+than a CTA's table holds, new positions at the edges of a warp's 32 positions and of a KV block (where the number of
+attention splits changes); teacher-forced logits against the float64 oracle within the stated tolerance."""
 import numpy as np
 import pytest
 
@@ -45,7 +45,7 @@ def test_teacher_forced_logits_by_rows_and_widths(pkg, shape, rows):
 
 
 @pytest.mark.parametrize("rows", [2, 20])
-@pytest.mark.parametrize("Lp", [30, 62, 126, 254])
+@pytest.mark.parametrize("Lp", [30, 62, 126, 254, 638])
 def test_new_position_at_tile_edges(pkg, Lp, rows):
     _check(pkg, ODD, rows, Lp, T=5)
 
