@@ -61,9 +61,9 @@ namespace sara {
 
 constexpr int kMegaThreads = 352;
 constexpr int kMegaCThreads = 256;  // compute warps 3..10
-constexpr int kWSlots = 4;  // weight / KV ring entries (a power of two: slot = index & 3)
+constexpr int kMaxWSlots = 5;  // weight / KV ring entries of a launch: ring_slots
 constexpr int kSlotBytes = 32768;
-constexpr int kRingBytes = 4 * 32768 + 65536;  // W slots, then the X stages
+constexpr int kRingBytes = 5 * kSlotBytes + 53248;  // W slots, then the X stages
 constexpr int kMaxXStages = 8;
 constexpr int kTileN = 256;           // weight rows (output features) per GEMM tile
 constexpr int kKVPos = 128;           // positions per KV block (an attention split holds `span` blocks)
@@ -83,6 +83,9 @@ constexpr uint32_t kTmemCols = 512;
 // Floats per head row of the attention states that a warp group joins in shared memory (128 dims,
 // padded so that the eight heads' rows start in distinct banks).
 constexpr int kAttORow = 132;
+constexpr int kMinXBytes = kRingBytes - kMaxWSlots * kSlotBytes;
+static_assert(2 * 4 * 8 * kAttORow * 4 <= kMinXBytes, "the joined attention states fit the X stages");
+static_assert(8 * kSmallUnits * 16 * 8 * 4 <= kMinXBytes, "small_k's sums fit the X stages");
 // Attention probabilities are taken against a running maximum that is re-based only when a
 // score exceeds it by more than this (log2 units): P <= 2^8 in fp16, and most blocks skip the
 // block maximum and the rescale of the output.
@@ -152,9 +155,19 @@ struct GemmPlan {
 };
 constexpr int kPlanTiles = 32;  // contributor table entries per phase (wider phases compute them)
 
+// W slots of a launch.  What the ring holds ahead is read while the step waits on a phase, so a fifth slot
+// (5 MB over the CTAs) shortens the phases that stream weights; the activation stages give up its room,
+// which costs more from 40 rows on, where a chunk takes 12 KB or more.  1.5B kernel, 4 -> 5 slots: one row
+// of 100 positions 1.063 -> 1.043 ms, 16 rows 1.182 -> 1.148, 26 rows of 758 1.380 -> 1.352, 40 rows of
+// 500 1.444 either way, 48 of 300 1.469 -> 1.474; the stages that need not be a power of two in
+// number: 80 rows of 300 1.915 -> 1.885, 96 2.022 -> 1.977.
+__host__ __device__ constexpr int ring_slots(int rows) { return rows <= 32 ? 5 : 4; }
+// Bytes of an activation chunk (64 wide) in a stage: hi and lo parts of the rows' 8-row groups.
+__host__ __device__ constexpr int x_chunk_bytes(int rows) { return rows <= 8 ? 2048 : (rows + 15) / 16 * 4096; }
+
 struct MegaSmem {
-    uint64_t wfull[kWSlots], wempty[kWSlots];
-    uint64_t kvready[2][kWSlots];  // attention: ring slot s holds warp group g's next KV tile
+    uint64_t wfull[kMaxWSlots], wempty[kMaxWSlots];
+    uint64_t kvready[2][kMaxWSlots];  // attention: ring slot s holds warp group g's next KV tile
     uint64_t xfull[kMaxXStages], xempty[kMaxXStages];
     uint64_t acc_full[2], acc_empty[2];
     uint64_t drain;
@@ -166,7 +179,7 @@ struct MegaSmem {
     uint32_t tmem_base;
     int abort;
     int last_flag;
-    int rows, rows16, nx, nx_lg, xgroup, n_items, att_span;  // nx = 2^nx_lg X stages of xgroup chunks
+    int rows, rows16, nws, nx, xgroup, xchunk, n_items, att_span;  // nws W slots; nx X stages of xgroup chunks
     GemmPlan plan[5];           // this CTA's share of each GEMM phase (the same for every layer)
     int2 tile_cta[3][kPlanTiles];  // first and last contributor of the tiles of q/k/v, O, down
     int small;                  // at most kSmallRows live rows
@@ -181,14 +194,14 @@ struct MegaSmem {
     int rowblk[128];
     int ablk_ok;
     float red[2][4][8], red2[2][4][8];  // per warp group and warp: attention max / weighted sum of each head
-    int kvrel[kWSlots];                  // warps that have read the slot's KV tile
+    int kvrel[kMaxWSlots];                // warps that have read the slot's KV tile
     float mw[2][8][kMegaMaxSplits];      // per warp group: split weights of a merge
     float ml[2][8];
     int last_flag2[2];
 };
 
-constexpr size_t kMegaSmemBytes =
-    1024 + (size_t)kRingBytes + sizeof(MegaSmem);
+constexpr size_t kMegaSmemBytes = 1024 + (size_t)kRingBytes + sizeof(MegaSmem);
+static_assert(kMegaSmemBytes <= 232448, "227 KB of shared memory per CTA");
 
 // ------------------------------------------------------------------------------ layouts
 // Pair-blocked activation (a GEMM operand held as bf16 hi + lo parts): per 64-wide k-chunk,
@@ -495,6 +508,9 @@ __device__ __forceinline__ void fill_att_blocks(const MegaParams &p, MegaSmem &S
     __syncwarp();
 }
 
+// Slot of ring entry e: e mod nws (mul = 2^32 / nws rounded up: exact far beyond a launch's entries).
+__device__ __forceinline__ uint32_t ring_slot(uint32_t e, uint32_t nws, uint32_t mul) { return e - __umulhi(e, mul) * nws; }
+
 // Counter of a GEMM phase of layer l.
 __device__ __forceinline__ int gemm_counter(int gk, int l) {
     return 1 + kPhasesPerLayer * l + (gk == kGQKV ? kPhQKV : gk == kGO ? kPhO : gk == kGGU ? kPhGU : kPhDown);
@@ -509,11 +525,13 @@ __device__ __forceinline__ void mega_w_producer(const MegaParams &p, MegaSmem &S
     const uint64_t lim = S.wait_ns;
     int *err = &p.c.v->err;
     const uint64_t pol = l2_policy_evict_first();
-    constexpr uint32_t nws = kWSlots;
-    uint32_t wi = 0;
+    const uint32_t nws = S.nws;
+    uint32_t wi = 0, ws = 0, wpar = 0;  // ring entries so far, the next one's slot, parity of its round
     bool ok = true;
-    auto acquire = [&](uint32_t i) -> bool {
-        return i < nws || mwait_warp(&S.wempty[i % nws], ((i / nws) & 1) ^ 1, err, ab, lim);
+    auto acquire = [&]() -> bool { return wi < nws || mwait_warp(&S.wempty[ws], wpar ^ 1, err, ab, lim); };
+    auto advance = [&]() {
+        ++wi;
+        if (++ws == nws) { ws = 0; wpar ^= 1; }
     };
     int a0, a1;
     att_range(p, S.n_items, a0, a1);
@@ -530,9 +548,9 @@ __device__ __forceinline__ void mega_w_producer(const MegaParams &p, MegaSmem &S
             const uint32_t cb = (uint32_t)sg.n * 128;  // a chunk's bytes
             const uint8_t *src = w + sg.kc0 * rowb + (int64_t)sg.col0 * 128;
 #pragma unroll 1
-            for (int kc = sg.kc0; kc < sg.kc1; kc += sg.cps, ++wi) {
-                if (!acquire(wi)) { ok = false; break; }
-                const int s = (int)(wi % nws), m = min(sg.cps, sg.kc1 - kc);
+            for (int kc = sg.kc0; kc < sg.kc1; kc += sg.cps) {
+                if (!acquire()) { ok = false; break; }
+                const int s = (int)ws, m = min(sg.cps, sg.kc1 - kc);
                 if (elect_one()) {
                     mbar_arrive_expect_tx(&S.wfull[s], (uint32_t)m * cb);
 #pragma unroll 1
@@ -540,6 +558,7 @@ __device__ __forceinline__ void mega_w_producer(const MegaParams &p, MegaSmem &S
                         bulk_load(sW + (size_t)s * kSlotBytes + (size_t)j * cb, src, cb, &S.wfull[s], pol);
                 }
                 src = w + (kc + m) * rowb + (int64_t)sg.col0 * 128;
+                advance();
             }
         }
         MEGA_STAMP(gk == kGLM ? 1 + kPhasesPerLayer * l : gemm_counter(gk, l), 2);
@@ -562,8 +581,8 @@ __device__ __forceinline__ void mega_w_producer(const MegaParams &p, MegaSmem &S
                     const int n = x ? ub.n : ua.n;
                     const uint8_t *blk = kv_block(p, S, l, x ? ub : ua, a - a0 + x, j) + kv * 32768;
                     const int nj = min(kKVPos, n - j * kKVPos);
-                    if (!acquire(wi)) { ok = false; break; }
-                    const int s = (int)(wi % nws);
+                    if (!acquire()) { ok = false; break; }
+                    const int s = (int)ws;
                     // K: rows = positions, halves of the dims; V^T: rows = dims, halves of the positions
                     const uint32_t hb = kv == 0 ? (uint32_t)(((nj + 7) & ~7) * 128) : (uint32_t)(p.hd * 128);
                     const bool both = kv == 0 ? p.hd > 64 : nj > 64;
@@ -572,7 +591,7 @@ __device__ __forceinline__ void mega_w_producer(const MegaParams &p, MegaSmem &S
                         bulk_load(sW + (size_t)s * kSlotBytes, blk, hb, &S.wfull[s], pol);
                         if (both) bulk_load(sW + (size_t)s * kSlotBytes + 16384, blk + 16384, hb, &S.wfull[s], pol);
                     }
-                    ++wi;
+                    advance();
                 }
             }
             MEGA_STAMP(1 + kPhasesPerLayer * l + kPhAtt, 2);
@@ -580,8 +599,8 @@ __device__ __forceinline__ void mega_w_producer(const MegaParams &p, MegaSmem &S
     }
     if (!ok) {  // every copy already issued lands before the CTA exits
         for (uint32_t s = 0; s < nws && s < wi; ++s) {
-            const uint32_t last = ((wi - 1 - s) / nws) * nws + s;
-            mbar_wait(&S.wfull[s], (last / nws) & 1, err);
+            const uint32_t last = (wi - 1 - s) / nws;  // round of its last use
+            mbar_wait(&S.wfull[s], last & 1, err);
         }
     }
 }
@@ -592,11 +611,13 @@ __device__ __forceinline__ void mega_x_producer(const MegaParams &p, MegaSmem &S
     const uint64_t lim = S.wait_ns;
     int *err = &p.c.v->err;
     const uint64_t pol = l2_policy_evict_last();
-    const int NX = S.nx, R16 = S.rows16, nxl = S.nx_lg, gx = S.xgroup;
-    const uint32_t chunk = (uint32_t)R16 * 256;  // hi + lo parts of the live rows' groups
+    const int NX = S.nx, gx = S.xgroup;
+    const uint32_t chunk = (uint32_t)S.xchunk;  // hi + lo parts of the live rows' groups
     const uint32_t stage = (uint32_t)gx * chunk;
     const int64_t chunk_stride = (int64_t)p.rows_cap16 * 256;
     uint32_t xi = 0;
+    int xs = 0;          // the next stage
+    uint32_t xpar = 0;   // parity of its round
     bool ok = true;
 #pragma unroll 1
     for (int i = 0; i <= 4 * p.layers && ok; ++i) {
@@ -615,8 +636,8 @@ __device__ __forceinline__ void mega_x_producer(const MegaParams &p, MegaSmem &S
             const uint8_t *src = g.x + sg.kc0 * chunk_stride;
 #pragma unroll 1
             for (int kc = sg.kc0; kc < sg.kc1; kc += gx, ++xi) {
-                const int s = (int)(xi & (uint32_t)(NX - 1)), m = min(gx, sg.kc1 - kc);
-                if (xi >= (uint32_t)NX && !mwait_warp(&S.xempty[s], ((xi >> nxl) & 1) ^ 1, err, ab, lim)) { ok = false; break; }
+                const int s = xs, m = min(gx, sg.kc1 - kc);
+                if (xi >= (uint32_t)NX && !mwait_warp(&S.xempty[s], xpar ^ 1, err, ab, lim)) { ok = false; break; }
                 if (elect_one()) {
                     mbar_arrive_expect_tx(&S.xfull[s], (uint32_t)m * chunk);
 #pragma unroll 1
@@ -624,13 +645,14 @@ __device__ __forceinline__ void mega_x_producer(const MegaParams &p, MegaSmem &S
                         bulk_load(sX + (size_t)s * stage + (size_t)j * chunk, src + j * chunk_stride, chunk, &S.xfull[s], pol);
                 }
                 src += gx * chunk_stride;
+                if (++xs == NX) { xs = 0; xpar ^= 1; }
             }
         }
     }
     if (!ok) {
         for (uint32_t s = 0; s < (uint32_t)NX && s < xi; ++s) {
-            const uint32_t last = (((xi - 1 - s) >> nxl) << nxl) + s;
-            mbar_wait(&S.xfull[s], (last >> nxl) & 1, err);
+            const uint32_t last = (xi - 1 - s) / (uint32_t)NX;  // round of its last use
+            mbar_wait(&S.xfull[s], last & 1, err);
         }
     }
 }
@@ -640,18 +662,21 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
     volatile int *ab = &S.abort;
     const uint64_t lim = S.wait_ns;
     int *err = &p.c.v->err;
-    const int NX = S.nx, R16 = S.rows16, nxl = S.nx_lg, gx = S.xgroup;
-    const uint32_t chunk = (uint32_t)R16 * 256, stage = (uint32_t)gx * chunk;
+    const int NX = S.nx, R16 = S.rows16, gx = S.xgroup;
+    const uint32_t chunk = (uint32_t)S.xchunk, stage = (uint32_t)gx * chunk;
     // at most 64 live rows: one MMA per k-step over the stacked hi / lo groups (M = 2 R16
     // rounded up to 64 or 128: the rows past the stage only feed accumulator rows nobody
     // reads); more: the hi and the lo groups as two 128-row operands into one accumulator
     const bool stacked = R16 <= 64;
     const uint32_t sbo = stacked ? 1024u : 2048u;
-    uint32_t wi = 0, xi = 0;
+    uint32_t ws = 0, wpar = 0, xs = 0, xpar = 0;  // the next W slot / X stage and the parity of its round
     uint32_t use[2] = {0, 0};  // accumulator buffer uses
     uint32_t tseg = 0;         // segments so far
     bool ok = true;
-    constexpr uint32_t nws = kWSlots;
+    const uint32_t nws = S.nws;
+    auto w_advance = [&]() {
+        if (++ws == nws) { ws = 0; wpar ^= 1; }
+    };
     int a0, a1;
     att_range(p, S.n_items, a0, a1);
     int gi = 0;  // attention units so far (unit i of a phase runs on group (gi + i) & 1)
@@ -666,12 +691,13 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
         while (ok && walk.next(g, sg)) {
             if (fwd) {  // small_k's weights: handed over to both compute groups as they land (see below)
 #pragma unroll 1
-                for (int e = sg.entries(); e > 0; --e, ++wi) {
-                    if (!mwait_warp(&S.wfull[wi % nws], (wi / nws) & 1, err, ab, lim)) { ok = false; break; }
+                for (int e = sg.entries(); e > 0; --e) {
+                    if (!mwait_warp(&S.wfull[ws], wpar, err, ab, lim)) { ok = false; break; }
                     if (elect_one()) {
-                        mbar_arrive(&S.kvready[0][wi % nws]);
-                        mbar_arrive(&S.kvready[1][wi % nws]);
+                        mbar_arrive(&S.kvready[0][ws]);
+                        mbar_arrive(&S.kvready[1][ws]);
                     }
+                    w_advance();
                 }
                 continue;
             }
@@ -688,16 +714,15 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
             int wj = 0, xj = 0;  // chunk within the weight slot / the activation stage
 #pragma unroll 1
             for (int kc = sg.kc0; kc < sg.kc1; kc += grp) {
-                if (wj == 0 && !mwait_warp(&S.wfull[wi % nws], (wi / nws) & 1, err, ab, lim)) { ok = false; break; }
-                const int xs = (int)(xi & (uint32_t)(NX - 1));
-                if (xj == 0 && !mwait_warp(&S.xfull[xs], (xi >> nxl) & 1, err, ab, lim)) { ok = false; break; }
+                if (wj == 0 && !mwait_warp(&S.wfull[ws], wpar, err, ab, lim)) { ok = false; break; }
+                if (xj == 0 && !mwait_warp(&S.xfull[xs], xpar, err, ab, lim)) { ok = false; break; }
                 tc_fence_after();
                 const int m = min(grp, sg.kc1 - kc);
                 const bool end = kc + m == sg.kc1;
                 const bool wlast = end || wj + grp == sg.cps, xlast = end || xj + grp == gx;
                 if (elect_one()) {
-                    uint32_t aw = smem_u32(sW) + (wi % nws) * kSlotBytes + (uint32_t)wj * cb;
-                    uint32_t ax = smem_u32(sX) + (uint32_t)xs * stage + (uint32_t)xj * chunk;
+                    uint32_t aw = smem_u32(sW) + ws * kSlotBytes + (uint32_t)wj * cb;
+                    uint32_t ax = smem_u32(sX) + xs * stage + (uint32_t)xj * chunk;
                     uint32_t acc = kc == sg.kc0 ? 0u : 1u;
 #pragma unroll 1
                     for (int j = 0; j < m; ++j, aw += cb, ax += chunk) {
@@ -710,14 +735,14 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
                         }
                     }
                     if (xlast) tc_commit(&S.xempty[xs]);
-                    if (wlast) tc_commit(&S.wempty[wi % nws]);
+                    if (wlast) tc_commit(&S.wempty[ws]);
                     if (end) tc_commit(&S.acc_full[a]);
                 }
                 __syncwarp();
                 wj = wlast ? 0 : wj + grp;
                 xj = xlast ? 0 : xj + grp;
-                wi += wlast ? 1 : 0;
-                xi += xlast ? 1 : 0;
+                if (wlast) w_advance();
+                if (xlast && ++xs == (uint32_t)NX) { xs = 0; xpar ^= 1; }
             }
             if (a) ++use[1]; else ++use[0];
             ++tseg;
@@ -741,9 +766,9 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
                 for (int q = 0; q < 4 * nbm; ++q) {  // the W producer's order
                     const int j = q >> 2, x = q & 1;
                     if (j >= (x ? nbb : nba)) continue;
-                    if (!mwait_warp(&S.wfull[wi % nws], (wi / nws) & 1, err, ab, lim)) { ok = false; break; }
-                    if (elect_one()) mbar_arrive(&S.kvready[(gi + u + x) & 1][wi % nws]);
-                    ++wi;
+                    if (!mwait_warp(&S.wfull[ws], wpar, err, ab, lim)) { ok = false; break; }
+                    if (elect_one()) mbar_arrive(&S.kvready[(gi + u + x) & 1][ws]);
+                    w_advance();
                 }
             }
             gi += n;
@@ -767,7 +792,7 @@ __device__ __forceinline__ void mega_mma(const MegaParams &p, MegaSmem &S, uint8
 // but as much lost to the larger code of the other phases).
 template <typename KvWait>
 __device__ __forceinline__ void small_k(MegaSmem &S, const uint8_t *sW, float *red, const uint8_t *X, int rows16, int kch,
-                                        const Seg &sg, uint32_t wring, int cw, int lane, KvWait &&kv_wait) {
+                                        const Seg &sg, uint32_t wring, int cw, int lane, KvWait &&kv_wait, uint32_t nws_mul) {
     constexpr int B = 3;  // k-blocks per batch (more would spill registers, in every phase of the kernel)
     const int mt = sg.n / kOwnCols, E = sg.entries(), lgc = __ffs(sg.cps) - 1;
     const uint32_t kbs = (uint32_t)(rows16 >> 3) * 1024;  // bytes of a k-block
@@ -778,8 +803,8 @@ __device__ __forceinline__ void small_k(MegaSmem &S, const uint8_t *sW, float *r
         for (int q = 0; q < 4; ++q) acc[m][q] = 0.f;
     const int arow = lane & 15;  // ldmatrix row of this lane
 #pragma unroll 1
-    for (int e0 = 0; e0 < E; e0 += kWSlots) {  // as many slots as the ring holds
-        const int e1 = min(E, e0 + kWSlots);
+    for (int e0 = 0; e0 < E; e0 += S.nws) {  // as many slots as the ring holds
+        const int e1 = min(E, e0 + S.nws);
         const int kb1 = min(2 * kch, 2 * sg.cps * e1);
         int seen = e0;  // slots handed over so far
 #pragma unroll 1
@@ -801,7 +826,7 @@ __device__ __forceinline__ void small_k(MegaSmem &S, const uint8_t *sW, float *r
                     const int e = (kb >> 1) >> lgc;
 #pragma unroll 1
                     for (; seen <= e; ++seen) kv_wait(wring + seen);
-                    const uint32_t wb = smem_u32(sW) + ((wring + e) % kWSlots) * kSlotBytes +
+                    const uint32_t wb = smem_u32(sW) + ring_slot(wring + e, S.nws, nws_mul) * kSlotBytes +
                                         (uint32_t)(((kb >> 1) - (e << lgc)) * sg.n * 128 + arow * 128);
 #pragma unroll
                     for (int ks = 0; ks < 2; ++ks) {
@@ -824,7 +849,7 @@ __device__ __forceinline__ void small_k(MegaSmem &S, const uint8_t *sW, float *r
         if (e1 < E) {
             named_bar_sync(1, kMegaCThreads);
             if (cw == 0 && lane == 0)
-                for (int e = e0; e < e1; ++e) mbar_arrive(&S.wempty[(wring + e) % kWSlots]);
+                for (int e = e0; e < e1; ++e) mbar_arrive(&S.wempty[ring_slot(wring + e, S.nws, nws_mul)]);
         }
     }
 #pragma unroll
@@ -872,8 +897,10 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
     const bool quarter_live = (R16 <= 32 ? quarter * 8 : pair ? quarter * 16 : quarter * 32) < R;
     uint32_t wring = 0;  // W ring entries of the phases before the current one (the producer's count)
     uint32_t kvpar = 0;  // per ring slot (bit s): parity of this warp group's next kvready wait
+    const uint32_t nws = S.nws, nws_mul = 0xffffffffu / nws + 1;
+    auto wslot = [&](uint32_t e) { return ring_slot(e, nws, nws_mul); };
     auto kv_wait = [&](uint32_t e) {
-        const uint32_t sl = e % kWSlots;
+        const uint32_t sl = wslot(e);
         mwait(&S.kvready[half][sl], (kvpar >> sl) & 1u, err, ab, lim);
         kvpar ^= 1u << sl;
     };
@@ -1160,9 +1187,9 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
             // a tile's slot goes back to the producer once the group's four warps have read it
             auto kv_release = [&](uint32_t e) {
                 __syncwarp();
-                if (lane == 0 && atom_add_acq_rel_cta(&S.kvrel[e % kWSlots], 1) == 3) {
-                    S.kvrel[e % kWSlots] = 0;
-                    mbar_arrive(&S.wempty[e % kWSlots]);
+                if (lane == 0 && atom_add_acq_rel_cta(&S.kvrel[wslot(e)], 1) == 3) {
+                    S.kvrel[wslot(e)] = 0;
+                    mbar_arrive(&S.wempty[wslot(e)]);
                 }
             };
 #pragma unroll 1
@@ -1217,7 +1244,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                     const bool add_new = mine_new && jb == u.nb - 1;
                     kv_wait(ek);
                     if (add_new) {  // into the tile that only this warp reads there, and into the cache
-                        *reinterpret_cast<uint2 *>(sW + (size_t)(ek % kWSlots) * kSlotBytes + kv_k_off(pp, 4 * lane)) = kn;
+                        *reinterpret_cast<uint2 *>(sW + (size_t)wslot(ek) * kSlotBytes + kv_k_off(pp, 4 * lane)) = kn;
                         *reinterpret_cast<uint2 *>(blkn + kv_k_off(pp, 4 * lane)) = kn;
                         fence_proxy_async_smem();
                     }
@@ -1225,7 +1252,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                     uint32_t pf[2][2];  // P^T of 16 positions each as mma B fragments
                     if (nj > 0) {
                         const int pr = 32 * hq + (lane & 15);
-                        const uint32_t krow = smem_u32(sW) + (ek % kWSlots) * kSlotBytes + pr * 128;
+                        const uint32_t krow = smem_u32(sW) + wslot(ek) * kSlotBytes + pr * 128;
                         float sc[2][4];
 #pragma unroll
                         for (int i = 0; i < 2; ++i)
@@ -1282,7 +1309,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                     kv_release(ek);
                     kv_wait(ev);
                     if (add_new) {
-                        uint8_t *tile = sW + (size_t)(ev % kWSlots) * kSlotBytes - 32768;
+                        uint8_t *tile = sW + (size_t)wslot(ev) * kSlotBytes - 32768;
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {
                             const uint16_t v = (uint16_t)((e < 2 ? vn.x : vn.y) >> (16 * (e & 1)));
@@ -1295,7 +1322,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                     __syncwarp();
                     if (nj > 0) {
                         const int dr = lane & 15;
-                        const uint32_t vrow = smem_u32(sW) + (ev % kWSlots) * kSlotBytes + (hq >> 1) * 16384 + dr * 128;
+                        const uint32_t vrow = smem_u32(sW) + wslot(ev) * kSlotBytes + (hq >> 1) * 16384 + dr * 128;
 #pragma unroll
                         for (int kk = 0; kk < 2; ++kk) {  // positions 16 kk .. of the warp's
                             const uint32_t off = ((uint32_t)((hq & 1) * 4 + 2 * kk + (lane >> 4)) ^ (dr & 7)) << 4;
@@ -1478,11 +1505,11 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                     }
                 }
                 if (k == 0) load_rstd(p.ssqA, d / 64);
-                small_k(S, sW, red, X, R16c, g.kch, sg, wring, cw, lane, kv_wait);
+                small_k(S, sW, red, X, R16c, g.kch, sg, wring, cw, lane, kv_wait, nws_mul);
                 named_bar_sync(1, kMegaCThreads);
                 const int E = sg.entries();
                 if (ctid == 0)  // the slots not yet returned
-                    for (int e = (E - 1) / kWSlots * kWSlots; e < E; ++e) mbar_arrive(&S.wempty[(wring + e) % kWSlots]);
+                    for (int e = (E - 1) / S.nws * S.nws; e < E; ++e) mbar_arrive(&S.wempty[wslot(wring + e)]);
                 wring += (uint32_t)E;
                 float v = 0.f;
                 if (live) {
@@ -1669,7 +1696,7 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
     StepVars *V = p.c.v;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kWSlots; ++s) {
+        for (int s = 0; s < kMaxWSlots; ++s) {
             mbar_init(&S.wfull[s], 1);
             mbar_init(&S.wempty[s], 1);
             mbar_init(&S.kvready[0][s], 1);
@@ -1688,16 +1715,12 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
         S.rows = rows;
         S.rows16 = max(16, (rows + 15) & ~15);
         S.small = live <= kSmallRows;
-        // X stages of up to 16 KB: 4, 2 or 1 k-chunks each (fewer waits and commits per MMA), and
-        // the largest power of two of them (at most kMaxXStages) that fits after the W slots
-        {
-            S.xgroup = S.rows16 <= 16 ? 4 : S.rows16 <= 32 ? 2 : 1;
-            const int fit = min(kMaxXStages, (kRingBytes - kWSlots * kSlotBytes) / (S.rows16 * 256 * S.xgroup));
-            int lg = 0;
-            while ((2 << lg) <= fit) ++lg;
-            S.nx = 1 << lg;
-            S.nx_lg = lg;
-        }
+        // X stages of several k-chunks each where the rows are few (fewer waits and commits per MMA), as
+        // many as fit after the W slots
+        S.nws = ring_slots(rows);
+        S.xchunk = x_chunk_bytes(rows);
+        S.xgroup = rows <= 16 ? 4 : rows <= 32 ? 2 : 1;
+        S.nx = min(kMaxXStages, (kRingBytes - S.nws * kSlotBytes) / (S.xchunk * S.xgroup));
         S.n_items = *(volatile int *)&V->att_items;
         S.att_span = max(1, *(volatile int *)&V->att_span);
         S.target = (*(volatile unsigned long long *)p.epoch + 1ull) * gridDim.x;
@@ -1735,7 +1758,7 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = S.tmem_base;
-    uint8_t *sX = sW + (size_t)kWSlots * kSlotBytes;
+    uint8_t *sX = sW + (size_t)S.nws * kSlotBytes;
     const bool run = !S.abort && S.rows > 0;
     if (run) {
         if (warp == 0) {
