@@ -43,8 +43,8 @@
 //           and up rows alternate in blocks of 8, a CTA holds whole features (counter 5 is unused)
 //   7 DOWN  h W_down^T -> partials
 //   8 FIN_D x += sum; x_g = x * g_next; sum of squares
-// then lm_head over whole 256-token tiles fused with the Gumbel-max sampler: per (row, tile,
-// half-tile) maximum of logit + noise; the logits are stored only under teacher forcing.
+// then lm_head, column-owned and fused with the Gumbel-max sampler: per (row, CTA, half of its columns)
+// maximum of logit + noise; the logits are stored only under teacher forcing.
 //
 // Layouts (all chosen so that bulk copies land MMA operands in shared memory in the
 // 128-byte-swizzled K-major form the tensor core reads):
@@ -312,10 +312,9 @@ __device__ __forceinline__ unsigned long long phase_target(const MegaParams &p, 
 
 // ------------------------------------------------------------------------------ phases
 // GEMM phases: N output features, K inputs.  Two ways to split the work:
-//   split-K: (256-feature tile, 64-column chunk) units in equal contiguous ranges over the CTAs
-//     (lm_head: on whole tiles); each CTA stores its fp32 partial tiles and a finalisation phase
-//     sums them.
-//   column-owned (gate / up; q/k/v and O at few live rows): 16-feature units in equal contiguous
+//   split-K: (256-feature tile, 64-column chunk) units in equal contiguous ranges over the CTAs;
+//     each CTA stores its fp32 partial tiles and a finalisation phase sums them.
+//   column-owned (gate / up; lm_head; q/k/v and O at few live rows): 16-feature units in equal contiguous
 //     ranges, each with the whole K, so that the CTA's epilogue applies what follows (SwiGLU;
 //     RoPE and the cache append; residual and norm input) itself and no partials and no
 //     finalisation phase are needed.  More activation traffic (every CTA reads the whole
@@ -343,10 +342,10 @@ __device__ __noinline__ void make_plan(const MegaParams &p, GemmPlan &g, int whi
     }
     g.kch = K / 64;
     g.t = g.kc = g.units = 0;
-    // at most one CTA per unit (tile for lm_head), so every participating CTA holds a
+    // at most one CTA per unit, so every participating CTA holds a
     // non-empty range and the CTAs between a tile's first and last owner all contributed
     const bool sm = small && (which == kGQKV || which == kGO);
-    if (which == kGGU || sm) {
+    if (which == kGGU || which == kGLM || sm) {
         const int U = g.N / kOwnCols, most = sm ? kSmallUnits : kOwnUnits;
         Gp = min(G, U);
         if (sm) {  // equal shares: a pass of small_k costs about the same for one unit or two
@@ -356,16 +355,22 @@ __device__ __noinline__ void make_plan(const MegaParams &p, GemmPlan &g, int whi
         if (c < Gp) {
             g.t = c * U / Gp;
             g.units = (c + 1) * U / Gp - g.t;
+            if (which == kGLM && U >= kOwnUnits * 2 * Gp) {
+                // a large vocabulary in whole passes: equal shares of 62.5 units read no faster
+                // (1.5B, 151,936 tokens, 26 rows: 1.189 ms in tiles, 1.191 in shares)
+                const int T = (U + kOwnUnits - 1) / kOwnUnits;
+                g.t = c * T / Gp * kOwnUnits;
+                g.units = min(U, (c + 1) * T / Gp * kOwnUnits) - g.t;
+            }
             const int np = (g.units + most - 1) / most;  // equal passes
             g.pass = (g.units + np - 1) / np;
         }
     } else {
-        const int T = (g.N + kTileN - 1) / kTileN;
-        const int U = which == kGLM ? T : T * g.kch, m = which == kGLM ? g.kch : 1;
+        const int U = (g.N + kTileN - 1) / kTileN * g.kch;
         Gp = min(Gp, U);
         if (c < Gp) {
-            const int u0 = c * U / Gp * m;
-            g.units = (c + 1) * U / Gp * m - u0;
+            const int u0 = c * U / Gp;
+            g.units = (c + 1) * U / Gp - u0;
             g.t = u0 / g.kch;
             g.kc = u0 - g.t * g.kch;
         }
@@ -1595,19 +1600,21 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
 
     // ---------------------------------------------------------------- lm_head + Gumbel-max
     // logits = (x_g W_lm^T) / rms(x) for the live rows, fused with the temperature-1 sampler:
-    // each thread scans its columns of a tile in increasing token order, adds the
+    // each thread scans its columns of the CTA's in increasing token order, adds the
     // Gumbel noise g(row key, token) and keeps the first maximum of logit + g; the per (row,
-    // tile, half) maxima go to the bookkeeping kernel, which takes the row's argmax (ties to
+    // CTA, half) maxima go to the bookkeeping kernel, which takes the row's argmax (ties to
     // the lowest token id).  Products and sums are rounded separately (no contraction), as
     // the sampler on stored logits would do them.  The logits themselves are written only
     // when requested (teacher forcing).
+    // (Each lane finishes its columns one after the other, so a small vocabulary in whole 256-token tiles
+    // on two CTAs took 12 us of 54: it is shared in 16-token units over all CTAs.  Vocabulary of 512
+    // and 2 rows, kernel: 51.1 -> 45.7 us; 25 rows: 66.4 -> 61.1.)
     wait_phase(kPhasesPerLayer * p.layers);
     load_rstd(p.ssqA, d / 64);
     named_bar_sync(1, kMegaCThreads);
     const GemmPlan &g = S.plan[kGLM];
     const float rs = act ? S.rstd[my_row] : 0.f;
     const uint64_t seed = act ? __ldg(&p.c.row_seed[my_row]) : 0ull;
-    const int nparts = 2 * ((g.N + kTileN - 1) / kTileN);
     float best = -INFINITY;  // running over this thread's tiles (its row and columns)
     int bi = 0x7fffffff;
     SegWalk walk(g);
@@ -1615,22 +1622,22 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
 #pragma unroll 1
     while (walk.next(g, sg)) {
         const uint32_t a = acc_wait();
-        if (quarter_live && half * 128 < sg.n) {
-            const float best0 = best;  // the maximum over this thread's earlier tiles
+        const int hc = 32 * ((sg.n + 63) / 64);  // a half's columns: from half * hc on
+        if (quarter_live) {
 #pragma unroll 1
-            for (int cc = 0; cc < 4; ++cc) {
+            for (int c0 = half * hc; c0 < min(sg.n, half * hc + hc); c0 += 32) {
                 float v[32];
-                tmem_ld_32x32b_x32(tmem + lane_base + a * kTileN + half * 128 + cc * 32, v);
+                tmem_ld_32x32b_x32(tmem + lane_base + a * kTileN + c0, v);
                 float w[16];
                 pair_part(v, w);
                 // 16 columns at a time; each lane of a pair takes one half of the 32
 #pragma unroll 1
                 for (int q = second ? 1 : 0; q < (pair && !second ? 1 : 2); ++q) {
-                    if (!act) continue;
+                    if (!act || c0 + q * 16 >= sg.n) continue;
                     float z[16];
 #pragma unroll
                     for (int e = 0; e < 16; ++e) z[e] = __fmul_rn((q ? v[16 + e] : v[e]) + w[e], rs);
-                    const int nb = sg.col0 + half * 128 + cc * 32 + q * 16;
+                    const int nb = sg.col0 + c0 + q * 16;
                     if (p.write_logits) {
                         float4 *o = reinterpret_cast<float4 *>(p.logits + (int64_t)my_row * p.V + nb);
 #pragma unroll
@@ -1641,13 +1648,26 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                     // so z_e + g(u_e) > best needs u_e > exp(-exp(-(best - max_e z_e))); the
                     // cut is taken 1e-3 lower in g and 4 codes lower in the 24-bit u, far
                     // beyond the rounding of the float evaluation, so no candidate is lost.
-                    // `best` runs over all of this thread's tiles: a (tile, half) whose
-                    // tokens cannot beat an earlier tile's maximum reports -inf, which the
-                    // row's argmax ignores (ties go to the lower token id either way).
+                    // `best` runs over all of this thread's columns; before the first maximum, the
+                    // token of the largest noise stands in for it.
+                    float low = best;
+                    if (best == -INFINITY) {
+                        uint32_t most = 0;
+                        int me = 0;
+#pragma unroll 1
+                        for (int e = 0; e < 16; ++e) {
+                            const uint32_t code = (uint32_t)(splitmix_at(seed, (uint64_t)(nb + e) + 1) >> 40);
+                            if (code > most) { most = code; me = e; }
+                        }
+                        float ze = z[0];
+#pragma unroll
+                        for (int i = 1; i < 16; ++i) ze = (i == me) ? z[i] : ze;
+                        low = __fadd_rn(ze, gumbel_from_hash(splitmix_at(seed, (uint64_t)(nb + me) + 1)));
+                    }
                     float vmax = z[0];
 #pragma unroll
                     for (int e = 1; e < 16; ++e) vmax = fmaxf(vmax, z[e]);
-                    const float ureq = expf(-expf(-(best - vmax - 1e-3f)));  // 0 while best = -inf
+                    const float ureq = expf(-expf(-(low - vmax - 1e-3f)));
                     const float cut = ureq * 16777216.0f - 4.0f;
                     const uint32_t thr = cut > 0.f ? (uint32_t)cut : 0u;
                     uint32_t cand = 0;
@@ -1666,21 +1686,19 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                     }
                 }
             }
-            // this (tile, half)'s maximum if it beats the earlier tiles, else -inf; the lanes of a
-            // pair hold disjoint columns (ties to the lower id)
-            float wv = best > best0 ? best : -INFINITY;
-            int wi = best > best0 ? bi : 0x7fffffff;
-            if (pair) {
-                const float ov = __shfl_xor_sync(0xffffffffu, wv, 8);
-                const int oi = __shfl_xor_sync(0xffffffffu, wi, 8);
-                if (ov > wv || (ov == wv && oi < wi)) { wv = ov; wi = oi; }
-            }
-            if (act && !second) {
-                p.c.arg_val[my_row * nparts + 2 * sg.t + half] = wv;
-                p.c.arg_idx[my_row * nparts + 2 * sg.t + half] = wi;
-            }
         }
         acc_release(a);
+    }
+    // this (CTA, half)'s maximum (-inf where it has no columns); the lanes of a pair hold disjoint
+    // columns (ties to the lower id)
+    if (pair) {
+        const float ov = __shfl_xor_sync(0xffffffffu, best, 8);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, 8);
+        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
+    }
+    if (act && !second) {
+        p.c.arg_val[(my_row * G + cta) * 2 + half] = best;
+        p.c.arg_idx[(my_row * G + cta) * 2 + half] = bi;
     }
     named_bar_sync(1, kMegaCThreads);
     if (ctid == 0) MEGA_STAMP(1 + kPhasesPerLayer * p.layers, 0);

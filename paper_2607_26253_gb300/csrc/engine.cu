@@ -369,7 +369,7 @@ void enqueue_decode_step(sara_handle &h, cudaStream_t s, bool write_logits = fal
     MegaParams mp = mega_params(h);
     mp.write_logits = write_logits ? 1 : 0;
     launch_ex(s, false, true, dim3(h.sms), dim3(kMegaThreads), kMegaSmemBytes, decode_step_kernel, mp);
-    launch(s, false, dim3(h.cfg.max_seqs), dim3(256), 0, sample_finish_kernel, h.ptrs, h.cfg.vocab,
+    launch(s, false, dim3(h.cfg.max_seqs), dim3(256), 0, sample_finish_kernel, h.ptrs,
            more ? *more : cudaGraphConditionalHandle{}, more ? 1 : 0);
 }
 
@@ -790,10 +790,10 @@ void create_impl(sara_handle &h, const sara_model_cfg *cfgp, const sara_weights 
         const int Gq = m.n_heads / KVH;
         h.attn_part = h.mem.alloc<float>((size_t)h.att_cap * KVH * Gq * (hd + 2), false);
         h.attn_cnt = h.mem.alloc<int>((size_t)S * KVH);
-        // the lm_head epilogue's sampler maxima: [rows][2 per 256-token tile]
-        c.lm_tiles = (m.vocab + kTileN - 1) / kTileN;
-        h.lm_val = h.mem.alloc<float>((size_t)S * 2 * c.lm_tiles, false);
-        h.lm_idx = h.mem.alloc<int>((size_t)S * 2 * c.lm_tiles, false);
+        // the lm_head epilogue's sampler maxima: [rows][2 per CTA]
+        c.lm_parts = 2 * h.sms;
+        h.lm_val = h.mem.alloc<float>((size_t)S * c.lm_parts, false);
+        h.lm_idx = h.mem.alloc<int>((size_t)S * c.lm_parts, false);
         h.logit_buf = h.mem.alloc<float>((size_t)S * m.vocab, false);
         c.arg_val = h.lm_val;
         c.arg_idx = h.lm_idx;

@@ -70,8 +70,8 @@ __device__ __forceinline__ int scan256(int v, int &total, int *warp_tot) {
 }
 
 // Sampling finish + step bookkeeping, after the decode-step kernel.  That kernel's lm_head
-// epilogue left, per live row, the first maximum of logit + Gumbel noise of every (256-token
-// tile, 128-token half) (arg_val / arg_idx [rows][2 * tiles]); CTA r reduces row r's maxima
+// epilogue left, per live row, the first maximum of logit + Gumbel noise of every (CTA, half of its
+// columns) (arg_val / arg_idx [rows][lm_parts]); CTA r reduces row r's maxima
 // to its token (ties: lowest token id).  The last CTA to finish appends each row's token to
 // its rollout, retires rollouts that reached their length, compacts the live rows (order
 // kept) and writes the next step's rows and attention items.
@@ -80,7 +80,7 @@ __device__ __forceinline__ int scan256(int v, int &total, int *warp_tot) {
 // follows unless the controller has work (a round's last rollout finished, or on the asynchronous
 // schedule a prompt's batch), an error was reported, or a bound is reached (the controller then
 // reports it).
-static __global__ void __launch_bounds__(256) sample_finish_kernel(StepPtrs c, int vocab, cudaGraphConditionalHandle more,
+static __global__ void __launch_bounds__(256) sample_finish_kernel(StepPtrs c, cudaGraphConditionalHandle more,
                                                                    int use_more) {
     __shared__ int span_sm[kAttCands + 1];
     __shared__ float sv[8];
@@ -94,11 +94,10 @@ static __global__ void __launch_bounds__(256) sample_finish_kernel(StepPtrs c, i
     const int r = blockIdx.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     if (r < live) {
-        const int tiles = (vocab + 255) / 256, nparts = 2 * tiles;
+        const int nparts = c.lm_parts;
         float best = -INFINITY;
         int bi = 0x7fffffff;
         for (int j = tid; j < nparts; j += blockDim.x) {
-            if ((j & 1) * 128 >= min(256, vocab - 256 * (j >> 1))) continue;  // a half tile past the vocabulary
             const float v = __ldcg(&c.arg_val[(int64_t)r * nparts + j]);
             const int id = __ldcg(&c.arg_idx[(int64_t)r * nparts + j]);
             if (v > best || (v == best && id < bi)) { best = v; bi = id; }

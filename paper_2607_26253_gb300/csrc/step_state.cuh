@@ -137,7 +137,7 @@ struct StepPtrs {
     // sampling partial argmax per (row, vocabulary chunk)
     float *arg_val;
     int32_t *arg_idx;
-    int32_t lm_tiles;
+    int32_t lm_parts;  // maxima per row: two per CTA of the decode-step kernel
     int32_t max_seqs, max_active, pre_cap, att_cap;
     // paged KV cache of 128-position blocks.  Block ids [0, n_shared) hold the prompts' full
     // blocks (prompt slot ps owns ids ps * nsh_max ..), ids [n_shared, n_shared + n_priv) are

@@ -1,7 +1,7 @@
 """The decode step's row-count and width branches: every accumulator layout of its projections (row counts around 8, 16,
-32, 64 and 128), MLP widths from a single 16-feature unit per CTA to more than one 256-feature pass, more attention units
-than a CTA's table holds, new positions at the edges of a warp's 32 positions and of a KV block (where the number of
-attention splits changes); teacher-forced logits against the float64 oracle within the stated tolerance."""
+32, 64 and 128), MLP widths and vocabularies from a single 16-feature unit per CTA to more than one 256-feature pass, more
+attention units than a CTA's table holds, new positions at the edges of a warp's 32 positions and of a KV block (where the
+number of attention splits changes); teacher-forced logits against the float64 oracle within the stated tolerance."""
 import numpy as np
 import pytest
 
@@ -33,12 +33,15 @@ WIDE = _shape("ffn 20032", layers=1, ffn=20032)                     # 2,504 unit
 DEEP = _shape("d 2048", layers=2, d_model=2048, n_heads=16, head_dim=128, ffn=448)
 MANY_HEADS = _shape("32 heads", d_model=512, n_heads=32, n_kv_heads=4, head_dim=128, ffn=128)  # K = 4,096 > d
 MANY_KV = _shape("48 kv heads", layers=2, d_model=128, n_heads=48, n_kv_heads=48, head_dim=32, ffn=64)  # 40 units per SM
+VOCAB_UNITS = _shape("vocab 40064", layers=1, d_model=128, n_heads=4, head_dim=32, ffn=64, vocab=40064)  # 2,504 units
+VOCAB_TILES = _shape("vocab 80000", layers=1, d_model=128, n_heads=4, head_dim=32, ffn=64, vocab=80000)  # whole tiles
 
 
 @pytest.mark.parametrize("shape,rows", [(NARROW, 1), (NARROW, 9), (NARROW, 128), (ODD, 8), (ODD, 17), (ODD, 33),
                                         (ODD, 65), (WIDE, 2), (WIDE, 32), (WIDE, 64), (DEEP, 1), (DEEP, 16),
                                         (DEEP, 31), (DEEP, 48), (MANY_HEADS, 3), (MANY_HEADS, 32), (MANY_HEADS, 40),
-                                        (MANY_KV, 128)],
+                                        (MANY_KV, 128), (VOCAB_UNITS, 3), (VOCAB_UNITS, 66),
+                                        (VOCAB_TILES, 3), (VOCAB_TILES, 66)],
                          ids=lambda v: getattr(v, "name", v))
 def test_teacher_forced_logits_by_rows_and_widths(pkg, shape, rows):
     _check(pkg, shape, rows, Lp=5, T=3)
