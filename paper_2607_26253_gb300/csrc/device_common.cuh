@@ -42,9 +42,8 @@ __device__ __forceinline__ uint64_t mix64(uint64_t z) {
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
     return z ^ (z >> 31);
 }
-__device__ __forceinline__ uint64_t splitmix_at(uint64_t seed, uint64_t c) {
-    return mix64(seed + c * 0x9E3779B97F4A7C15ull);
-}
+constexpr uint64_t kSplitmixGamma = 0x9E3779B97F4A7C15ull;  // golden
+__device__ __forceinline__ uint64_t splitmix_at(uint64_t seed, uint64_t c) { return mix64(seed + c * kSplitmixGamma); }
 
 // Gumbel(0,1) noise from a 64-bit hash: u = (top 24 bits + 0.5) / 2^24, g = -log(-log u).
 __device__ __forceinline__ float gumbel_from_hash(uint64_t h) {

@@ -309,16 +309,21 @@ static __global__ void __launch_bounds__(kCtlThreads, 1) teacher_setup_kernel(St
 
 // Gumbel-max over given fp32 logits (kernel-level entry point): one cluster of kSampleCtas CTAs per
 // row, each a contiguous share of the vocabulary, the row's maximum joined through distributed
-// shared memory.  Bound by instruction issue (a 64-bit hash per token), so the noise's logarithms
-// are taken only for tokens that could beat the warp's best so far (g(u) increases with the
-// hash's top 24 bits; see the lm_head phase for the cut).  64 rows x 151,936, whole call: 37 us;
-// 277 us with one CTA per row (64 of 152 SMs) and the noise of every token.
+// shared memory.  Bound by instruction issue (a 64-bit hash per token; 51 instructions a token in all),
+// so the noise's logarithms are taken only for tokens that could beat the CTA's best so far (g(u)
+// increases with the hash's top 24 bits; see the lm_head phase for the cut), the hash's input is
+// advanced by additions, and a step's logits load during the one before.  64 rows x 151,936, whole
+// call: 277 us with one CTA per row (64 of 152 SMs) and the noise of every token, 37 us with the
+// bound per warp and all of the first step's tokens evaluated, 26 us now (kernel 35.6 -> 25.0).
 constexpr int kSampleCtas = 8;
 static __global__ void __launch_bounds__(256) sample_rows_kernel(const float *logits, int V, uint64_t sample_seed,
                                                                  const int64_t *uid, const int32_t *t, int *token) {
     __shared__ float sv[8];
     __shared__ int si[8];
     __shared__ uint32_t cv[kSampleCtas], ci[kSampleCtas];  // (rank 0) the cluster's maxima
+    __shared__ volatile float wb[8];                       // each warp's best so far
+    if (threadIdx.x < 8) wb[threadIdx.x] = -INFINITY;
+    __syncthreads();
     const int r = blockIdx.x / kSampleCtas, rank = (int)cluster_rank();
     const uint64_t rs = sampler_row_seed(sample_seed, uid[r], t[r]);
     const float *row = logits + (int64_t)r * V;
@@ -327,20 +332,51 @@ static __global__ void __launch_bounds__(256) sample_rows_kernel(const float *lo
     const bool vec = (reinterpret_cast<uintptr_t>(row) & 15) == 0;
     float best = -INFINITY, wbest = -INFINITY;  // this thread's, and the warp's as of the last step
     int bi = 0x7fffffff;
-#pragma unroll 1
-    for (int b = rank * per; b < v1; b += 2048) {
-        float z[8];  // tokens b + 4 tid .. and b + 1024 + 4 tid ..
-        uint32_t cand = 0;
+    bool first = true;
+    // a step's tokens: b + 4 tid .. and b + 1024 + 4 tid ..
+    auto load = [&](int b, float (&y)[8]) {
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int v = b + q * 1024 + (int)threadIdx.x * 4;
             if (vec && v + 3 < v1) {
                 const float4 x = __ldg(reinterpret_cast<const float4 *>(row + v));
-                z[4 * q] = x.x; z[4 * q + 1] = x.y; z[4 * q + 2] = x.z; z[4 * q + 3] = x.w;
+                y[4 * q] = x.x; y[4 * q + 1] = x.y; y[4 * q + 2] = x.z; y[4 * q + 3] = x.w;
             } else {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) z[4 * q + e] = v + e < v1 ? __ldg(row + v + e) : -INFINITY;
+                for (int e = 0; e < 4; ++e) y[4 * q + e] = v + e < v1 ? __ldg(row + v + e) : -INFINITY;
             }
+        }
+    };
+    float next[8];
+    load(rank * per, next);
+#pragma unroll 1
+    for (int b = rank * per; b < v1; b += 2048) {
+        float z[8];
+        uint32_t cand = 0;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) z[e] = next[e];
+        if (v1 - b > 2048) load(b + 2048, next);  // (in flight during this step)
+        // the hash's input is linear in the token: one product per four of them
+        uint32_t code[8];  // the hash's top 24 bits
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int v = b + q * 1024 + (int)threadIdx.x * 4;
+            const uint64_t x = rs + (uint64_t)(v + 1) * kSplitmixGamma;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) code[4 * q + e] = (uint32_t)(mix64(x + (uint64_t)e * kSplitmixGamma) >> 40);
+        }
+        const int n0 = v1 - b - (int)threadIdx.x * 4, n1 = n0 - 1024;  // this thread's tokens of each four
+        const uint32_t valid = (n0 >= 4 ? 0xfu : n0 > 0 ? (1u << n0) - 1 : 0u) | (n1 >= 4 ? 0xf0u : n1 > 0 ? (16u << n1) - 16 : 0u);
+        if (first) {  // before the first maximum, the warp's best of the tokens of largest noise stands in for it
+            first = false;
+            uint32_t most = 0;
+            float zmost = -INFINITY;
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (code[e] >= most && (valid >> e & 1)) { most = code[e]; zmost = z[e]; }
+            wbest = __fadd_rn(zmost, gumbel_from_hash((uint64_t)most << 40));
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) wbest = fmaxf(wbest, __shfl_xor_sync(0xffffffffu, wbest, o));
         }
         float vmax = z[0];
 #pragma unroll
@@ -349,24 +385,30 @@ static __global__ void __launch_bounds__(256) sample_rows_kernel(const float *lo
         const float cut = ureq * 16777216.0f - 4.0f;
         const uint32_t thr = cut > 0.f ? (uint32_t)cut : 0u;
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            const int v = b + (e >> 2) * 1024 + (int)threadIdx.x * 4 + (e & 3);
-            cand |= (uint32_t)(v < v1 && (uint32_t)(splitmix_at(rs, (uint64_t)v + 1) >> 40) >= thr) << e;
-        }
+        for (int e = 0; e < 8; ++e) cand |= (uint32_t)(code[e] >= thr) << e;
+        cand &= valid;
 #pragma unroll 1
         while (cand) {  // in increasing token order: the first maximum is kept
             const int e = __ffs(cand) - 1;
             cand &= cand - 1;
             float ze = z[0];
+            uint32_t k = code[0];
 #pragma unroll
-            for (int i = 1; i < 8; ++i) ze = (i == e) ? z[i] : ze;
+            for (int i = 1; i < 8; ++i) {
+                ze = (i == e) ? z[i] : ze;
+                k = (i == e) ? code[i] : k;
+            }
             const int v = b + (e >> 2) * 1024 + (int)threadIdx.x * 4 + (e & 3);
-            ze = __fadd_rn(ze, gumbel_from_hash(splitmix_at(rs, (uint64_t)v + 1)));
+            ze = __fadd_rn(ze, gumbel_from_hash((uint64_t)k << 40));  // (the noise is of the top 24 bits)
             if (ze > best) { best = ze; bi = v; }
         }
-        wbest = best;
+        // the next step's bound: the CTA's best so far (a warp that is behind reads an older one)
+        wbest = fmaxf(wbest, best);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) wbest = fmaxf(wbest, __shfl_xor_sync(0xffffffffu, wbest, o));
+        if ((threadIdx.x & 31) == 0) wb[threadIdx.x >> 5] = wbest;
+        __syncwarp();
+        for (int w = 0; w < 8; ++w) wbest = fmaxf(wbest, wb[w]);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
