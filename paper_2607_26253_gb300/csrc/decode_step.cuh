@@ -31,12 +31,13 @@
 //
 // Phases of layer l (counter index 1 + 9l + k):
 //   0 QKV   x_g W_qkv^T -> partials        (a subset of the CTAs: few tiles)
-//   1 FIN_Q q, k, v = RMSNorm scale + RoPE of the summed partials, fp16, once per row
-//   2 ATT   softmax(q K^T) V, 128-position KV blocks, online softmax over a split's blocks
-//           with warp-level MMAs (mma.sync: N = 8 heads, operands and accumulators in
-//           registers, no exchange between warps inside a split; the new k, v join the tiles and
-//           the KV cache here; the tcgen05 path's issue / commit / tensor-memory round trips cost more
-//           than these products); the last split of a row to finish merges the splits
+//   2 ATT   q, k, v = RMSNorm scale + RoPE of the summed partials, fp16 (counter 1: of the few rows'
+//           q/k/v phase, which does that itself); softmax(q K^T) V, 128-position KV blocks,
+//           online softmax over a split's blocks with warp-level MMAs (mma.sync: N = 8 heads,
+//           operands and accumulators in registers, no exchange between warps inside a split; the
+//           tcgen05 path's issue / commit / tensor-memory round trips cost more than these
+//           products); the new k, v join the tiles and the KV cache here; the last split of a row
+//           to finish merges the splits
 //   3 O     att W_o^T -> partials           (a subset of the CTAs)
 //   4 FIN_O x += sum; x_g = x * g_mlp (bf16 hi/lo, blocked); per-row sum of squares
 //   6 GU    h = silu(r g) * (r u), g | u = x_g W_gu^T, r = 1/rms(x)  (bf16 hi/lo, blocked): gate
@@ -968,13 +969,14 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
     auto contributors = [&](int which, int t) -> int2 {
         return t < kPlanTiles ? S.tile_cta[which][t] : tile_ctas(p, S.plan[which], which, t, G);
     };
-    // Four columns' sum of a tile's partials for one row: lanes 0-15 and 16-31 of a warp take
-    // alternate contributors (up to 16 loads in flight each), then add up.  `off`: row and column
-    // inside a segment, in floats.
-    auto part_sum = [&](int2 ct, int t, int off) -> float4 {
+    // Four columns' sum of a tile's partials for one row.  split: lanes 0-15 and 16-31 of a warp have
+    // the same columns, take alternate contributors (up to 16 loads in flight each), then add up.
+    // `off`: row and column inside a segment, in floats.
+    auto part_sum = [&](int2 ct, int t, int off, bool split) -> float4 {
         const int64_t seg = (int64_t)p.rows_cap * kTileN;
-        const float *src = p.gpart + (int64_t)(ct.x + (lane >> 4) + t) * seg + off;
-        int n = (ct.y - ct.x - (lane >> 4) + 2) >> 1;  // contributors of this half
+        const int c0 = split ? lane >> 4 : 0, step = split ? 2 : 1;
+        const float *src = p.gpart + (int64_t)(ct.x + c0 + t) * seg + off;
+        int n = (ct.y - ct.x - c0 + step) / step;  // contributors of this lane
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
         while (__any_sync(0xffffffffu, n > 0)) {
@@ -983,12 +985,13 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
             for (int k = 0; k < 16; ++k) {
                 v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (k < n) v[k] = __ldcg(reinterpret_cast<const float4 *>(src));
-                src += 2 * seg;
+                src += step * seg;
             }
 #pragma unroll
             for (int k = 0; k < 16; ++k) { s.x += v[k].x; s.y += v[k].y; s.z += v[k].z; s.w += v[k].w; }
             n -= 16;
         }
+        if (!split) return s;
         s.x += __shfl_xor_sync(0xffffffffu, s.x, 16);
         s.y += __shfl_xor_sync(0xffffffffu, s.y, 16);
         s.z += __shfl_xor_sync(0xffffffffu, s.z, 16);
@@ -1046,7 +1049,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                 } else {
                     x = __ldcg(reinterpret_cast<const float4 *>(xp));
                     const int t = f / kTileN;
-                    const float4 s = part_sum(contributors(which, t), t, r * kTileN + f - t * kTileN);
+                    const float4 s = part_sum(contributors(which, t), t, r * kTileN + f - t * kTileN, true);
                     x.x += s.x; x.y += s.y; x.z += s.z; x.w += s.w;
                 }
                 uint16_t h[4], lo[4];
@@ -1120,53 +1123,72 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                 arrive(base + kPhGU, true);
             }
         } else if (k == 1) {
-          if (!small) {
-            // -------------------------------------------------------- q, k, v (once per row)
-            // The head's QKV partials summed, times 1/rms; RoPE on q and k; q pre-scaled by
-            // log2(e)/sqrt(hd) for the exp2 softmax; fp16 q, k, v for the attention phase.  Unit =
-            // (row, 64 weight rows): a
-            // head's weight rows come in 16s, 8 dims and their rotation partners, so lane % 16
-            // holds 4 dims and lane ^ 2 their partners; the warp's halves split the contributors.
-            wait_phase(base + kPhQKV);
-            const int n64 = p.nqkv / 64, half_hd = hd >> 1;
-#pragma unroll 1
-            for (int u = gw; u < R * n64; u += nw) {
-                const int r = u / n64, n0 = (u - r * n64) * 64 + (lane & 15) * 4;
-                const int head = n0 / hd, j = n0 - head * hd;
-                const bool isq = head < p.H, isk = !isq && head < p.H + p.KVH, hi = (j & 8) != 0;
-                const int fr = (j >> 4) * 8 + (j & 7), d0 = hi ? fr + half_hd : fr;
-                // the row's sum-of-squares partials and rotation factors load with the QKV partials
-                const float sq = lane < d / 64 ? __ldcg(&p.ssqA[lane * p.rows_cap + r]) : 0.f;
-                const int pos = S.rowpos[r];
-                float4 c0 = make_float4(1.f, 0.f, 1.f, 0.f), c1 = c0;  // (cos, sin) of two dims each
-                if (isq || isk) {
-                    const float4 *rp = reinterpret_cast<const float4 *>(p.rope + (int64_t)pos * half_hd + fr);
-                    c0 = __ldg(rp);
-                    c1 = __ldg(rp + 1);
-                }
-                const int t = n0 / kTileN;
-                const float4 x = part_sum(contributors(kGQKV, t), t, r * kTileN + n0 - t * kTileN);
-                const float rs = rsqrtf(warp_sum(sq) / (float)d + p.eps) * (isq ? p.scale_log2 : 1.f);
-                float4 o;
-                o.x = __shfl_xor_sync(0xffffffffu, x.x, 2);
-                o.y = __shfl_xor_sync(0xffffffffu, x.y, 2);
-                o.z = __shfl_xor_sync(0xffffffffu, x.z, 2);
-                o.w = __shfl_xor_sync(0xffffffffu, x.w, 2);
-                const float sg = hi ? 1.f : -1.f;  // rotate the pairs (i, i + hd/2); identity for v
-                const uint16_t h[4] = {f32_to_f16_sat((x.x * c0.x + sg * (o.x * c0.y)) * rs),
-                                       f32_to_f16_sat((x.y * c0.z + sg * (o.y * c0.w)) * rs),
-                                       f32_to_f16_sat((x.z * c1.x + sg * (o.z * c1.y)) * rs),
-                                       f32_to_f16_sat((x.w * c1.z + sg * (o.w * c1.w)) * rs)};
-                if (lane < 16) *reinterpret_cast<uint2 *>(p.qkv16 + r * p.nqkv + head * hd + d0) = pack4(h);
-            }
-            arrive(base + kPhFinQ, false);
-          }
-            // -------------------------------------------------------- attention
             int a0, a1;
             att_range(p, S.n_items, a0, a1);
             const int n = a1 - a0;
             if (l == 0) mwait(&S.units_ready, 0, err, ab, lim);
-            wait_phase(base + kPhFinQ);
+            if (small) {
+                wait_phase(base + kPhFinQ);
+            } else {
+                // ------------------------------------------------ q, k, v of this CTA's attention units
+                // The QKV partials summed, times 1/rms; RoPE on q and k; q pre-scaled by log2(e)/sqrt(hd)
+                // for the exp2 softmax; fp16.  Splits of a row on several CTAs sum the same partials (and
+                // store the same values): cheaper than a phase of its own, with an arrival and a wait.
+                // 1.5B kernel, ms as a phase of its own -> here: 16 rows of 60 positions 1.145 -> 1.112, 26 rows
+                // 1.202 -> 1.155, 64 rows 1.526 -> 1.445, 128 rows of 500 2.378 -> 2.273; 16 rows of 2000
+                // positions, eight splits each, 1.355 -> 1.328.  (With a warp per group, whose halves
+                // split the contributors: 80 rows 1.782 -> 1.800, 3B 26 rows 1.950 -> 1.989.)
+                // A half warp takes a group of 64 weight rows; a head's weight rows come in 16s, 8 dims and
+                // their rotation partners, so lane % 16 holds 4 dims and lane ^ 2 their partners.
+                wait_phase(base + kPhQKV);
+                const int half_hd = hd >> 1;
+                int w = 2 * cw;  // this warp's next two groups, counted from the current unit's first
+#pragma unroll 1
+                for (int i = 0; i < n; ++i) {
+                    const AttUnit &u = cta_unit(p, S, a0, i, 0);
+                    const int r = u.row;
+                    if (i >= p.KVH && cta_unit(p, S, a0, i - p.KVH, 1).row == r) continue;  // (an earlier split of the row)
+                    // the groups that hold the unit's q heads, its k and its v
+                    const int q0 = u.kvh * Gq * hd / 64, nq = ((u.kvh + 1) * Gq * hd + 63) / 64 - q0;
+                    const int k0 = (p.H + u.kvh) * hd / 64, nk = ((p.H + u.kvh + 1) * hd + 63) / 64 - k0;
+                    const int v0 = (p.H + p.KVH + u.kvh) * hd / 64, ng = nq + nk + ((p.H + p.KVH + u.kvh + 1) * hd + 63) / 64 - v0;
+#pragma unroll 1
+                    for (; w < ng; w += 16) {
+                        const int y = min(w + (lane >> 4), ng - 1);  // (both halves the last one: the same values stored twice)
+                        const int n0 = (y < nq ? q0 + y : y < nq + nk ? k0 + y - nq : v0 + y - nq - nk) * 64 + (lane & 15) * 4;
+                        const int head = n0 / hd, j = n0 - head * hd;
+                        const bool isq = head < p.H, isk = !isq && head < p.H + p.KVH, hi = (j & 8) != 0;
+                        const int fr = (j >> 4) * 8 + (j & 7), d0 = hi ? fr + half_hd : fr;
+                        // the row's sum-of-squares partials and rotation factors load with the QKV partials
+                        const float sq = lane < d / 64 ? __ldcg(&p.ssqA[lane * p.rows_cap + r]) : 0.f;
+                        const int pos = S.rowpos[r];
+                        float4 c0 = make_float4(1.f, 0.f, 1.f, 0.f), c1 = c0;  // (cos, sin) of two dims each
+                        if (isq || isk) {
+                            const float4 *rp = reinterpret_cast<const float4 *>(p.rope + (int64_t)pos * half_hd + fr);
+                            c0 = __ldg(rp);
+                            c1 = __ldg(rp + 1);
+                        }
+                        const int t = n0 / kTileN;
+                        const float4 x = part_sum(contributors(kGQKV, t), t, r * kTileN + n0 - t * kTileN, false);
+                        const float rs = rsqrtf(warp_sum(sq) / (float)d + p.eps) * (isq ? p.scale_log2 : 1.f);
+                        float4 o;
+                        o.x = __shfl_xor_sync(0xffffffffu, x.x, 2);
+                        o.y = __shfl_xor_sync(0xffffffffu, x.y, 2);
+                        o.z = __shfl_xor_sync(0xffffffffu, x.z, 2);
+                        o.w = __shfl_xor_sync(0xffffffffu, x.w, 2);
+                        const float sg = hi ? 1.f : -1.f;  // rotate the pairs (i, i + hd/2); identity for v
+                        const uint16_t h[4] = {f32_to_f16_sat((x.x * c0.x + sg * (o.x * c0.y)) * rs),
+                                               f32_to_f16_sat((x.y * c0.z + sg * (o.y * c0.w)) * rs),
+                                               f32_to_f16_sat((x.z * c1.x + sg * (o.z * c1.y)) * rs),
+                                               f32_to_f16_sat((x.w * c1.z + sg * (o.w * c1.w)) * rs)};
+                        *reinterpret_cast<uint2 *>(p.qkv16 + r * p.nqkv + head * hd + d0) = pack4(h);
+                    }
+                    w -= (ng + 1) & ~1;
+                }
+                named_bar_sync(1, kMegaCThreads);
+                if (ctid == 0) atomicAdd(&p.cnt[(base + kPhFinQ) * kCntStride], 1ull);  // (few rows count on it)
+            }
+            // -------------------------------------------------------- attention
             // units alternate between the two warp groups: group h (warps 3..6 / 7..10, named
             // barrier 2 + h) runs the units (gi + i) & 1 == h.  Each warp of a group takes 32 positions
             // of every KV block by itself -- scores, probabilities and output sum stay in its registers
@@ -1750,6 +1772,7 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
         if (S.stall_idx > 0) {
             const int ph = (S.stall_idx - 1) % kPhasesPerLayer;
             if (ph == kPhGU - 1 || (S.small && (ph == kPhQKV || ph == kPhO))) ++S.stall_idx;
+            if (ph == kPhFinQ && !S.small) --S.stall_idx;  // (the attention units' sums wait on the projection)
         }
         S.p_headroom = p.c.kc->eager_softmax ? 0.f : kSoftmaxHeadroom;
         S.abort = (*(volatile int *)&V->err & ERR_WAIT_TIMEOUT) != 0;
