@@ -974,9 +974,10 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
     // `off`: row and column inside a segment, in floats.
     auto part_sum = [&](int2 ct, int t, int off, bool split) -> float4 {
         const int64_t seg = (int64_t)p.rows_cap * kTileN;
-        const int c0 = split ? lane >> 4 : 0, step = split ? 2 : 1;
+        const int c0 = split ? lane >> 4 : 0;
+        const int64_t step = split ? 2 * seg : seg;
         const float *src = p.gpart + (int64_t)(ct.x + c0 + t) * seg + off;
-        int n = (ct.y - ct.x - c0 + step) / step;  // contributors of this lane
+        int n = split ? (ct.y - ct.x - c0 + 2) >> 1 : ct.y - ct.x + 1;  // contributors of this lane
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 1
         while (__any_sync(0xffffffffu, n > 0)) {
@@ -985,7 +986,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
             for (int k = 0; k < 16; ++k) {
                 v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (k < n) v[k] = __ldcg(reinterpret_cast<const float4 *>(src));
-                src += step * seg;
+                src += step;
             }
 #pragma unroll
             for (int k = 0; k < 16; ++k) { s.x += v[k].x; s.y += v[k].y; s.z += v[k].z; s.w += v[k].w; }
@@ -1022,15 +1023,22 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
             // ---------------------------------------------------- residual, next norm input
             // x += sum of the GEMM's partials (x = E[tok] at the start); x_g = x * gn as a blocked
             // hi/lo pair; per (row, 64 features) sum of squares.  Unit = (row, 64 features): lane
-            // % 16 = 4 features; the two halves of the warp split the contributors, then the first
-            // stores x and the hi parts, the second the lo parts.
+            // % 16 = 4 features.  While no warp has more than one unit its two halves split the
+            // contributors, then the first stores x and the hi parts, the second the lo parts; above,
+            // a half warp takes a unit, so that fewer of them follow one another in a warp.  Kernel,
+            // ms with split units -> with half warps: 1.5B 48 rows of 60 positions (one unit) 1.317 ->
+            // 1.332, 64 rows (two) 1.439 -> 1.395, 100 rows 1.806 -> 1.761; 3B 48 rows 2.212 -> 2.147.
             const int which = k == 0 ? kGDown : kGO;
             const uint16_t *gn = k == 2 ? p.mlp_norm + l * d : l < p.layers ? p.attn_norm + l * d : p.final_norm;
             float *ssq = k == 2 ? p.ssqM : p.ssqA;
             if (step > 0) wait_phase(k == 2 ? base + kPhO : base - kPhasesPerLayer + kPhDown);
-            const int d64 = d / 64;
+            const int d64 = d / 64, nu = R * d64;
+            const bool split = small || nu <= nw;
+            const int per = split ? 1 : 2, add = split ? 0 : lane >> 4;  // units of a warp, of which this lane's
 #pragma unroll 1
-            for (int u = gw; u < R * d64; u += nw) {
+            for (int u0 = per * gw; u0 < nu; u0 += per * nw) {
+                const bool own = u0 + add < nu;
+                const int u = own ? u0 + add : u0;
                 const int r = u / d64, h64 = u - r * d64;
                 const int f = h64 * 64 + (lane & 15) * 4;
                 // the norm weights load with the residual and the partials
@@ -1040,7 +1048,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                 if (step == 0) {
                     int tok = p.c.row_tok[r];
                     if (tok < 0 || tok >= p.V) {
-                        if (lane == 0) report_error(err, ERR_BOUNDS);
+                        if ((lane & 15) == 0) report_error(err, ERR_BOUNDS);
                         tok = 0;
                     }
                     const uint2 e = __ldg(reinterpret_cast<const uint2 *>(p.embed + (int64_t)tok * d + f));
@@ -1049,7 +1057,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                 } else {
                     x = __ldcg(reinterpret_cast<const float4 *>(xp));
                     const int t = f / kTileN;
-                    const float4 s = part_sum(contributors(which, t), t, r * kTileN + f - t * kTileN, true);
+                    const float4 s = part_sum(contributors(which, t), t, r * kTileN + f - t * kTileN, split);
                     x.x += s.x; x.y += s.y; x.z += s.z; x.w += s.w;
                 }
                 uint16_t h[4], lo[4];
@@ -1057,21 +1065,22 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                 split_bf16(x.y * bf16_to_f32(gb.x >> 16), h[1], lo[1]);
                 split_bf16(x.z * bf16_to_f32(gb.y & 0xffff), h[2], lo[2]);
                 split_bf16(x.w * bf16_to_f32(gb.y >> 16), h[3], lo[3]);
-                float sq = 0.f;
-                if (lane < 16) {
-                    *reinterpret_cast<float4 *>(xp) = x;
-                    sq = (x.x * x.x + x.y * x.y) + (x.z * x.z + x.w * x.w);
-                }
-                const uint2 w = lane < 16 ? pack4(h) : pack4(lo);
+                const bool first = lane < 16 || !split;  // stores x (and the hi parts)
+                float sq = first ? (x.x * x.x + x.y * x.y) + (x.z * x.z + x.w * x.w) : 0.f;
+                if (first && own) *reinterpret_cast<float4 *>(xp) = x;
+                const uint2 w = first ? pack4(h) : pack4(lo);
                 if (small && l < p.layers) {  // small_k's operand
-                    uint8_t *dst = p.xg + frag_off(r, f, R16c) + (lane < 16 ? 0 : kFragLo);
+                    uint8_t *dst = p.xg + frag_off(r, f, R16c) + (first ? 0 : kFragLo);
                     *reinterpret_cast<uint32_t *>(dst) = w.x;
                     *reinterpret_cast<uint32_t *>(dst + 16) = w.y;
-                } else {
-                    *reinterpret_cast<uint2 *>(p.xg + xblk_off(r, f, R16c) + (lane < 16 ? 0 : kLoOff)) = w;
+                } else if (own) {
+                    uint8_t *dst = p.xg + xblk_off(r, f, R16c);
+                    *reinterpret_cast<uint2 *>(dst + (first ? 0 : kLoOff)) = w;
+                    if (!split) *reinterpret_cast<uint2 *>(dst + kLoOff) = pack4(lo);
                 }
-                sq = warp_sum(sq);
-                if (lane == 0) ssq[h64 * p.rows_cap + r] = sq;
+#pragma unroll
+                for (int o2 = 8; o2 > 0; o2 >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o2);
+                if ((lane & 15) == 0 && first && own) ssq[h64 * p.rows_cap + r] = sq;
             }
             arrive(k == 2 ? base + kPhFinO : base - 1, true);
             if (l == p.layers) break;

@@ -31,6 +31,7 @@ NARROW = _shape("ffn 64", d_model=128, n_heads=4, head_dim=32, ffn=64)
 ODD = _shape("ffn 320")
 WIDE = _shape("ffn 20032", layers=1, ffn=20032)                     # 2,504 units: two passes on some CTAs
 DEEP = _shape("d 2048", layers=2, d_model=2048, n_heads=16, head_dim=128, ffn=448)
+ODD_D = _shape("d 1664", layers=1, d_model=1664, n_heads=4, head_dim=128, ffn=128)  # 26 units of 64: 1,222 at 47 rows
 MANY_HEADS = _shape("32 heads", d_model=512, n_heads=32, n_kv_heads=4, head_dim=128, ffn=128)  # K = 4,096 > d
 MANY_KV = _shape("48 kv heads", layers=2, d_model=128, n_heads=48, n_kv_heads=48, head_dim=32, ffn=64)  # 40 units per SM
 VOCAB_UNITS = _shape("vocab 40064", layers=1, d_model=128, n_heads=4, head_dim=32, ffn=64, vocab=40064)  # 2,504 units
@@ -39,7 +40,7 @@ VOCAB_TILES = _shape("vocab 80000", layers=1, d_model=128, n_heads=4, head_dim=3
 
 @pytest.mark.parametrize("shape,rows", [(NARROW, 1), (NARROW, 9), (NARROW, 128), (ODD, 8), (ODD, 17), (ODD, 33),
                                         (ODD, 65), (WIDE, 2), (WIDE, 32), (WIDE, 64), (DEEP, 1), (DEEP, 16),
-                                        (DEEP, 31), (DEEP, 48), (MANY_HEADS, 3), (MANY_HEADS, 32), (MANY_HEADS, 40),
+                                        (DEEP, 31), (DEEP, 48), (ODD_D, 47), (MANY_HEADS, 3), (MANY_HEADS, 32), (MANY_HEADS, 40),
                                         (MANY_KV, 128), (VOCAB_UNITS, 3), (VOCAB_UNITS, 66),
                                         (VOCAB_TILES, 3), (VOCAB_TILES, 66)],
                          ids=lambda v: getattr(v, "name", v))
