@@ -440,11 +440,11 @@ def run_mine(args):
         "clocks": clocks,
         "wall_s": round(time.time() - t_start, 1),
     }
-    # kernels launched: per decode step the controller, the decode-step kernel and the
-    # sampling/bookkeeping kernel; per round start (or, asynchronous, per decision event) at most
-    # the prefill (embedding + 5 per layer but the last layer's 4) and the KV set-up; per call
-    # the init kernel
-    line["gpu_launches"] = int(3 * dsteps + rounds * (1 + 5 * m.layers - 4 + 1) + args.steps * world)
+    # kernels launched: per decode step the decode-step kernel and the sampling/bookkeeping
+    # kernel; per round start (or, asynchronous, per decision event) the controller and at most
+    # the prefill (embedding, the choice of its GEMM, 5 per layer but the last layer's 1) and the
+    # KV set-up; per call the init kernel and the controller's last run
+    line["gpu_launches"] = int(2 * dsteps + rounds * (1 + 2 + 5 * m.layers - 4 + 1) + 2 * args.steps * world)
     line["committed_per_step"] = groups / world / args.steps
     line["kv_blocks_peak"] = max(o.kv_blocks_peak for o in outs)
     print(json.dumps(line), flush=True)

@@ -240,7 +240,8 @@ SARA_API int sara_profile(sara_handle *h, int32_t kernel, int32_t rows, int32_t 
  *                   iterations (0: only the built-in round bounds).
  *   stall_phase:    -1, or a phase-counter index of the decode-step kernel (0 = embedding,
  *                   1 + 9 l + j = phase j of layer l) whose waits are made to wait for a value
- *                   no launch reaches: they time out after wait_limit_ns.
+ *                   no launch reaches: they time out after wait_limit_ns.  (A counter that this
+ *                   launch has no phase of its own for stands for a neighbour that it waits on.)
  *   eager_softmax:  the decode attention's online softmax takes each KV block's
  *                   probabilities against a running maximum.  0 (default): the maximum is
  *                   re-based only when a probability against it would exceed 2^8, so
