@@ -17,17 +17,17 @@
 //
 // Split-K: a phase's (tile, k-chunk) units are cut into equal contiguous ranges over its
 // CTAs; each CTA stores its fp32 partial tile with plain stores and the consuming phase
-// sums a tile's partials in CTA order (deterministic, no atomics).  The gate / up projection is
-// column-owned instead: each CTA takes 16-feature units with the whole K and applies the SwiGLU
-// in its epilogue (no partials, no finalisation phase).
+// sums a tile's partials in CTA order (deterministic, no atomics).  Gate / up, lm_head and, up to
+// 8 rows, q/k/v and O are column-owned instead: each CTA takes 16-feature units with the whole K
+// and applies what follows in its epilogue (no partials, no finalisation phase).
 //
 // Warp roles (352 threads, 11 warps):
 //   warp 0   W producer: bulk copies of pre-swizzled weight tiles and KV blocks
 //   warp 1   tcgen05 issuer and tensor-memory owner; hands the attention phase's KV tiles
 //            to the compute warp group that runs their unit
 //   warp 2   X producer: activation chunks, after the phase they come from has completed
-//   warps 3..10  compute: GEMM epilogues, attention softmax / merge, residual + RMSNorm +
-//                SwiGLU finalisation, embedding, logits
+//   warps 3..10  compute: GEMM epilogues, attention, residual + RMSNorm finalisation, embedding,
+//                logits
 //
 // Phases of layer l (counter index 1 + 9l + k):
 //   0 QKV   x_g W_qkv^T -> partials        (a subset of the CTAs: few tiles)
