@@ -195,7 +195,6 @@ __global__ void __launch_bounds__(kSplitThreads) attn_split_kernel(AttnSplitPara
             }
         p.out[((int64_t)row * p.H + kvh * G) * HD + e] = f32_to_bf16(acc / L);
     }
-    __syncwarp();
     cluster_sync();  // no CTA leaves while its state is read
 }
 

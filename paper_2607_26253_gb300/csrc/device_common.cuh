@@ -349,14 +349,25 @@ __device__ __forceinline__ void named_bar_sync(int id, int nthreads) {
 }
 
 // Thread-block clusters: this CTA's rank, the barrier over every thread of the cluster (release /
-// acquire), and accesses to the same shared-memory object of another CTA.
+// acquire; converges the warp itself), and accesses to the same shared-memory object of another
+// CTA.  That CTA has to have started: an access comes after a barrier, of which the arrival and
+// the wait may be apart.
 __device__ __forceinline__ uint32_t cluster_rank() {
     uint32_t r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 __device__ __forceinline__ uint32_t cluster_addr(const void *p, uint32_t rank) {
     uint32_t a;

@@ -184,7 +184,6 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 p.y[(int64_t)r * p.nout + unit * kRowsTileM + mrow] = __fadd_rn(s, c);
             }
         }
-        __syncwarp();
         cluster_sync();  // no CTA leaves while its partial tile is read
     }
     tc_fence_before();

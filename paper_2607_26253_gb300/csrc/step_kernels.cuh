@@ -322,6 +322,7 @@ static __global__ void __launch_bounds__(256) sample_rows_kernel(const float *lo
     __shared__ int si[8];
     __shared__ uint32_t cv[kSampleCtas], ci[kSampleCtas];  // (rank 0) the cluster's maxima
     __shared__ volatile float wb[8];                       // each warp's best so far
+    cluster_arrive();  // (waited for before the store into rank 0's shared memory)
     if (threadIdx.x < 8) wb[threadIdx.x] = -INFINITY;
     __syncthreads();
     const int r = blockIdx.x / kSampleCtas, rank = (int)cluster_rank();
@@ -418,6 +419,7 @@ static __global__ void __launch_bounds__(256) sample_rows_kernel(const float *lo
     }
     if ((threadIdx.x & 31) == 0) { sv[threadIdx.x >> 5] = best; si[threadIdx.x >> 5] = bi; }
     __syncthreads();
+    cluster_wait();  // every CTA of the cluster has started
     if (threadIdx.x == 0) {
         for (int w = 1; w < 8; ++w)
             if (sv[w] > best || (sv[w] == best && si[w] < bi)) { best = sv[w]; bi = si[w]; }

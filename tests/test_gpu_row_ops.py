@@ -37,6 +37,22 @@ def test_sampler_vocabulary_edges(pkg, V):
             assert tok[r] == want, (r, tok[r], want, margin)
 
 
+# many rows of few tokens: most CTAs of a cluster have none and reach the join of the maxima at once, while others may
+# not have started
+@pytest.mark.parametrize("V", [1, 3, 40])
+def test_sampler_many_rows_of_few_tokens(pkg, V):
+    rng = np.random.default_rng(V)
+    R = 6000
+    logits = (rng.standard_normal((R, V)) * 2).astype(np.float32)
+    uid, t = np.arange(R, dtype=np.int64), np.zeros(R, np.int32)
+    tok = pkg.sample(_dev(logits), _dev(uid), _dev(t), 4).cpu().numpy()
+    assert tok.min() >= 0 and tok.max() < V
+    for r in range(R if V > 1 else 0):
+        want, margin = o2.sample_token(logits[r], 4, r, 0)
+        if margin > 1e-5:
+            assert tok[r] == want, (r, tok[r], want, margin)
+
+
 def test_sampler_infinities_and_nan(pkg):
     V, R = 4099, 4
     logits = np.full((R, V), -np.inf, np.float32)
