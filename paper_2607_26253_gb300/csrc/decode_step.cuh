@@ -1674,13 +1674,9 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
 #pragma unroll
                         for (int e = 0; e < 4; ++e) o[e] = make_float4(z[4 * e], z[4 * e + 1], z[4 * e + 2], z[4 * e + 3]);
                     }
-                    // Only tokens whose noise could lift them over the best so far are
-                    // evaluated exactly: g(u) increases with u = (top 24 hash bits + 0.5) / 2^24,
-                    // so z_e + g(u_e) > best needs u_e > exp(-exp(-(best - max_e z_e))); the
-                    // cut is taken 1e-3 lower in g and 4 codes lower in the 24-bit u, far
-                    // beyond the rounding of the float evaluation, so no candidate is lost.
-                    // `best` runs over all of this thread's columns; before the first maximum, the
-                    // token of the largest noise stands in for it.
+                    // Only tokens whose noise could lift them to the best so far are evaluated
+                    // exactly (noise_cut).  `best` runs over all of this thread's columns; before the
+                    // first maximum, the sum of the token of the largest noise stands in for it.
                     float low = best;
                     if (best == -INFINITY) {
                         uint32_t most = 0;
@@ -1698,9 +1694,7 @@ __device__ __forceinline__ void mega_compute(const MegaParams &p, MegaSmem &S, u
                     float vmax = z[0];
 #pragma unroll
                     for (int e = 1; e < 16; ++e) vmax = fmaxf(vmax, z[e]);
-                    const float ureq = expf(-expf(-(low - vmax - 1e-3f)));
-                    const float cut = ureq * 16777216.0f - 4.0f;
-                    const uint32_t thr = cut > 0.f ? (uint32_t)cut : 0u;
+                    const uint32_t thr = noise_cut(low, vmax);
                     uint32_t cand = 0;
 #pragma unroll
                     for (int e = 0; e < 16; ++e)

@@ -50,6 +50,17 @@ __device__ __forceinline__ float gumbel_from_hash(uint64_t h) {
     const float u = ((float)(uint32_t)(h >> 40) + 0.5f) * 5.9604644775390625e-08f;  // 2^-24
     return -logf(-logf(u));
 }
+// The smallest top-24-bit code whose noise could lift a value of at most vmax to `best`, a sum value +
+// noise that a token reached.  g(u) increases with u, so a token needs u > exp(-exp(-(best - vmax))).  The
+// cut is taken lower by 1e-3 in g and by 4 codes for the evaluation's own rounding, and by twice the
+// spacing of floats at `best`: there the sums are rounded, so the token that reached it, and others that tie
+// with it (the lowest id wins), may have that much less noise than the difference says.
+// best = -inf, or NaN in between: every code.  (The largest code's noise is infinite.)
+__device__ __forceinline__ uint32_t noise_cut(float best, float vmax) {
+    const float margin = fminf(fmaf(fabsf(best), 2.38418579e-7f, 1e-3f), 3.40282347e38f);  // 2^-22; finite
+    const float cut = expf(-expf(-(best - vmax - margin))) * 16777216.0f - 4.0f;
+    return cut > 0.f ? (uint32_t)cut : 0u;
+}
 
 // ---------------------------------------------------------------------------------------
 __device__ __forceinline__ float bf16_to_f32(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }

@@ -310,8 +310,8 @@ static __global__ void __launch_bounds__(kCtlThreads, 1) teacher_setup_kernel(St
 // Gumbel-max over given fp32 logits (kernel-level entry point): one cluster of kSampleCtas CTAs per
 // row, each a contiguous share of the vocabulary, the row's maximum joined through distributed
 // shared memory.  Bound by instruction issue (a 64-bit hash per token; 51 instructions a token in all),
-// so the noise's logarithms are taken only for tokens that could beat the CTA's best so far (g(u)
-// increases with the hash's top 24 bits; see the lm_head phase for the cut), the hash's input is
+// so the noise's logarithms are taken only for tokens that could reach the CTA's best so far
+// (noise_cut), the hash's input is
 // advanced by additions, and a step's logits load during the one before.  64 rows x 151,936, whole
 // call: 277 us with one CTA per row (64 of 152 SMs) and the noise of every token, 37 us with the
 // bound per warp and all of the first step's tokens evaluated, 26 us now (kernel 35.6 -> 25.0).
@@ -382,9 +382,7 @@ static __global__ void __launch_bounds__(256) sample_rows_kernel(const float *lo
         float vmax = z[0];
 #pragma unroll
         for (int e = 1; e < 8; ++e) vmax = fmaxf(vmax, z[e]);
-        const float ureq = expf(-expf(-(wbest - vmax - 1e-3f)));  // 0 while wbest = -inf; NaN: every token
-        const float cut = ureq * 16777216.0f - 4.0f;
-        const uint32_t thr = cut > 0.f ? (uint32_t)cut : 0u;
+        const uint32_t thr = noise_cut(wbest, vmax);
 #pragma unroll
         for (int e = 0; e < 8; ++e) cand |= (uint32_t)(code[e] >= thr) << e;
         cand &= valid;

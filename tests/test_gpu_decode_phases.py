@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 import synth
-from gpu_util import LOGIT_MAX_ABS, LOGIT_REL_L2, logit_errors
+from gpu_util import LOGIT_MAX_ABS, LOGIT_REL_L2, assert_drawn_by_the_rule, logit_errors
 from oracle import decode as o2
 
 pytestmark = pytest.mark.gpu
@@ -52,6 +52,27 @@ def test_teacher_forced_logits_by_rows_and_widths(pkg, shape, rows):
 @pytest.mark.parametrize("Lp", [30, 62, 126, 254, 638])
 def test_new_position_at_tile_edges(pkg, Lp, rows):
     _check(pkg, ODD, rows, Lp, T=5)
+
+
+# every row of the head is the same large vector: all logits of a position are equal, so large that their sums with the
+# noise are rounded and tie
+@pytest.mark.parametrize("shape,rows", [(NARROW, 3), (NARROW, 40), (VOCAB_TILES, 9)], ids=lambda v: getattr(v, "name", v))
+def test_draws_from_large_logits(pkg, shape, rows):
+    weights = dict(synth.model_weights(shape, 3))
+    base = np.random.default_rng(1).standard_normal(shape.d_model).astype(np.float32) * 1e5
+    weights["lm_head"] = np.ascontiguousarray(np.broadcast_to(synth.f32_to_bf16_bits(base), (shape.vocab, shape.d_model)))
+    Lp, T = 4, 4
+    rng = np.random.default_rng(rows)
+    prompts = rng.integers(0, shape.vocab, size=(rows, Lp)).astype(np.int32)
+    forced = rng.integers(0, shape.vocab, size=(rows, T)).astype(np.int32)
+    uids = np.arange(rows, dtype=np.int64) * 64 + 3
+    cfg = pkg.model_cfg(shape, max_prompts=rows, max_active=rows, max_seqs=rows, max_prompt_len=Lp, max_gen_len=T + 1,
+                        max_k=2)
+    with pkg.Handle(cfg, weights) as h:
+        logits, sampled = h.teacher_force(prompts, forced, uids, sample_seed=9)
+    assert np.abs(logits).min(axis=-1).max() > 1e5
+    clear = sum(assert_drawn_by_the_rule(sampled[i, t], logits[i, t], 9, int(uids[i]), t) for i in range(rows) for t in range(T))
+    assert clear >= rows * T // 2
 
 
 def _check(pkg, shape, rows, Lp, T):

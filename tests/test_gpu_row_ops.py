@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 import synth
+from gpu_util import assert_drawn_by_the_rule
 from oracle import decode as o2
 
 pytestmark = pytest.mark.gpu
@@ -51,6 +52,19 @@ def test_sampler_many_rows_of_few_tokens(pkg, V):
         want, margin = o2.sample_token(logits[r], 4, r, 0)
         if margin > 1e-5:
             assert tok[r] == want, (r, tok[r], want, margin)
+
+
+# logits so large that the sum with the noise is rounded (spacing 0.008 to 0.06), equal or nearly so: the token that
+# bounds the others keeps its place, and ties go to the lowest id
+@pytest.mark.parametrize("V", [512, 40003])
+@pytest.mark.parametrize("mean,std", [(65536.0, 0.0), (65536.0, 1.0), (-65536.0, 1.0), (1e6, 0.0), (1e6, 1.0)])
+def test_sampler_large_logits(pkg, V, mean, std):
+    rng = np.random.default_rng(V)
+    R = 60
+    logits = (mean + std * rng.standard_normal((R, V))).astype(np.float32)
+    tok = pkg.sample(_dev(logits), _dev(np.arange(R, dtype=np.int64)), _dev(np.zeros(R, np.int32)), 5).cpu().numpy()
+    clear = sum(assert_drawn_by_the_rule(tok[r], logits[r], 5, r, 0) for r in range(R))
+    assert clear >= R * 3 // 4
 
 
 def test_sampler_infinities_and_nan(pkg):
