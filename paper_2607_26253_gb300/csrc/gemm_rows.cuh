@@ -173,7 +173,8 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                 float v[kRowsMaxSplit];
 #pragma unroll
                 for (int q = 0; q < kRowsMaxSplit; ++q) v[q] = q < p.split ? ld_cluster_f32(cluster_addr(src, q)) : 0.f;
-                // compensated (Knuth's two-sum): splitting K adds no rounding of its own
+                // compensated (Knuth's two-sum): splitting K adds no rounding of its own; an infinite
+                // or NaN sum has no error term
                 float s = v[0], c = 0.f;
 #pragma unroll
                 for (int q = 1; q < kRowsMaxSplit; ++q) {
@@ -181,7 +182,7 @@ gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
                     c = __fadd_rn(c, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v[q], b)));
                     s = t;
                 }
-                p.y[(int64_t)r * p.nout + unit * kRowsTileM + mrow] = __fadd_rn(s, c);
+                p.y[(int64_t)r * p.nout + unit * kRowsTileM + mrow] = isfinite(s) ? __fadd_rn(s, c) : s;
             }
         }
         cluster_sync();  // no CTA leaves while its partial tile is read

@@ -96,6 +96,26 @@ def test_gemm_splits_and_tile_walks(pkg, R, N, K, static):
     assert (np.abs(Y - xf @ wf.T) <= bound).all()
 
 
+# infinite and NaN activations and sums past the largest float: the same results with K split over a cluster and not
+@pytest.mark.parametrize("N,K", [(128, 128), (256, 1088), (2048, 1536), (40064, 192)])
+def test_gemm_infinities_and_nan(pkg, N, K):
+    import torch
+    rng = np.random.default_rng(N + K)
+    X = torch.from_numpy(rng.standard_normal((6, K)).astype(np.float32)).bfloat16().cuda()
+    W = torch.from_numpy(rng.uniform(0.5, 1.0, (N, K)).astype(np.float32)).bfloat16().cuda()
+    W[1::2] *= -1
+    X[1, 5], X[2, K - 1], X[3, 7], X[3, K - 7], X[4, K // 2] = np.inf, -np.inf, np.inf, np.inf, np.nan
+    X[5] = 3e38  # every partial sum overflows
+    Y = pkg.gemm_bf16(X, W).cpu()
+    sign = torch.ones(N)
+    sign[1::2] = -1
+    want = X[:1].double().cpu() @ W.double().cpu().t()
+    assert torch.allclose(Y[:1].double(), want, rtol=1e-4, atol=1e-3)
+    for r, s in ((1, 1), (2, -1), (3, 1), (5, 1)):
+        assert torch.equal(Y[r], s * sign * np.inf), r
+    assert Y[4].isnan().all()
+
+
 def _attention_ref(q, kv, ctx, n_kv):
     b, H, hd = q.shape
     out = np.zeros((b, H, hd))
