@@ -7,8 +7,10 @@
 //     32 j + 8 t .. + 7 of a position, and the same dims of its head, so the order of the dims
 //     inside a k-step does not matter and no fragment needs rearranging.
 //   - Output: A = P, straight from the score accumulators, B = V, whose 8 x 8 blocks movmatrix
-//     transposes.  Probabilities stay in 32-bit precision: P = hi + lo in fp16, two MMAs, scaled
-//     by 2^8 so that the small ones keep their low bits.
+//     transposes.  Probabilities enter as fp16 pairs, P = hi + lo, two MMAs: 22 bits, and multiples of
+//     2^-33 of the maximum (they are scaled by 2^8).  Against 64 bits the results are as far off as
+//     with fp32 probabilities (their rounding to bf16); infinite values of V are not: 0 for a small
+//     probability, times infinity.  A warp whose sums are not all finite takes them again in fp32.
 // Online softmax per warp; the warps' states meet in shared memory, the CTAs' in distributed
 // shared memory (no workspace, no counters, so no work list from the host either).  26 ragged rows
 // of median context 758, 12 heads / 2 KV heads of 128, whole call with its synchronisation: 46 us;
@@ -56,96 +58,135 @@ __global__ void __launch_bounds__(kSplitThreads) attn_split_kernel(AttnSplitPara
     const uint16_t *kb = p.kv + row * p.kv_stride + (int64_t)kvh * p.cap * HD + 8 * t;
     const uint16_t *vb = kb + (int64_t)p.KVH * p.cap * HD;
     const int nblk = (ctx + 15) >> 4, b0 = rank * nblk / S, b1 = (rank + 1) * nblk / S;
-    float m, l, o[NJ][4][4];
-    // with: the low parts of P take part.  Left out in a second run if a value came out infinite or
-    // NaN: an infinite V element times a zero or negative low part would turn it into NaN.
+    float m = -INFINITY, l = 0.f, o[NJ][4][4];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[j][i][e] = 0.f;
+    // K rows of step b, and its scores: s[h][e], e < 2: head g, position 16 b + 8 h + 2 t + e
+    auto load = [&](int b, int h, const uint16_t *base, uint4 (&r)[NJ]) {
+        const int64_t off = (int64_t)min(b * 16 + 8 * h + g, ctx - 1) * HD;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) r[j] = __ldg(reinterpret_cast<const uint4 *>(base + off + 32 * j));
+    };
+    auto scores = [&](int b, const uint4 (&kr)[2][NJ], float (&s)[2][4]) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[h][e] = 0.f;
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                const uint32_t a0[4] = {q[j].x, 0u, q[j].y, 0u}, a1[4] = {q[j].z, 0u, q[j].w, 0u};
+                mma_f16_16816(s[h], a0, kr[h][j].x, kr[h][j].y);
+                mma_f16_16816(s[h], a1, kr[h][j].z, kr[h][j].w);
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e)
+                s[h][e] = b * 16 + 8 * h + 2 * t + e < ctx ? s[h][e] * p.scale_log2 : -INFINITY;
+        }
+    };
 #pragma unroll 1
-    for (bool with = true;;) {
-        m = -INFINITY;
-        l = 0.f;
+    for (int b = b0 + warp; b < b1; b += kSplitWarps) {
+        uint4 kr[2][NJ], vr[2][NJ];
 #pragma unroll
-        for (int j = 0; j < NJ; ++j)
+        for (int h = 0; h < 2; ++h) {
+            load(b, h, kb, kr[h]);
+            load(b, h, vb, vr[h]);
+            if (b * 16 + 8 * h + g >= ctx) {  // (its probability is 0)
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+                for (int j = 0; j < NJ; ++j) vr[h][j] = make_uint4(0, 0, 0, 0);
+            }
+        }
+        float s[2][4];
+        scores(b, kr, s);
+        float mx = m;
 #pragma unroll
-                for (int e = 0; e < 4; ++e) o[j][i][e] = 0.f;
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) mx = fmaxf(mx, s[h][e]);
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        const float mr = mx == -INFINITY ? 0.f : mx;  // (every score so far is -inf: weights 0)
+        const float alpha = exp2f(m - mr);
+        m = mx;
+        l *= alpha;
+        uint32_t hi[4] = {0u, 0u, 0u, 0u}, lo[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const float p0 = exp2f(s[h][0] - mr + kSplitPScale), p1 = exp2f(s[h][1] - mr + kSplitPScale);
+            l += p0 + p1;
+            hi[2 * h] = pack_half2(p0, p1);
+            const __half2 hh = *reinterpret_cast<const __half2 *>(&hi[2 * h]);
+            lo[2 * h] = pack_half2(p0 - __low2float(hh), p1 - __high2float(hh));
+        }
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+            const uint32_t v0[4] = {vr[0][j].x, vr[0][j].y, vr[0][j].z, vr[0][j].w};
+            const uint32_t v1[4] = {vr[1][j].x, vr[1][j].y, vr[1][j].z, vr[1][j].w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t w0 = movmatrix_trans(v0[i]), w1 = movmatrix_trans(v1[i]);
+                o[j][i][0] *= alpha;
+                o[j][i][1] *= alpha;
+                mma_f16_16816(o[j][i], hi, w0, w1);
+                mma_f16_16816(o[j][i], lo, w0, w1);
+            }
+        }
+    }
+    bool fin = true;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) fin = fin && isfinite(o[j][i][0]) && isfinite(o[j][i][1]);
+    fin = __all_sync(0xffffffffu, fin);
+    if (!fin) {
+        // the warp's sums of P V once more, in fp32: each step's probabilities against the final maximum by way
+        // of the room of the sums (head, position), dims NJ lane .. of every head in this lane
+        float acc[8][NJ];
+#pragma unroll
+        for (int h = 0; h < 8; ++h)
+#pragma unroll
+            for (int i = 0; i < NJ; ++i) acc[h][i] = 0.f;
+        const float mr = m == -INFINITY ? 0.f : m;
 #pragma unroll 1
         for (int b = b0 + warp; b < b1; b += kSplitWarps) {
-            uint4 kr[2][NJ], vr[2][NJ];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int pos = b * 16 + 8 * h + g;
-                const int64_t off = (int64_t)min(pos, ctx - 1) * HD;
-#pragma unroll
-                for (int j = 0; j < NJ; ++j) {
-                    kr[h][j] = __ldg(reinterpret_cast<const uint4 *>(kb + off + 32 * j));
-                    vr[h][j] = pos < ctx ? __ldg(reinterpret_cast<const uint4 *>(vb + off + 32 * j)) : make_uint4(0, 0, 0, 0);
-                }
-            }
+            uint4 kr[2][NJ];
+            load(b, 0, kb, kr[0]);
+            load(b, 1, kb, kr[1]);
             float s[2][4];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-#pragma unroll
-                for (int e = 0; e < 4; ++e) s[h][e] = 0.f;
-#pragma unroll
-                for (int j = 0; j < NJ; ++j) {
-                    const uint32_t a0[4] = {q[j].x, 0u, q[j].y, 0u}, a1[4] = {q[j].z, 0u, q[j].w, 0u};
-                    mma_f16_16816(s[h], a0, kr[h][j].x, kr[h][j].y);
-                    mma_f16_16816(s[h], a1, kr[h][j].z, kr[h][j].w);
-                }
-            }
-            // s[h][e], e < 2: head g, position 16 b + 8 h + 2 t + e
-            float mx = m;
+            scores(b, kr, s);
+            __syncwarp();
 #pragma unroll
             for (int h = 0; h < 2; ++h)
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    s[h][e] = b * 16 + 8 * h + 2 * t + e < ctx ? s[h][e] * p.scale_log2 : -INFINITY;
-                    mx = fmaxf(mx, s[h][e]);
-                }
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-            const float mr = mx == -INFINITY ? 0.f : mx;  // (every score so far is -inf: weights 0)
-            const float alpha = exp2f(m - mr);
-            m = mx;
-            l *= alpha;
-            uint32_t hi[4] = {0u, 0u, 0u, 0u}, lo[4] = {0u, 0u, 0u, 0u};
+                for (int e = 0; e < 2; ++e) s_o[warp][g][8 * h + 2 * t + e] = exp2f(s[h][e] - mr + kSplitPScale);
+            __syncwarp();
+#pragma unroll 1
+            for (int x = 0; x < min(16, ctx - 16 * b); ++x) {
+                const uint16_t *v = vb - 8 * t + (int64_t)(16 * b + x) * HD + NJ * lane;
+                float f[NJ];
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float p0 = exp2f(s[h][0] - mr + kSplitPScale), p1 = exp2f(s[h][1] - mr + kSplitPScale);
-                l += p0 + p1;
-                hi[2 * h] = pack_half2(p0, p1);
-                const __half2 hh = *reinterpret_cast<const __half2 *>(&hi[2 * h]);
-                lo[2 * h] = pack_half2(p0 - __low2float(hh), p1 - __high2float(hh));
-            }
+                for (int i = 0; i < NJ; ++i) f[i] = __half2float(__ushort_as_half(__ldg(v + i)));
 #pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-                const uint32_t v0[4] = {vr[0][j].x, vr[0][j].y, vr[0][j].z, vr[0][j].w};
-                const uint32_t v1[4] = {vr[1][j].x, vr[1][j].y, vr[1][j].z, vr[1][j].w};
+                for (int h = 0; h < 8; ++h)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const uint32_t w0 = movmatrix_trans(v0[i]), w1 = movmatrix_trans(v1[i]);
-                    o[j][i][0] *= alpha;
-                    o[j][i][1] *= alpha;
-                    mma_f16_16816(o[j][i], hi, w0, w1);
-                    if (with) mma_f16_16816(o[j][i], lo, w0, w1);
-                }
+                    for (int i = 0; i < NJ; ++i) acc[h][i] = fmaf(s_o[warp][h][x], f[i], acc[h][i]);
             }
         }
-        bool fin = true;
+        __syncwarp();
 #pragma unroll
-        for (int j = 0; j < NJ; ++j)
+        for (int h = 0; h < 8; ++h)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) fin = fin && isfinite(o[j][i][0]) && isfinite(o[j][i][1]);
-        if (!with || __all_sync(0xffffffffu, fin)) break;
-        with = false;
+            for (int i = 0; i < NJ; ++i) s_o[warp][h][NJ * lane + i] = acc[h][i];
     }
     // o[j][i][e], e < 2: head g, dim 32 j + 8 t + 2 i + e
     l += __shfl_xor_sync(0xffffffffu, l, 1);
     l += __shfl_xor_sync(0xffffffffu, l, 2);
     if (t == 0) { s_m[warp][g] = m; s_l[warp][g] = l; }
 #pragma unroll
-    for (int j = 0; j < NJ; ++j) {
+    for (int j = 0; j < NJ && fin; ++j) {
         float4 *dst = reinterpret_cast<float4 *>(&s_o[warp][g][32 * j + 8 * t]);
         dst[0] = make_float4(o[j][0][0], o[j][0][1], o[j][1][0], o[j][1][1]);
         dst[1] = make_float4(o[j][2][0], o[j][2][1], o[j][3][0], o[j][3][1]);

@@ -178,6 +178,33 @@ def test_attention_infinite_value(pkg):
     assert np.all(np.abs(out - want)[mask] <= 2.0 ** -8 * np.abs(want)[mask] + 2e-3)
 
 
+def test_attention_infinite_value_of_small_probability(pkg):
+    # position 0 outweighs the others by e^40: their probabilities (2^-58) are far below what fp16 holds
+    q = np.ones((1, 8, 128), np.float16)
+    kv = np.zeros((1, 2, 1, 303, 128), np.float16)
+    kv[0, 0, 0, 0], kv[0, 1] = 40 / np.sqrt(128), np.random.default_rng(5).standard_normal((1, 303, 128))
+    want = kv[0, 1, 0, 0].astype(np.float32)
+    kv[0, 1, 0, 3, 17], kv[0, 1, 0, 299, 90] = np.inf, -np.inf  # in the same warp's step, in another CTA
+    out = pkg.attention_decode(_dev(q), _dev(kv), _dev(np.array([300], np.int32)), 1, 303).float().cpu().numpy()[0]
+    assert np.all(out[:, 17] == np.inf) and np.all(out[:, 90] == -np.inf)
+    mask = np.isfinite(out[0])
+    assert mask.sum() == 126 and np.all(np.abs(out - want)[:, mask] <= 2.0 ** -8 * np.abs(want)[mask])
+
+
+def test_attention_infinite_value_beside_cancelling_ones(pkg):
+    # values of +-1000 under nearly equal probabilities cancel to ~0.06: the other dims of a row with an infinite value
+    # need all of the probabilities' 24 bits (1000 * 2^-24 of each of 300, averaged: below 1e-5)
+    q, kv, ctx, cap = _attention_case(np.random.default_rng(6), 6, 1, 128, [300])
+    q *= np.float16(0.001)
+    kv[0, 1] = np.where(np.arange(cap) % 2 == 0, 1000, -1000).astype(np.float16)[None, :, None]
+    want = _attention_ref(q.astype(np.float64), kv.astype(np.float64), ctx, 1)
+    kv[0, 1, 0, 7, 5] = np.inf
+    out = pkg.attention_decode(_dev(q), _dev(kv), _dev(ctx), 1, cap).float().cpu().numpy()
+    assert np.all(out[0, :, 5] == np.inf)
+    mask = np.arange(128) != 5
+    assert np.all(np.abs(out - want)[..., mask] <= 2.0 ** -8 * np.abs(want)[..., mask] + 1e-4)
+
+
 @pytest.mark.parametrize("bad", [0, -1, 301])
 def test_attention_context_out_of_range_refused(pkg, bad):
     q, kv, ctx, cap = _attention_case(np.random.default_rng(3), 4, 2, 32, [300, 20, 5])
