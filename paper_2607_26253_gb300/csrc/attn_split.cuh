@@ -31,11 +31,21 @@ struct AttnSplitParams {
     const uint16_t *kv;  // sequence i at kv + i * kv_stride: [2][KVH][cap][hd] fp16
     const int *ctx;      // [b]
     uint16_t *out;       // [b][H][hd] bf16
-    int *bad;            // [b] 1: ctx out of range (the row is skipped)
+    int *bad;            // whether a row's ctx is out of range: then nothing is written
     int64_t kv_stride;
     int H, KVH, cap, max_ctx;
     float scale_log2;
 };
+
+// The verdict on the rows' contexts.  A kernel of its own, so that every row's counts before the first
+// result is written; the attention runs beside it and waits for it only there.
+static __global__ void __launch_bounds__(1024) attn_ctx_check_kernel(const int *ctx, int b, int max_ctx, int *bad) {
+    pdl_allow_dependents();
+    bool any = false;
+    for (int i = threadIdx.x; i < b; i += blockDim.x) any = any || ctx[i] < 1 || ctx[i] > max_ctx;
+    any = __syncthreads_or(any);
+    if (threadIdx.x == 0) *bad = any ? 1 : 0;
+}
 
 template <int HD>
 __global__ void __launch_bounds__(kSplitThreads) attn_split_kernel(AttnSplitParams p) {
@@ -46,9 +56,7 @@ __global__ void __launch_bounds__(kSplitThreads) attn_split_kernel(AttnSplitPara
     const int kvh = blockIdx.y, row = blockIdx.z, rank = (int)cluster_rank(), S = (int)gridDim.x;
     const int G = p.H / p.KVH;
     const int ctx = p.ctx[row];
-    const bool bad = ctx < 1 || ctx > p.max_ctx;
-    if (rank == 0 && kvh == 0 && threadIdx.x == 0) p.bad[row] = bad ? 1 : 0;
-    if (bad) return;  // (every CTA of the cluster has the same row)
+    if (ctx < 1 || ctx > p.max_ctx) return;  // (every CTA of the cluster has the same row)
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     uint4 q[NJ];
 #pragma unroll
@@ -192,6 +200,8 @@ __global__ void __launch_bounds__(kSplitThreads) attn_split_kernel(AttnSplitPara
         dst[1] = make_float4(o[j][2][0], o[j][2][1], o[j][3][0], o[j][3][1]);
     }
     __syncthreads();
+    pdl_wait_prior_grids();
+    if (*reinterpret_cast<volatile int *>(p.bad)) return;
     const int per = G * HD;
     for (int e = threadIdx.x; e < per; e += kSplitThreads) {
         const int h = e / HD, dd = e % HD;
@@ -244,10 +254,12 @@ __global__ void __launch_bounds__(kSplitThreads) attn_split_kernel(AttnSplitPara
 inline void launch_attn_split(cudaStream_t s, int sms, int b, int hd, const AttnSplitParams &p) {
     int split = 1;
     while (split < kSplitMaxCtas && p.max_ctx > 64 * split && (int64_t)b * p.KVH * split < 4 * sms) split *= 2;
+    attn_ctx_check_kernel<<<1, 1024, 0, s>>>(p.ctx, b, p.max_ctx, p.bad);
+    CK(cudaGetLastError());
     const dim3 grid((unsigned)split, (unsigned)p.KVH, (unsigned)b);
-    if (hd == 32) launch_cluster(s, grid, dim3(kSplitThreads), 0, (unsigned)split, attn_split_kernel<32>, p);
-    else if (hd == 64) launch_cluster(s, grid, dim3(kSplitThreads), 0, (unsigned)split, attn_split_kernel<64>, p);
-    else launch_cluster(s, grid, dim3(kSplitThreads), 0, (unsigned)split, attn_split_kernel<128>, p);
+    if (hd == 32) launch_cluster(s, true, grid, dim3(kSplitThreads), 0, (unsigned)split, attn_split_kernel<32>, p);
+    else if (hd == 64) launch_cluster(s, true, grid, dim3(kSplitThreads), 0, (unsigned)split, attn_split_kernel<64>, p);
+    else launch_cluster(s, true, grid, dim3(kSplitThreads), 0, (unsigned)split, attn_split_kernel<128>, p);
 }
 
 }  // namespace sara

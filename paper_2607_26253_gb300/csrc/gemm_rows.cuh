@@ -210,7 +210,7 @@ inline void launch_gemm_rows(cudaStream_t s, int sms, const uint16_t *X, const u
     const size_t smem = 1024 + (size_t)p.stages * stage;
     const CUtensorMap tw = make_tmap_bf16(W, K, nout, kRowsTileK, kRowsTileM);
     const CUtensorMap tx = make_tmap_bf16(X, K, R, kRowsTileK, kRowsBox);
-    launch_cluster(s, dim3((unsigned)grid), dim3(kRowsThreads), smem, (unsigned)p.split, gemm_rows_kernel, tw, tx, p);
+    launch_cluster(s, false, dim3((unsigned)grid), dim3(kRowsThreads), smem, (unsigned)p.split, gemm_rows_kernel, tw, tx, p);
 }
 
 // SM count of the current device, its kernel attributes set (looked up once per device).

@@ -55,20 +55,24 @@ inline CUtensorMap make_tmap_bf16(const void *base, int inner, int outer, int bo
     return tm;
 }
 
-// Launch with thread-block clusters of `cluster` CTAs along x.
+// Launch with thread-block clusters of `cluster` CTAs along x.  pdl: the kernel may start before the
+// preceding one on the stream has completed (it waits for that itself).
 template <typename Kern, typename... Args>
-inline void launch_cluster(cudaStream_t s, dim3 grid, dim3 block, size_t smem, unsigned cluster, Kern kern, Args... args) {
+inline void launch_cluster(cudaStream_t s, bool pdl, dim3 grid, dim3 block, size_t smem, unsigned cluster, Kern kern,
+                           Args... args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = cluster;
-    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 2 : 1;
     CK(cudaLaunchKernelEx(&cfg, kern, args...));
 }
 

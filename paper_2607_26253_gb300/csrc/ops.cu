@@ -151,7 +151,7 @@ int sara_attention_decode(const uint16_t *q, const uint16_t *kv, int64_t kv_stri
             a.kv = kv;
             a.ctx = ctx;
             a.out = out;
-            a.bad = reinterpret_cast<int *>(workspace);  // (b ints: far below the workspace's size)
+            a.bad = reinterpret_cast<int *>(workspace);
             a.kv_stride = kv_stride;
             a.H = n_heads;
             a.KVH = n_kv_heads;
@@ -159,11 +159,10 @@ int sara_attention_decode(const uint16_t *q, const uint16_t *kv, int64_t kv_stri
             a.max_ctx = max_ctx;
             a.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)head_dim));
             launch_attn_split(s, sms, b, head_dim, a);
-            std::vector<int> bad(b);
-            CK(cudaMemcpyAsync(bad.data(), a.bad, b * sizeof(int), cudaMemcpyDeviceToHost, s));
+            int bad = 0;
+            CK(cudaMemcpyAsync(&bad, a.bad, sizeof(int), cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
-            for (int i = 0; i < b; ++i)
-                if (bad[i]) throw SaraError(SARA_EINVAL, "ctx out of range");
+            if (bad) throw SaraError(SARA_EINVAL, "ctx out of range");
             return;
         }
         const size_t splits = (size_t)(max_ctx + 127) / 128;
@@ -227,7 +226,7 @@ int sara_sample(const float *logits, int32_t R, int32_t V, uint64_t sample_seed,
                 int32_t *token, void *stream) {
     if (!logits || !uid || !t || !token || R < 1 || V < 1) return SARA_EINVAL;
     return op_guard([&] {
-        launch_cluster(static_cast<cudaStream_t>(stream), dim3((unsigned)R * kSampleCtas), dim3(256), 0, kSampleCtas,
+        launch_cluster(static_cast<cudaStream_t>(stream), false, dim3((unsigned)R * kSampleCtas), dim3(256), 0, kSampleCtas,
                        sample_rows_kernel, logits, (int)V, sample_seed, uid, t, (int *)token);
     });
 }

@@ -212,3 +212,23 @@ def test_attention_context_out_of_range_refused(pkg, bad):
     with pytest.raises(pkg.SaraError) as e:
         pkg.attention_decode(_dev(q), _dev(kv), _dev(ctx), 2, cap, max_ctx=300)
     assert e.value.code == pkg.SARA_EINVAL
+
+
+@pytest.mark.parametrize("where", [0, 1700, 2999])
+def test_attention_refused_call_writes_nothing(pkg, where):
+    import torch
+    b, H, KVH, hd, cap = 3000, 4, 2, 32, 70
+    q = torch.ones((b, H, hd), dtype=torch.float16, device="cuda")
+    kv = torch.ones((b, 2, KVH, cap, hd), dtype=torch.float16, device="cuda")
+    ctx = torch.full((b,), 64, dtype=torch.int32, device="cuda")
+    ctx[where] = 71
+    out = torch.full((b, H, hd), 7.0, dtype=torch.bfloat16, device="cuda")
+    ws = torch.empty(pkg.load().sara_attention_workspace_bytes(b, H, hd, cap), dtype=torch.uint8, device="cuda")
+
+    def call():
+        return pkg.load().sara_attention_decode(q.data_ptr(), kv.data_ptr(), kv.stride(0), ctx.data_ptr(), out.data_ptr(), b,
+                                                H, KVH, hd, cap, cap, ws.data_ptr(), ws.numel(),
+                                                torch.cuda.current_stream().cuda_stream)
+    assert call() == pkg.SARA_EINVAL and bool((out == 7).all())
+    ctx[where] = 64
+    assert call() == pkg.SARA_OK and bool((out == 1).all())
