@@ -93,6 +93,8 @@ struct sara_handle {
     // workspaces
     unsigned long long *gemm_acc = nullptr;
     int *gemm_cnt = nullptr;
+    size_t gemm_cnt_n = 0;
+    bool finished = true;  // the last call ran to its end: the GEMM sums and counters are back at zero
     float *big_part = nullptr;  // partial tiles of the many-row prefill GEMM, two per SM
     float *attn_part = nullptr;
     int *attn_cnt = nullptr;
@@ -389,7 +391,9 @@ void enqueue_prefill_embed(sara_handle &h, cudaStream_t s) {
 void enqueue_prefill_layers(sara_handle &h, cudaStream_t s, bool pdl, bool big) {
     const sara_model_cfg &m = h.cfg;
     for (int l = 0; l < m.layers; ++l) {
-        enqueue_prefill_kernel(h, s, K_QKV, l, pdl, big);
+        // (the first not beside the embedding, which may still report a token out of range: the GEMM's CTAs skip
+        // their work on an error, all or none)
+        enqueue_prefill_kernel(h, s, K_QKV, l, pdl && l > 0, big);
         if (l == m.layers - 1) break;
         enqueue_prefill_kernel(h, s, K_ATTN, l, pdl, big);
         enqueue_prefill_kernel(h, s, K_OPROJ, l, pdl, big);
@@ -621,12 +625,18 @@ void alloc_decode(sara_handle &h) {
     h.phase_cnt = h.mem.alloc<unsigned long long>(((size_t)h.n_phase_cnt + 1) * kCntStride);
 }
 
-// Phase counters and split counters back to zero (start of every call: a step that failed
-// part-way may have left them anywhere).
+// Phase counters and split counters back to zero (start of every call: a step that failed part-way may
+// have left them anywhere); after a call that did not finish also the prefill GEMMs' sums and tile
+// counters, which a kernel leaves at zero only if all of its CTAs ran.
 void reset_decode_state(sara_handle &h, cudaStream_t s) {
     const sara_model_cfg &m = h.cfg;
     CK(cudaMemsetAsync(h.phase_cnt, 0, ((size_t)h.n_phase_cnt + 1) * kCntStride * 8, s));
     CK(cudaMemsetAsync(h.attn_cnt, 0, (size_t)m.max_seqs * m.n_kv_heads * 4, s));
+    if (!h.finished) {
+        CK(cudaMemsetAsync(h.gemm_acc, 0, (size_t)h.sms * kTileR * kTileM * sizeof(unsigned long long), s));
+        CK(cudaMemsetAsync(h.gemm_cnt, 0, h.gemm_cnt_n * sizeof(int), s));
+    }
+    h.finished = false;
 }
 
 void make_tensor_maps(sara_handle &h) {
@@ -786,7 +796,8 @@ void create_impl(sara_handle &h, const sara_model_cfg *cfgp, const sara_weights 
         h.big_part = h.mem.alloc<float>((size_t)2 * h.sms * kBigPartFloats, false);
         h.gemm_acc = h.mem.alloc<unsigned long long>((size_t)h.sms * kTileR * kTileM);
         const int max_m = std::max({(m.n_heads + 2 * KVH) * hd, d, 2 * m.ffn, m.vocab}) / 128;
-        h.gemm_cnt = h.mem.alloc<int>((size_t)max_m * ((h.pre_cap + kTileR - 1) / kTileR + 1));
+        h.gemm_cnt_n = (size_t)max_m * ((h.pre_cap + kTileR - 1) / kTileR + 1);
+        h.gemm_cnt = h.mem.alloc<int>(h.gemm_cnt_n);
         const int Gq = m.n_heads / KVH;
         h.attn_part = h.mem.alloc<float>((size_t)h.att_cap * KVH * Gq * (hd + 2), false);
         h.attn_cnt = h.mem.alloc<int>((size_t)S * KVH);
@@ -808,7 +819,8 @@ void create_impl(sara_handle &h, const sara_model_cfg *cfgp, const sara_weights 
     CK(cudaStreamSynchronize(h.stream));
 }
 
-void check_step_error(const StepVars &v) {
+void check_step_error(sara_handle &h, const StepVars &v) {
+    h.finished = v.err == 0;
     if (v.err & ERR_WAIT_TIMEOUT) throw SaraError(SARA_ETIMEOUT, "a bounded device wait timed out");
     if (v.err & ERR_ITER_BOUND) throw SaraError(SARA_ETIMEOUT, "the step exceeded its iteration bound");
     if (v.err & ERR_CAPACITY) throw SaraError(SARA_ENOMEM, "a round exceeded the handle's capacities");
@@ -923,7 +935,7 @@ void collect_impl(sara_handle &h, const sara_prompts *pr, int64_t N, int32_t k, 
             CK(cudaMemcpyAsync(out->tokens, h.gen_tok, (size_t)P * k * m.max_gen_len * 4, kout, s));
     }
     CK(cudaStreamSynchronize(s));
-    check_step_error(v);
+    check_step_error(h, v);
     float ms = 0.f;
     CK(cudaEventElapsedTime(&ms, h.ev0, h.ev1));
     out->rollouts = v.used;
@@ -1003,7 +1015,7 @@ void teacher_impl(sara_handle &h, int n, int Lp, const int32_t *prompts, int T, 
     StepVars v{};
     CK(cudaMemcpyAsync(&v, h.vars, sizeof(v), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
-    check_step_error(v);
+    check_step_error(h, v);
     if (v.live != 0 || v.exec_steps != T) throw SaraError(SARA_EDEVICE, "teacher forcing ran an unexpected number of steps");
 }
 
@@ -1148,7 +1160,7 @@ void profile_impl(sara_handle &h, int which, int rows, int ctx, int iters, doubl
     float t = 0.f;
     CK(cudaEventElapsedTime(&t, h.ev0, h.ev1));
     CK(cudaMemcpy(&v, h.vars, sizeof(v), cudaMemcpyDeviceToHost));
-    check_step_error(v);
+    check_step_error(h, v);
     *ms = (double)t / iters;
 #ifdef SARA_STAMPS
     if (which == 1) print_stamps(h, rows, ctx);

@@ -6,6 +6,7 @@ call return SARA_ETIMEOUT within the wait limit, and a bound on the step loop's 
 must end the loop with SARA_ETIMEOUT; in both cases the handle must stay usable, i.e. the next
 call with the default limits reproduces the oracle's schedule bit-exactly.
 """
+import ctypes
 import time
 
 import numpy as np
@@ -131,3 +132,38 @@ def test_kv_pool_exhaustion_and_exact_fit(pkg):
         for j in range(int(out.n[q])):
             L = int(si.lengths[q, j])
             assert np.array_equal(out.tokens[q, j, :L], ref.tokens[q, j, :L])
+
+
+@pytest.mark.parametrize("rows,Lp", [(128, 250), (2, 12)])  # the many-row and the few-row prefill GEMM
+def test_bad_prompt_token_leaves_no_trace(pkg, rows, Lp):
+    """Prompts on the device are not checked before they run: a token out of range ends the call with an error, and the
+    next call on the same handle gives what a fresh handle gives, bit for bit."""
+    import torch
+    shape = synth.ModelShape("d 512", layers=3, d_model=512, n_heads=8, n_kv_heads=2, head_dim=64, ffn=1280, vocab=640)
+    weights = synth.model_weights(shape, 3)
+    T = 2
+    g = torch.Generator(device="cuda").manual_seed(1)
+    prompts = torch.randint(0, shape.vocab, (rows, Lp), generator=g, device="cuda", dtype=torch.int32)
+    forced = torch.randint(0, shape.vocab, (rows, T), generator=g, device="cuda", dtype=torch.int32)
+    uid = torch.arange(rows, dtype=torch.int64, device="cuda")
+    cfg = pkg.model_cfg(shape, max_prompts=rows, max_active=rows, max_seqs=rows, max_prompt_len=Lp, max_gen_len=T + 1,
+                        max_k=2)
+
+    def call(h, p):
+        logits = torch.zeros((rows, T, shape.vocab), device="cuda")
+        ptr = [ctypes.c_void_p(x.data_ptr()) for x in (p, forced, uid, logits)]
+        torch.cuda.synchronize()
+        rc = pkg.load().sara_teacher_force(h._h, rows, Lp, ptr[0], T, ptr[1], ptr[2], 9, ptr[3], None, 1)
+        return rc, logits
+
+    with pkg.Handle(cfg, weights) as h:
+        rc, want = call(h, prompts)
+        assert rc == pkg.SARA_OK
+    with pkg.Handle(cfg, weights) as h:
+        for r in np.linspace(0, rows - 1, min(rows, 12)).astype(int):
+            for value in (shape.vocab, -1):
+                p = prompts.clone()
+                p[r, Lp - 2] = value
+                assert call(h, p)[0] == pkg.SARA_EINVAL
+                rc, got = call(h, prompts)
+                assert rc == pkg.SARA_OK and torch.equal(got, want), (r, value)
