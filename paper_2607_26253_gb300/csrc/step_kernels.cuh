@@ -327,9 +327,11 @@ static __global__ void __launch_bounds__(256) sample_rows_kernel(const float *lo
     __syncthreads();
     const int r = blockIdx.x / kSampleCtas, rank = (int)cluster_rank();
     const uint64_t rs = sampler_row_seed(sample_seed, uid[r], t[r]);
-    const float *row = logits + (int64_t)r * V;
-    const int per = ((V + kSampleCtas - 1) / kSampleCtas + 3) & ~3;
-    const int v1 = min(V, (rank + 1) * per);
+    // this CTA's share: n tokens from tok0 on (in 32 bits only what stays below 2^28 or V)
+    const int per = ((V - 1) / kSampleCtas + 4) & ~3;
+    const int64_t tok0 = (int64_t)rank * per;
+    const int n = (int)max((int64_t)0, min((int64_t)V - tok0, (int64_t)per));
+    const float *row = logits + (int64_t)r * V + tok0;
     const bool vec = (reinterpret_cast<uintptr_t>(row) & 15) == 0;
     float best = -INFINITY, wbest = -INFINITY;  // this thread's, and the warp's as of the last step
     int bi = 0x7fffffff;
@@ -339,34 +341,34 @@ static __global__ void __launch_bounds__(256) sample_rows_kernel(const float *lo
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int v = b + q * 1024 + (int)threadIdx.x * 4;
-            if (vec && v + 3 < v1) {
+            if (vec && v + 3 < n) {
                 const float4 x = __ldg(reinterpret_cast<const float4 *>(row + v));
                 y[4 * q] = x.x; y[4 * q + 1] = x.y; y[4 * q + 2] = x.z; y[4 * q + 3] = x.w;
             } else {
 #pragma unroll
-                for (int e = 0; e < 4; ++e) y[4 * q + e] = v + e < v1 ? __ldg(row + v + e) : -INFINITY;
+                for (int e = 0; e < 4; ++e) y[4 * q + e] = v + e < n ? __ldg(row + v + e) : -INFINITY;
             }
         }
     };
     float next[8];
-    load(rank * per, next);
+    load(0, next);
 #pragma unroll 1
-    for (int b = rank * per; b < v1; b += 2048) {
+    for (int b = 0; b < n; b += 2048) {
         float z[8];
         uint32_t cand = 0;
 #pragma unroll
         for (int e = 0; e < 8; ++e) z[e] = next[e];
-        if (v1 - b > 2048) load(b + 2048, next);  // (in flight during this step)
+        if (n - b > 2048) load(b + 2048, next);  // (in flight during this step)
         // the hash's input is linear in the token: one product per four of them
         uint32_t code[8];  // the hash's top 24 bits
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-            const int v = b + q * 1024 + (int)threadIdx.x * 4;
-            const uint64_t x = rs + (uint64_t)(v + 1) * kSplitmixGamma;
+            const uint64_t v = (uint64_t)tok0 + (uint32_t)(b + q * 1024) + threadIdx.x * 4;
+            const uint64_t x = rs + (v + 1) * kSplitmixGamma;
 #pragma unroll
             for (int e = 0; e < 4; ++e) code[4 * q + e] = (uint32_t)(mix64(x + (uint64_t)e * kSplitmixGamma) >> 40);
         }
-        const int n0 = v1 - b - (int)threadIdx.x * 4, n1 = n0 - 1024;  // this thread's tokens of each four
+        const int n0 = n - b - (int)threadIdx.x * 4, n1 = n0 - 1024;  // this thread's tokens of each four
         const uint32_t valid = (n0 >= 4 ? 0xfu : n0 > 0 ? (1u << n0) - 1 : 0u) | (n1 >= 4 ? 0xf0u : n1 > 0 ? (16u << n1) - 16 : 0u);
         if (first) {  // before the first maximum, the warp's best of the tokens of largest noise stands in for it
             first = false;
@@ -397,7 +399,7 @@ static __global__ void __launch_bounds__(256) sample_rows_kernel(const float *lo
                 ze = (i == e) ? z[i] : ze;
                 k = (i == e) ? code[i] : k;
             }
-            const int v = b + (e >> 2) * 1024 + (int)threadIdx.x * 4 + (e & 3);
+            const int v = (int)tok0 + b + (e >> 2) * 1024 + (int)threadIdx.x * 4 + (e & 3);
             ze = __fadd_rn(ze, gumbel_from_hash((uint64_t)k << 40));  // (the noise is of the top 24 bits)
             if (ze > best) { best = ze; bi = v; }
         }

@@ -38,6 +38,19 @@ def test_sampler_vocabulary_edges(pkg, V):
             assert tok[r] == want, (r, tok[r], want, margin)
 
 
+# the largest vocabulary whose token ids are 32-bit: shares and their steps end within 2,048 of 2^31
+@pytest.mark.parametrize("V", [2 ** 31 - 1, 2 ** 31 - 900])
+def test_sampler_largest_vocabulary(pkg, V):
+    import torch
+    per = (-(-V // 8) + 3) // 4 * 4
+    logits = torch.full((1, V), -np.inf, device="cuda")
+    one = torch.ones(1, dtype=torch.int64, device="cuda")
+    for v in (0, per - 1, 7 * per, V - 1):
+        logits[0, v] = 0
+        assert int(pkg.sample(logits, one, one.int(), 4)) == v
+        logits[0, v] = -np.inf
+
+
 # many rows of few tokens: most CTAs of a cluster have none and reach the join of the maxima at once, while others may
 # not have started
 @pytest.mark.parametrize("V", [1, 3, 40])
