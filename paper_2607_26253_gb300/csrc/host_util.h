@@ -55,8 +55,8 @@ inline CUtensorMap make_tmap_bf16(const void *base, int inner, int outer, int bo
     return tm;
 }
 
-// Launch with thread-block clusters of `cluster` CTAs along x.  pdl: the kernel may start before the
-// preceding one on the stream has completed (it waits for that itself).
+// Launch with thread-block clusters of `cluster` CTAs along x (1: none).  pdl: the kernel may start before
+// the preceding one on the stream has completed (it waits for that itself).
 template <typename Kern, typename... Args>
 inline void launch_cluster(cudaStream_t s, bool pdl, dim3 grid, dim3 block, size_t smem, unsigned cluster, Kern kern,
                            Args... args) {
@@ -66,13 +66,18 @@ inline void launch_cluster(cudaStream_t s, bool pdl, dim3 grid, dim3 block, size
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2] = {};
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = cluster;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 2 : 1;
+    if (cluster > 1) {
+        cudaLaunchAttribute &a = attr[cfg.numAttrs++];
+        a.id = cudaLaunchAttributeClusterDimension;
+        a.val.clusterDim.x = cluster;
+        a.val.clusterDim.y = a.val.clusterDim.z = 1;
+    }
+    if (pdl) {
+        cudaLaunchAttribute &a = attr[cfg.numAttrs++];
+        a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        a.val.programmaticStreamSerializationAllowed = 1;
+    }
     CK(cudaLaunchKernelEx(&cfg, kern, args...));
 }
 

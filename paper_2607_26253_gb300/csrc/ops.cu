@@ -226,8 +226,15 @@ int sara_sample(const float *logits, int32_t R, int32_t V, uint64_t sample_seed,
                 int32_t *token, void *stream) {
     if (!logits || !uid || !t || !token || R < 1 || V < 1) return SARA_EINVAL;
     return op_guard([&] {
-        launch_cluster(static_cast<cudaStream_t>(stream), false, dim3((unsigned)R * kSampleCtas), dim3(256), 0, kSampleCtas,
-                       sample_rows_kernel, logits, (int)V, sample_seed, uid, t, (int *)token);
+        cudaStream_t s = static_cast<cudaStream_t>(stream);
+        if (V <= kSampleShort) {
+            sample_short_rows_kernel<<<R, 256, 0, s>>>(logits, V, sample_seed, uid, t, token);
+            CK(cudaGetLastError());
+            return;
+        }
+        const int ctas = sample_ctas(R, V, sm_count());
+        launch_cluster(s, false, dim3((unsigned)R * ctas), dim3(256), 0, ctas,
+                       sample_rows_kernel, logits, (int)V, sample_seed, uid, t, (int *)token, ctas);
     });
 }
 

@@ -307,30 +307,68 @@ static __global__ void __launch_bounds__(kCtlThreads, 1) teacher_setup_kernel(St
     }
 }
 
-// Gumbel-max over given fp32 logits (kernel-level entry point): one cluster of kSampleCtas CTAs per
-// row, each a contiguous share of the vocabulary, the row's maximum joined through distributed
-// shared memory.  Bound by instruction issue (a 64-bit hash per token; 51 instructions a token in all),
-// so the noise's logarithms are taken only for tokens that could reach the CTA's best so far
-// (noise_cut), the hash's input is
-// advanced by additions, and a step's logits load during the one before.  64 rows x 151,936, whole
-// call: 277 us with one CTA per row (64 of 152 SMs) and the noise of every token, 37 us with the
-// bound per warp and all of the first step's tokens evaluated, 26 us now (kernel 35.6 -> 25.0).
+// Gumbel-max over given fp32 logits (kernel-level entry point), short vocabularies: one CTA per row, the
+// noise of every token.  Bound by the CTAs' latency chain, where the bounds of sample_rows_kernel cost more than
+// the logarithms they save: 65,536 rows x 512: 148 us against 426, 4,096 x 2,048 29 against 36,
+// 4,096 x 4,096 49 against 47.
+constexpr int kSampleShort = 2048;
+static __global__ void __launch_bounds__(256) sample_short_rows_kernel(const float *logits, int V, uint64_t sample_seed,
+                                                                       const int64_t *uid, const int32_t *t, int *token) {
+    __shared__ float sv[8];
+    __shared__ int si[8];
+    const int r = blockIdx.x;
+    const uint64_t rs = sampler_row_seed(sample_seed, uid[r], t[r]);
+    float best = -INFINITY;
+    int bi = 0x7fffffff;
+    for (int v = threadIdx.x; v < V; v += 256) {
+        const float z = __fadd_rn(logits[(int64_t)r * V + v], gumbel_from_hash(splitmix_at(rs, (uint64_t)v + 1)));
+        if (z > best) { best = z; bi = v; }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ov > best || (ov == best && oi < bi)) { best = ov; bi = oi; }
+    }
+    if ((threadIdx.x & 31) == 0) { sv[threadIdx.x >> 5] = best; si[threadIdx.x >> 5] = bi; }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w)
+            if (sv[w] > best || (sv[w] == best && si[w] < bi)) { best = sv[w]; bi = si[w]; }
+        token[r] = bi;
+    }
+}
+
+// Longer vocabularies: 1 to 8 CTAs per row (sample_ctas, a
+// cluster), each a contiguous share of the vocabulary, the row's maximum joined through distributed
+// shared memory.  Bound by instruction issue (a 64-bit hash per token), so the noise's logarithms are
+// taken only for tokens that could reach the CTA's best so far (noise_cut), the hash's input is
+// advanced by additions, and a step's logits load during the one before.
 constexpr int kSampleCtas = 8;
+// The split doubles while a CTA would still hold more than a thousand tokens and the CTAs fit the SMs at
+// once (8 an SM): a cluster costs ~48 ns of launch, so rows that fill the SMs by themselves take one CTA each
+// and no cluster (4,096 rows x 4,096: 212 us in clusters of 8, 47 without).
+inline int sample_ctas(int R, int V, int sms) {
+    int n = 1;
+    while (n < kSampleCtas && V > 1024 * n && (int64_t)R * 2 * n <= (int64_t)8 * sms) n *= 2;
+    return n;
+}
 static __global__ void __launch_bounds__(256) sample_rows_kernel(const float *logits, int V, uint64_t sample_seed,
-                                                                 const int64_t *uid, const int32_t *t, int *token) {
+                                                                 const int64_t *uid, const int32_t *t, int *token,
+                                                                 int ctas) {
     __shared__ float sv[8];
     __shared__ int si[8];
     __shared__ uint32_t cv[kSampleCtas], ci[kSampleCtas];  // (rank 0) the cluster's maxima
     __shared__ volatile float wb[8];                       // each warp's best so far
-    cluster_arrive();  // (waited for before the store into rank 0's shared memory)
+    if (ctas > 1) cluster_arrive();  // (waited for before the store into rank 0's shared memory)
     if (threadIdx.x < 8) wb[threadIdx.x] = -INFINITY;
     __syncthreads();
-    const int r = blockIdx.x / kSampleCtas, rank = (int)cluster_rank();
+    const int r = blockIdx.x / ctas, rank = (int)(blockIdx.x - (unsigned)r * ctas);
     const uint64_t rs = sampler_row_seed(sample_seed, uid[r], t[r]);
-    // this CTA's share: n tokens from tok0 on (in 32 bits only what stays below 2^28 or V)
-    const int per = ((V - 1) / kSampleCtas + 4) & ~3;
-    const int64_t tok0 = (int64_t)rank * per;
-    const int n = (int)max((int64_t)0, min((int64_t)V - tok0, (int64_t)per));
+    // this CTA's share: n tokens from tok0 on (n < 2^29: rows of more fit no memory in such numbers that
+    // they get one CTA each)
+    const int64_t per = (((int64_t)V - 1) / ctas + 4) & ~(int64_t)3, tok0 = rank * per;
+    const int n = (int)max((int64_t)0, min(V - tok0, per));
     const float *row = logits + (int64_t)r * V + tok0;
     const bool vec = (reinterpret_cast<uintptr_t>(row) & 15) == 0;
     float best = -INFINITY, wbest = -INFINITY;  // this thread's, and the warp's as of the last step
@@ -419,18 +457,23 @@ static __global__ void __launch_bounds__(256) sample_rows_kernel(const float *lo
     }
     if ((threadIdx.x & 31) == 0) { sv[threadIdx.x >> 5] = best; si[threadIdx.x >> 5] = bi; }
     __syncthreads();
-    cluster_wait();  // every CTA of the cluster has started
+    if (ctas > 1) cluster_wait();  // every CTA of the cluster has started
     if (threadIdx.x == 0) {
         for (int w = 1; w < 8; ++w)
             if (sv[w] > best || (sv[w] == best && si[w] < bi)) { best = sv[w]; bi = si[w]; }
-        st_cluster_u32(cluster_addr(&cv[rank], 0), __float_as_uint(best));
-        st_cluster_u32(cluster_addr(&ci[rank], 0), (uint32_t)bi);
+        if (ctas == 1) {
+            token[r] = bi;
+        } else {
+            st_cluster_u32(cluster_addr(&cv[rank], 0), __float_as_uint(best));
+            st_cluster_u32(cluster_addr(&ci[rank], 0), (uint32_t)bi);
+        }
     }
+    if (ctas == 1) return;
     cluster_sync();
     if (rank == 0 && threadIdx.x == 0) {
         best = -INFINITY;
         bi = 0x7fffffff;
-        for (int w = 0; w < kSampleCtas; ++w) {
+        for (int w = 0; w < ctas; ++w) {
             const float ov = __uint_as_float(cv[w]);
             if (ov > best || (ov == best && (int)ci[w] < bi)) { best = ov; bi = (int)ci[w]; }
         }

@@ -51,12 +51,12 @@ def test_sampler_largest_vocabulary(pkg, V):
         logits[0, v] = -np.inf
 
 
-# many rows of few tokens: most CTAs of a cluster have none and reach the join of the maxima at once, while others may
-# not have started
-@pytest.mark.parametrize("V", [1, 3, 40])
-def test_sampler_many_rows_of_few_tokens(pkg, V):
+# many rows of few tokens; the lines between the kernels and of the split: 8, 4, 2 and 1 CTAs a row, the last with few
+# tokens, so that it reaches the join of the maxima at once
+@pytest.mark.parametrize("R,V", [(6000, 1), (6000, 40), (1, 2048), (1, 2049), (1, 4097), (152, 8193), (153, 8193),
+                                 (304, 2049), (305, 2049), (609, 2050)])
+def test_sampler_rows_and_splits(pkg, R, V):
     rng = np.random.default_rng(V)
-    R = 6000
     logits = (rng.standard_normal((R, V)) * 2).astype(np.float32)
     uid, t = np.arange(R, dtype=np.int64), np.zeros(R, np.int32)
     tok = pkg.sample(_dev(logits), _dev(uid), _dev(t), 4).cpu().numpy()
@@ -67,9 +67,18 @@ def test_sampler_many_rows_of_few_tokens(pkg, V):
             assert tok[r] == want, (r, tok[r], want, margin)
 
 
+def test_sampler_most_rows(pkg):
+    # more rows than a grid holds clusters of 8 CTAs
+    import torch
+    R = 2 ** 28 + 5
+    uid, t = torch.arange(R, device="cuda"), torch.zeros(R, dtype=torch.int32, device="cuda")
+    tok = pkg.sample(torch.zeros((R, 1), device="cuda"), uid, t, 4)
+    assert int(tok.min()) == 0 and int(tok.max()) == 0
+
+
 # logits so large that the sum with the noise is rounded (spacing 0.008 to 0.06), equal or nearly so: the token that
 # bounds the others keeps its place, and ties go to the lowest id
-@pytest.mark.parametrize("V", [512, 40003])
+@pytest.mark.parametrize("V", [512, 5000, 40003])
 @pytest.mark.parametrize("mean,std", [(65536.0, 0.0), (65536.0, 1.0), (-65536.0, 1.0), (1e6, 0.0), (1e6, 1.0)])
 def test_sampler_large_logits(pkg, V, mean, std):
     rng = np.random.default_rng(V)
