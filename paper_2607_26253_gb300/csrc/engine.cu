@@ -512,11 +512,13 @@ void run_host_loop(sara_handle &h, int schedule) {
 // ------------------------------------------------------------------------ weights
 
 // A row-major bf16 matrix [n_src][K] (host or device) into chunk-major blocks at dst (a matrix of
-// N rows; rows, row0: see block_weights_kernel).  Host and misaligned sources go through the
-// device staging buffer tmp.
-void block_matrix(cudaStream_t s, const void *src, bool on_device, uint16_t *tmp, uint8_t *dst, int n_src, int K, int N,
-                  int rows = kRowsPlain, int row0 = 0, int head_dim = 0) {
-    if (!on_device || (reinterpret_cast<uintptr_t>(src) & 15)) {
+// N rows; rows, row0: see block_weights_kernel).  Sources that are not aligned memory of this GPU go
+// through the device staging buffer tmp.
+void block_matrix(cudaStream_t s, int device, const void *src, bool on_device, uint16_t *tmp, uint8_t *dst, int n_src,
+                  int K, int N, int rows = kRowsPlain, int row0 = 0, int head_dim = 0) {
+    cudaPointerAttributes attr{};
+    if (on_device) CK(cudaPointerGetAttributes(&attr, src));
+    if (!on_device || !readable_in_place(src, attr, device)) {
         CK(cudaMemcpyAsync(tmp, src, (size_t)n_src * K * 2, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, s));
         src = tmp;
     }
@@ -558,18 +560,18 @@ void load_weights(sara_handle &h, const sara_weights *w) {
     uint16_t *tmp = nullptr;
     if (cudaMalloc(&tmp, stage * 2) != cudaSuccess) throw SaraError(SARA_ENOMEM, "cudaMalloc of the weight staging buffer failed");
     try {
-        block_matrix(s, w->lm_head, dev, tmp, h.wb_lm, V, d, V);
+        block_matrix(s, h.device, w->lm_head, dev, tmp, h.wb_lm, V, d, V);
         for (int l = 0; l < L; ++l) {
             CK(cudaMemcpyAsync(h.norm_attn + (size_t)l * d, w->attn_norm[l], (size_t)d * 2, kind, s));
             CK(cudaMemcpyAsync(h.norm_mlp + (size_t)l * d, w->mlp_norm[l], (size_t)d * 2, kind, s));
             uint8_t *qkv = h.wb_qkv + l * h.ls_qkv, *gu = h.wb_gu + l * h.ls_gu;
-            block_matrix(s, w->wq[l], dev, tmp, qkv, H * hd, d, nqkv, kRowsHead, 0, hd);
-            block_matrix(s, w->wk[l], dev, tmp, qkv, KVH * hd, d, nqkv, kRowsHead, H * hd, hd);
-            block_matrix(s, w->wv[l], dev, tmp, qkv, KVH * hd, d, nqkv, kRowsHead, (H + KVH) * hd, hd);
-            block_matrix(s, w->wo[l], dev, tmp, h.wb_o + l * h.ls_o, d, H * hd, d);
-            block_matrix(s, w->wgate[l], dev, tmp, gu, F, d, 2 * F, kRowsAlt, 0);
-            block_matrix(s, w->wup[l], dev, tmp, gu, F, d, 2 * F, kRowsAlt, 8);
-            block_matrix(s, w->wdown[l], dev, tmp, h.wb_down + l * h.ls_down, d, F, d);
+            block_matrix(s, h.device, w->wq[l], dev, tmp, qkv, H * hd, d, nqkv, kRowsHead, 0, hd);
+            block_matrix(s, h.device, w->wk[l], dev, tmp, qkv, KVH * hd, d, nqkv, kRowsHead, H * hd, hd);
+            block_matrix(s, h.device, w->wv[l], dev, tmp, qkv, KVH * hd, d, nqkv, kRowsHead, (H + KVH) * hd, hd);
+            block_matrix(s, h.device, w->wo[l], dev, tmp, h.wb_o + l * h.ls_o, d, H * hd, d);
+            block_matrix(s, h.device, w->wgate[l], dev, tmp, gu, F, d, 2 * F, kRowsAlt, 0);
+            block_matrix(s, h.device, w->wup[l], dev, tmp, gu, F, d, 2 * F, kRowsAlt, 8);
+            block_matrix(s, h.device, w->wdown[l], dev, tmp, h.wb_down + l * h.ls_down, d, F, d);
         }
         CK(cudaStreamSynchronize(s));
     } catch (...) {

@@ -55,6 +55,12 @@ inline CUtensorMap make_tmap_bf16(const void *base, int inner, int outer, int bo
     return tm;
 }
 
+// Whether a kernel on `device` may read src (attributes a) where it lies, 16 bytes at a time: this GPU's own
+// memory.  Another GPU's would need peer access, which a copy does without.
+inline bool readable_in_place(const void *src, const cudaPointerAttributes &a, int device) {
+    return a.type == cudaMemoryTypeDevice && a.device == device && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
+}
+
 // Launch with thread-block clusters of `cluster` CTAs along x (1: none).  pdl: the kernel may start before
 // the preceding one on the stream has completed (it waits for that itself).
 template <typename Kern, typename... Args>

@@ -4,6 +4,7 @@ import ctypes
 import glob
 import os
 import re
+import subprocess
 
 import pytest
 
@@ -64,3 +65,28 @@ def test_missing_library_fails_loudly(tmp_path):
     import paper_2607_26253_gb300.sara as s
     with pytest.raises(ImportError):
         s.load(str(tmp_path / "libsara.so"))
+
+
+def test_weights_are_read_in_place_only_on_the_handles_gpu(tmp_path):
+    """Aligned memory of the handle's own GPU is read by a kernel where it lies; another GPU's, managed and host memory and
+    misaligned pointers are copied first."""
+    csrc = os.path.join(ROOT, "paper_2607_26253_gb300", "csrc")
+    src = tmp_path / "t.cpp"
+    src.write_text("""
+#include "host_util.h"
+int main() {
+    auto in_place = [](cudaMemoryType type, int gpu, uintptr_t at) {
+        cudaPointerAttributes a{};
+        a.type = type;
+        a.device = gpu;
+        return sara::readable_in_place(reinterpret_cast<const void *>(at), a, 1);
+    };
+    if (!in_place(cudaMemoryTypeDevice, 1, 4096) || in_place(cudaMemoryTypeDevice, 0, 4096)) return 1;
+    if (in_place(cudaMemoryTypeDevice, 1, 4104) || in_place(cudaMemoryTypeHost, 1, 4096)) return 2;
+    if (in_place(cudaMemoryTypeManaged, 1, 4096) || in_place(cudaMemoryTypeUnregistered, 1, 4096)) return 3;
+    return 0;
+}
+""")
+    exe = str(tmp_path / "t")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", csrc, "-I", "/usr/local/cuda/include", str(src), "-o", exe], check=True)
+    assert subprocess.run([exe]).returncode == 0
