@@ -25,7 +25,8 @@ int gemm_rows_sms() {
     int dev = 0, sms = 0;
     CK(cudaGetDevice(&dev));
     if (dev >= 0 && dev < kMaxDevices && (sms = known[dev].load(std::memory_order_acquire)) > 0) return sms;
-    CK(cudaFuncSetAttribute(gemm_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 + kRowsRing));
+    CK(cudaFuncSetAttribute(gemm_rows_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 + kRowsRing));
+    CK(cudaFuncSetAttribute(gemm_rows_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, 1024 + kRowsRing));
     CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     if (dev >= 0 && dev < kMaxDevices) known[dev].store(sms, std::memory_order_release);
     return sms;

@@ -101,9 +101,11 @@ def test_sampler_infinities_and_nan(pkg):
     assert tok[0] == 0x7FFFFFFF and tok[1] == 17 and tok[2] == 3001 and tok[3] % 2 == 1
 
 
-# one tile: K splits 1, 2, 4 and 8, uneven shares; tile counts at which the split halves; more tiles than CTAs
+# one tile: K splits 1, 2, 4 and 8, uneven shares; tile counts at which the split halves, up to 64 rows and above (other
+# CTAs per SM); more tiles than CTAs
 @pytest.mark.parametrize("R,N,K", [(1, 128, 64), (31, 128, 128), (32, 128, 448), (33, 128, 1088), (128, 4864, 640),
-                                   (5, 4992, 640), (64, 9856, 320), (65, 19584, 192), (127, 40064, 192)])
+                                   (5, 4992, 640), (64, 9856, 320), (65, 19584, 192), (127, 40064, 192),
+                                   (65, 128, 704), (97, 1920, 1088), (96, 4352, 640), (72, 9728, 640), (70, 9856, 640)])
 @pytest.mark.parametrize("static", [False, True])
 def test_gemm_splits_and_tile_walks(pkg, R, N, K, static):
     import torch
@@ -116,6 +118,22 @@ def test_gemm_splits_and_tile_walks(pkg, R, N, K, static):
     # fp32 accumulation of exact bf16 products: |error| <= K 2^-23 sum |x w|
     bound = K * 2.0 ** -23 * (np.abs(xf) @ np.abs(wf).T) + 1e-6
     assert (np.abs(Y - xf @ wf.T) <= bound).all()
+
+
+# The tensor core's accumulation truncates: about 1e-9 of the result per element of K in one chain (1.25e-9 allowed), so
+# chains are cut to half of what an even split over the SMs gives one, 64 elements at least; beyond that only the result
+# is rounded (2^-24).
+@pytest.mark.parametrize("R,N,K", [(8, 128, 2368), (100, 256, 4096), (4, 2048, 1536), (128, 2048, 1536), (16, 2048, 11008),
+                                   (15, 1536, 8960), (33, 17920, 1536), (64, 40064, 1536), (128, 40064, 1536), (3, 19584, 9024)])
+def test_gemm_accumulation_chains(pkg, R, N, K):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(N + K)
+    X = torch.randn((R, K), generator=g, device="cuda").bfloat16()
+    W = torch.randn((N, K), generator=g, device="cuda").bfloat16()
+    want = X.double() @ W.double().t()
+    chain = max(1, min(K // 64, N // 128 * (K // 64) // torch.cuda.get_device_properties(0).multi_processor_count) // 2)
+    rel = float((pkg.gemm_bf16(X, W).double() - want).norm() / want.norm())
+    assert rel < 1.25e-9 * 64 * chain + 2.0 ** -24, (rel, chain)
 
 
 # infinite and NaN activations and sums past the largest float: the same results with K split over a cluster and not
