@@ -3,7 +3,7 @@
 // The attention entry point's path for operands that are not 16-byte aligned (attn_split.cuh
 // serves the others).
 //
-// q and the KV cache are fp16; the output is a bf16 hi/lo pair (the next GEMM's operand).
+// q and the KV cache are fp16, the output bf16.
 //
 // Work item = (row, split of `chunk` positions) for one KV head (blockIdx.y): the CTA loads
 // the G = n_heads / n_kv query heads that share the KV head once and streams the split's K
@@ -26,43 +26,25 @@ constexpr int kAttnMaxSplits = 96;  // largest split count the merge handles in 
 
 struct AttnParams {
     const uint16_t *q;        // [rows][n_heads][hd] fp16
-    uint16_t *out;            // [rows][n_heads][hd] bf16 hi
-    uint16_t *out_lo;         // [rows][n_heads][hd] bf16 lo (may be null)
+    uint16_t *out;            // [rows][n_heads][hd] bf16
     const uint16_t *kv;       // slot s at kv + s * slot_stride: [2][n_kv][cap][hd] fp16
     int64_t slot_stride;
     int cap;
     const int *row_slot;      // [rows]
     const int *row_pos;       // [rows] position of the query token (ctx = pos + 1)
     const int2 *items;        // [n_items] (row, split)
-    const int *n_items_dev;   // device item count (nullptr -> n_items_fixed)
-    int n_items_fixed;
+    int n_items;
     const int *row_item0;     // [rows] index of the row's first item
     int n_heads, n_kv, chunk;
     float scale_log2;         // log2(e) / sqrt(hd)
     float *part;              // [items][n_kv][G][hd + 2] fp32 partials (m, l, o[hd])
     int *cnt;                 // [rows][n_kv] arrival counters, zero between launches
-    int *err;
-    uint64_t *stamps;         // optional [blocks][16] phase timestamps (profiling builds)
 };
-
-#ifdef SARA_STAMPS
-#define ATTN_STAMP(i) do { if (p.stamps && threadIdx.x == 0 && blockIdx.y == 0 && blockIdx.x < 152) p.stamps[(size_t)blockIdx.x * 16 + (i)] = globaltimer_ns(); } while (0)
-#else
-#define ATTN_STAMP(i) do { } while (0)
-#endif
 
 __device__ __forceinline__ float2 half2_bits_to_float2(uint32_t w) {
     __half2 h;
     *reinterpret_cast<uint32_t *>(&h) = w;
     return __half22float2(h);
-}
-
-// bf16 hi/lo store of one output element
-__device__ __forceinline__ void attn_store(const AttnParams &p, int64_t idx, float v) {
-    uint16_t hi, lo;
-    split_bf16(v, hi, lo);
-    p.out[idx] = hi;
-    if (p.out_lo) p.out_lo[idx] = lo;
 }
 
 template <int DPL>
@@ -91,19 +73,14 @@ attn_rows_kernel(AttnParams p) {
     __shared__ float s_w[G][kAttnMaxSplits];
     __shared__ int s_last;
 
-    ATTN_STAMP(0);
-    pdl_wait_prior_grids();
-    pdl_allow_dependents();
-    const int n_items = p.n_items_dev ? *p.n_items_dev : p.n_items_fixed;
     const int kvh = blockIdx.y;
-    ATTN_STAMP(1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int half = lane >> 4, dl = lane & 15;
     const int hw = warp * 2 + half;  // half-warp id 0..7
     const unsigned fmask = 0xffffffffu;
     constexpr int kStride = 8 * kAttnPPI;  // positions per CTA iteration
 
-    for (int item = blockIdx.x; item < n_items; item += gridDim.x) {
+    for (int item = blockIdx.x; item < p.n_items; item += gridDim.x) {
         const int2 it = p.items[item];
         const int row = it.x, split = it.y;
         const int ctx = p.row_pos[row] + 1;
@@ -146,7 +123,6 @@ attn_rows_kernel(AttnParams p) {
                 attn_load_words<DPL>(Vb + (int64_t)pc * HD, V[j]);
             }
         };
-        ATTN_STAMP(2);
         if (wstart < p1) load_rows(wstart, kw, vw);
         for (int wbase = wstart; wbase < p1; wbase += kStride) {
             uint32_t nk[kAttnPPI][NW], nv[kAttnPPI][NW];
@@ -204,7 +180,6 @@ attn_rows_kernel(AttnParams p) {
                     for (int i = 0; i < NW; ++i) { kw[j][i] = nk[j][i]; vw[j][i] = nv[j][i]; }
             }
         }
-        ATTN_STAMP(3);
         // merge the 8 half-warp states
 #pragma unroll
         for (int g = 0; g < G; ++g) {
@@ -232,7 +207,7 @@ attn_rows_kernel(AttnParams p) {
 #pragma unroll
                 for (int h = 0; h < 8; ++h)
                     if (s_m[h][g] != -INFINITY) acc += s_o[h][g][d] * exp2f(s_m[h][g] - M);
-                attn_store(p, ((int64_t)row * p.n_heads + kvh * G + g) * HD + d, acc / s_fin_l[g]);
+                p.out[((int64_t)row * p.n_heads + kvh * G + g) * HD + d] = f32_to_bf16(acc / s_fin_l[g]);
             }
         } else {
             float *mine = p.part + ((int64_t)item * p.n_kv + kvh) * G * (HD + 2);
@@ -251,14 +226,12 @@ attn_rows_kernel(AttnParams p) {
             }
             __threadfence();
             __syncthreads();
-            ATTN_STAMP(4);
             if (threadIdx.x == 0) {
                 const int old = atomicAdd(&p.cnt[row * p.n_kv + kvh], 1);
                 s_last = (old == nsplit - 1);
                 if (s_last) p.cnt[row * p.n_kv + kvh] = 0;
             }
             __syncthreads();
-            ATTN_STAMP(5);
             if (s_last) {
                 __threadfence();
                 const int i0 = p.row_item0[row];
@@ -288,14 +261,12 @@ attn_rows_kernel(AttnParams p) {
                     const float *src = base + g * (HD + 2) + 2 + d;
 #pragma unroll 4
                     for (int sp = 0; sp < nsplit; ++sp) acc += s_w[g][sp] * __ldcg(src + sp * sp_stride);
-                    attn_store(p, ((int64_t)row * p.n_heads + kvh * G + g) * HD + d, acc / s_fin_l[g]);
+                    p.out[((int64_t)row * p.n_heads + kvh * G + g) * HD + d] = f32_to_bf16(acc / s_fin_l[g]);
                 }
-                ATTN_STAMP(6);
             }
         }
         __syncthreads();  // shared state reused by the next item
     }
-    ATTN_STAMP(7);
 }
 
 }  // namespace sara

@@ -179,7 +179,6 @@ struct MegaSmem {
     int stall_idx;              // test hook: the phase counter whose waits never complete (-1: none)
     uint32_t tmem_base;
     int abort;
-    int last_flag;
     int rows, rows16, nws, nx, xgroup, xchunk, n_items, att_span;  // nws W slots; nx X stages of xgroup chunks
     GemmPlan plan[5];           // this CTA's share of each GEMM phase (the same for every layer)
     int2 tile_cta[3][kPlanTiles];  // first and last contributor of the tiles of q/k/v, O, down
@@ -201,6 +200,23 @@ struct MegaSmem {
     int last_flag2[2];
 };
 
+// An MMA reads the operand rows of its M whether a chunk holds them or not (they feed accumulator rows that
+// nobody reads): bytes past the last X stage's chunk, at most over the row counts.
+__host__ __device__ constexpr int x_stage_chunks(int rows) { return rows <= 16 ? 4 : rows <= 32 ? 2 : 1; }
+__host__ __device__ constexpr int x_stages(int rows) {
+    const int n = (kRingBytes - ring_slots(rows) * kSlotBytes) / (x_chunk_bytes(rows) * x_stage_chunks(rows));
+    return n < kMaxXStages ? n : kMaxXStages;
+}
+constexpr int x_overread() {
+    int most = 0;
+    for (int rows = 1; rows <= 128; ++rows) {
+        const int operand = rows <= 32 ? 64 * 128 : rows <= 64 ? 128 * 128 : 2 * 128 * 128;
+        const int end = ring_slots(rows) * kSlotBytes + (x_stages(rows) * x_stage_chunks(rows) - 1) * x_chunk_bytes(rows) + operand;
+        most = end - kRingBytes > most ? end - kRingBytes : most;
+    }
+    return most;
+}
+static_assert(x_overread() <= (int)sizeof(MegaSmem), "the operands' don't-care rows stay inside the shared memory");
 constexpr size_t kMegaSmemBytes = 1024 + (size_t)kRingBytes + sizeof(MegaSmem);
 static_assert(kMegaSmemBytes <= 232448, "227 KB of shared memory per CTA");
 
@@ -1762,8 +1778,8 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
         // many as fit after the W slots
         S.nws = ring_slots(rows);
         S.xchunk = x_chunk_bytes(rows);
-        S.xgroup = rows <= 16 ? 4 : rows <= 32 ? 2 : 1;
-        S.nx = min(kMaxXStages, (kRingBytes - S.nws * kSlotBytes) / (S.xchunk * S.xgroup));
+        S.xgroup = x_stage_chunks(rows);
+        S.nx = x_stages(rows);
         S.n_items = *(volatile int *)&V->att_items;
         S.att_span = max(1, *(volatile int *)&V->att_span);
         S.target = (*(volatile unsigned long long *)p.epoch + 1ull) * gridDim.x;
@@ -1779,7 +1795,6 @@ __global__ void __launch_bounds__(kMegaThreads, 1) decode_step_kernel(const __gr
         }
         S.p_headroom = p.c.kc->eager_softmax ? 0.f : kSoftmaxHeadroom;
         S.abort = (*(volatile int *)&V->err & ERR_WAIT_TIMEOUT) != 0;
-        S.last_flag = 0;
         fence_mbar_init();
     }
     if (threadIdx.x == 0) MEGA_STAMP(p.n_stamp_ph - 1, 0);  // kernel start

@@ -203,8 +203,7 @@ int sara_attention_decode(const uint16_t *q, const uint16_t *kv, int64_t kv_stri
         a.row_slot = row_slot;
         a.row_pos = row_pos;
         a.items = items;
-        a.n_items_dev = nullptr;
-        a.n_items_fixed = (int)hitems.size();
+        a.n_items = (int)hitems.size();
         a.row_item0 = row_item0;
         a.n_heads = n_heads;
         a.n_kv = n_kv_heads;
@@ -212,7 +211,6 @@ int sara_attention_decode(const uint16_t *q, const uint16_t *kv, int64_t kv_stri
         a.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)head_dim));
         a.part = part;
         a.cnt = cnt;
-        a.err = nullptr;
         CK(cudaMemsetAsync(cnt, 0, (size_t)b * n_heads * sizeof(int), s));
         dim3 grid(std::max(1, sms * 4 / n_kv_heads), n_kv_heads);
         if (head_dim == 32) launch_g<32>(grid, G, s, a);
