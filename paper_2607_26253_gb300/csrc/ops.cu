@@ -136,6 +136,10 @@ int sara_attention_decode(const uint16_t *q, const uint16_t *kv, int64_t kv_stri
     if (b < 1 || n_kv_heads < 1 || n_heads % n_kv_heads || n_heads / n_kv_heads > kAttnMaxG) return SARA_EINVAL;
     if (head_dim != 32 && head_dim != 64 && head_dim != 128) return SARA_EINVAL;
     if (max_ctx < 1 || max_ctx > cap || (max_ctx + 127) / 128 > kAttnMaxSplits) return SARA_EINVAL;
+    // a row is read in loads of head_dim / 16 elements at least
+    if (((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(kv)) & (head_dim / 8 - 1)) ||
+        (b > 1 && kv_stride % (head_dim / 16)))
+        return SARA_EINVAL;
     return op_guard([&] {
         if (workspace_bytes < sara_attention_workspace_bytes(b, n_heads, head_dim, max_ctx))
             throw SaraError(SARA_EINVAL, "workspace too small");

@@ -205,6 +205,18 @@ def test_attention_unaligned_operands(pkg):
     _check_attention(pkg.attention_decode(off(q), off(kv), _dev(ctx), 2, cap), q, kv, ctx, 2)
 
 
+@pytest.mark.parametrize("hd,elements", [(128, 4), (64, 2), (32, 1)])
+def test_attention_operands_below_their_loads_alignment_refused(pkg, hd, elements):
+    # a head dim's rows are read hd / 16 elements at a time: less alignment is an error, not a fault
+    import torch
+    q = torch.zeros(2 * 4 * hd + 8, dtype=torch.float16, device="cuda")[elements:][:2 * 4 * hd].view(2, 4, hd)
+    kv = torch.zeros((2, 2, 2, 20, hd), dtype=torch.float16, device="cuda")
+    ctx = torch.full((2,), 20, dtype=torch.int32, device="cuda")
+    with pytest.raises(pkg.SaraError) as e:
+        pkg.attention_decode(q, kv, ctx, 2, 20)
+    assert e.value.code == pkg.SARA_EINVAL
+
+
 def test_attention_infinite_value(pkg):
     # an infinite V element reaches the result with its sign, beside exact values in the other dims
     q, kv, ctx, cap = _attention_case(np.random.default_rng(2), 12, 2, 128, [40, 300])
