@@ -303,13 +303,15 @@ SARA_API int sara_gemm_bf16_static(const uint16_t *X, const uint16_t *W, float *
                                    int32_t Nout, int32_t K, void *stream);
 
 /*
- * Attention of b query rows against their own KV ranges (the prefill's attention kernel),
- * one query each (softmax(q K^T / sqrt(hd)) V with grouped-query heads): q [b][n_heads][hd] fp16; kv cache of sequence i at kv + i*kv_stride
+ * Attention of b query rows against their own KV ranges, one query each (softmax(q K^T / sqrt(hd)) V
+ * with grouped-query heads): q [b][n_heads][hd] fp16; kv cache of sequence i at kv + i*kv_stride
  * elements, laid out [2 (K,V)][n_kv_heads][cap][hd] fp16, valid for positions < ctx[i];
- * out [b][n_heads][hd] bf16 (the high part of the step's bf16 hi/lo output pair).  Split over the context in chunks of 128 positions with an
- * fp32 log-sum-exp combine.  hd in {32, 64, 128}; n_heads / n_kv_heads in {1, 2, 4, 6, 8};
- * max_ctx <= 96 * 128.
- * workspace: >= sara_attention_workspace_bytes(b, n_heads, hd, max_ctx), counter area zero.
+ * out [b][n_heads][hd] bf16.  A cluster of up to 8 CTAs shares a (row, KV head)'s positions, with an fp32
+ * log-sum-exp combine.  hd in {32, 64, 128}; n_heads / n_kv_heads in {1, 2, 4, 6, 8};
+ * 1 <= ctx[i] <= max_ctx <= min(cap, 96 * 128), else SARA_EINVAL and out stays as it is.  q and every row of kv
+ * at least hd / 8 bytes aligned (SARA_EINVAL); operands that are not 16-byte aligned take a slower kernel.
+ * workspace: >= sara_attention_workspace_bytes(b, n_heads, hd, max_ctx); its contents do not matter.
+ * The call waits for its own work.
  */
 SARA_API size_t sara_attention_workspace_bytes(int32_t b, int32_t n_heads, int32_t head_dim,
                                                int32_t max_ctx);
@@ -320,7 +322,7 @@ SARA_API int sara_attention_decode(const uint16_t *q, const uint16_t *kv, int64_
                                    void *stream);
 
 /*
- * Temperature-1 sampling by Gumbel-max (the decode step's sampling rule, one CTA per row):
+ * Temperature-1 sampling by Gumbel-max (the decode step's sampling rule; one to eight CTAs per row):
  * token[r] = argmax_v (logits[r][v] + g(r, v)) with
  * g = -log(-log u), u from SplitMix64 keyed by (sample_seed, uid[r], t[r], v), decided in
  * fp32, ties to the lowest index.  logits [R][V] fp32, uid/t/token [R], all device.
