@@ -242,20 +242,6 @@ __device__ __forceinline__ uint64_t sub_f32x2(uint64_t a, uint64_t b) {
     return d;
 }
 
-// s += v, the rounding error and v's own (e) to c (Knuth's two-sum).  Below: two sums at once, without e.
-__device__ __forceinline__ void two_sum(float &s, float &c, float v, float e) {
-    const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
-    c = __fadd_rn(c, __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b))));
-    s = t;
-}
-__device__ __forceinline__ void two_sum(uint64_t &s, uint64_t &c, uint64_t v) {
-    const uint64_t t = add_f32x2(s, v), b = sub_f32x2(t, s);
-    c = add_f32x2(c, add_f32x2(sub_f32x2(s, sub_f32x2(t, b)), sub_f32x2(v, b)));
-    s = t;
-}
-// The sum; an infinite or NaN one has no error term.
-__device__ __forceinline__ float sum_of(float s, float c) { return isfinite(s) ? __fadd_rn(s, c) : s; }
-
 // 1-D bulk copy global -> shared memory, completing `bytes` on `bar`; both addresses 16-byte
 // aligned and `bytes` a multiple of 16.
 __device__ __forceinline__ void bulk_load(void *smem_dst, const void *src, uint32_t bytes, uint64_t *bar,

@@ -53,6 +53,20 @@ struct GemmRowsSmem {
 __host__ __device__ inline int gemm_rows_stage(int R) {
     return kRowsTileM * 128 + (R + kRowsBox - 1) / kRowsBox * kRowsBox * 128;
 }
+// s += v, the rounding error and v's own (e) to c.  Below: two sums at once, without e.
+__device__ __forceinline__ void two_sum(float &s, float &c, float v, float e) {
+    const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
+    c = __fadd_rn(c, __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b))));
+    s = t;
+}
+__device__ __forceinline__ void two_sum(uint64_t &s, uint64_t &c, uint64_t v) {
+    const uint64_t t = add_f32x2(s, v), b = sub_f32x2(t, s);
+    c = add_f32x2(c, add_f32x2(sub_f32x2(s, sub_f32x2(t, b)), sub_f32x2(v, b)));
+    s = t;
+}
+// The sum; an infinite or NaN one has no error term.
+__device__ __forceinline__ float sum_of(float s, float c) { return isfinite(s) ? __fadd_rn(s, c) : s; }
+
 template <int C>
 __global__ void __launch_bounds__(kRowsThreads, 2)
 gemm_rows_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmX, GemmRowsParams p) {

@@ -227,9 +227,8 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
                     if (whole) {
                         tmem_ld_32x32b_x32(tmem + lane_base + (uint32_t)(a * kBigCols + half * 128 + cc * 32), v);
                     } else {
-                        float err[32];  // the sums' rounding errors: cutting a tile adds none of its own
 #pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = err[e] = 0.f;
+                        for (int e = 0; e < 32; ++e) v[e] = 0.f;
 #pragma unroll 1
                         for (int c = ca; c <= cb; c += 2) {  // in CTA order, two contributors' loads in flight
                             const int off = (half * 128 + cc * 32) * kBigRows + lrow;
@@ -241,13 +240,8 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
 #pragma unroll
                             for (int e = 0; e < 32; ++e) w1[e] = c < cb ? __ldcg(s1 + e * kBigRows) : 0.f;
 #pragma unroll
-                            for (int e = 0; e < 32; ++e) {
-                                two_sum(v[e], err[e], w0[e], 0.f);
-                                two_sum(v[e], err[e], w1[e], 0.f);
-                            }
+                            for (int e = 0; e < 32; ++e) v[e] = (v[e] + w0[e]) + w1[e];
                         }
-#pragma unroll
-                        for (int e = 0; e < 32; ++e) v[e] = sum_of(v[e], err[e]);
                     }
                     if (!live) continue;
                     const int n = n0 + cc * 32;
