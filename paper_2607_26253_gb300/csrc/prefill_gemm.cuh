@@ -23,10 +23,10 @@ namespace sara {
 // Up to kPrefillFewRows rows a model with long reductions (more than kPrefillFewChunks chunks) runs the
 // few-row GEMM (gemm_tc.cuh) instead: there the finishing CTA's sum of the contributors' partial
 // tiles weighs more than the units.  A 5-layer prefill and decode step, few-row / this kernel, ms:
-// 1.5B shape, 32 rows 0.80 / 0.83, 64 rows 0.96 / 0.88, 255 rows 1.42 / 1.10, 16,320 rows 19.2 /
-// 11.1; 3B shape, 32 rows 0.92 / 0.96, 16,320 rows 31.3 / 17.7; 8 chunks (2 layers, d 128), 1 row
-// 0.70 / 0.32, 16,320 rows 1.70 / 0.74.
-constexpr int kPrefillFewRows = 32, kPrefillFewChunks = 16;
+// 1.5B shape, 32 rows 0.79 / 0.94, 48 rows 0.92 / 0.96, 64 rows 0.95 / 0.98, 96 rows 1.12 / 1.05, 255 rows 1.39 /
+// 1.14, 16,320 rows 18.4 / 11.0; 3B shape, 32 rows 0.91 / 1.00, 48 rows 1.04 / 1.02, 64 rows 1.08 / 1.04, 16,320
+// rows 30.9 / 17.4; 8 chunks (2 layers, d 128), 1 row 0.27 / 0.23, 16,320 rows 0.57 / 0.29.
+constexpr int kPrefillFewRows = 48, kPrefillFewChunks = 16;
 constexpr int kBigThreads = 320;
 constexpr int kBigRows = 128, kBigCols = 256, kBigStages = 3;
 constexpr int kBigStage = kBigCols * 128 + 2 * kBigRows * 128;  // 64 KB
@@ -71,9 +71,14 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_consta
     const int64_t U = (int64_t)nt * ((rows + kBigRows - 1) / kBigRows) * kch;
     // At most one CTA per unit, so that every CTA between a tile's first and last contributes; with
     // few tiles fewer, so that the time of a CTA's units (~0.5 us each) and of summing a tile's
-    // contributors (~1.4 us each) balance.
+    // contributors (~1.4 us each) balance, but half of the grid at least: the tensor core's accumulation
+    // truncates along a chain, about 1e-9 of the result per element of K, and a CTA's units of a tile are one;
+    // half of the grid makes it as long as an even split of 128 x 128 tiles over all of it does.  Relative
+    // error against 64 bits and time, with and without that: 80 x 2,048 x 2,048 4.9e-7, 38.7 us / 1.19e-6,
+    // 32.9; 255 x 1,536 x 1,536 5.2e-7, 48.3 / 1.10e-6, 41.4; from 300 rows on it changes nothing.
     const int tiles = nt * ((rows + kBigRows - 1) / kBigRows);
-    const int G = (int)min64(min64(gridDim.x, U > 0 ? U : 1), max(tiles, (int)sqrtf(0.37f * (float)U * (float)tiles) + 1));
+    const int G = (int)min64(min64(gridDim.x, U > 0 ? U : 1),
+                             max(max(tiles, (int)(gridDim.x + 1) / 2), (int)sqrtf(0.37f * (float)U * (float)tiles) + 1));
     const int64_t u0 = cta < G ? unit_begin(cta, U, G) : 0, u1 = cta < G ? unit_begin(cta + 1, U, G) : 0;
     volatile int *ab = &S.abort;
 
