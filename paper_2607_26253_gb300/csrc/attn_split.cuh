@@ -13,8 +13,8 @@
 //     probability, times infinity.  A warp whose sums are not all finite takes them again in fp32.
 // Online softmax per warp; the warps' states meet in shared memory, the CTAs' in distributed
 // shared memory (no workspace, no counters, so no work list from the host either).  26 ragged rows
-// of median context 758, 12 heads / 2 KV heads of 128, whole call with its synchronisation: 46 us;
-// 91 us with scalar products over a work list that the host built from the copied contexts.
+// of median context 758, 12 heads / 2 KV heads of 128, whole call with its synchronisation: 45 to 50 us (kernel 18,
+// caches cold); 89 to 97 us with scalar products over a work list that the host built from the copied contexts.
 #pragma once
 #include "device_common.cuh"
 #include "host_util.h"
