@@ -1,9 +1,8 @@
 """GPU check of sara_gemm_bf16_static, the GEMM entry point that allocates nothing.
 
 Some callers cannot allocate device memory themselves (their framework's pool owns the
-GPU, or their interface only passes inputs and outputs); this entry point keeps its scratch
-in a fixed array inside the library.  The test calls it twice in a row through the C ABI
-(the second call must not be disturbed by what the first left in the shared scratch) and
+GPU, or their interface only passes inputs and outputs); this entry point needs no scratch.
+The test calls it twice in a row through the C ABI and
 compares both results with sara_gemm_bf16, which takes a caller workspace, within the fp32
 accumulation bound the GEMM tests use.  This file is collected last on purpose.
 """
